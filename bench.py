@@ -285,9 +285,9 @@ def launches_per_step(w, precision):
         # (then reduce and finish): kernel (0, 1); shadow copy + screening kernel (2, 4); BF16 copy, tensor-core
         # tiles, SIMT leftovers (3)
         return 3 if precision < 2 else (4 if precision in (2, 4) or w.d > 128 else 5)
-    # refine: run count, scan, run clusters, then cluster-sorted copy + Gram + exact recompute + merge (tensor
-    # cores) or the two FP32 tile widths
-    ref = 1 + 3 + 1 + (4 if tc_refine(precision, w.d, w.storage) else 2)
+    # refine: the run lists, then cluster-sorted copy + Gram + exact recompute + merge (tensor cores) or the two FP32
+    # tile widths (runs of max_cluster = 128 members at most)
+    ref = 1 + (4 if tc_refine(precision, w.d, w.storage) else 2)
     graph = 1 + 1 + grp(w.k0) + upd + w.tau * (asg(w.k0) + grp(w.k0) + upd + ref)
     fit = 1 + grp(w.k) + upd + w.iters * (asg(w.k) + grp(w.k) + upd)
     return graph + fit

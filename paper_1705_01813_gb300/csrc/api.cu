@@ -107,6 +107,7 @@ struct Layout {
     int32_t *labels_b;
     float *cent;
     double *elog;
+    int32_t *prev[2];  // BUILD: each sample's run in the last two refinements
     size_t bytes;
 };
 
@@ -138,6 +139,8 @@ Layout carve(void *ws, int op, int64_t n, int64_t d, int32_t k)
     if (op == GK_OP_BUILD) {
         L.labels_a = cv.take<int32_t>((size_t)n);
         L.cent = cv.take<float>((size_t)k * (size_t)d);
+        L.prev[0] = cv.take<int32_t>((size_t)n);
+        L.prev[1] = cv.take<int32_t>((size_t)n);
     }
     if (op == GK_OP_RECALL)  // k: the number of queries
         L.rec_scratch = cv.take<char>(recall_scratch_bytes(n, k));
@@ -717,7 +720,8 @@ static int build_knn_graph_impl(const void *X, bool bf16, int64_t n, int64_t d, 
                                   L.elog + 2 + 2 * t, L.upd_scratch, L.st, s));
             // exhaustive pairs inside the clusters of the new partition
             GK_CUDA(launch_refine(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k0, p->kappa, p->max_cluster, g_idx,
-                                  g_dist, L.ref_scratch, L.st, s, p->precision & 0xff));
+                                  g_dist, L.ref_scratch, L.st, s, p->precision & 0xff, t > 0 ? L.prev[(t + 1) & 1] : nullptr,
+                                  L.prev[t & 1], true));
             int32_t *tmp = cur;
             cur = nxt;
             nxt = tmp;
@@ -849,7 +853,8 @@ static int batch_fit_impl(const void *X, bool bf16, int64_t d, int64_t ld, int32
             GK_CUDA(launch_update(X, bf16, N, d, ld, L.grp.offsets, L.grp.members, bd.K0, L.cent, L.grp.counts,
                                   nullptr, L.upd_scratch, L.st, s));
             GK_CUDA(launch_refine(X, bf16, N, d, ld, L.grp.offsets, L.grp.members, bd.K0, p->kappa, p->max_cluster,
-                                  g_idx, g_dist, L.ref_scratch, L.st, s, p->precision & 0xff));
+                                  g_idx, g_dist, L.ref_scratch, L.st, s, p->precision & 0xff, t > 0 ? L.prev[(t + 1) & 1] : nullptr,
+                                  L.prev[t & 1], true));
             int32_t *tmp = cur;
             cur = nxt;
             nxt = tmp;

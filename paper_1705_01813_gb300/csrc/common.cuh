@@ -271,15 +271,23 @@ cudaError_t launch_assign(const void *X, bool bf16, int64_t n, int64_t d, int64_
 
 void set_last_error(const char *msg);
 
+// Runs listed for a refinement (refine.cu): at most `split` members (a), longer (b), and inexact tensor-core runs (x).
+struct RunCounts {
+    int a, b, x, pad;
+};
 size_t refine_scratch_bytes(int64_t n, int32_t k, int64_t d);
-// precision 0: FP32 pair distances on the SIMT cores; 1: tensor-core Gram with exact FP32 rerank
+// precision 0: FP32 pair distances on the SIMT cores; 1: tensor-core Gram with exact FP32 rerank.  prev_in, prev_out
+// (n each, distinct; NULL: not kept): the run of every sample in the previous refinement of the same graph, whose
+// pairs are not compared again, and in this one.  canon: every distance in the graph has the bits that the library
+// computes for the pair (a graph that init_graph and refinements made), see merge.cuh.
 cudaError_t launch_refine(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                           const int32_t *members, int32_t k, int32_t kappa, int32_t max_cluster, int32_t *g_idx,
-                          float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision);
+                          float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision,
+                          const int32_t *prev_in = nullptr, int32_t *prev_out = nullptr, bool canon = false);
 size_t refine_tc_scratch_bytes(int64_t n, int32_t k, int64_t d);
-cudaError_t launch_refine_tc(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
-                             const int32_t *members, const int32_t *run_off, const int32_t *run_cl, int32_t k,
-                             int32_t kappa, int32_t max_cluster, int64_t grid, int32_t *g_idx, float *g_dist,
-                             void *scratch, DevStatus *st, cudaStream_t s);
+cudaError_t launch_refine_tc(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *members,
+                             const int2 *runs, RunCounts *cnt, int64_t bound, int32_t k, int32_t kappa,
+                             const int32_t *prev, bool canon, int32_t *g_idx, float *g_dist, void *scratch,
+                             DevStatus *st, cudaStream_t s);
 
 }  // namespace gkm

@@ -4,11 +4,16 @@
 //
 // A cluster of m members (CSR, ascending id) larger than max_cluster is cut
 // into ceil(m / max_cluster) runs of consecutive members whose sizes differ by
-// at most one; pairs are formed inside a run only.  One block per cluster (the
-// hardware hands clusters to SMs as blocks finish, which balances uneven
-// cluster sizes).  Two instances of the kernel run back to back: a 64-wide
-// tile for clusters whose runs hold at most 64 members (the common case, small
-// shared memory, several blocks per SM) and a 128-wide tile for the others.
+// at most one; pairs are formed inside a run only.  k_refine_plan lists the
+// runs; within a graph construction it leaves out those whose members all were
+// in one run in the previous round, and the kernels below compare only pairs
+// that were not: such a pair has been offered to both rows, and a kappa-th key
+// only decreases, so it can neither be missing nor enter again (after the first
+// round 1-67% of the pairs are new on the workloads' data; the refinements of a
+// graph construction at 2M x 512 BF16 go from 62.1 to 16.4 ms, at 200k x 960
+// FP32 from 16.3 to 12.9, at 1.3M x 64 in 16 jobs from 20.0 to 13.0).  Blocks walk the
+// lists grid-stride: a 64-wide tile for runs of at most 64 members (the common
+// case, several blocks per SM) and a 128-wide tile for longer ones.
 // A run is covered by T x T tiles (rows x columns of the run); for each tile
 // the block stages 32 coordinates of the row and column samples at a time in
 // shared memory (the row samples twice over, as broadcast pairs) and every
@@ -17,12 +22,7 @@
 // difference as fma(y, -1, x), then fma(e, e, acc): per pair the operations of
 // pair_d2_seq), with one accumulator in ascending coordinate order, so a
 // pair's distance has the same bits here, in the initial graph and in any
-// later round.  Each
-// warp then merges the tile's candidates into the graph rows of its rows:
-// candidates that beat the row's kappa-th key and are not already in the row
-// are compacted, ranked among themselves, located in the row by binary
-// search (all on 64-bit packed keys), and the kappa smallest keys of the union
-// are written back.  Every
+// later round.  Each warp then merges the tile's distances into the graph rows of its rows (merge.cuh).  Every
 // row belongs to exactly one run per refinement, so blocks never write the
 // same row.
 #include "common.cuh"
@@ -33,111 +33,252 @@
 
 namespace gkm {
 
-// Cluster of every run: run_cl[run_off[r] + c] = r for c < nruns[r].
-__global__ void k_run_clusters(const int32_t *__restrict__ run_off, int k, int32_t *__restrict__ run_cl)
-{
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < k; r += gridDim.x * blockDim.x)
-        for (int q = run_off[r]; q < run_off[r + 1]; q++)
-            run_cl[q] = r;
-}
+// The runs of a refinement: int2 records {first position in the grouping, members}.  One array holds the runs of at
+// most `split` members from its front (RunCounts::a of them) and the longer ones from its back (RunCounts::b).  A run
+// whose members all shared one run in the previous refinement has no pair left to compare and is not listed.
+constexpr int PL_WARPS = 8;
 
-// Runs of each cluster: ceil(m / cap) for m >= 2, else none.
-__global__ void k_count_runs(const int32_t *__restrict__ off, int k, int cap, int32_t *__restrict__ nruns)
+// One warp per `chunk` clusters (at most 32); the runs of a cluster that is cut are shared out over the block's warps
+// (the SIFT- and GIST-shaped graphs grow clusters of thousands, 40 and 65 us a round with one warp each).  prev_in
+// (may be NULL) and prev_out (may be NULL): per sample the run it
+// belonged to in the previous and in this refinement, named by the run's first position; -1 for none.  The order in
+// which runs are listed varies from call to call and decides nothing but which block takes a run.  This one kernel
+// replaces counting the runs, scanning the counts and mapping runs to clusters (five launches, about 12 us a round).
+__global__ void __launch_bounds__(PL_WARPS * 32) k_refine_plan(const int32_t *__restrict__ off,
+                                                               const int32_t *__restrict__ mem, int64_t n, int k,
+                                                               int cap, int split, int chunk,
+                                                               const int32_t *__restrict__ prev_in,
+                                                               int32_t *__restrict__ prev_out, int2 *__restrict__ runs,
+                                                               int64_t runs_cap, RunCounts *__restrict__ cnt)
 {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < k; r += gridDim.x * blockDim.x) {
-        int m = off[r + 1] - off[r];
-        nruns[r] = m >= 2 ? (m + cap - 1) / cap : 0;
+    __shared__ int s_ncut;
+    __shared__ int2 s_cut[PL_WARPS * 32];  // {first member position, members} of the block's cut clusters
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    if (threadIdx.x == 0)
+        s_ncut = 0;
+    __syncthreads();
+    const int64_t c0 = ((int64_t)blockIdx.x * PL_WARPS + w) * chunk;
+    const int nq = (int)max((int64_t)0, min((int64_t)chunk, k - c0));
+    int my_beg = 0, my_m = 0;
+    if (lane < nq) {
+        my_beg = off[c0 + lane];
+        my_m = off[c0 + lane + 1] - my_beg;
+        if (my_m > cap) {
+            s_cut[atomicAdd(&s_ncut, 1)] = make_int2(my_beg, my_m);
+            my_m = 0;
+        }
+    }
+    // records the run of the members first .. first + sz - 1 in prev_out; has it a pair that was not compared before?
+    auto visit = [&](int first, int sz) -> bool {
+        bool same = prev_in != nullptr;
+        if (same || prev_out) {
+            int ref = -1;
+#pragma unroll 2
+            for (int t0 = 0; t0 < sz; t0 += 32) {
+                const int t = t0 + lane;
+                const int a = t < sz ? mem[first + t] : -1;
+                const bool in = (unsigned)a < (unsigned)n;
+                const int p = prev_in && in ? prev_in[a] : -1;
+                if (t0 == 0)
+                    ref = __shfl_sync(FULL_MASK, p, 0);
+                same = same && (t >= sz || (p == ref && p >= 0));
+                if (prev_out && in)
+                    prev_out[a] = sz >= 2 ? first : -1;
+            }
+            same = __all_sync(FULL_MASK, same);
+        }
+        return sz >= 2 && !same;
+    };
+    int2 rec = make_int2(0, 0);
+    // the lanes' records into the two lists, one atomic per list
+    auto append = [&]() {
+        const unsigned la = __ballot_sync(FULL_MASK, rec.y > 0 && rec.y <= split);
+        const unsigned lb = __ballot_sync(FULL_MASK, rec.y > split);
+        int ba = 0, bb = 0;
+        if (lane == 0) {
+            if (la)
+                ba = atomicAdd(&cnt->a, __popc(la));
+            if (lb)
+                bb = atomicAdd(&cnt->b, __popc(lb));
+        }
+        ba = __shfl_sync(FULL_MASK, ba, 0);
+        bb = __shfl_sync(FULL_MASK, bb, 0);
+        if (rec.y > split)
+            runs[runs_cap - 1 - (bb + __popc(lb & lanemask_lt()))] = rec;
+        else if (rec.y > 0)
+            runs[ba + __popc(la & lanemask_lt())] = rec;
+        rec = make_int2(0, 0);
+    };
+    for (int q = 0; q < nq; q++) {
+        const int beg = __shfl_sync(FULL_MASK, my_beg, q), m = __shfl_sync(FULL_MASK, my_m, q);
+        if (m > 0 && visit(beg, m) && lane == q)
+            rec = make_int2(beg, m);
+    }
+    append();
+    __syncthreads();
+    const int ncut = s_ncut;
+    for (int z = 0; z < ncut; z++) {
+        const int beg = s_cut[z].x, m = s_cut[z].y;
+        const int nc = (m + cap - 1) / cap, base = m / nc, rem = m % nc;
+        for (int b0 = 0; b0 < nc; b0 += PL_WARPS * 32) {
+            for (int q = 0; q < 32; q++) {
+                const int c = b0 + q * PL_WARPS + w;
+                if (c >= nc)
+                    break;
+                const int first = beg + c * base + min(c, rem), sz = base + (c < rem ? 1 : 0);
+                if (visit(first, sz) && lane == q)
+                    rec = make_int2(first, sz);
+            }
+            append();
+        }
     }
 }
 
-template <int T, typename XT, bool VEC>
-__global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT *__restrict__ X, int64_t n, int d, int64_t ld,
-                                                       const int32_t *__restrict__ off,
-                                                       const int32_t *__restrict__ mem,
-                                                       const int32_t *__restrict__ run_off,
-                                                       const int32_t *__restrict__ run_cl, int k, int kappa,
-                                                       int cap, int lo_run, int32_t *__restrict__ g_idx,
-                                                       float *__restrict__ g_dist, DevStatus *st)
+// Dynamic shared memory of k_refine: the stage buffers (the distance tile aliases them), ids and previous runs of the
+// rows and columns, the members before they are sorted (a second id and run array), the list of blocks to compute.
+template <int T>
+__host__ __device__ constexpr size_t refine_smem_bytes()
 {
     using TL = RefineTile<T>;
-    constexpr int DS = TL::DS;
+    return sizeof(float) * (TL::stage_floats > TL::tile_floats ? TL::stage_floats : TL::tile_floats) +
+           sizeof(int) * 6 * T + T + sizeof(unsigned short) * ((TL::NBLK + 3) & ~3) + sizeof(int) * RF_WARPS +
+           sizeof(MergeBuf<T / 32>) * RF_WARPS;
+}
+
+// The members of a run of sz <= T samples, read by the threads t < T of a group: ids (-1 for a corrupt entry, which is
+// recorded, and past the end) and previous runs, in member order or, with prev, sorted by (previous run, member
+// order), so that members that were together before are neighbours.  sid gets the ids in member order (ascending) and
+// smap each one's place in rid (with prev only; else rid is in that order); spr: T entries of scratch.
+template <int T, typename Sync>
+__device__ __forceinline__ void load_members(const int32_t *__restrict__ S, int sz, int64_t n,
+                                             const int32_t *__restrict__ prev, int *rid, int *rpr, int *sid,
+                                             unsigned char *smap, int *spr, int t, int first, DevStatus *st, Sync sync)
+{
+    int a = -1, p = -1;
+    if (t < T) {
+        a = t < sz ? S[t] : -1;
+        if (a >= n) {  // corrupt grouping: record, skip the sample
+            flag_error(st, GK_ERR_INVALID, (unsigned)first);
+            a = -1;
+        }
+        if (prev && a >= 0)
+            p = prev[a];
+        sid[t] = a;
+        if (!prev || t >= sz) {
+            rid[t] = a;
+            rpr[t] = -1;
+        }
+    }
+    if (prev) {
+        if (t < T)
+            spr[t] = p;
+        sync();
+        if (t < sz) {
+            int r = 0;
+            for (int q = 0; q < sz; q++)
+                r += (spr[q] < p || (spr[q] == p && q < t)) ? 1 : 0;
+            rid[r] = a;
+            rpr[r] = p;
+            smap[t] = (unsigned char)r;
+        }
+    }
+    sync();
+}
+
+// Listed runs blockIdx.x, + gridDim.x, ... (LONG: the list from the back of the array), T-wide tiles.
+template <int T, typename XT, bool VEC>
+__global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT *__restrict__ X, int64_t n, int d,
+                                                                        int64_t ld, const int32_t *__restrict__ mem,
+                                                                        const int2 *__restrict__ runs,
+                                                                        int64_t runs_cap,
+                                                                        const RunCounts *__restrict__ cnt, bool longs,
+                                                                        const int32_t *__restrict__ prev, bool canon, int kappa,
+                                                                        int32_t *__restrict__ g_idx,
+                                                                        float *__restrict__ g_dist, DevStatus *st)
+{
+    using TL = RefineTile<T>;
+    constexpr int DS = TL::DS, NC = T / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *xr = reinterpret_cast<float *>(smem_raw);  // staging buffers of the pair tiles (tiles.cuh)
     float *dt = xr;  // aliases the staging buffers
     constexpr size_t span = TL::stage_floats > TL::tile_floats ? TL::stage_floats : TL::tile_floats;
     int *rid = reinterpret_cast<int *>(xr + span);
-    int *cid = rid + T;
+    int *cid = rid + T, *rpr = cid + T, *cpr = rpr + T, *sid = cpr + T, *spr = sid + T;
+    int *wcnt = spr + T;
     const int tid = threadIdx.x, w = tid >> 5;
-    unsigned char *wbase = reinterpret_cast<unsigned char *>(cid + T) + w * TL::warp_bytes(kappa);
-    uint64_t *rk = reinterpret_cast<uint64_t *>(wbase);
-    uint64_t *nk = rk + kappa;
-    uint64_t *bk = nk + kappa;
-    unsigned *dup = reinterpret_cast<unsigned *>(bk + T);
-
-    // block `run` handles that run: find its cluster r, run_off[r] <= run < run_off[r + 1]
-    const int run = blockIdx.x;
-    if (run >= run_off[k])
-        return;
-    const int r = run_cl[run];
-    const int beg = off[r], m = off[r + 1] - beg;
-    const int nc = (m + cap - 1) / cap, base = m / nc, rem = m % nc;
-    const int c = run - run_off[r];
-    const int s0 = c * base + min(c, rem), sz = base + (c < rem ? 1 : 0);
-    // the 64-wide instance (lo_run = 0) takes runs of <= 64 members, the
-    // 128-wide instance (lo_run = 64) all longer runs
-    const bool mine = lo_run == 0 ? sz <= T : sz > lo_run;
-    if (!mine || sz < 2)
-        return;
-    {
-        const int32_t *S = mem + beg + s0;
+    MergeBuf<NC> &mb = reinterpret_cast<MergeBuf<NC> *>(wcnt + RF_WARPS)[w];
+    unsigned char *smap = reinterpret_cast<unsigned char *>(reinterpret_cast<MergeBuf<NC> *>(wcnt + RF_WARPS) + RF_WARPS);
+    unsigned short *list = reinterpret_cast<unsigned short *>(smap + T);
+    auto sync = [] { __syncthreads(); };
+    const int nrun = longs ? cnt->b : cnt->a;
+    for (int run = blockIdx.x; run < nrun; run += gridDim.x) {
+        const int2 rec = longs ? runs[runs_cap - 1 - run] : runs[run];
+        const int first = rec.x, sz = rec.y;
+        const int32_t *S = mem + first;
+        // the merges of the rows of one tile
+        auto merge_rows = [&](int nr, int ncl, const int *ci, const int *cp, const int *si, const unsigned char *sm) {
+            RowRegs cur, nxt;
+            if (w < nr && rid[w] >= 0)
+                load_row(cur, g_idx + (int64_t)rid[w] * kappa, g_dist + (int64_t)rid[w] * kappa, kappa);
+            for (int row = w; row < nr; row += RF_WARPS) {
+                const int i = rid[row];
+                const int rn = row + RF_WARPS;
+                if (rn < nr && rid[rn] >= 0)  // next row's list in flight during this merge
+                    load_row(nxt, g_idx + (int64_t)rid[rn] * kappa, g_dist + (int64_t)rid[rn] * kappa, kappa);
+                if (i >= 0)
+                    merge_row<NC>(i, rpr[row], canon, ci, cp, si, sm, dt + row * DS, ncl, kappa, cur,
+                                  g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mb);
+                cur = nxt;
+            }
+        };
+        __syncthreads();  // the previous run's merges are done
+        if (sz <= T) {
+            load_members<T>(S, sz, n, prev, rid, rpr, sid, smap, spr, tid, first, st, sync);
+            const int nlive = live_blocks<T, RF_THREADS>(sz, prev ? rpr : nullptr, list, wcnt, tid, sync);
+            // the arithmetic goes to the block's warps rot, rot + 1, ... (rot = blockIdx.x % 4): each warp of an SM
+            // issues on scheduler (its index % 4), so blocks that share an SM spread their few busy warps over all
+            // four schedulers instead of all starting at scheduler 0
+            const int t = (tid - (int)(blockIdx.x & 3) * 32) & (RF_THREADS - 1);
+            const int code = t < nlive ? list[t] : 0;
+            tile_distances<T, true, VEC>(X, d, ld, rid, rid, code >> 8, code & 255, t < nlive, xr, dt);
+            __syncthreads();
+            merge_rows(sz, sz, rid, rpr, sid, prev ? smap : nullptr);
+            continue;
+        }
         for (int rb = 0; rb < sz; rb += T) {
             const int nr = min(T, sz - rb);
             for (int cb = 0; cb < sz; cb += T) {
                 const int ncl = min(T, sz - cb);
-                const bool same = rb == cb;
                 __syncthreads();
                 for (int q = tid; q < T; q += RF_THREADS) {
                     int a = q < nr ? S[rb + q] : -1;
                     int b = q < ncl ? S[cb + q] : -1;
                     if (a >= n || b >= n) {  // corrupt grouping: record, skip the sample
-                        flag_error(st, GK_ERR_INVALID, (unsigned)r);
+                        flag_error(st, GK_ERR_INVALID, (unsigned)first);
                         a = a >= n ? -1 : a;
                         b = b >= n ? -1 : b;
                     }
                     rid[q] = a;
                     cid[q] = b;
+                    rpr[q] = prev && a >= 0 ? prev[a] : -1;
+                    cpr[q] = prev && b >= 0 ? prev[b] : -1;
                 }
                 __syncthreads();
-                if (same)
-                    tile_distances<T, true, VEC>(X, d, ld, rid, cid, nr, xr, dt);
-                else
-                    tile_distances<T, false, VEC>(X, d, ld, rid, cid, nr, xr, dt);
+                tile_distances<T, false, VEC>(X, d, ld, rid, cid, tid >> 4, tid & 15, TL::Q * (tid >> 4) < nr, xr, dt);
                 __syncthreads();
-                RowRegs cur, nxt;
-                if (w < nr && rid[w] >= 0)
-                    load_row(cur, g_idx + (int64_t)rid[w] * kappa, g_dist + (int64_t)rid[w] * kappa, kappa);
-                for (int row = w; row < nr; row += RF_WARPS) {
-                    const int i = rid[row];
-                    const int rn = row + RF_WARPS;
-                    if (rn < nr && rid[rn] >= 0)  // next row's list in flight during this merge
-                        load_row(nxt, g_idx + (int64_t)rid[rn] * kappa, g_dist + (int64_t)rid[rn] * kappa, kappa);
-                    if (i >= 0)
-                        merge_row(i, cid, dt + row * DS, ncl, kappa, cur, g_idx + (int64_t)i * kappa,
-                                  g_dist + (int64_t)i * kappa, rk, bk, nk, dup);
-                    cur = nxt;
-                }
+                merge_rows(nr, ncl, cid, cpr, cid, nullptr);
             }
         }
     }
 }
 
-// Runs of at most 64 members, warp-specialised: a persistent block takes runs blockIdx.x, + gridDim.x, ...; five
+// Listed runs of at most 64 members, warp-specialised: a persistent block takes runs blockIdx.x, + gridDim.x, ...; five
 // of its nine warps (the compute group, WS_NC threads, rotated over the block's warps by blockIdx.x so that the
 // blocks of an SM spread them over its four schedulers) stage and compute a run's pair tile while the other four
 // merge the previous run's rows.  The two hand the distance tile over through named barriers: FULL (the compute group
 // arrives when the tile and the run's ids are written, the merge warps wait) and EMPTY (the merge warps arrive
 // when they no longer read it, the compute group waits before writing the next one).  Both sides walk the same
-// runs with the same skips, so the barriers pair up: per run one FULL and one EMPTY phase, plus the EMPTY phase
+// list, so the barriers pair up: per run one FULL and one EMPTY phase, plus the EMPTY phase
 // the merge warps open before the first run and the compute group closes after the last.  Pair arithmetic,
 // merge order and results are those of k_refine<64>.
 constexpr int WS_NC = 160;  // compute group: 5 warps, covers the 136 pair blocks of a 64-row triangle
@@ -145,20 +286,22 @@ constexpr int WS_NM = 4;    // merge warps
 constexpr int WS_THREADS = WS_NC + 32 * WS_NM;
 constexpr int WS_BAR_C = 1, WS_BAR_FULL = 2, WS_BAR_EMPTY = 3;
 
-// dynamic shared memory: two stage buffers, the distance tile, the run ids of two runs, the merge warps' buffers
-__host__ __device__ inline size_t refine_ws_smem_bytes(int kappa)
+// dynamic shared memory: two stage buffers, the distance tile, two runs' members (ids and previous runs, ids in
+// member order and their places), scratch of the sort, the merge warps' buffers, the list of blocks to compute
+__host__ __device__ constexpr size_t refine_ws_smem_bytes()
 {
     using TL = RefineTile<64>;
-    return sizeof(float) * (TL::stage_floats + TL::tile_floats) + sizeof(int) * 2 * 64 + WS_NM * TL::warp_bytes(kappa);
+    return sizeof(float) * (TL::stage_floats + TL::tile_floats) + sizeof(int) * 7 * 64 + 2 * 64 +
+           sizeof(int) * 8 + sizeof(MergeBuf<2>) * WS_NM + sizeof(unsigned short) * ((TL::NBLK + 3) & ~3);
 }
 
 template <typename XT, bool VEC>
 __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restrict__ X, int64_t n, int d, int64_t ld,
-                                                             const int32_t *__restrict__ off,
                                                              const int32_t *__restrict__ mem,
-                                                             const int32_t *__restrict__ run_off,
-                                                             const int32_t *__restrict__ run_cl, int k, int kappa,
-                                                             int cap, int32_t *__restrict__ g_idx,
+                                                             const int2 *__restrict__ runs,
+                                                             const RunCounts *__restrict__ cnt,
+                                                             const int32_t *__restrict__ prev, bool canon, int kappa,
+                                                             int32_t *__restrict__ g_idx,
                                                              float *__restrict__ g_dist, DevStatus *st)
 {
     constexpr int T = 64;
@@ -169,41 +312,31 @@ __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restric
     float *stage = reinterpret_cast<float *>(smem_raw);
     float *dt = stage + TL::stage_floats;
     int *rids = reinterpret_cast<int *>(dt + TL::tile_floats);  // [2][T]: the ids of runs j and j + 1
-    unsigned char *mbase = reinterpret_cast<unsigned char *>(rids + 2 * T);
+    int *rprs = rids + 2 * T;                                   // [2][T]: their previous runs
+    int *sids = rprs + 2 * T;                                   // [2][T]: the ids in member order
+    int *spr = sids + 2 * T, *wcnt = spr + T;
+    MergeBuf<2> *mbufs = reinterpret_cast<MergeBuf<2> *>(wcnt + 8);
+    unsigned char *smaps = reinterpret_cast<unsigned char *>(mbufs + WS_NM);  // [2][T]: and their places
+    unsigned short *list = reinterpret_cast<unsigned short *>(smaps + 2 * T);
     const int w = threadIdx.x >> 5, lane = lane_id();
     const int rr = (w + WARPS - (int)(blockIdx.x & 3)) % WARPS;  // 0 .. 4: compute group, 5 .. 8: merge warps
-    const int nruns = run_off[k];
-    // run `run`: its cluster, first member (in mem) and size, as k_refine cuts clusters into runs
-    auto geometry = [&](int run, int &r, int &first, int &sz) {
-        r = run_cl[run];
-        const int beg = off[r], m = off[r + 1] - beg;
-        const int nc = (m + cap - 1) / cap, base = m / nc, rem = m % nc;
-        const int c = run - run_off[r];
-        first = beg + c * base + min(c, rem);
-        sz = base + (c < rem ? 1 : 0);
-    };
+    const int nrun = cnt->a;
     if (rr < 5) {
         // ---- compute group ----
         const int ct = rr * 32 + lane;
+        auto sync = [] { bar_sync(WS_BAR_C, WS_NC); };
         int j = 0;
-        for (int run = blockIdx.x; run < nruns; run += gridDim.x) {
-            int r, first, sz;
-            geometry(run, r, first, sz);
-            if (sz < 2 || sz > T)
-                continue;  // a run of the 128-wide kernel, or no pairs: skipped alike by the merge warps
-            int *rid = rids + (j & 1) * T;
-            if (ct < T) {
-                int a = ct < sz ? mem[first + ct] : -1;
-                if (a >= n) {  // corrupt grouping: record, skip the sample
-                    flag_error(st, GK_ERR_INVALID, (unsigned)r);
-                    a = -1;
-                }
-                rid[ct] = a;  // the merges of run j - 2, which read this slot, ended before EMPTY of run j - 1
-            }
-            bar_sync(WS_BAR_C, WS_NC);
+        for (int run = blockIdx.x; run < nrun; run += gridDim.x) {
+            const int2 rec = runs[run];
+            // the merges of run j - 2, which read this slot, ended before EMPTY of run j - 1
+            int *rid = rids + (j & 1) * T, *rpr = rprs + (j & 1) * T;
+            load_members<T>(mem + rec.x, rec.y, n, prev, rid, rpr, sids + (j & 1) * T, smaps + (j & 1) * T, spr, ct, rec.x,
+                            st, sync);
+            const int nlive = live_blocks<T, WS_NC>(rec.y, prev ? rpr : nullptr, list, wcnt, ct, sync);
+            const bool live = ct < nlive;
+            const int code = live ? list[ct] : 0, by = code >> 8, bx = code & 255;
             float2 acc[Q][Q / 2];
-            int by, bx;
-            const bool live = tile_distances_group<WS_NC, VEC>(X, d, ld, rid, sz, stage, ct, WS_BAR_C, acc, by, bx);
+            tile_distances_group<WS_NC, VEC>(X, d, ld, rid, by, bx, live, stage, ct, WS_BAR_C, acc);
             bar_sync(WS_BAR_EMPTY, WS_THREADS);  // the merge warps no longer read the distance tile
             if (live) {
 #pragma unroll
@@ -226,19 +359,13 @@ __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restric
     } else {
         // ---- merge warps ----
         const int mw = rr - 5;
-        unsigned char *wb = mbase + mw * TL::warp_bytes(kappa);
-        uint64_t *rk = reinterpret_cast<uint64_t *>(wb);
-        uint64_t *nk = rk + kappa;
-        uint64_t *bk = nk + kappa;
-        unsigned *dup = reinterpret_cast<unsigned *>(bk + T);
         bar_arrive(WS_BAR_EMPTY, WS_THREADS);  // the distance tile starts free
         int j = 0;
-        for (int run = blockIdx.x; run < nruns; run += gridDim.x) {
-            int r, first, sz;
-            geometry(run, r, first, sz);
-            if (sz < 2 || sz > T)
-                continue;
-            const int *rid = rids + (j & 1) * T;
+        for (int run = blockIdx.x; run < nrun; run += gridDim.x) {
+            const int sz = runs[run].y;
+            const int *rid = rids + (j & 1) * T, *rpr = rprs + (j & 1) * T;
+            const int *sid = sids + (j & 1) * T;
+            const unsigned char *smap = prev ? smaps + (j & 1) * T : nullptr;
             bar_sync(WS_BAR_FULL, WS_THREADS);  // run j's ids and distances
             RowRegs cur, nxt;
             if (mw < sz && rid[mw] >= 0)
@@ -249,8 +376,8 @@ __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restric
                 if (rn < sz && rid[rn] >= 0)  // next row's list in flight during this merge
                     load_row(nxt, g_idx + (int64_t)rid[rn] * kappa, g_dist + (int64_t)rid[rn] * kappa, kappa);
                 if (i >= 0)
-                    merge_row(i, rid, dt + row * DS, sz, kappa, cur, g_idx + (int64_t)i * kappa,
-                              g_dist + (int64_t)i * kappa, rk, bk, nk, dup);
+                    merge_row<T / 32>(i, rpr[row], canon, rid, rpr, sid, smap, dt + row * DS, sz, kappa, cur,
+                                      g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mbufs[mw]);
                 cur = nxt;
             }
             __threadfence_block();
@@ -260,44 +387,26 @@ __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restric
     }
 }
 
-static size_t run_bytes(int32_t k) { return ((size_t)(2 * (k + 1)) * sizeof(int32_t) + 255) / 256 * 256; }
-// runs per refinement are at most k + n / max_cluster (max_cluster >= 2)
-static size_t run_cl_bytes(int64_t n, int32_t k) { return ((size_t)(k + n / 2 + 1) * sizeof(int32_t) + 255) / 256 * 256; }
+// runs per refinement: sum over clusters of ceil(m / max_cluster), at most k + n / max_cluster (max_cluster >= 2)
+static int64_t max_runs(int64_t n, int32_t k) { return (int64_t)k + n / 2 + 1; }
+static size_t runs_bytes(int64_t n, int32_t k) { return ((size_t)max_runs(n, k) * sizeof(int2) + 255) / 256 * 256; }
 
 size_t refine_scratch_bytes(int64_t n, int32_t k, int64_t d)
 {
-    return run_bytes(k) + run_cl_bytes(n, k) + scan_scratch_bytes(k) + refine_tc_scratch_bytes(n, k, d);
+    return 256 + runs_bytes(n, k) + refine_tc_scratch_bytes(n, k, d);
 }
 
 template <typename XT, bool VEC>
 static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
-                            const int32_t *members, int32_t k, int32_t kappa, int32_t max_cluster, int32_t *g_idx,
-                            float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision)
+                             const int32_t *members, int32_t k, int32_t kappa, int32_t max_cluster, int32_t *g_idx,
+                             float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision,
+                             const int32_t *prev_in, int32_t *prev_out, bool canon)
 {
-    int32_t *nruns = static_cast<int32_t *>(scratch);
-    int32_t *run_off = nruns + (k + 1);
-    int32_t *run_cl = reinterpret_cast<int32_t *>(static_cast<char *>(scratch) + run_bytes(k));
-    void *sc = static_cast<char *>(scratch) + run_bytes(k) + run_cl_bytes(n, k);
-    void *tc_scratch = static_cast<char *>(sc) + scan_scratch_bytes(k);
-    const size_t shm64 = RefineTile<64>::smem_bytes(kappa), shm128 = RefineTile<128>::smem_bytes(kappa),
-                 shm_ws = refine_ws_smem_bytes(kappa);
+    RunCounts *cnt = static_cast<RunCounts *>(scratch);
+    int2 *runs = reinterpret_cast<int2 *>(static_cast<char *>(scratch) + 256);
+    void *tc_scratch = static_cast<char *>(scratch) + 256 + runs_bytes(n, k);
+    const int64_t runs_cap = max_runs(n, k);
     cudaError_t e;
-    if constexpr (VEC)
-        e = set_max_smem(reinterpret_cast<const void *>(k_refine_ws<XT, VEC>), (int)refine_ws_smem_bytes(MAX_KAPPA));
-    else
-        e = set_max_smem(reinterpret_cast<const void *>(k_refine<64, XT, VEC>),
-                         (int)RefineTile<64>::smem_bytes(MAX_KAPPA));
-    if (e != cudaSuccess)
-        return e;
-    if ((e = set_max_smem(reinterpret_cast<const void *>(k_refine<128, XT, VEC>),
-                          (int)RefineTile<128>::smem_bytes(MAX_KAPPA))) != cudaSuccess)
-        return e;
-    k_count_runs<<<(k + 255) / 256 < 1024 ? (k + 255) / 256 : 1024, 256, 0, s>>>(offsets, k, max_cluster, nruns);
-    if ((e = launch_scan(nruns, run_off, k, sc, s)) != cudaSuccess)
-        return e;
-    k_run_clusters<<<(k + 255) / 256 < 1024 ? (k + 255) / 256 : 1024, 256, 0, s>>>(run_off, k, run_cl);
-    // an upper bound of the number of runs: sum over clusters of (m / cap + 1)
-    const int64_t grid = (int64_t)k + n / max_cluster + 1;
     // The tensor-core path for 64 <= d <= 128.  Its Gram is exact only for integer data with 2 d 255^2 < 2^24
     // (d <= 128), and wider rows made the recompute of every kept pair dearer than the FP32 tile kernels
     // (1M x 960 FP32: 91 ms against 25 ms per call; 10M x 512 BF16 unit vectors, whose Gram carries no BF16
@@ -305,38 +414,55 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
     // tile kernels'
     // cost, proportional to d, is below the fixed per-run cost of the Gram path (20k x 32: 0.18 ms against
     // 0.12 ms per call).
-    if (precision >= 1 && d >= 64 && d <= 128) {
-        // tensor-core Gram for runs of <= 128 members, the FP32 kernel for longer runs
-        constexpr bool bf16 = std::is_same_v<XT, __nv_bfloat16>;
-        if ((e = launch_refine_tc(X, bf16, n, d, ld, offsets, members, run_off, run_cl, k, kappa, max_cluster, grid,
-                                  g_idx, g_dist, tc_scratch, st, s)) != cudaSuccess)
+    const bool tensor = precision >= 1 && d >= 64 && d <= 128;
+    const int split = tensor ? 128 : 64;
+    if ((e = cudaMemsetAsync(cnt, 0, sizeof(RunCounts), s)) != cudaSuccess)
+        return e;
+    // clusters per warp: enough warps to fill the chip first, then fewer atomics on the list counters
+    const int64_t per = k / (152 * 32);
+    const int chunk = per < 1 ? 1 : per > 32 ? 32 : (int)per;
+    const int64_t pblocks = ((int64_t)k + (int64_t)chunk * PL_WARPS - 1) / ((int64_t)chunk * PL_WARPS);
+    k_refine_plan<<<(unsigned)pblocks, PL_WARPS * 32, 0, s>>>(offsets, members, n, k, max_cluster, split, chunk, prev_in,
+                                                              prev_out, runs, runs_cap, cnt);
+    // an upper bound of the number of runs: sum over clusters of (m / cap + 1)
+    const int64_t bound = (int64_t)k + n / max_cluster + 1;
+    auto blocks = [&](int resident) { return (unsigned)(bound < resident ? bound : resident); };
+    int grid = 0;
+    // runs of more than `split` members (FP32 tiles of 128; longer runs in several tiles)
+    if (max_cluster > split) {
+        constexpr size_t shm = refine_smem_bytes<128>();
+        const void *f = reinterpret_cast<const void *>(k_refine<128, XT, VEC>);
+        if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, RF_THREADS, shm, &grid)) != cudaSuccess)
             return e;
-        if (max_cluster > 128)
-            k_refine<128, XT, VEC><<<(unsigned)grid, RF_THREADS, shm128, s>>>(X, n, (int)d, ld, offsets, members, run_off,
-                                                                     run_cl, k, kappa, max_cluster, 128, g_idx,
-                                                                     g_dist, st);
-        return cudaGetLastError();
+        k_refine<128, XT, VEC><<<blocks(grid), RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, true,
+                                                                     prev_in, canon, kappa, g_idx, g_dist, st);
     }
-    // runs of <= 64 members, then the longer runs (up to 128 per tile, longer runs in tiles).  Rows staged by
+    if (tensor) {
+        // tensor-core Gram for runs of <= 128 members
+        constexpr bool bf16 = std::is_same_v<XT, __nv_bfloat16>;
+        return launch_refine_tc(X, bf16, n, d, ld, members, runs, cnt, bound, k, kappa, prev_in, canon, g_idx, g_dist, tc_scratch,
+                                st, s);
+    }
+    // runs of <= 64 members.  Rows staged by
     // 16-byte loads take the persistent warp-specialised kernel (one wave of blocks; 10M x 512 BF16: 32.0 ->
-    // 31.3 ms per call, 98 -> 75 ms for runs of about ten); rows staged element by element keep the block per
-    // run, where five warps' share of the element loads made the specialised form slower (1M x 960 FP32: 7.6
+    // 31.3 ms per call, 98 -> 75 ms for runs of about ten); rows staged element by element keep the plain block,
+    // where five warps' share of the element loads made the specialised form slower (1M x 960 FP32: 7.6
     // against 7.7 ms; 1M x 128 FP32: 3.7 against 3.9 ms)
     if constexpr (VEC) {
-        int wgrid = 0;
-        if ((e = resident_grid(reinterpret_cast<const void *>(k_refine_ws<XT, VEC>), WS_THREADS, shm_ws, &wgrid)) !=
-            cudaSuccess)
+        constexpr size_t shm = refine_ws_smem_bytes();
+        const void *f = reinterpret_cast<const void *>(k_refine_ws<XT, VEC>);
+        if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, WS_THREADS, shm, &grid)) != cudaSuccess)
             return e;
-        k_refine_ws<XT, VEC><<<(unsigned)(grid < wgrid ? grid : wgrid), WS_THREADS, shm_ws, s>>>(
-            X, n, (int)d, ld, offsets, members, run_off, run_cl, k, kappa, max_cluster, g_idx, g_dist, st);
+        k_refine_ws<XT, VEC><<<blocks(grid), WS_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, cnt, prev_in, canon, kappa,
+                                                                   g_idx, g_dist, st);
     } else {
-        (void)shm_ws;
-        k_refine<64, XT, VEC><<<(unsigned)grid, RF_THREADS, shm64, s>>>(X, n, (int)d, ld, offsets, members, run_off,
-                                                                        run_cl, k, kappa, max_cluster, 0, g_idx,
-                                                                        g_dist, st);
+        constexpr size_t shm = refine_smem_bytes<64>();
+        const void *f = reinterpret_cast<const void *>(k_refine<64, XT, VEC>);
+        if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, RF_THREADS, shm, &grid)) != cudaSuccess)
+            return e;
+        k_refine<64, XT, VEC><<<blocks(grid), RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, false,
+                                                                    prev_in, canon, kappa, g_idx, g_dist, st);
     }
-    k_refine<128, XT, VEC><<<(unsigned)grid, RF_THREADS, shm128, s>>>(X, n, (int)d, ld, offsets, members, run_off, run_cl, k,
-                                                             kappa, max_cluster, 64, g_idx, g_dist, st);
     return cudaGetLastError();
 }
 
@@ -345,24 +471,26 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
 template <typename XT>
 static cudaError_t refine_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                             const int32_t *members, int32_t k, int32_t kappa, int32_t max_cluster, int32_t *g_idx,
-                            float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision)
+                            float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision,
+                            const int32_t *prev_in, int32_t *prev_out, bool canon)
 {
     if (std::is_same_v<XT, __nv_bfloat16> && tile_vec16(X, (int)d, ld))
         return refine_tv<XT, true>(X, n, d, ld, offsets, members, k, kappa, max_cluster, g_idx, g_dist, scratch, st, s,
-                                   precision);
+                                   precision, prev_in, prev_out, canon);
     return refine_tv<XT, false>(X, n, d, ld, offsets, members, k, kappa, max_cluster, g_idx, g_dist, scratch, st, s,
-                                precision);
+                                precision, prev_in, prev_out, canon);
 }
 
 cudaError_t launch_refine(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                           const int32_t *members, int32_t k, int32_t kappa, int32_t max_cluster, int32_t *g_idx,
-                          float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision)
+                          float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision,
+                          const int32_t *prev_in, int32_t *prev_out, bool canon)
 {
     if (bf16)
         return refine_t(static_cast<const __nv_bfloat16 *>(X), n, d, ld, offsets, members, k, kappa, max_cluster,
-                        g_idx, g_dist, scratch, st, s, precision);
+                        g_idx, g_dist, scratch, st, s, precision, prev_in, prev_out, canon);
     return refine_t(static_cast<const float *>(X), n, d, ld, offsets, members, k, kappa, max_cluster, g_idx, g_dist,
-                    scratch, st, s, precision);
+                    scratch, st, s, precision, prev_in, prev_out, canon);
 }
 
 }  // namespace gkm

@@ -31,9 +31,12 @@
 // marked (recorded by its column in the run instead of its id), and the run is
 // flagged.
 //
-// k_refine_exact, one CTA per flagged run: the run's FP32 rows are staged in
+// k_refine_exact, over the listed inexact runs: the run's FP32 rows are staged in
 // shared memory once and every marked pair is recomputed exactly in the order
 // of pair_d2_seq, in place.
+//
+// Pairs that shared a run in the previous refinement of the same graph (prev)
+// are left out (refine.cu says why).
 //
 // k_refine_merge, one warp per graph row that received candidates: the
 // candidates are merged into the row as in the FP32 path (merge.cuh).  Rows
@@ -64,7 +67,7 @@ constexpr unsigned TC_RERANK = 0x80000000u;  // candidate id flag: distance need
 constexpr size_t TC_STAGE = (size_t)TC_KCH * TC_KB_BYTES;
 constexpr size_t TC_BUF = (size_t)2 * TC_M * 32 * sizeof(int);  // ids and distances of one 32-column chunk
 static_assert(TC_BUF <= TC_STAGE, "the epilogue's candidate buffers reuse the staging area");
-constexpr size_t TC_SMEM = 1024 /*alignment slack*/ + TC_STAGE + sizeof(float) * TC_M + sizeof(int) * TC_M * 3 + 64;
+constexpr size_t TC_SMEM = 1024 /*alignment slack*/ + TC_STAGE + sizeof(float) * TC_M * 2 + sizeof(int) * TC_M * 4 + 64;
 
 // Columns of a row of the cluster-sorted copy: d rounded up to 8 (16-byte rows for the tensor map).
 static int64_t perm_cols(int64_t d) { return (d + 7) & ~int64_t(7); }
@@ -74,35 +77,19 @@ static int64_t perm_cols(int64_t d) { return (d + 7) & ~int64_t(7); }
 // their m-th entries, and a warp reading one row, touch 32 distinct banks.
 __device__ __forceinline__ int buf_slot(int r, int m) { return r * 32 + (m ^ (r & 31)); }
 
-// The run of block `run`: its cluster r, first member position p0 (in members / Xp) and size sz.
-__device__ __forceinline__ void run_range(int run, const int32_t *__restrict__ off, const int32_t *__restrict__ run_off,
-                                          const int32_t *__restrict__ run_cl, int cap, int *p0, int *sz, int *r)
-{
-    *r = run_cl[run];
-    const int beg = off[*r], m = off[*r + 1] - beg;
-    const int nc = (m + cap - 1) / cap, rbase = m / nc, rem = m % nc;
-    const int c = run - run_off[*r];
-    *p0 = beg + c * rbase + min(c, rem);
-    *sz = rbase + (c < rem ? 1 : 0);
-}
-
 template <typename XT>
 __global__ void __launch_bounds__(TC_THREADS) k_refine_perm(const XT *__restrict__ X, int64_t n, int d, int64_t ld,
-                                                            const int32_t *__restrict__ off,
                                                             const int32_t *__restrict__ mem,
-                                                            const int32_t *__restrict__ run_off,
-                                                            const int32_t *__restrict__ run_cl, int k, int cap,
-                                                            int dp, __nv_bfloat16 *__restrict__ Xp,
+                                                            const int2 *__restrict__ runs,
+                                                            RunCounts *__restrict__ cnt, int dp,
+                                                            __nv_bfloat16 *__restrict__ Xp,
                                                             float *__restrict__ pnrm, int32_t *__restrict__ run_flags,
-                                                            DevStatus *st)
+                                                            int32_t *__restrict__ inexact_runs, DevStatus *st)
 {
     const int run = blockIdx.x;
-    if (run >= run_off[k])
+    if (run >= cnt->a)
         return;
-    int p0, sz, r;
-    run_range(run, off, run_off, run_cl, cap, &p0, &sz, &r);
-    if (sz < 2 || sz > TC_M)  // no pairs, or a run of the FP32 kernel
-        return;
+    const int p0 = runs[run].x, sz = runs[run].y;
     const int tid = threadIdx.x, w = tid >> 5, lane = lane_id();
     // BF16 samples are copied as they are: their values, products and the Gram's accumulation carry no BF16
     // rounding (centring would round the differences)
@@ -116,7 +103,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_perm(const XT *__restrict
         int a = mem[p];
         if ((unsigned)a >= (unsigned)n) {
             if (lane == 0)
-                flag_error(st, GK_ERR_INVALID, (unsigned)r);
+                flag_error(st, GK_ERR_INVALID, (unsigned)p0);
             a = -1;
         }
         float part = 0.f;
@@ -157,22 +144,27 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_perm(const XT *__restrict
             pnrm[p] = part;
     }
     const int any_inexact = __syncthreads_or(inexact ? 1 : 0), any_lossy = __syncthreads_or(lossy ? 1 : 0);
-    if (tid == 0)
-        run_flags[run] = (any_inexact ? 1 : 0) | (any_lossy ? 2 : 0);
+    if (tid == 0) {
+        // integer run with |x| <= 255: exact only while 2 d 255^2 < 2^24
+        const bool exact = !any_inexact && 2.0 * d * 255.0 * 255.0 < 16777216.0;
+        run_flags[run] = (exact ? 0 : 1) | (any_lossy ? 2 : 0);
+        if (!exact)
+            inexact_runs[atomicAdd(&cnt->x, 1)] = run;  // k_refine_exact recomputes its marked pairs
+    }
 }
 
 __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constant__ CUtensorMap tmap, int64_t n,
-                                                            int d, const int32_t *__restrict__ off,
-                                                            const int32_t *__restrict__ mem,
-                                                            const int32_t *__restrict__ run_off,
-                                                            const int32_t *__restrict__ run_cl, int k, int kappa,
-                                                            int cap, const int32_t *__restrict__ g_idx,
+                                                            int d, const int32_t *__restrict__ mem,
+                                                            const int2 *__restrict__ runs,
+                                                            const RunCounts *__restrict__ cnt,
+                                                            const int32_t *__restrict__ prev, int kappa,
+                                                            const int32_t *__restrict__ g_idx,
                                                             const float *__restrict__ g_dist,
                                                             const float *__restrict__ pnrm,
                                                             const int32_t *__restrict__ run_flags,
                                                             int32_t *__restrict__ cand_id,
                                                             float *__restrict__ cand_d, int32_t *__restrict__ cand_n,
-                                                            int32_t *__restrict__ run_tag, DevStatus *st)
+                                                            DevStatus *st)
 {
     extern __shared__ unsigned char smem_raw[];
     unsigned char *stage = reinterpret_cast<unsigned char *>(
@@ -181,17 +173,16 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
     int *rid = reinterpret_cast<int *>(nrm + TC_M);
     int *bcnt = rid + TC_M;   // candidates of each row in the current chunk
     int *btot = bcnt + TC_M;  // candidates of each row written so far
-    uint64_t *bar = reinterpret_cast<uint64_t *>(btot + TC_M);  // [0] the tile's copies, [1] the MMAs
+    int *rpr = btot + TC_M;   // previous run of each row
+    float *srt = reinterpret_cast<float *>(rpr + TC_M);         // square roots of nrm
+    uint64_t *bar = reinterpret_cast<uint64_t *>(srt + TC_M);  // [0] the tile's copies, [1] the MMAs
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bar + 2);
     const int tid = threadIdx.x, w = tid >> 5, lane = lane_id();
 
     const int run = blockIdx.x;
-    if (run >= run_off[k])
+    if (run >= cnt->a)
         return;
-    int p0, sz, r;
-    run_range(run, off, run_off, run_cl, cap, &p0, &sz, &r);
-    if (sz < 2 || sz > TC_M)  // longer runs (max_cluster > 128) go to the FP32 kernel
-        return;
+    const int p0 = runs[run].x, sz = runs[run].y;
     const int N = (sz + 15) & ~15;
     const uint32_t ncols = sz <= 32 ? 32u : sz <= 64 ? 64u : 128u;
     const int nkb = (d + TC_KB - 1) / TC_KB;
@@ -212,11 +203,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
     // this thread's graph row, its kappa-th key and its norm, while the tile is in flight
     int gi_row = tid < sz ? mem[p0 + tid] : -1;
     if (gi_row >= n) {
-        flag_error(st, GK_ERR_INVALID, (unsigned)r);
+        flag_error(st, GK_ERR_INVALID, (unsigned)p0);
         gi_row = -1;
     }
     rid[tid] = gi_row;
-    nrm[tid] = tid < sz ? pnrm[p0 + tid] : 0.f;
+    const int my_prev = prev && gi_row >= 0 ? prev[gi_row] : -1;
+    rpr[tid] = my_prev;
+    srt[tid] = tid < sz ? sqrtf(pnrm[p0 + tid]) : 0.f;
+    nrm[tid] = tid < sz ? pnrm[p0 + tid] : __int_as_float(0x7f800000);  // no distance to a column past the run passes
     float thd = 0.f;
     int thi = 0;
     if (gi_row >= 0) {
@@ -269,10 +263,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
             tc::tmem_dealloc(taddr, ncols);
         return;
     }
-    // integer run with |x| <= 255: exact only while 2 d 255^2 < 2^24
-    const bool exact = (rf & 1) == 0 && 2.0 * d * 255.0 * 255.0 < 16777216.0;
-    if (tid == 0)
-        run_tag[run] = exact ? 0 : 1;  // k_refine_exact recomputes the marked pairs of this run
+    const bool exact = (rf & 1) == 0;
 
     // ---- candidates of row tid (TMEM lane tid), 32 columns at a time ----
     // Each thread collects its row's candidates of the chunk in shared memory
@@ -282,13 +273,16 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
     float *bdv = reinterpret_cast<float *>(bid + TC_M * 32);
     const bool rows_here = 32 * w < sz;  // warp-uniform
     const int row = tid;
-    const float n_i = nrm[row];
+    const float n_i = nrm[row], s_i = sqrtf(n_i);
+    // a column of the row's own previous run is left out: a code no column has when there is none
+    const int skip = my_prev >= 0 ? my_prev : -2;
     const float u = 1.0f / 256.0f;
     const float rnd = (rf & 2) != 0 ? 4.f * u + 2.f * u * u : 0.f;  // BF16 rounding of the operands
     // accumulation of G: exact products, each 16-deep step aligned to its largest term and truncated (an
     // error below 16 units of 2^-23 of the step's terms), over d / 16 steps, doubled by the factor 2 of
-    // 2 G and once more as a margin
-    const float c1 = 1.02f * (rnd + 8.f * (d + 2) * 5.9604645e-8f);
+    // 2 G and once more as a margin.  The factor 1.02 covers the rounding of the bound's own terms (|x_t| |x_j| is
+    // a product of two rounded square roots).
+    const float c1 = 1.02f * (rnd + 8.f * (d + 2) * 5.9604645e-8f) * s_i;
     const float c2 = 1.02f * (d + 8) * 1.1920929e-7f;
     btot[tid] = 0;
     for (int c0 = 0; c0 < N; c0 += 32) {
@@ -298,26 +292,44 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
             tc::tmem_ld32(taddr + ((uint32_t)(32 * w) << 16) + (uint32_t)c0, g);
             tc::tmem_ld_wait();
             if (gi_row >= 0) {
+                auto keep = [&](int j, float d2, unsigned tag) {
+                    const int jid = rid[j];
+                    // exact: the whole key decides; a marked pair records the run column of j (k_refine_exact
+                    // writes the id back)
+                    if (j != row && jid >= 0 && (tag || key_less(d2, jid, thd, thi))) {
+                        bid[buf_slot(row, m)] = tag ? (int)(TC_RERANK | (unsigned)j) : jid;
+                        bdv[buf_slot(row, m)] = d2;
+                        m++;
+                    }
+                };
+                if (exact) {
 #pragma unroll
-                for (int q = 0; q < 32; q++) {
-                    const int j = c0 + q;
-                    if (j < sz && j != row) {
-                        const int jid = rid[j];
-                        const float d2 = (n_i + nrm[j]) - 2.f * g[q];
-                        bool keep;
-                        unsigned tag = 0;
-                        if (exact) {
-                            keep = key_less(d2, jid, thd, thi);
-                        } else {
-                            const float e = c1 * sqrtf(n_i * nrm[j]) + c2 * (n_i + nrm[j]);
-                            keep = d2 - e <= thd;
-                            tag = TC_RERANK;
+                    for (int q4 = 0; q4 < 32; q4 += 4) {
+                        const float4 nj = *reinterpret_cast<const float4 *>(nrm + c0 + q4);
+                        const int4 pj = *reinterpret_cast<const int4 *>(rpr + c0 + q4);
+                        const float nn[4] = {nj.x, nj.y, nj.z, nj.w};
+                        const int pp[4] = {pj.x, pj.y, pj.z, pj.w};
+#pragma unroll
+                        for (int e = 0; e < 4; e++) {
+                            const float d2 = (n_i + nn[e]) - 2.f * g[q4 + e];
+                            if (d2 <= thd && pp[e] != skip)
+                                keep(c0 + q4 + e, d2, 0u);
                         }
-                        if (keep && jid >= 0) {
-                            // a marked pair records the run column of j (k_refine_exact writes the id back)
-                            bid[buf_slot(row, m)] = tag ? (int)(TC_RERANK | (unsigned)j) : jid;
-                            bdv[buf_slot(row, m)] = d2;
-                            m++;
+                    }
+                } else {
+#pragma unroll
+                    for (int q4 = 0; q4 < 32; q4 += 4) {
+                        const float4 nj = *reinterpret_cast<const float4 *>(nrm + c0 + q4);
+                        const float4 sj = *reinterpret_cast<const float4 *>(srt + c0 + q4);
+                        const int4 pj = *reinterpret_cast<const int4 *>(rpr + c0 + q4);
+                        const float nn[4] = {nj.x, nj.y, nj.z, nj.w}, ss[4] = {sj.x, sj.y, sj.z, sj.w};
+                        const int pp[4] = {pj.x, pj.y, pj.z, pj.w};
+#pragma unroll
+                        for (int e = 0; e < 4; e++) {
+                            const float d2 = (n_i + nn[e]) - 2.f * g[q4 + e];
+                            const float err = c1 * ss[e] + c2 * (n_i + nn[e]);
+                            if (d2 - err <= thd && pp[e] != skip)
+                                keep(c0 + q4 + e, d2, TC_RERANK);
                         }
                     }
                 }
@@ -352,38 +364,32 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
 // stages the run's rows in FP32 in shared memory (row stride d + 1 words) and
 // the threads share out all (row, candidate) pairs of the run; each marked
 // pair (t, column c) is recomputed by one thread in the order of pair_d2_seq
-// and written back in place with the id of column c.  Runs the Gram kernel
-// found exact return at once.
+// and written back in place with the id of column c.  The blocks walk the list
+// of inexact runs: none on integer data, where a block per run cost 37 us a
+// round at 1M x 128 to find that out.
 constexpr int EX_THREADS = TC_M;
 
 template <typename XT>
 __global__ void __launch_bounds__(EX_THREADS) k_refine_exact(const XT *__restrict__ X, int64_t n, int d,
-                                                             int64_t ld, const int32_t *__restrict__ off,
-                                                             const int32_t *__restrict__ mem,
-                                                             const int32_t *__restrict__ run_off,
-                                                             const int32_t *__restrict__ run_cl, int k, int cap,
-                                                             const int32_t *__restrict__ run_tag,
+                                                             int64_t ld, const int32_t *__restrict__ mem,
+                                                             const int2 *__restrict__ runs,
+                                                             const RunCounts *__restrict__ cnt,
+                                                             const int32_t *__restrict__ inexact_runs,
                                                              int32_t *__restrict__ cand_id,
                                                              float *__restrict__ cand_d,
                                                              const int32_t *__restrict__ cand_n, DevStatus *st)
 {
     extern __shared__ float xs[];  // [sz][d + 1], d <= 128
     __shared__ int rid[TC_M], pre[TC_M + 1], wsum[EX_THREADS / 32];
-    const int run = blockIdx.x;
-    if (run >= run_off[k] || run_tag[run] == 0)
-        return;
-    const int r = run_cl[run];
-    const int beg = off[r], m = off[r + 1] - beg;
-    const int nc = (m + cap - 1) / cap, rbase = m / nc, rem = m % nc;
-    const int c = run - run_off[r];
-    const int s0 = c * rbase + min(c, rem), sz = rbase + (c < rem ? 1 : 0);
-    if (sz < 2 || sz > TC_M)
-        return;
+    const int nrun = cnt->x;
+    for (int q = blockIdx.x; q < nrun; q += gridDim.x) {
+    const int2 rec = runs[inexact_runs[q]];
+    const int p0 = rec.x, sz = rec.y;
     const int tid = threadIdx.x, w = tid >> 5, lane = lane_id();
     const int ds = d + 1;
     int cnt = 0;
     if (tid < sz) {
-        const int a = mem[beg + s0 + tid];
+        const int a = mem[p0 + tid];
         rid[tid] = (a >= 0 && a < n) ? a : -1;
         cnt = rid[tid] >= 0 ? cand_n[rid[tid]] : 0;
     }
@@ -428,7 +434,7 @@ __global__ void __launch_bounds__(EX_THREADS) k_refine_exact(const XT *__restric
             continue;
         const int col = (int)(raw & ~TC_RERANK);
         if (col >= sz || rid[col] < 0) {
-            flag_error(st, GK_ERR_INVALID, (unsigned)r);
+            flag_error(st, GK_ERR_INVALID, (unsigned)p0);
             continue;
         }
         const float *xa = xs + row * ds, *xb = xs + col * ds;
@@ -440,54 +446,64 @@ __global__ void __launch_bounds__(EX_THREADS) k_refine_exact(const XT *__restric
         cand_d[slot] = acc;
         cand_id[slot] = rid[col];
     }
+    __syncthreads();  // the next run rewrites the staged rows and ids
+    }
 }
 
 // One warp per graph row that received candidates (all exact by now): the
 // merge of the FP32 path.  Candidate ids arrive in ascending order.
 constexpr int MG_WARPS = 8;
 
-// per warp: candidate keys (TC_CAP), row and merged-row keys (kappa each), candidate ids and distances, dup bits
-__host__ __device__ inline size_t merge_warp_bytes(int kappa)
-{
-    return sizeof(uint64_t) * (size_t)(TC_CAP + 2 * kappa) + (sizeof(int) + sizeof(float)) * TC_CAP + 16;
-}
-
-__global__ void __launch_bounds__(MG_WARPS * 32) k_refine_merge(int64_t n, int kappa,
+__global__ void __launch_bounds__(MG_WARPS * 32) k_refine_merge(int64_t n, int kappa, bool canon,
                                                                 const int32_t *__restrict__ cand_id,
                                                                 const float *__restrict__ cand_d,
                                                                 const int32_t *__restrict__ cand_n,
                                                                 int32_t *__restrict__ g_idx,
                                                                 float *__restrict__ g_dist)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int NC = TC_CAP / 32;
+    __shared__ MergeBuf<NC> mbuf[MG_WARPS];
+    __shared__ int s_cid[MG_WARPS][TC_CAP];
     const int w = threadIdx.x >> 5, lane = lane_id();
-    unsigned char *wb = smem_raw + (size_t)w * merge_warp_bytes(kappa);
-    uint64_t *bk = reinterpret_cast<uint64_t *>(wb);
-    uint64_t *rk = bk + TC_CAP;
-    uint64_t *nk = rk + kappa;
-    int *cid = reinterpret_cast<int *>(nk + kappa);
-    float *cdv = reinterpret_cast<float *>(cid + TC_CAP);
-    unsigned *dup = reinterpret_cast<unsigned *>(cdv + TC_CAP);
+    int *cid = s_cid[w];
+    // all lanes take part: nc slots of candidates
+    auto merge = [&](auto slots, int64_t i, int cnt, const RowRegs &cur) {
+        constexpr int S = decltype(slots)::value;
+        uint64_t ck[S];
+        bool ok[S];
+        const uint64_t th = pack_key(cur.thd, cur.thi);
+#pragma unroll
+        for (int v = 0; v < S; v++) {
+            const int q = lane + 32 * v;
+            ck[v] = ~0ull;
+            if (q < cnt) {
+                const int j = (int)((unsigned)__ldcg(cand_id + i * TC_CAP + q) & ~TC_RERANK);
+                cid[q] = j;  // ascending
+                ck[v] = pack_key(__ldcg(cand_d + i * TC_CAP + q), j);
+            }
+            ok[v] = ck[v] < th;  // a recomputed pair may miss the row after all (~0 for no candidate)
+        }
+        __syncwarp();
+        merge_slots<S>(ck, ok, canon, cid, nullptr, cnt, kappa, cur, g_idx + i * kappa, g_dist + i * kappa,
+                       reinterpret_cast<MergeBuf<S> &>(mbuf[w]));
+        __syncwarp();
+    };
     for (int64_t i = (int64_t)blockIdx.x * MG_WARPS + w; i < n; i += (int64_t)gridDim.x * MG_WARPS) {
         const int cnt = cand_n[i];
         if (cnt == 0)
             continue;
         RowRegs cur;
         load_row(cur, g_idx + i * kappa, g_dist + i * kappa, kappa);
-        for (int q = lane; q < cnt; q += 32) {
-            cid[q] = (int)((unsigned)__ldcg(cand_id + i * TC_CAP + q) & ~TC_RERANK);
-            cdv[q] = __ldcg(cand_d + i * TC_CAP + q);
-        }
-        __syncwarp();
-        merge_row((int)i, cid, cdv, cnt, kappa, cur, g_idx + i * kappa, g_dist + i * kappa, rk, bk, nk, dup);
-        __syncwarp();
+        if (cnt <= 64)
+            merge(std::integral_constant<int, 2>{}, i, cnt, cur);
+        else
+            merge(std::integral_constant<int, NC>{}, i, cnt, cur);
     }
 }
 
-// candidate ids and distances (n x TC_CAP each), counts (n), run flags (at most k + n / 2 + 1 runs)
 static size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
-// candidate ids and distances (n x TC_CAP each), counts (n), run tags and run flags (at most k + n / 2 + 1 runs
+// candidate ids and distances (n x TC_CAP each), counts (n), run flags and inexact runs (at most k + n / 2 + 1 runs
 // each), and for 64 <= d <= 128 the cluster-sorted BF16 copy (n x perm_cols(d)) with its row norms (n)
 size_t refine_tc_scratch_bytes(int64_t n, int32_t k, int64_t d)
 {
@@ -543,10 +559,9 @@ static cudaError_t perm_tensor_map(CUtensorMap *tm, const __nv_bfloat16 *Xp, int
 }
 
 template <typename XT>
-static cudaError_t refine_tc_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
-                               const int32_t *members, const int32_t *run_off, const int32_t *run_cl, int32_t k,
-                               int32_t kappa, int32_t max_cluster, int64_t grid, int32_t *g_idx, float *g_dist,
-                               void *scratch, DevStatus *st, cudaStream_t s)
+static cudaError_t refine_tc_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *members, const int2 *runs,
+                               RunCounts *cnt, int64_t bound, int32_t k, int32_t kappa, const int32_t *prev, bool canon,
+                               int32_t *g_idx, float *g_dist, void *scratch, DevStatus *st, cudaStream_t s)
 {
     const size_t a = al256((size_t)n * TC_CAP * sizeof(int32_t));
     const size_t t = al256((size_t)(k + n / 2 + 1) * sizeof(int32_t));
@@ -554,7 +569,7 @@ static cudaError_t refine_tc_t(const XT *X, int64_t n, int64_t d, int64_t ld, co
     int32_t *cand_id = reinterpret_cast<int32_t *>(sp);
     float *cand_d = reinterpret_cast<float *>(sp + a);
     int32_t *cand_n = reinterpret_cast<int32_t *>(sp + 2 * a);
-    int32_t *run_tag = reinterpret_cast<int32_t *>(sp + 2 * a + al256((size_t)n * 4));
+    int32_t *inexact_runs = reinterpret_cast<int32_t *>(sp + 2 * a + al256((size_t)n * 4));
     int32_t *run_flags = reinterpret_cast<int32_t *>(sp + 2 * a + al256((size_t)n * 4) + t);
     __nv_bfloat16 *Xp = reinterpret_cast<__nv_bfloat16 *>(sp + 2 * a + al256((size_t)n * 4) + 2 * t);
     const int64_t dp = perm_cols(d);
@@ -569,40 +584,33 @@ static cudaError_t refine_tc_t(const XT *X, int64_t n, int64_t d, int64_t ld, co
     if ((e = set_max_smem(reinterpret_cast<const void *>(k_refine_exact<XT>),
                           (int)(sizeof(float) * TC_M * (128 + 1)))) != cudaSuccess)
         return e;
-    const size_t shm_merge = MG_WARPS * merge_warp_bytes(kappa);
-    if ((e = set_max_smem(reinterpret_cast<const void *>(k_refine_merge),
-                          (int)(MG_WARPS * merge_warp_bytes(MAX_KAPPA)))) != cudaSuccess)
-        return e;
     if ((e = cudaMemsetAsync(cand_n, 0, sizeof(int32_t) * (size_t)n, s)) != cudaSuccess)
         return e;
-    if ((e = cudaMemsetAsync(run_tag, 0, sizeof(int32_t) * (size_t)grid, s)) != cudaSuccess)
-        return e;
-    k_refine_perm<XT><<<(unsigned)grid, TC_THREADS, 0, s>>>(X, n, (int)d, ld, offsets, members, run_off, run_cl, k,
-                                                            max_cluster, (int)dp, Xp, pnrm, run_flags, st);
-    k_refine_gram<<<(unsigned)grid, TC_THREADS, TC_SMEM, s>>>(tmap, n, (int)d, offsets, members, run_off, run_cl, k,
-                                                              kappa, max_cluster, g_idx, g_dist, pnrm, run_flags,
-                                                              cand_id, cand_d, cand_n, run_tag, st);
-    k_refine_exact<XT><<<(unsigned)grid, EX_THREADS, shm_exact, s>>>(X, n, (int)d, ld, offsets, members, run_off, run_cl,
-                                                                 k, max_cluster, run_tag, cand_id, cand_d, cand_n,
-                                                                 st);
+    k_refine_perm<XT><<<(unsigned)bound, TC_THREADS, 0, s>>>(X, n, (int)d, ld, members, runs, cnt, (int)dp, Xp, pnrm,
+                                                             run_flags, inexact_runs, st);
+    k_refine_gram<<<(unsigned)bound, TC_THREADS, TC_SMEM, s>>>(tmap, n, (int)d, members, runs, cnt, prev, kappa, g_idx,
+                                                               g_dist, pnrm, run_flags, cand_id, cand_d, cand_n, st);
+    // the inexact runs are listed: three blocks per SM fit at d = 128, more at smaller d
+    const int64_t ex_blocks = bound < 152 * 6 ? bound : 152 * 6;
+    k_refine_exact<XT><<<(unsigned)ex_blocks, EX_THREADS, shm_exact, s>>>(X, n, (int)d, ld, members, runs, cnt,
+                                                                          inexact_runs, cand_id, cand_d, cand_n, st);
     int64_t mblocks = (n + MG_WARPS - 1) / MG_WARPS;
     if (mblocks > 152 * 64)
         mblocks = 152 * 64;
-    k_refine_merge<<<(unsigned)mblocks, MG_WARPS * 32, shm_merge, s>>>(n, kappa, cand_id, cand_d, cand_n, g_idx,
-                                                                        g_dist);
+    k_refine_merge<<<(unsigned)mblocks, MG_WARPS * 32, 0, s>>>(n, kappa, canon, cand_id, cand_d, cand_n, g_idx, g_dist);
     return cudaGetLastError();
 }
 
-cudaError_t launch_refine_tc(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
-                             const int32_t *members, const int32_t *run_off, const int32_t *run_cl, int32_t k,
-                             int32_t kappa, int32_t max_cluster, int64_t grid, int32_t *g_idx, float *g_dist,
-                             void *scratch, DevStatus *st, cudaStream_t s)
+cudaError_t launch_refine_tc(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *members,
+                             const int2 *runs, RunCounts *cnt, int64_t bound, int32_t k, int32_t kappa,
+                             const int32_t *prev, bool canon, int32_t *g_idx, float *g_dist, void *scratch,
+                             DevStatus *st, cudaStream_t s)
 {
     if (bf16)
-        return refine_tc_t(static_cast<const __nv_bfloat16 *>(X), n, d, ld, offsets, members, run_off, run_cl, k,
-                           kappa, max_cluster, grid, g_idx, g_dist, scratch, st, s);
-    return refine_tc_t(static_cast<const float *>(X), n, d, ld, offsets, members, run_off, run_cl, k, kappa,
-                       max_cluster, grid, g_idx, g_dist, scratch, st, s);
+        return refine_tc_t(static_cast<const __nv_bfloat16 *>(X), n, d, ld, members, runs, cnt, bound, k, kappa, prev,
+                           canon, g_idx, g_dist, scratch, st, s);
+    return refine_tc_t(static_cast<const float *>(X), n, d, ld, members, runs, cnt, bound, k, kappa, prev, canon, g_idx,
+                       g_dist, scratch, st, s);
 }
 
 }  // namespace gkm

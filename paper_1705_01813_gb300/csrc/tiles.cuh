@@ -28,13 +28,7 @@ struct RefineTile {
     static constexpr size_t tile_floats = (size_t)T * DS;
     static constexpr size_t fixed_bytes =
         sizeof(float) * (stage_floats > tile_floats ? stage_floats : tile_floats) + sizeof(int) * 2 * T;
-    // per warp: row keys (kappa), merged-row keys (kappa), candidate keys (T), dup bits
-    __host__ __device__ static size_t warp_bytes(int kappa)
-    {
-        return sizeof(uint64_t) * (size_t)(2 * kappa + T) + 4 * sizeof(unsigned);
-    }
-    static_assert(fixed_bytes % 8 == 0, "the per-warp key buffers need 8-byte alignment");
-    __host__ __device__ static size_t smem_bytes(int kappa) { return fixed_bytes + RF_WARPS * warp_bytes(kappa); }
+    static constexpr int NBLK = 16 * 17 / 2;  // Q x Q blocks on and above the diagonal
 };
 
 // 16 bytes of sample elements (4 FP32 or 8 BF16) widened to floats.
@@ -63,43 +57,57 @@ __host__ __device__ inline bool tile_vec16(const XT *X, int d, int64_t ld)
     return d % E == 0 && ld % E == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
 }
 
+// The Q x Q blocks of a run's own tile (rows = columns = the run's nr members) that have to be computed, as codes
+// by << 8 | bx in list[].  The tile is symmetric, d(i, j) = d(j, i) bit for bit (the difference only changes sign),
+// so only blocks with by <= bx < nb = ceil(nr / Q) count (a run of 50 has 91 at Q = 4); and with prun, the run each
+// member belonged to in the previous refinement (members sorted by it, -1: none), a block whose rows and columns all
+// come from one such run holds only pairs that were compared then, and is left out.  Called by NT threads with index
+// t in [0, NT), NT a multiple of 32 and >= NBLK; sync() is their barrier, wcnt has NT / 32 entries.  Returns the
+// number of blocks (the list is valid after the call).
+template <int T, int NT, typename Sync>
+__device__ __forceinline__ int live_blocks(int nr, const int *prun, unsigned short *list, int *wcnt, int t, Sync sync)
+{
+    constexpr int Q = RefineTile<T>::Q;
+    static_assert(NT >= RefineTile<T>::NBLK && NT % 32 == 0, "one thread per block");
+    const int nb = (nr + Q - 1) / Q;
+    int bx = t, by = 0;
+    while (by < nb && bx >= nb - by) {
+        bx -= nb - by;
+        by++;
+    }
+    bx += by;
+    bool live = by < nb;
+    if (live && prun)
+        live = prun[Q * by] < 0 || prun[Q * by] != prun[min(Q * bx + Q, nr) - 1];
+    const unsigned bal = __ballot_sync(FULL_MASK, live);
+    if ((t & 31) == 0)
+        wcnt[t >> 5] = __popc(bal);
+    sync();
+    int before = 0, total = 0;
+    for (int w = 0; w < NT / 32; w++) {
+        before += w < (t >> 5) ? wcnt[w] : 0;
+        total += wcnt[w];
+    }
+    if (live)
+        list[before + __popc(bal & lanemask_lt())] = (unsigned short)(by << 8 | bx);
+    sync();
+    return total;
+}
+
 // Pair distances of one T x T tile into dt[row * DS + col]: rows are the samples rid[0 .. nr),
 // columns the samples cid[] (SAME: the rows again).  stage points at the block's staging area
 // (RefineTile<T>::stage_floats floats), dt at the distance tile, which may alias it.  Called by all threads
-// of the block; the caller synchronises before reading dt.  VEC: the rows meet tile_vec16, and each stage is
+// of the block; the caller synchronises before reading dt.  This thread computes the Q x Q block of rows Q by .. and
+// columns Q bx .. when rows_live is set (SAME: by <= bx, the block is also written mirrored); a warp without such a
+// thread skips the arithmetic.  VEC: the rows meet tile_vec16, and each stage is
 // fetched as 16-byte vectors (one load per 4 or 8 elements) instead of element by element.
 template <int T, bool SAME, bool VEC, typename XT>
 __device__ __forceinline__ void tile_distances(const XT *__restrict__ X, int d, int64_t ld, const int *rid,
-                                               const int *cid, int nr, float *stage, float *dt)
+                                               const int *cid, int by, int bx, bool rows_live, float *stage, float *dt)
 {
     using TL = RefineTile<T>;
     constexpr int XR = TL::XR, XC = TL::XC, DS = TL::DS, Q = TL::Q;
     const int tid = threadIdx.x;
-    // this thread: rows Q by .. Q by + Q - 1, columns Q bx .. Q bx + Q - 1 of the tile.  Two tiles: block
-    // (by, bx) = (tid / 16, tid % 16), and warps whose rows all lie beyond the run skip the arithmetic.  A run's
-    // own tile (SAME) is symmetric, d(i, j) = d(j, i) bit for bit (the difference only changes sign): only the
-    // nb (nb + 1) / 2 blocks with by <= bx < nb = ceil(nr / Q) hold pairs of the run, and they go to threads
-    // 0, 1, ... row by row (a run of 50 fills 91 threads, three warps; the other warps skip the arithmetic);
-    // each block is also written mirrored.
-    int by = tid >> 4, bx = tid & 15;
-    bool rows_live;
-    if constexpr (SAME) {
-        // the arithmetic goes to the block's warps rot, rot + 1, ... (rot = blockIdx.x % 4): each warp of an SM
-        // issues on scheduler (its index % 4), so blocks that share an SM spread their few busy warps over all
-        // four schedulers instead of all starting at scheduler 0
-        const int rot = (int)(blockIdx.x & 3) * 32;
-        const int nb = (nr + Q - 1) / Q;
-        int t = (tid - rot) & (RF_THREADS - 1), r = 0;
-        while (r < nb && t >= nb - r) {
-            t -= nb - r;
-            r++;
-        }
-        by = r;
-        bx = r + t;
-        rows_live = r < nb;
-    } else {
-        rows_live = Q * by < nr;
-    }
     const float2 m1 = make_float2(-1.f, -1.f);
     float2 acc[Q][Q / 2];
 #pragma unroll
@@ -246,30 +254,19 @@ __device__ __forceinline__ void tile_distances(const XT *__restrict__ X, int d, 
     }
 }
 
-// A run's own 64 x 64 tile (rows = columns = rid[0 .. nr)) computed by a group of NC threads of the block, with
+// A run's own 64 x 64 tile (rows = columns = rid[]) computed by a group of NC threads of the block, with
 // index ct in [0, NC), that synchronise on named barrier bar (the rest of the block does other work meanwhile):
 // the arithmetic, the stages and the pair order of tile_distances<64, true, VEC>, so every distance has the same
-// bits.  Nothing is written to a distance tile: a thread that holds a block of pairs (returns true) gets the
-// block's position (by, bx) and its Q x Q distances in acc, for the caller to store when the tile is free.
+// bits.  Nothing is written to a distance tile: a thread with rows_live set gets the Q x Q distances of its block
+// (by, bx) in acc, for the caller to store when the tile is free.
 template <int NC, bool VEC, typename XT>
-__device__ __forceinline__ bool tile_distances_group(const XT *__restrict__ X, int d, int64_t ld, const int *rid,
-                                                     int nr, float *stage, int ct, int bar,
-                                                     float2 (&acc)[RefineTile<64>::Q][RefineTile<64>::Q / 2],
-                                                     int &by_out, int &bx_out)
+__device__ __forceinline__ void tile_distances_group(const XT *__restrict__ X, int d, int64_t ld, const int *rid,
+                                                     int by, int bx, bool rows_live, float *stage, int ct, int bar,
+                                                     float2 (&acc)[RefineTile<64>::Q][RefineTile<64>::Q / 2])
 {
     constexpr int T = 64;
     using TL = RefineTile<T>;
     constexpr int XR = TL::XR, XC = TL::XC, Q = TL::Q;
-    static_assert(NC % 32 == 0 && NC >= 136, "the group covers the 136 pair blocks of a 64-row triangle");
-    const int nb = (nr + Q - 1) / Q;
-    int t = ct, r = 0;
-    while (r < nb && t >= nb - r) {
-        t -= nb - r;
-        r++;
-    }
-    const int by = r, bx = r + t;
-    const bool rows_live = r < nb;
-    by_out = by, bx_out = bx;
     const float2 m1 = make_float2(-1.f, -1.f);
 #pragma unroll
     for (int a = 0; a < Q; a++)
@@ -376,7 +373,6 @@ __device__ __forceinline__ bool tile_distances_group(const XT *__restrict__ X, i
             store(stage + (sidx ^ 1) * TL::buf_floats);  // read last in the previous stage, before its barrier
         bar_sync(bar, NC);
     }
-    return rows_live;
 }
 
 }  // namespace gkm
