@@ -107,7 +107,10 @@ struct Layout {
     int32_t *labels_b;
     float *cent;
     double *elog;
-    int32_t *prev[2];  // BUILD: each sample's run in the last two refinements
+    int32_t *prev[2];      // BUILD: each sample's run in the last two refinements
+    uint8_t *dirty[2];     // FIT, BUILD: clusters changed by the last two assignments
+    uint8_t *row_changed;  // BUILD: graph rows changed since the last assignment
+    int32_t *todo_n;       // FIT, BUILD: Track's counters
     size_t bytes;
 };
 
@@ -135,12 +138,16 @@ Layout carve(void *ws, int op, int64_t n, int64_t d, int32_t k)
     if (op == GK_OP_FIT || op == GK_OP_BUILD) {
         L.labels_b = cv.take<int32_t>((size_t)n);
         L.elog = cv.take<double>(MAX_LOG);
+        L.todo_n = cv.take<int32_t>(64);  // 256 bytes, followed by dirty[0]: one memset clears both
+        L.dirty[0] = cv.take<uint8_t>((size_t)k);
+        L.dirty[1] = cv.take<uint8_t>((size_t)k);
     }
     if (op == GK_OP_BUILD) {
         L.labels_a = cv.take<int32_t>((size_t)n);
         L.cent = cv.take<float>((size_t)k * (size_t)d);
         L.prev[0] = cv.take<int32_t>((size_t)n);
         L.prev[1] = cv.take<int32_t>((size_t)n);
+        L.row_changed = cv.take<uint8_t>((size_t)n);
     }
     if (op == GK_OP_RECALL)  // k: the number of queries
         L.rec_scratch = cv.take<char>(recall_scratch_bytes(n, k));
@@ -148,6 +155,20 @@ Layout carve(void *ws, int op, int64_t n, int64_t d, int32_t k)
         L.tree_scratch = cv.take<char>(tree_scratch_bytes(n, d, k));
     L.bytes = cv.off;
     return L;
+}
+
+// What assignment t of a fit or a graph construction knows from the one before (Track).  Precision 3 does not keep it:
+// its tile kernels evaluate whole candidate unions.  Nor do sample sets of less than 4M values (16 MB): their
+// assignments take about 10 us, no more than sorting the samples into lists (a fit of 20,000 x 32 took 1.23 ms with
+// it and 1.13 without; one of 2M x 512 takes 19 and 104).
+constexpr int64_t TRACK_MIN_VALUES = (int64_t)1 << 22;
+
+Track track_of(const Layout &L, int t, int64_t n, int64_t d, int32_t precision, bool rows)
+{
+    if ((precision & 0xff) == 3 || n * d < TRACK_MIN_VALUES)
+        return Track{};
+    return Track{t > 0 ? L.dirty[(t + 1) & 1] : nullptr, L.dirty[t & 1], rows ? L.row_changed : nullptr,
+                 L.dirty[(t + 1) & 1], L.todo_n};
 }
 
 int32_t build_k0(int64_t n, int32_t xi) { return (int32_t)(n / xi > 0 ? n / xi : 1); }
@@ -636,12 +657,15 @@ static int kmeans_fit_impl(const void *X, bool bf16, int64_t n, int64_t d, int64
         GK_CUDA(launch_group(cur, n, k, L.grp.offsets, L.grp.members, cnt, L.grp.scratch, L.st, s));
         GK_CUDA(launch_update(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k, C_out, cnt, L.elog + 0,
                               L.upd_scratch, L.st, s));
+        if (track_of(L, 0, n, d, precision, false).dirty_out)
+            GK_CUDA(cudaMemsetAsync(L.todo_n, 0, 256 + (size_t)k, s));
         for (int t = 0; t < iters; t++) {
+            const Track trk = track_of(L, t, n, d, precision, false);
             GK_CUDA(launch_assign(X, bf16, n, d, ld, g_idx, kappa, C_out, k, cur, nxt, nullptr, L.elog + 1 + 2 * t,
-                                  nullptr, L.asg_scratch, L.st, s, precision, L.grp.members));
+                                  nullptr, L.asg_scratch, L.st, s, precision, L.grp.members, trk));
             GK_CUDA(launch_group(nxt, n, k, L.grp.offsets, L.grp.members, cnt, L.grp.scratch, L.st, s));
             GK_CUDA(launch_update(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k, C_out, cnt, L.elog + 2 + 2 * t,
-                                  L.upd_scratch, L.st, s));
+                                  L.upd_scratch, L.st, s, trk.dirty_out));
             int32_t *tmp = cur;
             cur = nxt;
             nxt = tmp;
@@ -711,17 +735,22 @@ static int build_knn_graph_impl(const void *X, bool bf16, int64_t n, int64_t d, 
         GK_CUDA(launch_group(cur, n, k0, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s));
         GK_CUDA(launch_update(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k0, L.cent, L.grp.counts, L.elog + 0,
                               L.upd_scratch, L.st, s));
+        if (track_of(L, 0, n, d, p->precision, true).dirty_out) {
+            GK_CUDA(cudaMemsetAsync(L.row_changed, 0, (size_t)n, s));
+            GK_CUDA(cudaMemsetAsync(L.todo_n, 0, 256 + (size_t)k0, s));
+        }
         for (int t = 0; t < tau; t++) {
+            const Track trk = track_of(L, t, n, d, p->precision, true);
             // one k-means iteration at k0 on the current graph (Sec. 4.5: t = 1 per round)
             GK_CUDA(launch_assign(X, bf16, n, d, ld, g_idx, p->kappa, L.cent, k0, cur, nxt, nullptr, L.elog + 1 + 2 * t,
-                                  nullptr, L.asg_scratch, L.st, s, p->precision, L.grp.members));
+                                  nullptr, L.asg_scratch, L.st, s, p->precision, L.grp.members, trk));
             GK_CUDA(launch_group(nxt, n, k0, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s));
             GK_CUDA(launch_update(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k0, L.cent, L.grp.counts,
-                                  L.elog + 2 + 2 * t, L.upd_scratch, L.st, s));
+                                  L.elog + 2 + 2 * t, L.upd_scratch, L.st, s, trk.dirty_out));
             // exhaustive pairs inside the clusters of the new partition
             GK_CUDA(launch_refine(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k0, p->kappa, p->max_cluster, g_idx,
                                   g_dist, L.ref_scratch, L.st, s, p->precision & 0xff, t > 0 ? L.prev[(t + 1) & 1] : nullptr,
-                                  L.prev[t & 1], true));
+                                  L.prev[t & 1], true, trk.row_changed));
             int32_t *tmp = cur;
             cur = nxt;
             nxt = tmp;
@@ -846,15 +875,21 @@ static int batch_fit_impl(const void *X, bool bf16, int64_t d, int64_t ld, int32
         GK_CUDA(launch_group(cur, N, bd.K0, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s));
         GK_CUDA(launch_update(X, bf16, N, d, ld, L.grp.offsets, L.grp.members, bd.K0, L.cent, L.grp.counts, nullptr,
                               L.upd_scratch, L.st, s));
+        const bool track = track_of(L, 0, N, d, p->precision, true).dirty_out != nullptr;
+        if (track) {
+            GK_CUDA(cudaMemsetAsync(L.row_changed, 0, (size_t)N, s));
+            GK_CUDA(cudaMemsetAsync(L.todo_n, 0, 256 + (size_t)bd.K0, s));
+        }
         for (int t = 0; t < p->tau; t++) {
+            const Track trk = track_of(L, t, N, d, p->precision, true);
             GK_CUDA(launch_assign(X, bf16, N, d, ld, g_idx, p->kappa, L.cent, bd.K0, cur, nxt, nullptr, nullptr,
-                                  nullptr, L.asg_scratch, L.st, s, p->precision, L.grp.members));
+                                  nullptr, L.asg_scratch, L.st, s, p->precision, L.grp.members, trk));
             GK_CUDA(launch_group(nxt, N, bd.K0, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s));
             GK_CUDA(launch_update(X, bf16, N, d, ld, L.grp.offsets, L.grp.members, bd.K0, L.cent, L.grp.counts,
-                                  nullptr, L.upd_scratch, L.st, s));
+                                  nullptr, L.upd_scratch, L.st, s, trk.dirty_out));
             GK_CUDA(launch_refine(X, bf16, N, d, ld, L.grp.offsets, L.grp.members, bd.K0, p->kappa, p->max_cluster,
                                   g_idx, g_dist, L.ref_scratch, L.st, s, p->precision & 0xff, t > 0 ? L.prev[(t + 1) & 1] : nullptr,
-                                  L.prev[t & 1], true));
+                                  L.prev[t & 1], true, trk.row_changed));
             int32_t *tmp = cur;
             cur = nxt;
             nxt = tmp;
@@ -868,12 +903,15 @@ static int batch_fit_impl(const void *X, bool bf16, int64_t d, int64_t ld, int32
         GK_CUDA(launch_group(cur, N, bd.K, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s));
         GK_CUDA(launch_update(X, bf16, N, d, ld, L.grp.offsets, L.grp.members, bd.K, C_out, L.grp.counts, nullptr,
                               L.upd_scratch, L.st, s));
+        if (track)
+            GK_CUDA(cudaMemsetAsync(L.todo_n, 0, 256 + (size_t)bd.K, s));
         for (int t = 0; t < iters; t++) {
+            const Track trk = track_of(L, t, N, d, p->precision, false);
             GK_CUDA(launch_assign(X, bf16, N, d, ld, g_idx, p->kappa, C_out, bd.K, cur, nxt, nullptr, nullptr, nullptr,
-                                  L.asg_scratch, L.st, s, p->precision, L.grp.members));
+                                  L.asg_scratch, L.st, s, p->precision, L.grp.members, trk));
             GK_CUDA(launch_group(nxt, N, bd.K, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s));
             GK_CUDA(launch_update(X, bf16, N, d, ld, L.grp.offsets, L.grp.members, bd.K, C_out, L.grp.counts,
-                                  nullptr, L.upd_scratch, L.st, s));
+                                  nullptr, L.upd_scratch, L.st, s, trk.dirty_out));
             int32_t *tmp = cur;
             cur = nxt;
             nxt = tmp;

@@ -3,11 +3,9 @@
 //   Q_i = { L[i] } u { L[G[i][j]] : j < kappa }          (candidate clusters)
 //   L'[i] = argmin over r in Q_i of (||x_i - C_r||^2, r)  (ties -> smaller label)
 //
-// One warp per sample.  The warp stages x_i in shared memory, gathers the
-// kappa + 1 candidate labels 32 at a time and removes repeats with
-// __match_any_sync plus a scan of the labels already kept, then each lane
-// takes candidates lane, lane + 32, ... and computes their distances with
-// 16-byte centroid loads; a shuffle reduction picks the (distance, label)
+// One warp per sample.  The warp collects the distinct labels of the kappa + 1
+// candidates (collect_labels) and takes the distances to their centroids; a
+// shuffle reduction picks the (distance, label)
 // minimum.  Per-block FP64 partial sums of the winning distances and the
 // count of changed labels are reduced in a fixed order afterwards, so every
 // run gives the same bits.
@@ -35,6 +33,224 @@ constexpr int AS_BLOCKS = 152 * 8;  // fixed grid: the FP64 partial sums have a 
 constexpr int AS_ROWS_PER_SM = 6;
 constexpr int AS_QCAP = MAX_KAPPA + 1;
 constexpr int AS_TILE = 128;  // samples per tile of the tensor-core assignment
+
+constexpr int AS_G = 8;
+constexpr int AS_HASH = 256;                                  // slots of the per-warp label set
+constexpr int AS_QROW = (AS_QCAP + AS_G + 3) / 4 * 4;         // candidate list row, padding included
+static_assert(AS_HASH > AS_QCAP, "the label set must never fill up");
+
+// The distinct candidate labels of sample i in list order (the own label first, then the neighbours'), written to
+// qlist; returns their number.  Repeats are dropped with __match_any_sync inside each batch of 32 and, across batches,
+// with a per-warp open-addressing set in shared memory (one atomicCAS per new label).
+__device__ __forceinline__ int collect_labels(int64_t i, int own, const int32_t *__restrict__ G, int kappa, int64_t n,
+                                              int k, const int32_t *__restrict__ Lin, int *qlist, int *tab,
+                                              DevStatus *st)
+{
+    const int lane = lane_id(), ncand = kappa + 1;
+#pragma unroll
+    for (int q = lane * 4; q < AS_HASH; q += 128)
+        *reinterpret_cast<int4 *>(tab + q) = make_int4(-1, -1, -1, -1);
+    __syncwarp();
+    int u = 0;
+    for (int c0 = 0; c0 < ncand; c0 += 32) {
+        int c = c0 + lane;
+        int lab = -1;
+        if (c == 0) {
+            lab = own;
+        } else if (c < ncand) {
+            int nb = __ldcs(G + i * kappa + (c - 1));
+            if ((unsigned)nb < (unsigned)n)
+                lab = Lin[nb];
+            else
+                flag_error(st, GK_ERR_INVALID, (unsigned)i);
+        }
+        if (c < ncand && (unsigned)lab >= (unsigned)k) {
+            flag_error(st, GK_ERR_INVALID, (unsigned)i);
+            lab = -1;
+        }
+        const unsigned peers = __match_any_sync(FULL_MASK, lab);
+        bool fresh = false;
+        if (lab >= 0 && (peers & lanemask_lt()) == 0u) {
+            unsigned h = ((unsigned)lab * 0x9E3779B1u) >> 24;  // 8-bit multiplicative hash
+            for (int probe = 0; probe < AS_HASH; probe++) {    // the set is never full: ends early
+                const int old = atomicCAS(tab + h, -1, lab);
+                if (old == -1) {
+                    fresh = true;
+                    break;
+                }
+                if (old == lab)
+                    break;
+                h = (h + 1) & (AS_HASH - 1);
+            }
+        }
+        const unsigned fr = __ballot_sync(FULL_MASK, fresh);
+        if (fresh)
+            qlist[u + __popc(fr & lanemask_lt())] = lab;
+        u += __popc(fr);
+    }
+    __syncwarp();
+    return u;
+}
+
+// Several assignments of the same samples in a row (Track): a sample whose graph row and own centroid are as they were
+// in the previous one still has its distance best[i] to that centroid, which every other candidate with an unchanged
+// centroid lost to then (its cluster has the same members, so it was a candidate then too); only candidates of changed
+// clusters can win now.  The result, and every bit of best[], is that of the whole evaluation.
+//
+// k_assign_select sorts the samples by what they need: none of a known sample's neighbours is in a changed cluster:
+// its label is written and it is done; otherwise it goes to the back list (candidates of changed clusters only), and
+// a sample whose own centroid or graph row changed goes to the front list (all candidates).  The assignment kernels
+// then walk the lists.  Doing the test inside them cost registers that the evaluation needs: 30 -> 32 ms for the
+// 1M x 128 graph construction, where almost no sample is done early (this kernel: 13 us of 1 ms there).  The lists' order varies from call to call and
+// decides nothing but which warp takes a sample.  Against evaluating everything: a fit of 2M x 512 BF16 (k = 200,000)
+// takes 1.0 ms an assignment instead of 9.0 once its labels have settled.
+constexpr int SL_WARPS = 8;
+
+template <int S>
+__global__ void __launch_bounds__(SL_WARPS * 32) k_assign_select(int64_t n, const int32_t *__restrict__ G, int kappa,
+                                                                 int k, const int32_t *__restrict__ Lin,
+                                                                 int32_t *__restrict__ Lout, const Track trk,
+                                                                 int32_t *__restrict__ todo)
+{
+    constexpr int B = S <= 2 ? 4 : 2;  // samples whose neighbours are looked up together, S slots of 32 each
+    __shared__ int s_n[2], s_at[2];
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const int64_t step = (int64_t)gridDim.x * SL_WARPS * 32;
+    for (int64_t b0 = (int64_t)blockIdx.x * SL_WARPS * 32; b0 < n; b0 += step) {
+        const int64_t i0 = b0 + w * 32, i = i0 + lane;
+        int own = -1;
+        bool known = false;
+        if (i < n) {
+            own = Lin[i];
+            known = (unsigned)own < (unsigned)k && trk.dirty[own] == 0;
+            if (trk.row_changed && trk.row_changed[i]) {
+                trk.row_changed[i] = 0;
+                known = false;
+            }
+        }
+        unsigned left = __ballot_sync(FULL_MASK, known);
+        unsigned touched = 0;  // known samples with a neighbour in a changed cluster (or an id out of range)
+        while (left) {
+            int src[B];
+            int nb[B][S];
+#pragma unroll
+            for (int q = 0; q < B; q++) {
+                src[q] = left ? __ffs(left) - 1 : -1;
+                left &= left - 1;
+#pragma unroll
+                for (int u = 0; u < S; u++) {
+                    const int c = lane + 32 * u;
+                    nb[q][u] = src[q] >= 0 && c < kappa ? __ldcs(G + (i0 + src[q]) * kappa + c) : -2;
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < B; q++)
+#pragma unroll
+                for (int u = 0; u < S; u++)
+                    if (nb[q][u] != -2)
+                        nb[q][u] = (unsigned)nb[q][u] < (unsigned)n ? Lin[nb[q][u]] : -1;
+#pragma unroll
+            for (int q = 0; q < B; q++) {
+                bool any = false;
+#pragma unroll
+                for (int u = 0; u < S; u++)
+                    if (nb[q][u] != -2)
+                        any |= (unsigned)nb[q][u] >= (unsigned)k || trk.dirty[nb[q][u]] != 0;
+                if (__any_sync(FULL_MASK, any) && src[q] >= 0)
+                    touched |= 1u << src[q];
+            }
+        }
+        const bool part = known && ((touched >> lane) & 1u) != 0, full = i < n && !known;
+        if (known && !part)
+            Lout[i] = own;
+        // places in the two lists, one atomic per block and list
+        if (threadIdx.x < 2)
+            s_n[threadIdx.x] = 0;
+        __syncthreads();
+        const unsigned bf = __ballot_sync(FULL_MASK, full), bp = __ballot_sync(FULL_MASK, part);
+        int wf = 0, wp = 0;
+        if (lane == 0) {
+            wf = atomicAdd(&s_n[0], __popc(bf));
+            wp = atomicAdd(&s_n[1], __popc(bp));
+        }
+        __syncthreads();
+        if (threadIdx.x < 2)
+            s_at[threadIdx.x] = s_n[threadIdx.x] ? atomicAdd(trk.todo_n + threadIdx.x, s_n[threadIdx.x]) : 0;
+        __syncthreads();
+        wf = __shfl_sync(FULL_MASK, wf, 0) + s_at[0];
+        wp = __shfl_sync(FULL_MASK, wp, 0) + s_at[1];
+        if (full)
+            todo[wf + __popc(bf & lanemask_lt())] = (int32_t)i;
+        else if (part)
+            todo[n - 1 - (wp + __popc(bp & lanemask_lt()))] = (int32_t)i;
+        __syncthreads();
+    }
+}
+
+// The samples of an assignment kernel: all of them, or the two lists; f(sample, std::true_type) for the back list.
+// (Taking all samples in their order where the lists hold 7/8 of them gained 1% at 1M x 128 and lost 5% at
+// 200k x 960 and 2M x 512, where the back list is long.)
+template <bool LISTS, typename F>
+__device__ __forceinline__ void each_sample(int64_t first, int64_t step, int64_t n, const Track &trk,
+                                            const int32_t *__restrict__ todo, F f)
+{
+    if constexpr (!LISTS) {
+        for (int64_t i = first; i < n; i += step)
+            f(i, std::false_type{});
+    } else {
+        const int nf = trk.todo_n[0], np = trk.todo_n[1];
+        int32_t nxt = first < nf ? todo[first] : 0;  // the entries are loaded a sample ahead
+        for (int64_t p = first; p < nf; p += step) {
+            const int64_t i = nxt;
+            if (p + step < nf)
+                nxt = todo[p + step];
+            f(i, std::false_type{});
+        }
+        for (int64_t p = first; p < np; p += step)
+            f((int64_t)todo[n - 1 - p], std::true_type{});
+    }
+}
+
+// The candidates of changed clusters among the u of a sample whose own distance is known, moved to the list's front.
+__device__ __forceinline__ int track_filter(const Track &trk, int *qlist, int u)
+{
+    const int lane = lane_id();
+    int m = 0;
+    for (int c0 = 0; c0 < u; c0 += 32) {
+        const int c = c0 + lane;
+        const int lab = c < u ? qlist[c] : -1;
+        const bool keep = c > 0 && c < u && trk.dirty[lab] != 0;  // entry 0 is the own label
+        const unsigned bal = __ballot_sync(FULL_MASK, keep);      // every lane has read its entry
+        if (keep)
+            qlist[m + __popc(bal & lanemask_lt())] = lab;
+        m += __popc(bal);
+    }
+    __syncwarp();
+    return m;
+}
+
+// The winner (bd, br) of sample i, written by lane 0.  Without a valid candidate (br still INT_MAX) the input label
+// stays, with distance 0, and its cluster counts as changed, so that the next assignment looks again.
+__device__ __forceinline__ void write_winner(int64_t i, int own, int k, float bd, int br, int32_t *__restrict__ Lout,
+                                             float *__restrict__ best, const Track &trk)
+{
+    if (lane_id() != 0)
+        return;
+    bool changed = br != own;
+    if (br == 0x7fffffff) {
+        br = own, bd = 0.f;
+        changed = true;
+    }
+    Lout[i] = br;
+    if (best)
+        best[i] = bd;
+    if (changed && trk.dirty_out) {
+        if ((unsigned)own < (unsigned)k)
+            trk.dirty_out[own] = 1;
+        if ((unsigned)br < (unsigned)k)
+            trk.dirty_out[br] = 1;
+    }
+}
 
 template <int VEC>
 __device__ __forceinline__ float cand_d2(const float *__restrict__ xs, const float *__restrict__ c, int d);
@@ -76,68 +292,47 @@ __device__ __forceinline__ float cand_d2<1>(const float *__restrict__ xs, const 
     return a0 + a1;
 }
 
-template <int VEC, typename XT>
+template <int VEC, typename XT, bool LISTS>
 __global__ void __launch_bounds__(AS_WARPS * 32) k_assign(const XT *__restrict__ X, int64_t n, int d, int64_t ld,
                                                           const int32_t *__restrict__ G, int kappa,
                                                           const float *__restrict__ C, int k,
                                                           const int32_t *__restrict__ Lin,
                                                           int32_t *__restrict__ Lout, float *__restrict__ best_out,
-                                                          DevStatus *st)
+                                                          DevStatus *st, const Track trk,
+                                                          const int32_t *__restrict__ todo)
 {
     extern __shared__ __align__(16) float smem[];
     const int w = threadIdx.x >> 5, lane = lane_id();
     const int dpad = (d + 3) & ~3;
     float *xs = smem + w * dpad;
-    int *qlist = reinterpret_cast<int *>(smem + AS_WARPS * dpad) + w * AS_QCAP;
+    int *tab = reinterpret_cast<int *>(smem + AS_WARPS * dpad) + w * (AS_HASH + AS_QROW);
+    int *qlist = tab + AS_HASH;
 
-    const int ncand = kappa + 1;
-    for (int64_t i = (int64_t)blockIdx.x * AS_WARPS + w; i < n; i += (int64_t)gridDim.x * AS_WARPS) {
-        // stage x_i
-        const XT *xi = X + i * ld;
-        if (VEC == 4) {
-            for (int t = lane; t < (d >> 2); t += 32)
-                reinterpret_cast<float4 *>(xs)[t] = ldx4<XT>(xi + 4 * t);
-        } else {
-            for (int t = lane; t < d; t += 32)
-                xs[t] = ldx(xi + t);
-        }
-        // candidate labels: slot 0 is the own label, slot 1 + j the label of neighbour j
+    each_sample<LISTS>((int64_t)blockIdx.x * AS_WARPS + w, (int64_t)gridDim.x * AS_WARPS, n, trk, todo,
+                       [&](int64_t i, auto part) {
+        constexpr bool PART = decltype(part)::value;
         const int own = Lin[i];
-        int u = 0;
-        for (int c0 = 0; c0 < ncand; c0 += 32) {
-            int c = c0 + lane;
-            int lab = -1;
-            if (c == 0) {
-                lab = own;
-            } else if (c < ncand) {
-                int nb = G[i * kappa + (c - 1)];
-                if ((unsigned)nb < (unsigned)n)
-                    lab = Lin[nb];
-                else
-                    flag_error(st, GK_ERR_INVALID, (unsigned)i);
+        int u = collect_labels(i, own, G, kappa, n, k, Lin, qlist, tab, st);
+        float bd = __int_as_float(0x7f800000);
+        int br = 0x7fffffff;
+        if constexpr (PART) {
+            u = track_filter(trk, qlist, u);
+            bd = best_out[i];
+            br = own;
+        }
+        if (u > 0) {
+            // stage x_i
+            const XT *xi = X + i * ld;
+            if (VEC == 4) {
+                for (int t = lane; t < (d >> 2); t += 32)
+                    reinterpret_cast<float4 *>(xs)[t] = ldx4<XT>(xi + 4 * t);
+            } else {
+                for (int t = lane; t < d; t += 32)
+                    xs[t] = ldx(xi + t);
             }
-            if (c < ncand && (unsigned)lab >= (unsigned)k) {
-                flag_error(st, GK_ERR_INVALID, (unsigned)i);
-                lab = -1;
-            }
-            unsigned peers = __match_any_sync(FULL_MASK, lab);
-            bool keep = lab >= 0 && (peers & lanemask_lt()) == 0u;
-            if (keep)
-                for (int q = 0; q < u; q++)
-                    if (qlist[q] == lab) {
-                        keep = false;
-                        break;
-                    }
-            unsigned keeps = __ballot_sync(FULL_MASK, keep);
-            __syncwarp();
-            if (keep)
-                qlist[u + __popc(keeps & lanemask_lt())] = lab;
-            u += __popc(keeps);
             __syncwarp();
         }
         // distances to the kept centroids, lane-parallel over candidates
-        float bd = __int_as_float(0x7f800000);
-        int br = 0x7fffffff;
         for (int q = lane; q < u; q += 32) {
             int r = qlist[q];
             float dv = cand_d2<VEC>(xs, C + (int64_t)r * d, d);
@@ -155,39 +350,26 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign(const XT *__restrict__
                 br = orr;
             }
         }
-        if (lane == 0) {
-            if (br == 0x7fffffff)  // no valid candidate (own label out of range): keep the input label
-                br = own, bd = 0.f;
-            Lout[i] = br;
-            if (best_out)
-                best_out[i] = bd;
-        }
+        write_winner(i, own, k, bd, br, Lout, best_out, trk);
         __syncwarp();
-    }
+    });
 }
 
 // Coalesced variant for 16-byte rows (d % 4 == 0, d <= 32 * 4 * NV): the warp
-// keeps x_i in registers (lane l owns vectors l, l + 32, ...).  Repeated
-// candidate labels are dropped with __match_any_sync inside each batch of 32
-// and, across batches, with a per-warp open-addressing set in shared memory
-// (one atomicCAS per new label).  Distances are taken AS_G candidates at a
+// keeps x_i in registers (lane l owns vectors l, l + 32, ...).  Distances are taken AS_G candidates at a
 // time (AS_G / 2 for rows over 512 floats): each lane loads one 16-byte vector
 // of every centroid of the group, and transpose_reduce completes the group's
 // sums together.  The candidate list is padded to a multiple of the group with
 // its first entry, whose second evaluation
 // cannot change the (distance, label) minimum.
-constexpr int AS_G = 8;
-constexpr int AS_HASH = 256;                                  // slots of the per-warp label set
-constexpr int AS_QROW = (AS_QCAP + AS_G + 3) / 4 * 4;         // candidate list row, padding included
-static_assert(AS_HASH > AS_QCAP, "the label set must never fill up");
-
-template <int NV, typename XT, int GS>
+template <int NV, typename XT, int GS, bool LISTS>
 __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k_assign_rows(const XT *__restrict__ X, int64_t n, int d,
                                                                int64_t ld, const int32_t *__restrict__ G, int kappa,
                                                                const float *__restrict__ C, int k,
                                                                const int32_t *__restrict__ Lin,
                                                                int32_t *__restrict__ Lout,
-                                                               float *__restrict__ best_out, DevStatus *st)
+                                                               float *__restrict__ best_out, DevStatus *st,
+                                                               const Track trk, const int32_t *__restrict__ todo)
 {
     __shared__ __align__(16) int s_q[AS_WARPS][AS_QROW];
     __shared__ __align__(16) int s_h[AS_WARPS][AS_HASH];
@@ -197,9 +379,10 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
     static_assert(GS == 4 || GS == 8, "candidates per group: 4 or 8");
     const int d4 = d >> 2;
     const float4 *C4 = reinterpret_cast<const float4 *>(C);
-    const int ncand = kappa + 1;
 
-    for (int64_t i = (int64_t)blockIdx.x * AS_WARPS + w; i < n; i += (int64_t)gridDim.x * AS_WARPS) {
+    each_sample<LISTS>((int64_t)blockIdx.x * AS_WARPS + w, (int64_t)gridDim.x * AS_WARPS, n, trk, todo,
+                       [&](int64_t i, auto part_list) {
+        constexpr bool PART = decltype(part_list)::value;
         const XT *xrow = X + i * ld;
         float4 xv[NV];
 #pragma unroll
@@ -207,56 +390,19 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
             int col = lane + 32 * v;
             xv[v] = col < d4 ? ldx4<XT, true>(xrow + 4 * col) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-#pragma unroll
-        for (int q = lane * 4; q < AS_HASH; q += 128)
-            *reinterpret_cast<int4 *>(tab + q) = make_int4(-1, -1, -1, -1);
-        __syncwarp();
-        // candidate labels: slot 0 is the own label, slot 1 + j the label of neighbour j
         const int own = Lin[i];
-        int u = 0;
-        for (int c0 = 0; c0 < ncand; c0 += 32) {
-            int c = c0 + lane;
-            int lab = -1;
-            if (c == 0) {
-                lab = own;
-            } else if (c < ncand) {
-                int nb = __ldcs(G + i * kappa + (c - 1));
-                if ((unsigned)nb < (unsigned)n)
-                    lab = Lin[nb];
-                else
-                    flag_error(st, GK_ERR_INVALID, (unsigned)i);
-            }
-            if (c < ncand && (unsigned)lab >= (unsigned)k) {
-                flag_error(st, GK_ERR_INVALID, (unsigned)i);
-                lab = -1;
-            }
-            const unsigned peers = __match_any_sync(FULL_MASK, lab);
-            bool fresh = false;
-            if (lab >= 0 && (peers & lanemask_lt()) == 0u) {
-                unsigned h = ((unsigned)lab * 0x9E3779B1u) >> 24;  // 8-bit multiplicative hash
-                for (int probe = 0; probe < AS_HASH; probe++) {    // the set is never full: ends early
-                    const int old = atomicCAS(tab + h, -1, lab);
-                    if (old == -1) {
-                        fresh = true;
-                        break;
-                    }
-                    if (old == lab)
-                        break;
-                    h = (h + 1) & (AS_HASH - 1);
-                }
-            }
-            const unsigned fr = __ballot_sync(FULL_MASK, fresh);
-            if (fresh)
-                qlist[u + __popc(fr & lanemask_lt())] = lab;
-            u += __popc(fr);
+        int u = collect_labels(i, own, G, kappa, n, k, Lin, qlist, tab, st);
+        float bd = __int_as_float(0x7f800000);
+        int br = 0x7fffffff;
+        if constexpr (PART) {
+            u = track_filter(trk, qlist, u);
+            bd = best_out[i];
+            br = own;
         }
-        __syncwarp();
         if (u > 0 && lane < GS)
             qlist[u + lane] = qlist[0];
         __syncwarp();
 
-        float bd = __int_as_float(0x7f800000);
-        int br = 0x7fffffff;
         for (int g0 = 0; g0 < u; g0 += GS) {
             int lab[GS];
 #pragma unroll
@@ -290,15 +436,9 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
                 br = orr;
             }
         }
-        if (lane == 0) {
-            if (br == 0x7fffffff)  // no valid candidate (own label out of range): keep the input label
-                br = own, bd = 0.f;
-            Lout[i] = br;
-            if (best_out)
-                best_out[i] = bd;
-        }
+        write_winner(i, own, k, bd, br, Lout, best_out, trk);
         __syncwarp();
-    }
+    });
 }
 
 // k_assign_rows with the candidate distances screened against a shadow copy of
@@ -317,12 +457,12 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
 // Shadow formats of the screening: FMT 0 BF16 rows (4 values per 8 bytes), FMT 1 int8 rows with a per-row
 // scale s_r (4 values per 4 bytes; see lane_partial_q8), half the bytes again; FMT 2 the same int8 rows stored
 // lane-major (d a multiple of 128), so that a lane's share of a row is one vector load.
-template <int NV, typename XT, int GS, int FMT>
+template <int NV, typename XT, int GS, int FMT, bool LISTS>
 __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV == 4 ? 4 : 3)) k_assign_rows_scr(
     const XT *__restrict__ X, int64_t n, int d, int64_t ld, const int32_t *__restrict__ G, int kappa,
     const float *__restrict__ C, const void *__restrict__ Cs, const float *__restrict__ delta,
     const float *__restrict__ scale, int k, const int32_t *__restrict__ Lin, int32_t *__restrict__ Lout,
-    float *__restrict__ best_out, DevStatus *st)
+    float *__restrict__ best_out, DevStatus *st, const Track trk, const int32_t *__restrict__ todo)
 {
     __shared__ __align__(16) int s_q[AS_WARPS][AS_QROW];
     __shared__ __align__(16) int s_h[AS_WARPS][AS_HASH];
@@ -337,9 +477,10 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV 
     const uint2 *Cb4 = static_cast<const uint2 *>(Cs);       // FMT 0: 4 BF16 per 8 bytes
     const uint32_t *Cq4 = static_cast<const uint32_t *>(Cs);  // FMT 1: 4 int8 per 4 bytes
     const float gam = (float)(d + 8) * 5.9604645e-8f;         // FP32 rounding of a d-term sum, relative
-    const int ncand = kappa + 1;
 
-    for (int64_t i = (int64_t)blockIdx.x * AS_WARPS + w; i < n; i += (int64_t)gridDim.x * AS_WARPS) {
+    each_sample<LISTS>((int64_t)blockIdx.x * AS_WARPS + w, (int64_t)gridDim.x * AS_WARPS, n, trk, todo,
+                       [&](int64_t i, auto part_list) {
+        constexpr bool PART = decltype(part_list)::value;
         const XT *xrow = X + i * ld;
         float4 xv[NV];
 #pragma unroll
@@ -347,55 +488,21 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV 
             int col = lane + 32 * v;
             xv[v] = col < d4 ? ldx4<XT, true>(xrow + 4 * col) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-#pragma unroll
-        for (int q = lane * 4; q < AS_HASH; q += 128)
-            *reinterpret_cast<int4 *>(tab + q) = make_int4(-1, -1, -1, -1);
-        __syncwarp();
         const int own = Lin[i];
-        int u = 0;
-        for (int c0 = 0; c0 < ncand; c0 += 32) {
-            int c = c0 + lane;
-            int lab = -1;
-            if (c == 0) {
-                lab = own;
-            } else if (c < ncand) {
-                int nb = __ldcs(G + i * kappa + (c - 1));
-                if ((unsigned)nb < (unsigned)n)
-                    lab = Lin[nb];
-                else
-                    flag_error(st, GK_ERR_INVALID, (unsigned)i);
-            }
-            if (c < ncand && (unsigned)lab >= (unsigned)k) {
-                flag_error(st, GK_ERR_INVALID, (unsigned)i);
-                lab = -1;
-            }
-            const unsigned peers = __match_any_sync(FULL_MASK, lab);
-            bool fresh = false;
-            if (lab >= 0 && (peers & lanemask_lt()) == 0u) {
-                unsigned h = ((unsigned)lab * 0x9E3779B1u) >> 24;
-                for (int probe = 0; probe < AS_HASH; probe++) {
-                    const int old = atomicCAS(tab + h, -1, lab);
-                    if (old == -1) {
-                        fresh = true;
-                        break;
-                    }
-                    if (old == lab)
-                        break;
-                    h = (h + 1) & (AS_HASH - 1);
-                }
-            }
-            const unsigned fr = __ballot_sync(FULL_MASK, fresh);
-            if (fresh)
-                qlist[u + __popc(fr & lanemask_lt())] = lab;
-            u += __popc(fr);
+        int u = collect_labels(i, own, G, kappa, n, k, Lin, qlist, tab, st);
+        float bd = __int_as_float(0x7f800000);
+        int br = 0x7fffffff;
+        if constexpr (PART) {
+            u = track_filter(trk, qlist, u);
+            bd = best_out[i];
+            br = own;
         }
-        __syncwarp();
         if (u > 0 && lane < GS)
             qlist[u + lane] = qlist[0];
         __syncwarp();
 
         // pass 1: BF16 distances with their bounds
-        float best_up = __int_as_float(0x7f800000);
+        float best_up = bd;  // the known distance, or infinity
         for (int g0 = 0; g0 < u; g0 += GS) {
             int lab[GS];
 #pragma unroll
@@ -436,8 +543,6 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV 
             best_up = fminf(best_up, __shfl_xor_sync(FULL_MASK, best_up, o));
         __syncwarp();
         // pass 2: exact FP32 distances of the candidates that may be the minimum
-        float bd = __int_as_float(0x7f800000);
-        int br = 0x7fffffff;
         for (int g0 = 0; g0 < u; g0 += 32) {
             const int cnt = min(32, u - g0);
             unsigned sel = __ballot_sync(FULL_MASK, lane < cnt && lov[g0 + lane] <= best_up);
@@ -453,25 +558,21 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV 
                 }
             }
         }
-        if (lane == 0) {
-            if (br == 0x7fffffff)  // no valid candidate (own label out of range): keep the input label
-                br = own, bd = 0.f;
-            Lout[i] = br;
-            if (best_out)
-                best_out[i] = bd;
-        }
+        write_winner(i, own, k, bd, br, Lout, best_out, trk);
         __syncwarp();
-    }
+    });
 }
 
 // ---------------------------------------------------------------------------
 // BF16 shadow of the centroids: Cb = bf16(C) and delta_r >= ||C_r - Cb_r||.
 // ---------------------------------------------------------------------------
 __global__ void k_shadow_bf16(const float *__restrict__ C, int k, int d, __nv_bfloat16 *__restrict__ Cb,
-                              float *__restrict__ delta, float *__restrict__ cnorm)
+                              float *__restrict__ delta, float *__restrict__ cnorm, const uint8_t *__restrict__ dirty)
 {
     const int lane = lane_id();
     for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < k; r += gridDim.x * (blockDim.x >> 5)) {
+        if (dirty && dirty[r] == 0)
+            continue;  // the row, and so its shadow, is as the previous assignment left it
         double e = 0.0, c2 = 0.0;
         for (int t = lane; t < d; t += 32) {
             const float c = C[(int64_t)r * d + t];
@@ -504,11 +605,14 @@ __global__ void k_shadow_bf16(const float *__restrict__ C, int k, int d, __nv_bf
 // evaluation's own roundings) and adds sqrt(d) 4e-15 max|C_r| (the absolute term, which also covers squares
 // below the normal range): a rigorous upper bound, no FP64.
 __global__ void k_shadow_i8(const float *__restrict__ C, int k, int d, bool lane_major, uint32_t *__restrict__ Cq,
-                            float *__restrict__ delta, float *__restrict__ scale)
+                            float *__restrict__ delta, float *__restrict__ scale,
+                            const uint8_t *__restrict__ dirty)
 {
     const int lane = lane_id();
     const int d4 = d >> 2;
     for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < k; r += gridDim.x * (blockDim.x >> 5)) {
+        if (dirty && dirty[r] == 0)
+            continue;  // the row, and so its shadow, is as the previous assignment left it
         const float4 *row = reinterpret_cast<const float4 *>(C + (int64_t)r * d);
         float mx = 0.f;
         for (int col = lane; col < d4; col += 32) {
@@ -722,8 +826,15 @@ __global__ void __launch_bounds__(256) k_assign_reduce(const float *__restrict__
                                                        const int32_t *__restrict__ Lin,
                                                        const int32_t *__restrict__ Lout, int64_t n,
                                                        double *__restrict__ blk_sum,
-                                                       unsigned long long *__restrict__ blk_changed)
+                                                       unsigned long long *__restrict__ blk_changed,
+                                                       const Track trk, int k)
 {
+    if (trk.clear) {  // Track's clears, here to save a launch
+        for (int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x; r < k; r += (int64_t)gridDim.x * 256)
+            trk.clear[r] = 0;
+        if (blockIdx.x == 0 && threadIdx.x < 2)
+            trk.todo_n[threadIdx.x] = 0;
+    }
     __shared__ double s[256];
     __shared__ unsigned long long c[256];
     const int64_t per = (n + gridDim.x - 1) / gridDim.x;
@@ -796,7 +907,7 @@ template <typename XT>
 static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *g_idx, int32_t kappa,
                             const float *C, int32_t k, const int32_t *labels_in, int32_t *labels_out, float *best_d2,
                             double *sum_d2, int64_t *n_changed, void *scratch, DevStatus *st, cudaStream_t s,
-                            int precision, const int32_t *members)
+                            int precision, const int32_t *members, Track trk)
 {
     char *sp = static_cast<char *>(scratch);
     double *blk_sum = reinterpret_cast<double *>(sp);
@@ -826,24 +937,41 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     cudaError_t e;
     int grid = 0;
     bool done = false;
+    if (trk.dirty) {  // the lists take the place that precision 3 alone uses otherwise
+        const int64_t sb = (n + SL_WARPS * 32 - 1) / (SL_WARPS * 32);
+        const unsigned sgrid = (unsigned)(sb < 152 * 8 ? sb : 152 * 8);
+        if (kappa <= 32)
+            k_assign_select<1><<<sgrid, SL_WARPS * 32, 0, s>>>(n, g_idx, kappa, k, labels_in, labels_out, trk, sel_lab);
+        else if (kappa <= 64)
+            k_assign_select<2><<<sgrid, SL_WARPS * 32, 0, s>>>(n, g_idx, kappa, k, labels_in, labels_out, trk, sel_lab);
+        else
+            k_assign_select<4><<<sgrid, SL_WARPS * 32, 0, s>>>(n, g_idx, kappa, k, labels_in, labels_out, trk, sel_lab);
+    }
     if ((precision == 2 || precision == 4) && vec4 && d4 <= 32 * 8) {
         // the shadow: BF16 (2) or int8 with a per-row scale (4); the int8 codes take the BF16 shadow's space
         const int sgrid = (k + 7) / 8 < 152 * 16 ? (k + 7) / 8 : 152 * 16;
         // int8 rows lane-major where every lane owns whole vectors (d a multiple of 128): one load per lane and row
         const bool lane_major = precision == 4 && d % 128 == 0;
         if (precision == 2)
-            k_shadow_bf16<<<sgrid, 256, 0, s>>>(C, k, (int)d, Cb, delta, cnorm);
+            k_shadow_bf16<<<sgrid, 256, 0, s>>>(C, k, (int)d, Cb, delta, cnorm, trk.dirty);
         else
             k_shadow_i8<<<sgrid, 256, 0, s>>>(C, k, (int)d, lane_major, reinterpret_cast<uint32_t *>(Cb), delta,
-                                              cnorm);
+                                              cnorm, trk.dirty);
 #define GK_ASB8F(NV, GS, F)                                                                                      \
     do {                                                                                                         \
-        if ((e = resident_grid(reinterpret_cast<const void *>(k_assign_rows_scr<NV, XT, GS, F>), AS_WARPS * 32,  \
-                               0, &grid)) != cudaSuccess)                                                        \
+        if (trk.dirty)                                                                                           \
+            GK_ASB8T(NV, GS, F, true);                                                                           \
+        else                                                                                                     \
+            GK_ASB8T(NV, GS, F, false);                                                                          \
+    } while (0)
+#define GK_ASB8T(NV, GS, F, T)                                                                                   \
+    do {                                                                                                         \
+        if ((e = resident_grid(reinterpret_cast<const void *>(k_assign_rows_scr<NV, XT, GS, F, T>),              \
+                               AS_WARPS * 32, 0, &grid)) != cudaSuccess)                                         \
             return e;                                                                                            \
-        k_assign_rows_scr<NV, XT, GS, F><<<grid, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, Cb,   \
-                                                                        delta, cnorm, k, labels_in, labels_out,  \
-                                                                        best, st);                               \
+        k_assign_rows_scr<NV, XT, GS, F, T><<<grid, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, Cb,  \
+                                                                           delta, cnorm, k, labels_in, labels_out, \
+                                                                           best, st, trk, sel_lab);                       \
     } while (0)
 #define GK_ASB8G(NV, GS)                                                                                         \
     do {                                                                                                         \
@@ -872,12 +1000,13 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
 #undef GK_ASB8
 #undef GK_ASB8G
 #undef GK_ASB8F
+#undef GK_ASB8T
         done = true;
     }
     if constexpr (std::is_same_v<XT, float>) {  // tensor-core screening: FP32 samples only
         if (precision == 3 && vec4 && d4 <= 32 * 8) {
             k_shadow_bf16<<<(k + 7) / 8 < 152 * 16 ? (k + 7) / 8 : 152 * 16, 256, 0, s>>>(C, k, (int)d, Cb, delta,
-                                                                                      cnorm);
+                                                                                      cnorm, nullptr);
             const bool tiles = members && assign_tc_supported(d, ld, X, C, kappa);
             if (tiles) {
                 if ((e = launch_assign_tc(X, n, d, ld, g_idx, kappa, C, Cb, delta, cnorm, k, labels_in, members,
@@ -907,11 +1036,18 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     } else if (vec4 && d4 <= 32 * 8) {
 #define GK_ASGG(NV, GS)                                                                                          \
     do {                                                                                                         \
-        if ((e = resident_grid(reinterpret_cast<const void *>(k_assign_rows<NV, XT, GS>), AS_WARPS * 32, 0,      \
+        if (trk.dirty)                                                                                           \
+            GK_ASGT(NV, GS, true);                                                                               \
+        else                                                                                                     \
+            GK_ASGT(NV, GS, false);                                                                              \
+    } while (0)
+#define GK_ASGT(NV, GS, T)                                                                                       \
+    do {                                                                                                         \
+        if ((e = resident_grid(reinterpret_cast<const void *>(k_assign_rows<NV, XT, GS, T>), AS_WARPS * 32, 0,   \
                                &grid)) != cudaSuccess)                                                           \
             return e;                                                                                            \
-        k_assign_rows<NV, XT, GS><<<grid, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, k, labels_in,  \
-                                                                 labels_out, best, st);                          \
+        k_assign_rows<NV, XT, GS, T><<<grid, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, k, labels_in, \
+                                                                    labels_out, best, st, trk, sel_lab);                  \
     } while (0)
 #define GK_ASG(NV)                                                                                               \
     do {                                                                                                         \
@@ -930,27 +1066,32 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
             GK_ASG(8);
 #undef GK_ASG
 #undef GK_ASGG
+#undef GK_ASGT
     } else {
         int dpad = (int)((d + 3) & ~3);
-        size_t shm = sizeof(float) * (size_t)AS_WARPS * dpad + sizeof(int) * AS_WARPS * AS_QCAP;
-        const int shm_max = (int)(sizeof(float) * (size_t)AS_WARPS * MAX_D + sizeof(int) * AS_WARPS * AS_QCAP);
-        if (vec4) {
-            if ((e = set_max_smem(reinterpret_cast<const void *>(k_assign<4, XT>), shm_max)) !=
-                cudaSuccess)
-                return e;
-            k_assign<4, XT><<<AS_BLOCKS, AS_WARPS * 32, shm, s>>>(X, n, (int)d, ld, g_idx, kappa, C, k, labels_in,
-                                                                labels_out, best, st);
-        } else {
-            if ((e = set_max_smem(reinterpret_cast<const void *>(k_assign<1, XT>), shm_max)) !=
-                cudaSuccess)
-                return e;
-            k_assign<1, XT><<<AS_BLOCKS, AS_WARPS * 32, shm, s>>>(X, n, (int)d, ld, g_idx, kappa, C, k, labels_in,
-                                                                labels_out, best, st);
-        }
+        size_t shm = sizeof(float) * (size_t)AS_WARPS * dpad + sizeof(int) * AS_WARPS * (AS_HASH + AS_QROW);
+        const int shm_max = (int)(sizeof(float) * (size_t)AS_WARPS * MAX_D + sizeof(int) * AS_WARPS * (AS_HASH + AS_QROW));
+        auto launch = [&](auto kernel) -> cudaError_t {
+            cudaError_t le = set_max_smem(reinterpret_cast<const void *>(kernel), shm_max);
+            if (le == cudaSuccess)
+                kernel<<<AS_BLOCKS, AS_WARPS * 32, shm, s>>>(X, n, (int)d, ld, g_idx, kappa, C, k, labels_in, labels_out,
+                                                             best, st, trk, sel_lab);
+            return le;
+        };
+        if (vec4)
+            e = trk.dirty ? launch(k_assign<4, XT, true>) : launch(k_assign<4, XT, false>);
+        else
+            e = trk.dirty ? launch(k_assign<1, XT, true>) : launch(k_assign<1, XT, false>);
+        if (e != cudaSuccess)
+            return e;
     }
     if (sum_d2 || n_changed) {
-        k_assign_reduce<<<AS_BLOCKS, 256, 0, s>>>(best, labels_in, labels_out, n, blk_sum, blk_chg);
+        k_assign_reduce<<<AS_BLOCKS, 256, 0, s>>>(best, labels_in, labels_out, n, blk_sum, blk_chg, trk, k);
         k_assign_finish<<<1, 1024, 0, s>>>(blk_sum, blk_chg, AS_BLOCKS, sum_d2, n_changed);
+    } else if (trk.clear) {
+        if ((e = cudaMemsetAsync(trk.clear, 0, (size_t)k, s)) != cudaSuccess ||
+            (e = cudaMemsetAsync(trk.todo_n, 0, 2 * sizeof(int32_t), s)) != cudaSuccess)
+            return e;
     }
     return cudaGetLastError();
 }
@@ -958,13 +1099,13 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
 cudaError_t launch_assign(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *g_idx,
                           int32_t kappa, const float *C, int32_t k, const int32_t *labels_in, int32_t *labels_out,
                           float *best_d2, double *sum_d2, int64_t *n_changed, void *scratch, DevStatus *st,
-                          cudaStream_t s, int precision, const int32_t *members)
+                          cudaStream_t s, int precision, const int32_t *members, Track trk)
 {
     if (bf16)
         return assign_t(static_cast<const __nv_bfloat16 *>(X), n, d, ld, g_idx, kappa, C, k, labels_in, labels_out,
-                        best_d2, sum_d2, n_changed, scratch, st, s, precision, members);
+                        best_d2, sum_d2, n_changed, scratch, st, s, precision, members, trk);
     return assign_t(static_cast<const float *>(X), n, d, ld, g_idx, kappa, C, k, labels_in, labels_out, best_d2,
-                    sum_d2, n_changed, scratch, st, s, precision, members);
+                    sum_d2, n_changed, scratch, st, s, precision, members, trk);
 }
 
 }  // namespace gkm

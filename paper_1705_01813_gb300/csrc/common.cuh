@@ -257,8 +257,18 @@ cudaError_t launch_batch_labels(const int32_t *labels, int64_t N, const BatchTab
                                 cudaStream_t s);
 cudaError_t launch_update(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                           const int32_t *members, int32_t k, float *C, int32_t *counts, double *sum_d2,
-                          void *scratch, DevStatus *st, cudaStream_t s);
+                          void *scratch, DevStatus *st, cudaStream_t s, const uint8_t *dirty = nullptr);
 
+// What changed since the previous assignment of the same samples, kept by the callers that run several in a row (one
+// fit, one graph construction); bytes, non-zero for "changed".  An update that finds a cluster's members unchanged
+// leaves its centroid's bits as they are, so distances to it need not be taken again (assign.cu).
+struct Track {
+    const uint8_t *dirty;      // k: the cluster gained or lost members in the previous assignment (NULL: the first)
+    uint8_t *dirty_out;        // k, zeroed: the clusters this assignment changes (NULL: not kept)
+    uint8_t *row_changed;      // n: the graph row changed since the previous assignment, read and cleared (NULL: none)
+    uint8_t *clear;            // k: zeroed after this assignment (the next one's dirty_out; may be `dirty`)
+    int32_t *todo_n;           // two counters, zeroed before and after the assignment
+};
 size_t assign_scratch_bytes(int64_t n, int32_t k, int64_t d);
 // precision 0 and 1: FP32 candidate rows; 2: BF16 screening on the SIMT cores; 3: on the tensor cores over
 // 128-sample tiles when members, the grouping of labels_in, is given and d <= 128; 4: int8 screening (per-row
@@ -267,7 +277,7 @@ size_t assign_scratch_bytes(int64_t n, int32_t k, int64_t d);
 cudaError_t launch_assign(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *g_idx,
                           int32_t kappa, const float *C, int32_t k, const int32_t *labels_in, int32_t *labels_out,
                           float *best_d2, double *sum_d2, int64_t *n_changed, void *scratch, DevStatus *st,
-                          cudaStream_t s, int precision, const int32_t *members);
+                          cudaStream_t s, int precision, const int32_t *members, Track trk = Track{});
 
 void set_last_error(const char *msg);
 
@@ -279,15 +289,17 @@ size_t refine_scratch_bytes(int64_t n, int32_t k, int64_t d);
 // precision 0: FP32 pair distances on the SIMT cores; 1: tensor-core Gram with exact FP32 rerank.  prev_in, prev_out
 // (n each, distinct; NULL: not kept): the run of every sample in the previous refinement of the same graph, whose
 // pairs are not compared again, and in this one.  canon: every distance in the graph has the bits that the library
-// computes for the pair (a graph that init_graph and refinements made), see merge.cuh.
+// computes for the pair (a graph that init_graph and refinements made), see merge.cuh.  row_changed (n, may be NULL):
+// set to 1 for every row that takes a new neighbour.
 cudaError_t launch_refine(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                           const int32_t *members, int32_t k, int32_t kappa, int32_t max_cluster, int32_t *g_idx,
                           float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision,
-                          const int32_t *prev_in = nullptr, int32_t *prev_out = nullptr, bool canon = false);
+                          const int32_t *prev_in = nullptr, int32_t *prev_out = nullptr, bool canon = false,
+                          uint8_t *row_changed = nullptr);
 size_t refine_tc_scratch_bytes(int64_t n, int32_t k, int64_t d);
 cudaError_t launch_refine_tc(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *members,
                              const int2 *runs, RunCounts *cnt, int64_t bound, int32_t k, int32_t kappa,
-                             const int32_t *prev, bool canon, int32_t *g_idx, float *g_dist, void *scratch,
-                             DevStatus *st, cudaStream_t s);
+                             const int32_t *prev, bool canon, uint8_t *row_changed, int32_t *g_idx, float *g_dist,
+                             void *scratch, DevStatus *st, cudaStream_t s);
 
 }  // namespace gkm

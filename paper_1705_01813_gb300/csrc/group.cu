@@ -268,7 +268,8 @@ size_t group_scratch_bytes(int64_t n, int32_t k)
     size_t b = 0;
     auto add = [&](size_t bytes) { b += (bytes + 255) & ~size_t(255); };
     add(sizeof(int32_t) * (size_t)k);           // counts (when the caller keeps none)
-    add(sizeof(int32_t) * (size_t)n * 4);        // keys / values, two buffers each
+    for (int q = 0; q < 4; q++)
+        add(sizeof(int32_t) * (size_t)n);        // keys / values, two buffers each, aligned one by one
     add(sizeof(int32_t) * (size_t)(hist + 1));   // tile histogram, scanned in place
     size_t sc = scan_scratch_bytes(hist > (int64_t)k ? hist : (int64_t)k);
     add(sc);

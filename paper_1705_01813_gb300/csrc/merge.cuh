@@ -69,7 +69,7 @@ __device__ __forceinline__ void load_row(RowRegs &r, const int32_t *__restrict__
 // key is found at its place; otherwise the row ids are looked up among the candidates' ids (ascending, in shared
 // memory).
 //
-// Only the entries that move are written.  Instruction issue bounds the merge: ranking, then binary searches for
+// Only the entries that move are written; the result says whether a candidate entered the row.  Instruction issue bounds the merge: ranking, then binary searches for
 // every candidate and row entry, took 1,400 warp instructions a row with 50 candidates and 830 with 15; with these
 // forms the merge of a 1M x 128 graph construction (kappa = 50) takes 0.64 ms a round instead of 0.94, the pairs left
 // out included.
@@ -83,7 +83,7 @@ struct alignas(16) MergeBuf {
 };
 
 template <int NU, int NC>
-__device__ __forceinline__ void merge_few(uint64_t (&ck)[NC], bool (&ok)[NC], int kappa, const RowRegs &cur,
+__device__ __forceinline__ bool merge_few(uint64_t (&ck)[NC], bool (&ok)[NC], int kappa, const RowRegs &cur,
                                           int32_t *__restrict__ gi, float *__restrict__ gd)
 {
     const int lane = lane_id();
@@ -139,14 +139,17 @@ __device__ __forceinline__ void merge_few(uint64_t (&ck)[NC], bool (&ok)[NC], in
             gd[q] = key_dist(rk[u]);
         }
     }
+    bool entered = false;
 #pragma unroll
     for (int v = 0; v < NC; v++) {
         const int q = pos[v] + rank[v];
         if (ok[v] && q < kappa) {
             gi[q] = key_id(ck[v]);
             gd[q] = key_dist(ck[v]);
+            entered = true;
         }
     }
+    return __any_sync(FULL_MASK, entered);
 }
 
 // Number of the 32 N sorted keys k[] smaller than key (fixed steps; N a power of two).
@@ -163,7 +166,7 @@ __device__ __forceinline__ int lower_rank(const uint64_t *k, uint64_t key)
 // sid[0 .. ns): the ids of all candidate columns, ascending; smap[t] (NULL: t) the column of sid[t] (not read with
 // canon).
 template <int NU, int NC>
-__device__ __forceinline__ void merge_many(uint64_t (&ck)[NC], bool (&ok)[NC], bool canon, const int *__restrict__ sid,
+__device__ __forceinline__ bool merge_many(uint64_t (&ck)[NC], bool (&ok)[NC], bool canon, const int *__restrict__ sid,
                                            const unsigned char *__restrict__ smap, int ns, int kappa,
                                            const RowRegs &cur, int32_t *__restrict__ gi, float *__restrict__ gd,
                                            MergeBuf<NC> &mb)
@@ -268,11 +271,12 @@ __device__ __forceinline__ void merge_many(uint64_t (&ck)[NC], bool (&ok)[NC], b
         }
     }
     __syncwarp();  // the buffers are rewritten by the next row
+    return below > 0;
 }
 
 // The form and the number of row slots that the flagged candidates and kappa ask for.
 template <int NC>
-__device__ __forceinline__ void merge_slots(uint64_t (&ck)[NC], bool (&ok)[NC], bool canon,
+__device__ __forceinline__ bool merge_slots(uint64_t (&ck)[NC], bool (&ok)[NC], bool canon,
                                             const int *__restrict__ sid, const unsigned char *__restrict__ smap, int ns,
                                             int kappa, const RowRegs &cur, int32_t *__restrict__ gi,
                                             float *__restrict__ gd, MergeBuf<NC> &mb)
@@ -282,22 +286,14 @@ __device__ __forceinline__ void merge_slots(uint64_t (&ck)[NC], bool (&ok)[NC], 
     for (int v = 0; v < NC; v++)
         m += __popc(__ballot_sync(FULL_MASK, ok[v]));
     if (m == 0)
-        return;
-    if (m <= MERGE_FEW) {
-        if (kappa <= 32)
-            merge_few<1, NC>(ck, ok, kappa, cur, gi, gd);
-        else if (kappa <= 64)
-            merge_few<2, NC>(ck, ok, kappa, cur, gi, gd);
-        else
-            merge_few<4, NC>(ck, ok, kappa, cur, gi, gd);
-    } else {
-        if (kappa <= 32)
-            merge_many<1, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb);
-        else if (kappa <= 64)
-            merge_many<2, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb);
-        else
-            merge_many<4, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb);
-    }
+        return false;
+    if (m <= MERGE_FEW)
+        return kappa <= 32   ? merge_few<1, NC>(ck, ok, kappa, cur, gi, gd)
+               : kappa <= 64 ? merge_few<2, NC>(ck, ok, kappa, cur, gi, gd)
+                             : merge_few<4, NC>(ck, ok, kappa, cur, gi, gd);
+    return kappa <= 32   ? merge_many<1, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb)
+           : kappa <= 64 ? merge_many<2, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb)
+                         : merge_many<4, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb);
 }
 
 // Merge a run's pair distances drow[0 .. ncol) (ncol <= 32 NC) to the members cid[] into graph row i of that run.
@@ -306,7 +302,7 @@ __device__ __forceinline__ void merge_slots(uint64_t (&ck)[NC], bool (&ok)[NC], 
 // which has only decreased since, so it is left out here (its distance need not have been computed).  canon, sid, smap: see
 // merge_many (the members in ascending id and the columns they have).
 template <int NC>
-__device__ __forceinline__ void merge_row(int i, int irun, bool canon, const int *__restrict__ cid,
+__device__ __forceinline__ bool merge_row(int i, int irun, bool canon, const int *__restrict__ cid,
                                           const int *__restrict__ crun,
                                           const int *__restrict__ sid, const unsigned char *__restrict__ smap,
                                           const float *__restrict__ drow, int ncol, int kappa, const RowRegs &cur,
@@ -329,7 +325,7 @@ __device__ __forceinline__ void merge_row(int i, int irun, bool canon, const int
             }
         }
     }
-    merge_slots<NC>(ck, ok, canon, sid, smap, ncol, kappa, cur, gi, gd, mb);
+    return merge_slots<NC>(ck, ok, canon, sid, smap, ncol, kappa, cur, gi, gd, mb);
 }
 
 }  // namespace gkm

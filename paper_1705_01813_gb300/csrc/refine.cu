@@ -192,7 +192,8 @@ __global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT
                                                                         const int2 *__restrict__ runs,
                                                                         int64_t runs_cap,
                                                                         const RunCounts *__restrict__ cnt, bool longs,
-                                                                        const int32_t *__restrict__ prev, bool canon, int kappa,
+                                                                        const int32_t *__restrict__ prev, bool canon,
+                                                                        uint8_t *__restrict__ row_changed, int kappa,
                                                                         int32_t *__restrict__ g_idx,
                                                                         float *__restrict__ g_dist, DevStatus *st)
 {
@@ -225,9 +226,10 @@ __global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT
                 const int rn = row + RF_WARPS;
                 if (rn < nr && rid[rn] >= 0)  // next row's list in flight during this merge
                     load_row(nxt, g_idx + (int64_t)rid[rn] * kappa, g_dist + (int64_t)rid[rn] * kappa, kappa);
-                if (i >= 0)
-                    merge_row<NC>(i, rpr[row], canon, ci, cp, si, sm, dt + row * DS, ncl, kappa, cur,
-                                  g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mb);
+                if (i >= 0 && merge_row<NC>(i, rpr[row], canon, ci, cp, si, sm, dt + row * DS, ncl, kappa, cur,
+                                            g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mb) &&
+                    row_changed && lane_id() == 0)
+                    row_changed[i] = 1;
                 cur = nxt;
             }
         };
@@ -300,7 +302,8 @@ __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restric
                                                              const int32_t *__restrict__ mem,
                                                              const int2 *__restrict__ runs,
                                                              const RunCounts *__restrict__ cnt,
-                                                             const int32_t *__restrict__ prev, bool canon, int kappa,
+                                                             const int32_t *__restrict__ prev, bool canon,
+                                                                        uint8_t *__restrict__ row_changed, int kappa,
                                                              int32_t *__restrict__ g_idx,
                                                              float *__restrict__ g_dist, DevStatus *st)
 {
@@ -375,9 +378,10 @@ __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restric
                 const int rn = row + WS_NM;
                 if (rn < sz && rid[rn] >= 0)  // next row's list in flight during this merge
                     load_row(nxt, g_idx + (int64_t)rid[rn] * kappa, g_dist + (int64_t)rid[rn] * kappa, kappa);
-                if (i >= 0)
-                    merge_row<T / 32>(i, rpr[row], canon, rid, rpr, sid, smap, dt + row * DS, sz, kappa, cur,
-                                      g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mbufs[mw]);
+                if (i >= 0 && merge_row<T / 32>(i, rpr[row], canon, rid, rpr, sid, smap, dt + row * DS, sz, kappa, cur,
+                                                g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mbufs[mw]) &&
+                    row_changed && lane == 0)
+                    row_changed[i] = 1;
                 cur = nxt;
             }
             __threadfence_block();
@@ -400,7 +404,7 @@ template <typename XT, bool VEC>
 static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                              const int32_t *members, int32_t k, int32_t kappa, int32_t max_cluster, int32_t *g_idx,
                              float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision,
-                             const int32_t *prev_in, int32_t *prev_out, bool canon)
+                             const int32_t *prev_in, int32_t *prev_out, bool canon, uint8_t *row_changed)
 {
     RunCounts *cnt = static_cast<RunCounts *>(scratch);
     int2 *runs = reinterpret_cast<int2 *>(static_cast<char *>(scratch) + 256);
@@ -435,12 +439,12 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
         if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, RF_THREADS, shm, &grid)) != cudaSuccess)
             return e;
         k_refine<128, XT, VEC><<<blocks(grid), RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, true,
-                                                                     prev_in, canon, kappa, g_idx, g_dist, st);
+                                                                     prev_in, canon, row_changed, kappa, g_idx, g_dist, st);
     }
     if (tensor) {
         // tensor-core Gram for runs of <= 128 members
         constexpr bool bf16 = std::is_same_v<XT, __nv_bfloat16>;
-        return launch_refine_tc(X, bf16, n, d, ld, members, runs, cnt, bound, k, kappa, prev_in, canon, g_idx, g_dist, tc_scratch,
+        return launch_refine_tc(X, bf16, n, d, ld, members, runs, cnt, bound, k, kappa, prev_in, canon, row_changed, g_idx, g_dist, tc_scratch,
                                 st, s);
     }
     // runs of <= 64 members.  Rows staged by
@@ -453,7 +457,7 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
         const void *f = reinterpret_cast<const void *>(k_refine_ws<XT, VEC>);
         if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, WS_THREADS, shm, &grid)) != cudaSuccess)
             return e;
-        k_refine_ws<XT, VEC><<<blocks(grid), WS_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, cnt, prev_in, canon, kappa,
+        k_refine_ws<XT, VEC><<<blocks(grid), WS_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, cnt, prev_in, canon, row_changed, kappa,
                                                                    g_idx, g_dist, st);
     } else {
         constexpr size_t shm = refine_smem_bytes<64>();
@@ -461,7 +465,7 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
         if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, RF_THREADS, shm, &grid)) != cudaSuccess)
             return e;
         k_refine<64, XT, VEC><<<blocks(grid), RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, false,
-                                                                    prev_in, canon, kappa, g_idx, g_dist, st);
+                                                                    prev_in, canon, row_changed, kappa, g_idx, g_dist, st);
     }
     return cudaGetLastError();
 }
@@ -472,25 +476,25 @@ template <typename XT>
 static cudaError_t refine_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                             const int32_t *members, int32_t k, int32_t kappa, int32_t max_cluster, int32_t *g_idx,
                             float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision,
-                            const int32_t *prev_in, int32_t *prev_out, bool canon)
+                            const int32_t *prev_in, int32_t *prev_out, bool canon, uint8_t *row_changed)
 {
     if (std::is_same_v<XT, __nv_bfloat16> && tile_vec16(X, (int)d, ld))
         return refine_tv<XT, true>(X, n, d, ld, offsets, members, k, kappa, max_cluster, g_idx, g_dist, scratch, st, s,
-                                   precision, prev_in, prev_out, canon);
+                                   precision, prev_in, prev_out, canon, row_changed);
     return refine_tv<XT, false>(X, n, d, ld, offsets, members, k, kappa, max_cluster, g_idx, g_dist, scratch, st, s,
-                                precision, prev_in, prev_out, canon);
+                                precision, prev_in, prev_out, canon, row_changed);
 }
 
 cudaError_t launch_refine(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                           const int32_t *members, int32_t k, int32_t kappa, int32_t max_cluster, int32_t *g_idx,
                           float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision,
-                          const int32_t *prev_in, int32_t *prev_out, bool canon)
+                          const int32_t *prev_in, int32_t *prev_out, bool canon, uint8_t *row_changed)
 {
     if (bf16)
         return refine_t(static_cast<const __nv_bfloat16 *>(X), n, d, ld, offsets, members, k, kappa, max_cluster,
-                        g_idx, g_dist, scratch, st, s, precision, prev_in, prev_out, canon);
+                        g_idx, g_dist, scratch, st, s, precision, prev_in, prev_out, canon, row_changed);
     return refine_t(static_cast<const float *>(X), n, d, ld, offsets, members, k, kappa, max_cluster, g_idx, g_dist,
-                    scratch, st, s, precision, prev_in, prev_out, canon);
+                    scratch, st, s, precision, prev_in, prev_out, canon, row_changed);
 }
 
 }  // namespace gkm

@@ -455,6 +455,7 @@ __global__ void __launch_bounds__(EX_THREADS) k_refine_exact(const XT *__restric
 constexpr int MG_WARPS = 8;
 
 __global__ void __launch_bounds__(MG_WARPS * 32) k_refine_merge(int64_t n, int kappa, bool canon,
+                                                                uint8_t *__restrict__ row_changed,
                                                                 const int32_t *__restrict__ cand_id,
                                                                 const float *__restrict__ cand_d,
                                                                 const int32_t *__restrict__ cand_n,
@@ -484,8 +485,10 @@ __global__ void __launch_bounds__(MG_WARPS * 32) k_refine_merge(int64_t n, int k
             ok[v] = ck[v] < th;  // a recomputed pair may miss the row after all (~0 for no candidate)
         }
         __syncwarp();
-        merge_slots<S>(ck, ok, canon, cid, nullptr, cnt, kappa, cur, g_idx + i * kappa, g_dist + i * kappa,
-                       reinterpret_cast<MergeBuf<S> &>(mbuf[w]));
+        if (merge_slots<S>(ck, ok, canon, cid, nullptr, cnt, kappa, cur, g_idx + i * kappa, g_dist + i * kappa,
+                           reinterpret_cast<MergeBuf<S> &>(mbuf[w])) &&
+            row_changed && lane == 0)
+            row_changed[i] = 1;
         __syncwarp();
     };
     for (int64_t i = (int64_t)blockIdx.x * MG_WARPS + w; i < n; i += (int64_t)gridDim.x * MG_WARPS) {
@@ -561,7 +564,7 @@ static cudaError_t perm_tensor_map(CUtensorMap *tm, const __nv_bfloat16 *Xp, int
 template <typename XT>
 static cudaError_t refine_tc_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *members, const int2 *runs,
                                RunCounts *cnt, int64_t bound, int32_t k, int32_t kappa, const int32_t *prev, bool canon,
-                               int32_t *g_idx, float *g_dist, void *scratch, DevStatus *st, cudaStream_t s)
+                               uint8_t *row_changed, int32_t *g_idx, float *g_dist, void *scratch, DevStatus *st, cudaStream_t s)
 {
     const size_t a = al256((size_t)n * TC_CAP * sizeof(int32_t));
     const size_t t = al256((size_t)(k + n / 2 + 1) * sizeof(int32_t));
@@ -597,20 +600,20 @@ static cudaError_t refine_tc_t(const XT *X, int64_t n, int64_t d, int64_t ld, co
     int64_t mblocks = (n + MG_WARPS - 1) / MG_WARPS;
     if (mblocks > 152 * 64)
         mblocks = 152 * 64;
-    k_refine_merge<<<(unsigned)mblocks, MG_WARPS * 32, 0, s>>>(n, kappa, canon, cand_id, cand_d, cand_n, g_idx, g_dist);
+    k_refine_merge<<<(unsigned)mblocks, MG_WARPS * 32, 0, s>>>(n, kappa, canon, row_changed, cand_id, cand_d, cand_n, g_idx, g_dist);
     return cudaGetLastError();
 }
 
 cudaError_t launch_refine_tc(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *members,
                              const int2 *runs, RunCounts *cnt, int64_t bound, int32_t k, int32_t kappa,
-                             const int32_t *prev, bool canon, int32_t *g_idx, float *g_dist, void *scratch,
-                             DevStatus *st, cudaStream_t s)
+                             const int32_t *prev, bool canon, uint8_t *row_changed, int32_t *g_idx, float *g_dist,
+                             void *scratch, DevStatus *st, cudaStream_t s)
 {
     if (bf16)
         return refine_tc_t(static_cast<const __nv_bfloat16 *>(X), n, d, ld, members, runs, cnt, bound, k, kappa, prev,
-                           canon, g_idx, g_dist, scratch, st, s);
-    return refine_tc_t(static_cast<const float *>(X), n, d, ld, members, runs, cnt, bound, k, kappa, prev, canon, g_idx,
-                       g_dist, scratch, st, s);
+                           canon, row_changed, g_idx, g_dist, scratch, st, s);
+    return refine_tc_t(static_cast<const float *>(X), n, d, ld, members, runs, cnt, bound, k, kappa, prev, canon,
+                       row_changed, g_idx, g_dist, scratch, st, s);
 }
 
 }  // namespace gkm

@@ -177,7 +177,8 @@ __global__ void __launch_bounds__(UP_WARPS * 32) k_update(const XT *__restrict__
                                                           const int32_t *__restrict__ off,
                                                           const int32_t *__restrict__ mem, int k, int small_max,
                                                           float *__restrict__ C, int32_t *__restrict__ counts,
-                                                          double *__restrict__ contrib, DevStatus *st)
+                                                          double *__restrict__ contrib,
+                                                          const uint8_t *__restrict__ dirty, DevStatus *st)
 {
     using V = typename VecT<VEC>::T;
     static_assert(!PIPE || std::is_same_v<XT, float>, "the cp.async ring moves FP32 rows");
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(UP_WARPS * 32) k_update(const XT *__restrict__
     // clusters r = blockIdx.x, + gridDim.x, ...; those of at most small_max members are k_update_small's
     for (int r = blockIdx.x; r < k; r += gridDim.x) {
     const int beg = off[r], m = off[r + 1] - beg;
-    if (m <= small_max)
+    if (m <= small_max || (dirty && dirty[r] == 0))
         continue;
     if (counts && threadIdx.x == 0)
         counts[r] = m;
@@ -389,7 +390,8 @@ __global__ void __launch_bounds__(US_WARPS * 32, 3) k_update_small(const XT *__r
                                                                 const int32_t *__restrict__ off,
                                                                 const int32_t *__restrict__ mem, int k, int maxm,
                                                                 float *__restrict__ C, int32_t *__restrict__ counts,
-                                                                double *__restrict__ contrib, DevStatus *st)
+                                                                double *__restrict__ contrib,
+                                                          const uint8_t *__restrict__ dirty, DevStatus *st)
 {
     constexpr int RIF = NVL == 1 ? 8 : NVL == 2 ? 4 : 2;  // member rows in flight (registers allowing)
     using RV = RawVec<XT>;
@@ -397,8 +399,8 @@ __global__ void __launch_bounds__(US_WARPS * 32, 3) k_update_small(const XT *__r
     const int nv = d / 4;
     for (int r = blockIdx.x * US_WARPS + w; r < k; r += gridDim.x * US_WARPS) {
         const int beg = off[r], m = off[r + 1] - beg;
-        if (m > maxm)
-            continue;  // a cluster of k_update
+        if (m > maxm || (dirty && dirty[r] == 0))
+            continue;  // a cluster of k_update, or one whose members, sums and distortion term are as they were
         if (counts && lane == 0)
             counts[r] = m;
         if (m == 0) {
@@ -498,7 +500,7 @@ const double *update_contrib(const void *scratch) { return static_cast<const dou
 template <typename XT>
 static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                             const int32_t *members, int32_t k, float *C, int32_t *counts, double *sum_d2,
-                            void *scratch, DevStatus *st, cudaStream_t s)
+                            void *scratch, DevStatus *st, cudaStream_t s, const uint8_t *dirty)
 {
     double *contrib = static_cast<double *>(scratch);
     const bool vec4 = x_vec4(X, d, ld);
@@ -521,7 +523,7 @@ static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
             cudaSuccess)                                                                                         \
             return e;                                                                                            \
         k_update_small<NVL, XT><<<(unsigned)g, US_WARPS * 32, 0, s>>>(X, dd, ld, offsets, members, k, small_max, \
-                                                                      C, counts, contrib, st);                   \
+                                                                      C, counts, contrib, dirty, st);            \
     } while (0)
         if (nv <= 32)
             GK_UPS(1);
@@ -551,7 +553,7 @@ static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     const unsigned grid = (unsigned)(mostly_small ? (k < bg ? k : bg) : k);
 #define GK_UPD(VEC, CPL, P) \
     k_update<VEC, CPL, P, XT><<<grid, UP_WARPS * 32, 0, s>>>(X, dd, ld, offsets, members, k, small_max, C, counts, \
-                                                             contrib, st)
+                                                             contrib, dirty, st)
     if (vec4) {
         if (need <= 1)
             GK_UPD(4, 1, PIPE);
@@ -579,12 +581,13 @@ static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
 
 cudaError_t launch_update(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                           const int32_t *members, int32_t k, float *C, int32_t *counts, double *sum_d2,
-                          void *scratch, DevStatus *st, cudaStream_t s)
+                          void *scratch, DevStatus *st, cudaStream_t s, const uint8_t *dirty)
 {
     if (bf16)
         return update_t(static_cast<const __nv_bfloat16 *>(X), n, d, ld, offsets, members, k, C, counts, sum_d2,
-                        scratch, st, s);
-    return update_t(static_cast<const float *>(X), n, d, ld, offsets, members, k, C, counts, sum_d2, scratch, st, s);
+                        scratch, st, s, dirty);
+    return update_t(static_cast<const float *>(X), n, d, ld, offsets, members, k, C, counts, sum_d2, scratch, st, s,
+                    dirty);
 }
 
 }  // namespace gkm
