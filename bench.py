@@ -270,21 +270,22 @@ class Path:
 
 
 def _radix_passes(k):
-    # 8-bit passes over the sort keys 0..k (k: the key of an out-of-range label)
-    return (int(k).bit_length() + 7) // 8
+    # passes of at most 10 bits over the sort keys 0..k (k: the key of an out-of-range label)
+    return (int(k).bit_length() + 9) // 10
 
 
 def launches_per_step(w, precision):
     """Kernels of this library launched by one step (mirrors the library's launch sequence)."""
-    grp = lambda k: 1 + 3 + 5 * _radix_passes(k)  # noqa: E731
+    # group: three launches a pass, and the offsets' search after several passes
+    grp = lambda k: 3 * _radix_passes(k) + (1 if _radix_passes(k) > 1 else 0)  # noqa: E731
     # update: the warp-per-cluster kernel for clusters of at most 32 members (16-byte rows of at most 512 values),
-    # the block kernel for the others, the FP64 sum
-    upd = 3 if (w.d % 4 == 0 and w.d <= 512) else 2
+    # the block kernel for the others, the FP64 sum (chains and tree: the step's groupings come from their own call)
+    upd = 4 if (w.d % 4 == 0 and w.d <= 512) else 3
 
     def asg(k):
-        # (then reduce and finish): kernel (0, 1); shadow copy + screening kernel (2, 4); BF16 copy, tensor-core
-        # tiles, SIMT leftovers (3)
-        return 3 if precision < 2 else (4 if precision in (2, 4) or w.d > 128 else 5)
+        # (then the reduction): kernel (0, 1); shadow copy + screening kernel (2, 4); BF16 copy, tensor-core tiles,
+        # SIMT leftovers (3)
+        return 2 if precision < 2 else (3 if precision in (2, 4) or w.d > 128 else 4)
     # refine: the run lists, then cluster-sorted copy + Gram + exact recompute + merge (tensor cores) or the two FP32
     # tile widths (runs of max_cluster = 128 members at most)
     ref = 1 + (4 if tc_refine(precision, w.d, w.storage) else 2)

@@ -460,8 +460,9 @@ static int update_step_impl(const void *X, bool bf16, int64_t n, int64_t d, int6
     int32_t *off = offsets ? offsets : L.grp.offsets;
     int32_t *mem = members ? members : L.grp.members;
     int32_t *cnt = counts ? counts : L.grp.counts;
-    GK_CUDA(launch_group(labels, n, k, off, mem, cnt, L.grp.scratch, L.st, s));
-    GK_CUDA(launch_update(X, bf16, n, d, ld, off, mem, k, C, cnt, sum_d2, L.upd_scratch, L.st, s));
+    unsigned *tick = update_ticket(L.upd_scratch, k);
+    GK_CUDA(launch_group(labels, n, k, off, mem, cnt, L.grp.scratch, L.st, s, tick));
+    GK_CUDA(launch_update(X, bf16, n, d, ld, off, mem, k, C, cnt, sum_d2, L.upd_scratch, L.st, s, nullptr, tick));
     return GK_OK;
 }
 
@@ -645,6 +646,7 @@ static int kmeans_fit_impl(const void *X, bool bf16, int64_t n, int64_t d, int64
     cudaStream_t s = (cudaStream_t)stream;
     int32_t *cnt = counts_out ? counts_out : L.grp.counts;
 
+    unsigned *tick = update_ticket(L.upd_scratch, k);
     auto enqueue = [&]() -> int {
         // ping-pong the labels so that the final ones land in labels_out
         int32_t *cur = (iters % 2 == 0) ? labels_out : L.labels_b;
@@ -654,18 +656,18 @@ static int kmeans_fit_impl(const void *X, bool bf16, int64_t n, int64_t d, int64
         else
             GK_CUDA(launch_init_labels(n, k, seed, cur, s));
         GK_CUDA(cudaMemsetAsync(C_out, 0, sizeof(float) * (size_t)k * (size_t)d, s));
-        GK_CUDA(launch_group(cur, n, k, L.grp.offsets, L.grp.members, cnt, L.grp.scratch, L.st, s));
+        GK_CUDA(launch_group(cur, n, k, L.grp.offsets, L.grp.members, cnt, L.grp.scratch, L.st, s, tick));
         GK_CUDA(launch_update(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k, C_out, cnt, L.elog + 0,
-                              L.upd_scratch, L.st, s));
+                              L.upd_scratch, L.st, s, nullptr, tick));
         if (track_of(L, 0, n, d, precision, false).dirty_out)
             GK_CUDA(cudaMemsetAsync(L.todo_n, 0, 256 + (size_t)k, s));
         for (int t = 0; t < iters; t++) {
             const Track trk = track_of(L, t, n, d, precision, false);
             GK_CUDA(launch_assign(X, bf16, n, d, ld, g_idx, kappa, C_out, k, cur, nxt, nullptr, L.elog + 1 + 2 * t,
                                   nullptr, L.asg_scratch, L.st, s, precision, L.grp.members, trk));
-            GK_CUDA(launch_group(nxt, n, k, L.grp.offsets, L.grp.members, cnt, L.grp.scratch, L.st, s));
+            GK_CUDA(launch_group(nxt, n, k, L.grp.offsets, L.grp.members, cnt, L.grp.scratch, L.st, s, tick));
             GK_CUDA(launch_update(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k, C_out, cnt, L.elog + 2 + 2 * t,
-                                  L.upd_scratch, L.st, s, trk.dirty_out));
+                                  L.upd_scratch, L.st, s, trk.dirty_out, tick));
             int32_t *tmp = cur;
             cur = nxt;
             nxt = tmp;
@@ -727,14 +729,15 @@ static int build_knn_graph_impl(const void *X, bool bf16, int64_t n, int64_t d, 
     L = carve(ws, GK_OP_BUILD, n, d, k0);
     cudaStream_t s = (cudaStream_t)stream;
     const int tau = p->tau;
+    unsigned *tick = update_ticket(L.upd_scratch, k0);
     auto enqueue = [&]() -> int {
         int32_t *cur = L.labels_a, *nxt = L.labels_b;
         GK_CUDA(launch_init_graph(X, bf16, n, d, ld, p->kappa, p->seed, g_idx, g_dist, L.st, s));
         GK_CUDA(launch_init_labels(n, k0, p->seed, cur, s));
         GK_CUDA(cudaMemsetAsync(L.cent, 0, sizeof(float) * (size_t)k0 * (size_t)d, s));
-        GK_CUDA(launch_group(cur, n, k0, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s));
+        GK_CUDA(launch_group(cur, n, k0, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s, tick));
         GK_CUDA(launch_update(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k0, L.cent, L.grp.counts, L.elog + 0,
-                              L.upd_scratch, L.st, s));
+                              L.upd_scratch, L.st, s, nullptr, tick));
         if (track_of(L, 0, n, d, p->precision, true).dirty_out) {
             GK_CUDA(cudaMemsetAsync(L.row_changed, 0, (size_t)n, s));
             GK_CUDA(cudaMemsetAsync(L.todo_n, 0, 256 + (size_t)k0, s));
@@ -744,9 +747,9 @@ static int build_knn_graph_impl(const void *X, bool bf16, int64_t n, int64_t d, 
             // one k-means iteration at k0 on the current graph (Sec. 4.5: t = 1 per round)
             GK_CUDA(launch_assign(X, bf16, n, d, ld, g_idx, p->kappa, L.cent, k0, cur, nxt, nullptr, L.elog + 1 + 2 * t,
                                   nullptr, L.asg_scratch, L.st, s, p->precision, L.grp.members, trk));
-            GK_CUDA(launch_group(nxt, n, k0, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s));
+            GK_CUDA(launch_group(nxt, n, k0, L.grp.offsets, L.grp.members, L.grp.counts, L.grp.scratch, L.st, s, tick));
             GK_CUDA(launch_update(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k0, L.cent, L.grp.counts,
-                                  L.elog + 2 + 2 * t, L.upd_scratch, L.st, s, trk.dirty_out));
+                                  L.elog + 2 + 2 * t, L.upd_scratch, L.st, s, trk.dirty_out, tick));
             // exhaustive pairs inside the clusters of the new partition
             GK_CUDA(launch_refine(X, bf16, n, d, ld, L.grp.offsets, L.grp.members, k0, p->kappa, p->max_cluster, g_idx,
                                   g_dist, L.ref_scratch, L.st, s, p->precision & 0xff, t > 0 ? L.prev[(t + 1) & 1] : nullptr,

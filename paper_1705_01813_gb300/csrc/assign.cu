@@ -194,6 +194,8 @@ template <bool LISTS, typename F>
 __device__ __forceinline__ void each_sample(int64_t first, int64_t step, int64_t n, const Track &trk,
                                             const int32_t *__restrict__ todo, F f)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        *trk.ticket = 0u;  // for k_assign_reduce
     if constexpr (!LISTS) {
         for (int64_t i = first; i < n; i += step)
             f(i, std::false_type{});
@@ -671,8 +673,11 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign_rows_bf(const float *_
                                                                   float *__restrict__ best_out,
                                                                   const int32_t *__restrict__ tmem_members, const int32_t *__restrict__ tile_flag,
                                                                const int32_t *__restrict__ sel_lab,
-                                                               const int32_t *__restrict__ sel_n, DevStatus *st)
+                                                               const int32_t *__restrict__ sel_n, DevStatus *st,
+                                                               unsigned *__restrict__ ticket)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        *ticket = 0u;  // for k_assign_reduce
     __shared__ int s_q[AS_WARPS][AS_QCAP];
     __shared__ float s_lo[AS_WARPS][AS_QCAP + 31];
     const int w = threadIdx.x >> 5, lane = lane_id();
@@ -819,24 +824,27 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign_rows_bf(const float *_
     }
 }
 
-// Per-block FP64 sums of best[] and counts of changed labels over fixed index
-// ranges (the same for every kernel that produced best[]), so the total has
-// the same bits whichever assignment kernel ran.
+// FP64 sum of best[] and count of changed labels: per block over fixed index ranges (the same for every kernel that
+// produced best[], so the total has the same bits whichever assignment kernel ran), then over the blocks in the order
+// of 1024 chains and a halving tree, by the last block to finish (trk.ticket; a launch of its own took 3.6 us and a
+// gap).
 __global__ void __launch_bounds__(256) k_assign_reduce(const float *__restrict__ best,
                                                        const int32_t *__restrict__ Lin,
                                                        const int32_t *__restrict__ Lout, int64_t n,
                                                        double *__restrict__ blk_sum,
-                                                       unsigned long long *__restrict__ blk_changed,
-                                                       const Track trk, int k)
+                                                       unsigned long long *__restrict__ blk_changed, const Track trk,
+                                                       int k, double *__restrict__ sum_d2,
+                                                       int64_t *__restrict__ n_changed)
 {
+    static_assert(AS_BLOCKS > 1024 && AS_BLOCKS <= 2048, "two blocks per chain at most");
     if (trk.clear) {  // Track's clears, here to save a launch
         for (int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x; r < k; r += (int64_t)gridDim.x * 256)
             trk.clear[r] = 0;
         if (blockIdx.x == 0 && threadIdx.x < 2)
             trk.todo_n[threadIdx.x] = 0;
     }
-    __shared__ double s[256];
-    __shared__ unsigned long long c[256];
+    __shared__ double s[1024];
+    __shared__ unsigned long long c[1024];
     const int64_t per = (n + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = (int64_t)blockIdx.x * per, b1 = min(n, b0 + per);
     double a = 0.0;
@@ -859,30 +867,21 @@ __global__ void __launch_bounds__(256) k_assign_reduce(const float *__restrict__
         blk_sum[blockIdx.x] = s[0];
         blk_changed[blockIdx.x] = c[0];
     }
-}
-
-__global__ void __launch_bounds__(1024) k_assign_finish(const double *__restrict__ blk_sum,
-                                                        const unsigned long long *__restrict__ blk_changed, int nb,
-                                                        double *__restrict__ sum_d2, int64_t *__restrict__ n_changed)
-{
-    __shared__ double s[1024];
-    __shared__ unsigned long long c[1024];
-    double a = 0.0;
-    unsigned long long b = 0;
-    for (int i = threadIdx.x; i < nb; i += 1024) {
-        a += blk_sum[i];
-        b += blk_changed[i];
-    }
-    s[threadIdx.x] = a;
-    c[threadIdx.x] = b;
-    __syncthreads();
-    for (int w = 512; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            s[threadIdx.x] += s[threadIdx.x + w];
-            c[threadIdx.x] += c[threadIdx.x + w];
+    if (!last_block(trk.ticket))
+        return;
+    for (int q = threadIdx.x; q < 1024; q += 256) {
+        double x = __ldcg(blk_sum + q);
+        unsigned long long y = __ldcg(blk_changed + q);
+        if (q + 1024 < (int)gridDim.x) {
+            x += __ldcg(blk_sum + q + 1024);
+            y += __ldcg(blk_changed + q + 1024);
         }
-        __syncthreads();
+        s[q] = x;
+        c[q] = y;
     }
+    __syncthreads();
+    halving_sum<256>(s, 1024);
+    halving_sum<256>(c, 1024);
     if (threadIdx.x == 0) {
         if (sum_d2)
             *sum_d2 = s[0];
@@ -895,7 +894,7 @@ static size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 
 size_t assign_scratch_bytes(int64_t n, int32_t k, int64_t d)
 {
-    const size_t part = al256((size_t)AS_BLOCKS * (sizeof(double) + sizeof(unsigned long long)));
+    const size_t part = al256((size_t)AS_BLOCKS * (sizeof(double) + sizeof(unsigned long long)) + sizeof(unsigned));
     const size_t shadow = al256((size_t)k * (size_t)d * 2) + 2 * al256((size_t)k * 4);
     const size_t best = al256((size_t)n * 4);
     const size_t tiles = al256((size_t)((n + AS_TILE - 1) / AS_TILE) * 4);
@@ -912,7 +911,8 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     char *sp = static_cast<char *>(scratch);
     double *blk_sum = reinterpret_cast<double *>(sp);
     unsigned long long *blk_chg = reinterpret_cast<unsigned long long *>(blk_sum + AS_BLOCKS);
-    sp += al256((size_t)AS_BLOCKS * (sizeof(double) + sizeof(unsigned long long)));
+    trk.ticket = reinterpret_cast<unsigned *>(blk_chg + AS_BLOCKS);
+    sp += al256((size_t)AS_BLOCKS * (sizeof(double) + sizeof(unsigned long long)) + sizeof(unsigned));
     __nv_bfloat16 *Cb = reinterpret_cast<__nv_bfloat16 *>(sp);
     sp += al256((size_t)k * (size_t)d * 2);
     float *delta = reinterpret_cast<float *>(sp);
@@ -1016,7 +1016,7 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
 #define GK_ASGB(NV, T)                                                                                           \
     k_assign_rows_bf<NV, T><<<AS_BLOCKS, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, Cb, delta, k,   \
                                                                 labels_in, labels_out, best,                        \
-                                                                members, tile_flag, sel_lab, sel_n, st)
+                                                                members, tile_flag, sel_lab, sel_n, st, trk.ticket)
             if (tiles) {
                 GK_ASGB(1, true);  // d <= 128 on the tensor-core path
             } else if (d4 <= 32) {
@@ -1086,8 +1086,8 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
             return e;
     }
     if (sum_d2 || n_changed) {
-        k_assign_reduce<<<AS_BLOCKS, 256, 0, s>>>(best, labels_in, labels_out, n, blk_sum, blk_chg, trk, k);
-        k_assign_finish<<<1, 1024, 0, s>>>(blk_sum, blk_chg, AS_BLOCKS, sum_d2, n_changed);
+        k_assign_reduce<<<AS_BLOCKS, 256, 0, s>>>(best, labels_in, labels_out, n, blk_sum, blk_chg, trk, k, sum_d2,
+                                                  n_changed);
     } else if (trk.clear) {
         if ((e = cudaMemsetAsync(trk.clear, 0, (size_t)k, s)) != cudaSuccess ||
             (e = cudaMemsetAsync(trk.todo_n, 0, 2 * sizeof(int32_t), s)) != cudaSuccess)

@@ -159,6 +159,33 @@ __device__ __forceinline__ void bar_arrive(int id, int count)
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
+// True in every thread of the last of the grid's blocks to get here: what the other blocks wrote before may be read
+// (through L2).  ticket counts the blocks and starts at zero.  Called by all threads of the block.
+__device__ __forceinline__ bool last_block(unsigned *ticket)
+{
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0)
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (last)
+        __threadfence();
+    return last;
+}
+
+// The pairwise sum s[0] of s[0 .. 1024) that halving steps of 1024 threads give (s[t] += s[t + w], w = 512, 256, ...,
+// 1), by T threads; entries from count on are zero, which the steps skip (x + 0 = x).
+template <int T, typename V>
+__device__ __forceinline__ void halving_sum(V *s, int count)
+{
+    for (int w = 512; w > 0; w >>= 1) {
+        for (int t = threadIdx.x; t < w && t + w < count; t += T)
+            s[t] += s[t + w];
+        __syncthreads();
+    }
+}
+
 // 16-byte asynchronous copy global -> shared (both 16-byte aligned, L2 only),
 // grouping of the copies issued so far, and waits on the groups.
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
@@ -236,14 +263,11 @@ cudaError_t launch_init_graph(const void *X, bool bf16, int64_t n, int64_t d, in
                               uint64_t seed, int32_t *g_idx, float *g_dist, DevStatus *st, cudaStream_t s,
                               int32_t id_offset = 0);
 
-// Grouping of samples by label (CSR).  Scratch sizes via group_scratch_bytes().
+// Grouping of samples by label (CSR).  Scratch sizes via group_scratch_bytes().  counts_out may be NULL; zero (may be
+// NULL): a counter that the grouping clears for a later kernel of the caller.
 size_t group_scratch_bytes(int64_t n, int32_t k);
 cudaError_t launch_group(const int32_t *labels, int64_t n, int32_t k, int32_t *offsets, int32_t *members,
-                         int32_t *counts_out, void *scratch, DevStatus *st, cudaStream_t s);
-
-// Exclusive scan of int32 counts (count elements) into out (count + 1 elements, out[count] = total).
-size_t scan_scratch_bytes(int64_t count);
-cudaError_t launch_scan(const int32_t *in, int32_t *out, int64_t count, void *scratch, cudaStream_t s);
+                         int32_t *counts_out, void *scratch, DevStatus *st, cudaStream_t s, unsigned *zero = nullptr);
 
 size_t update_scratch_bytes(int64_t n, int32_t k);
 // the per-cluster distortion terms the last launch_update left in its scratch (k doubles)
@@ -257,7 +281,10 @@ cudaError_t launch_batch_labels(const int32_t *labels, int64_t N, const BatchTab
                                 cudaStream_t s);
 cudaError_t launch_update(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                           const int32_t *members, int32_t k, float *C, int32_t *counts, double *sum_d2,
-                          void *scratch, DevStatus *st, cudaStream_t s, const uint8_t *dirty = nullptr);
+                          void *scratch, DevStatus *st, cudaStream_t s, const uint8_t *dirty = nullptr,
+                          unsigned *ticket = nullptr);
+// a counter in the update's scratch that launch_group can clear (its `zero`) for launch_update's ticket
+unsigned *update_ticket(void *scratch, int32_t k);
 
 // What changed since the previous assignment of the same samples, kept by the callers that run several in a row (one
 // fit, one graph construction); bytes, non-zero for "changed".  An update that finds a cluster's members unchanged
@@ -268,6 +295,7 @@ struct Track {
     uint8_t *row_changed;      // n: the graph row changed since the previous assignment, read and cleared (NULL: none)
     uint8_t *clear;            // k: zeroed after this assignment (the next one's dirty_out; may be `dirty`)
     int32_t *todo_n;           // two counters, zeroed before and after the assignment
+    unsigned *ticket;          // set by launch_assign: block counter of the distance sum, cleared by the row kernels
 };
 size_t assign_scratch_bytes(int64_t n, int32_t k, int64_t d);
 // precision 0 and 1: FP32 candidate rows; 2: BF16 screening on the SIMT cores; 3: on the tensor cores over

@@ -120,8 +120,9 @@ extern "C" GK_API int gk_update_step_noalloc(const float *X, int64_t n, int64_t 
     // the status word keeps the previous call's value: clear it (the grouping
     // zeroes its own counters; everything else is overwritten before it is read)
     if ((e = cudaMemsetAsync(st, 0, sizeof(DevStatus), s)) == cudaSuccess &&
-        (e = launch_group(labels, n, k, off, mem, cnt, gscratch, st, s)) == cudaSuccess)
-        e = launch_update(X, false, n, d, ld, off, mem, k, C, cnt, sum_d2, uscratch, st, s);
+        (e = launch_group(labels, n, k, off, mem, cnt, gscratch, st, s, update_ticket(uscratch, k))) == cudaSuccess)
+        e = launch_update(X, false, n, d, ld, off, mem, k, C, cnt, sum_d2, uscratch, st, s, nullptr,
+                          update_ticket(uscratch, k));
     if (e != cudaSuccess) {
         return report(GK_ERR_CUDA, "launch failed: %s", cudaGetErrorString(e));
     }

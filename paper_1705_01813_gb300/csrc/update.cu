@@ -474,33 +474,62 @@ __global__ void __launch_bounds__(US_WARPS * 32, 3) k_update_small(const XT *__r
     }
 }
 
-// Deterministic FP64 sum of `count` values (one block, fixed order).
-__global__ void __launch_bounds__(1024) k_sum_f64(const double *__restrict__ v, int64_t count,
-                                                  double *__restrict__ out)
+// Deterministic FP64 sum of `count` values: 1024 chains, chain t adding every 1024th value from t on in order, then the
+// halving tree over the chains.  A warp per 32 chains (SUM_BLOCKS of them, on as many SMs: FP64 additions bound the sum,
+// one block took 63 us at 200,000 values), eight loads ahead of their additions; the last block to finish adds the
+// chains up (ticket), or the caller launches the tree as one block of its own (ticket NULL: partial only).
+constexpr int SUM_BLOCKS = 32;
+
+__global__ void __launch_bounds__(32) k_sum_f64(const double *__restrict__ v, int64_t count, double *__restrict__ part,
+                                                unsigned *__restrict__ ticket, double *__restrict__ out)
 {
     __shared__ double s[1024];
-    double a = 0.0;
-    for (int64_t i = threadIdx.x; i < count; i += 1024)
-        a += v[i];
-    s[threadIdx.x] = a;
-    __syncthreads();
-    for (int w = 512; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w)
-            s[threadIdx.x] += s[threadIdx.x + w];
-        __syncthreads();
+    const int t = blockIdx.x * 32 + threadIdx.x;
+    if (part) {
+        constexpr int Q = 8;
+        double a = 0.0;
+        int64_t i = t;
+        for (; i + (Q - 1) * 1024 < count; i += Q * 1024) {
+            double x[Q];
+#pragma unroll
+            for (int q = 0; q < Q; q++)
+                x[q] = v[i + q * 1024];
+#pragma unroll
+            for (int q = 0; q < Q; q++)
+                a += x[q];
+        }
+        for (; i < count; i += 1024)
+            a += v[i];
+        part[t] = a;
+        if (!ticket || !last_block(ticket))
+            return;
+        v = part;
     }
+    const int m = count < 1024 ? (int)count : 1024;
+    for (int q = threadIdx.x; q < m; q += 32)
+        s[q] = __ldcg(v + q);
+    __syncthreads();
+    halving_sum<32>(s, m);
     if (threadIdx.x == 0)
         *out = s[0];
 }
 
-size_t update_scratch_bytes(int64_t, int32_t k) { return ((size_t)k * sizeof(double) + 255) & ~size_t(255); }
+// the clusters' terms, the 1024 chains of their sum, the counter
+static size_t contrib_bytes(int32_t k) { return ((size_t)k * sizeof(double) + 255) & ~size_t(255); }
+
+size_t update_scratch_bytes(int64_t, int32_t k) { return contrib_bytes(k) + 1024 * sizeof(double) + 256; }
+
+unsigned *update_ticket(void *scratch, int32_t k)
+{
+    return reinterpret_cast<unsigned *>(static_cast<char *>(scratch) + contrib_bytes(k) + 1024 * sizeof(double));
+}
 
 const double *update_contrib(const void *scratch) { return static_cast<const double *>(scratch); }
 
 template <typename XT>
 static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                             const int32_t *members, int32_t k, float *C, int32_t *counts, double *sum_d2,
-                            void *scratch, DevStatus *st, cudaStream_t s, const uint8_t *dirty)
+                            void *scratch, DevStatus *st, cudaStream_t s, const uint8_t *dirty, unsigned *ticket)
 {
     double *contrib = static_cast<double *>(scratch);
     const bool vec4 = x_vec4(X, d, ld);
@@ -574,20 +603,24 @@ static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
             GK_UPD(1, 8, false);
     }
 #undef GK_UPD
-    if (sum_d2)
-        k_sum_f64<<<1, 1024, 0, s>>>(contrib, k, sum_d2);
+    if (sum_d2) {
+        double *part = reinterpret_cast<double *>(static_cast<char *>(scratch) + contrib_bytes(k));
+        k_sum_f64<<<SUM_BLOCKS, 32, 0, s>>>(contrib, k, part, ticket, sum_d2);
+        if (!ticket)
+            k_sum_f64<<<1, 32, 0, s>>>(part, k, nullptr, nullptr, sum_d2);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_update(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *offsets,
                           const int32_t *members, int32_t k, float *C, int32_t *counts, double *sum_d2,
-                          void *scratch, DevStatus *st, cudaStream_t s, const uint8_t *dirty)
+                          void *scratch, DevStatus *st, cudaStream_t s, const uint8_t *dirty, unsigned *ticket)
 {
     if (bf16)
         return update_t(static_cast<const __nv_bfloat16 *>(X), n, d, ld, offsets, members, k, C, counts, sum_d2,
-                        scratch, st, s, dirty);
+                        scratch, st, s, dirty, ticket);
     return update_t(static_cast<const float *>(X), n, d, ld, offsets, members, k, C, counts, sum_d2, scratch, st, s,
-                    dirty);
+                    dirty, ticket);
 }
 
 }  // namespace gkm
