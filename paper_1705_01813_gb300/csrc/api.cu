@@ -150,7 +150,7 @@ Layout carve(void *ws, int op, int64_t n, int64_t d, int32_t k)
         L.row_changed = cv.take<uint8_t>((size_t)n);
     }
     if (op == GK_OP_RECALL)  // k: the number of queries
-        L.rec_scratch = cv.take<char>(recall_scratch_bytes(n, k));
+        L.rec_scratch = cv.take<char>(recall_scratch_bytes(n, d, k));
     if (op == GK_OP_TREE)
         L.tree_scratch = cv.take<char>(tree_scratch_bytes(n, d, k));
     L.bytes = cv.off;

@@ -235,7 +235,7 @@ cudaError_t set_max_smem(const void *kernel, int bytes);
 cudaError_t resident_grid(const void *kernel, int threads, size_t smem, int *grid);
 
 // top-1 recall of a graph on sampled queries (recall.cu)
-size_t recall_scratch_bytes(int64_t n, int32_t m);
+size_t recall_scratch_bytes(int64_t n, int64_t d, int32_t m);
 cudaError_t launch_recall(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *g_idx,
                           int32_t kappa, const int32_t *queries, int32_t m, int32_t *nn_idx, float *nn_dist,
                           int64_t *hits, void *scratch, DevStatus *st, cudaStream_t s);

@@ -10,14 +10,19 @@
 //
 // k_nn_tiles: block (b, s) takes the 64 queries of query block b and the
 // samples of slice s, 64 at a time, as 64 x 64 distance tiles; each warp keeps
-// the smallest (distance, id) key of eight queries over the slice.
-// k_nn_finish: per query the smallest key over the slices, the hit test, and
-// the count of hits.
+// the smallest (distance, id) key of eight queries over the slice, and the
+// slices meet in best[] by atomic minimum.  Where there is enough to screen
+// (recall_screened) the tensor cores find the keys first (recall_tc.cu) and
+// the tiles take only the queries that are left, mostly none.
+// k_nn_finish: the hit test, and the count of hits.
 #include "common.cuh"
 #include "merge.cuh"
+#include "recall.cuh"
 #include "tiles.cuh"
 
 #include <cuda_bf16.h>
+
+#include <type_traits>
 
 namespace gkm {
 
@@ -35,15 +40,26 @@ int recall_slices(int64_t n, int32_t m)
     return (int)(s > tiles ? tiles : s);
 }
 
-size_t recall_scratch_bytes(int64_t n, int32_t m)
+// The screening pays from RECALL_SCREEN_MIN pair coordinates on: 10,000 x 128, 1,000 queries 144 against 184 us,
+// 1M x 32, 40 queries 203 against 243, 8,000 x 960, 200 queries 221 against 250; at 6.4e8 (10,000 x 64, 1,000 queries)
+// the tiles take 110 us, the screening's seven launches and 256 queries at a time about as much.
+constexpr double RECALL_SCREEN_MIN = 1.0e9;
+
+static bool recall_screened(int64_t n, int64_t d, int32_t m) { return (double)n * (double)d * (double)m >= RECALL_SCREEN_MIN; }
+
+static size_t best_bytes(int32_t m) { return ((size_t)m * sizeof(uint64_t) + 255) & ~size_t(255); }
+
+size_t recall_scratch_bytes(int64_t n, int64_t d, int32_t m)
 {
-    return (((size_t)m * (size_t)recall_slices(n, m) * sizeof(uint64_t)) + 255) & ~size_t(255);
+    return best_bytes(m) + (recall_screened(n, d, m) ? recall_screen_bytes(d, m) : 0);
 }
 
 template <typename XT>
 __global__ void __launch_bounds__(RF_THREADS) k_nn_tiles(const XT *__restrict__ X, int64_t n, int d, int64_t ld,
                                                         const int32_t *__restrict__ queries, int m, int slices,
-                                                        uint64_t *__restrict__ part, DevStatus *st)
+                                                        const int32_t *__restrict__ left,
+                                                        const int32_t *__restrict__ nleft,
+                                                        uint64_t *__restrict__ bestq, DevStatus *st)
 {
     using TL = RefineTile<NN_T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -54,13 +70,17 @@ __global__ void __launch_bounds__(RF_THREADS) k_nn_tiles(const XT *__restrict__ 
     int *cid = rid + NN_T;
     uint64_t *best = reinterpret_cast<uint64_t *>(cid + NN_T);
     const int tid = threadIdx.x, w = tid >> 5, lane = lane_id();
-    const int q0 = blockIdx.x * NN_T, nr = min(NN_T, m - q0);
+    // left (may be NULL): the queries to take, *nleft of them, instead of all m
+    const int q0 = blockIdx.x * NN_T, nr = min(NN_T, (left ? *nleft : m) - q0);
+    if (nr <= 0)
+        return;
+    auto index = [&](int t) { return left ? left[q0 + t] : q0 + t; };
     const int64_t tiles = (n + NN_T - 1) / NN_T;
     const int64_t t_lo = tiles * blockIdx.y / slices, t_hi = tiles * (blockIdx.y + 1) / slices;
     if (tid < NN_T) {
-        int q = tid < nr ? queries[q0 + tid] : -1;
+        int q = tid < nr ? queries[index(tid)] : -1;
         if (q >= n) {
-            flag_error(st, GK_ERR_INVALID, (unsigned)(q0 + tid));
+            flag_error(st, GK_ERR_INVALID, (unsigned)index(tid));
             q = -1;
         }
         rid[tid] = q;
@@ -94,19 +114,17 @@ __global__ void __launch_bounds__(RF_THREADS) k_nn_tiles(const XT *__restrict__ 
     }
     __syncthreads();
     if (tid < nr)
-        part[(int64_t)(q0 + tid) * slices + blockIdx.y] = best[tid];
+        atomicMin(reinterpret_cast<unsigned long long *>(bestq + index(tid)), (unsigned long long)best[tid]);
 }
 
-__global__ void k_nn_finish(const uint64_t *__restrict__ part, int m, int slices, const int32_t *__restrict__ queries,
-                            int64_t n, const int32_t *__restrict__ g_idx, int kappa, int32_t *__restrict__ nn_idx,
+__global__ void k_nn_finish(const uint64_t *__restrict__ best, int m, const int32_t *__restrict__ queries, int64_t n,
+                            const int32_t *__restrict__ g_idx, int kappa, int32_t *__restrict__ nn_idx,
                             float *__restrict__ nn_dist, unsigned long long *__restrict__ hits)
 {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= m)
         return;
-    uint64_t k = ~0ull;
-    for (int s = 0; s < slices; s++)
-        k = min(k, part[(int64_t)q * slices + s]);
+    const uint64_t k = best[q];
     const int qi = queries[q];
     const bool found = k != ~0ull && qi >= 0 && qi < n;
     const int id = found ? key_id(k) : -1;
@@ -129,11 +147,18 @@ static cudaError_t recall_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     if ((e = cudaMemsetAsync(hits, 0, sizeof(int64_t), s)) != cudaSuccess)
         return e;
     const int slices = recall_slices(n, m);
-    uint64_t *part = static_cast<uint64_t *>(scratch);
+    uint64_t *best = static_cast<uint64_t *>(scratch);
+    if ((e = cudaMemsetAsync(best, 0xff, sizeof(uint64_t) * (size_t)m, s)) != cudaSuccess)
+        return e;
+    const int32_t *left = nullptr, *nleft = nullptr;
+    if (recall_screened(n, d, m) &&
+        (e = launch_recall_screen(X, std::is_same_v<XT, __nv_bfloat16>, n, d, ld, g_idx, kappa, queries, m, best,
+                                  static_cast<char *>(scratch) + best_bytes(m), &left, &nleft, st, s)) != cudaSuccess)
+        return e;
     const dim3 grid((unsigned)nn_qblocks(m), (unsigned)slices);
-    k_nn_tiles<XT><<<grid, RF_THREADS, NN_SMEM, s>>>(X, n, (int)d, ld, queries, m, slices, part, st);
-    k_nn_finish<<<(m + 255) / 256, 256, 0, s>>>(part, m, slices, queries, n, g_idx, kappa, nn_idx, nn_dist,
-                                                 reinterpret_cast<unsigned long long *>(hits));
+    k_nn_tiles<XT><<<grid, RF_THREADS, NN_SMEM, s>>>(X, n, d, ld, queries, m, slices, left, nleft, best, st);
+    k_nn_finish<<<(m + 255) / 256, 256, 0, s>>>(best, m, queries, n, g_idx, kappa, nn_idx, nn_dist,
+                                                reinterpret_cast<unsigned long long *>(hits));
     return cudaGetLastError();
 }
 
