@@ -950,8 +950,9 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     if ((precision == 2 || precision == 4) && vec4 && d4 <= 32 * 8) {
         // the shadow: BF16 (2) or int8 with a per-row scale (4); the int8 codes take the BF16 shadow's space
         const int sgrid = (k + 7) / 8 < 152 * 16 ? (k + 7) / 8 : 152 * 16;
-        // int8 rows lane-major where every lane owns whole vectors (d a multiple of 128): one load per lane and row
-        const bool lane_major = precision == 4 && d % 128 == 0;
+        // int8 rows lane-major where a screening kernel has whole vectors in every lane (d = 128, 256, 512, 1024: the
+        // kernels' d4 == 32 NV below): one load per lane and row
+        const bool lane_major = precision == 4 && (d4 == 32 || d4 == 64 || d4 == 128 || d4 == 256);
         if (precision == 2)
             k_shadow_bf16<<<sgrid, 256, 0, s>>>(C, k, (int)d, Cb, delta, cnorm, trk.dirty);
         else
