@@ -283,9 +283,11 @@ def launches_per_step(w, precision):
     upd = 4 if (w.d % 4 == 0 and w.d <= 512) else 3
 
     def asg(k):
-        # (then the reduction): kernel (0, 1); shadow copy + screening kernel (2, 4); BF16 copy, tensor-core tiles,
-        # SIMT leftovers (3)
-        return 2 if precision < 2 else (3 if precision in (2, 4) or w.d > 128 else 4)
+        # (then the reduction): kernel (0, 1; wide rows of large sets take the int8 screening); shadow copy + screening
+        # kernel (2, 4); BF16 copy, tensor-core tiles, SIMT leftovers (3)
+        if precision < 2:
+            return 3 if w.d % 4 == 0 and 320 < w.d <= 1024 and w.n * w.d >= 1 << 22 else 2
+        return 3 if precision in (2, 4) or w.d > 128 else 4
     # refine: the run lists, then cluster-sorted copy + Gram + exact recompute + merge (tensor cores) or the two FP32
     # tile widths (runs of max_cluster = 128 members at most)
     ref = 1 + (4 if tc_refine(precision, w.d, w.storage) else 2)

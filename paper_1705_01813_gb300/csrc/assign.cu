@@ -443,9 +443,8 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
     });
 }
 
-// k_assign_rows with the candidate distances screened against a shadow copy of
-// the centroids: BF16 rows (FMT 0, half the bytes per candidate row) or int8
-// rows with a per-row scale (FMT 1, a quarter).  Pass 1 takes every
+// k_assign_rows with the candidate distances screened against a BF16 shadow of
+// the centroids (half the bytes per candidate row).  Pass 1 takes every
 // candidate's distance D~ to the shadow row as k_assign_rows does (same lane
 // layout, same candidate groups, shadow values widened exactly); with delta_r >=
 // ||C_r - Cb_r||, |D - D~| <= delta_r (2 sqrt(D~) + delta_r) for the exact
@@ -456,14 +455,10 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
 // so the winner and its distance are that kernel's bit for bit.  The samples
 // (FP32 or BF16, widened exactly) enter both passes unrounded: the bound covers
 // the centroids' rounding alone.
-// Shadow formats of the screening: FMT 0 BF16 rows (4 values per 8 bytes), FMT 1 int8 rows with a per-row
-// scale s_r (4 values per 4 bytes; see lane_partial_q8), half the bytes again; FMT 2 the same int8 rows stored
-// lane-major (d a multiple of 128), so that a lane's share of a row is one vector load.
-template <int NV, typename XT, int GS, int FMT, bool LISTS>
+template <int NV, typename XT, int GS, bool LISTS>
 __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV == 4 ? 4 : 3)) k_assign_rows_scr(
     const XT *__restrict__ X, int64_t n, int d, int64_t ld, const int32_t *__restrict__ G, int kappa,
-    const float *__restrict__ C, const void *__restrict__ Cs, const float *__restrict__ delta,
-    const float *__restrict__ scale, int k, const int32_t *__restrict__ Lin, int32_t *__restrict__ Lout,
+    const float *__restrict__ C, const void *__restrict__ Cs, const float *__restrict__ delta, int k, const int32_t *__restrict__ Lin, int32_t *__restrict__ Lout,
     float *__restrict__ best_out, DevStatus *st, const Track trk, const int32_t *__restrict__ todo)
 {
     __shared__ __align__(16) int s_q[AS_WARPS][AS_QROW];
@@ -476,8 +471,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV 
     static_assert(GS == 4 || GS == 8, "candidates per group: 4 or 8");
     const int d4 = d >> 2;
     const float4 *C4 = reinterpret_cast<const float4 *>(C);
-    const uint2 *Cb4 = static_cast<const uint2 *>(Cs);       // FMT 0: 4 BF16 per 8 bytes
-    const uint32_t *Cq4 = static_cast<const uint32_t *>(Cs);  // FMT 1: 4 int8 per 4 bytes
+    const uint2 *Cb4 = static_cast<const uint2 *>(Cs);  // 4 BF16 per 8 bytes
     const float gam = (float)(d + 8) * 5.9604645e-8f;         // FP32 rounding of a d-term sum, relative
 
     each_sample<LISTS>((int64_t)blockIdx.x * AS_WARPS + w, (int64_t)gridDim.x * AS_WARPS, n, trk, todo,
@@ -518,18 +512,8 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV 
             float part[GS];
 #pragma unroll
             for (int c = 0; c < GS; c++) {
-                if constexpr (FMT == 0) {
-                    const uint2 *row = Cb4 + (int64_t)lab[c] * d4;
-                    part[c] = lane_partial<NV>(xv, d4, [&](int col) { return bf16x4_to_float4(__ldg(row + col)); });
-                } else if constexpr (FMT == 1) {
-                    const uint32_t *row = Cq4 + (int64_t)lab[c] * d4;
-                    part[c] = lane_partial_q8<NV>(xv, d4, -__ldg(scale + lab[c]),
-                                                  [&](int col) { return __ldg(row + col); });
-                } else {  // FMT 2: lane-major int8 rows, d = 128 NV
-                    uint32_t wq[NV];
-                    load_q8w<NV>(Cq4 + (int64_t)lab[c] * d4, wq);
-                    part[c] = lane_partial_q8w<NV>(xv, -__ldg(scale + lab[c]), wq);
-                }
+                const uint2 *row = Cb4 + (int64_t)lab[c] * d4;
+                part[c] = lane_partial<NV>(xv, d4, [&](int col) { return bf16x4_to_float4(__ldg(row + col)); });
             }
             const float dt = transpose_reduce<GS>(part);
             const int cl = lane / (32 / GS);
@@ -596,8 +580,9 @@ __global__ void k_shadow_bf16(const float *__restrict__ C, int k, int d, __nv_bf
 }
 
 // Int8 shadow of the centroids: per row r the scale s_r = max_t |C_rt| / 127 (1 for a zero row), codes
-// q_rt = rint(C_rt / s_r) (the quotient taken as a product with 1 / s_r) clamped to [-127, 127] and stored as
-// q + 128, four per 32-bit word in the order of the row's values, and delta_r >= ||C_r - q_r s_r||, in FP32
+// q_rt = rint(C_rt / s_r) (the quotient taken as a product with 1 / s_r) in [-127, 127], coordinate t at byte t of a
+// row of 16 * units bytes (zeros past d), and meta[r] = {s_r, s_r^2 sum q^2, delta_r, 0} with
+// delta_r >= ||C_r - q_r s_r||, in FP32
 // only.  Each error v - q s is formed as (v - p) - e with p = fl(q s) and e = fma(q, s, -p) (q s = p + e
 // exactly); v - p is exact where p/2 <= v <= 2p (Sterbenz; |q| >= 1 puts v within half a step of q s), so the
 // computed error is within 2u |v - q s| + 1.01 u^2 max|C_r| of the true one (u = 2^-24).  The errors are squared
@@ -605,53 +590,245 @@ __global__ void k_shadow_bf16(const float *__restrict__ C, int k, int d, __nv_bf
 // summed in FP32 (d fma steps and the warp's 5 additions: relative error below gamma_(d+5), one more u for the
 // division by w); delta_r inflates the square root by (d + 24) 1.2e-7 and 1e-5 (the 1 / (1 - 2u) above and this
 // evaluation's own roundings) and adds sqrt(d) 4e-15 max|C_r| (the absolute term, which also covers squares
-// below the normal range): a rigorous upper bound, no FP64.
-__global__ void k_shadow_i8(const float *__restrict__ C, int k, int d, bool lane_major, uint32_t *__restrict__ Cq,
-                            float *__restrict__ delta, float *__restrict__ scale,
-                            const uint8_t *__restrict__ dirty)
+// below the normal range): a rigorous upper bound, no FP64.  sum q^2 <= 1024 * 127^2 is exact in FP32.  A row that is
+// not finite has zero codes and an infinite delta_r (always recomputed).
+__global__ void k_shadow_i8(const float *__restrict__ C, int k, int d, int units, uint32_t *__restrict__ Cq,
+                            float4 *__restrict__ meta, const uint8_t *__restrict__ dirty)
 {
     const int lane = lane_id();
-    const int d4 = d >> 2;
+    const int d4 = d >> 2, words = units * 4;
     for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < k; r += gridDim.x * (blockDim.x >> 5)) {
         if (dirty && dirty[r] == 0)
             continue;  // the row, and so its shadow, is as the previous assignment left it
         const float4 *row = reinterpret_cast<const float4 *>(C + (int64_t)r * d);
-        float mx = 0.f;
+        unsigned mb = 0;  // the largest magnitude's bits (in order; infinities and NaN above every number)
         for (int col = lane; col < d4; col += 32) {
             const float4 v = row[col];
-            mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+            mb = max(max(mb, __float_as_uint(fabsf(v.x))), __float_as_uint(fabsf(v.y)));
+            mb = max(max(mb, __float_as_uint(fabsf(v.z))), __float_as_uint(fabsf(v.w)));
         }
-        for (int o = 16; o > 0; o >>= 1)
-            mx = fmaxf(mx, __shfl_xor_sync(FULL_MASK, mx, o));
+        mb = __reduce_max_sync(FULL_MASK, mb);
+        const bool finite = mb < 0x7f800000u;
+        const float mx = finite ? __uint_as_float(mb) : 0.f;
         const float sc = mx > 0.f ? mx / 127.f : 1.f;
         const float inv = 1.f / sc;
         const float wu = fmaxf(sc, 1.17549435e-38f), winv = 1.f / wu;  // error unit (FLT_MIN at least)
         float e = 0.f;
-        for (int col = lane; col < d4; col += 32) {
-            const float4 v = row[col];
-            const float vals[4] = {v.x, v.y, v.z, v.w};
+        int qq = 0;
+        for (int col = lane; col < words; col += 32) {
             uint32_t word = 0;
+            if (finite && col < d4) {
+                const float4 v = row[col];
+                const float vals[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const float qf = fminf(127.f, fmaxf(-127.f, rintf(vals[q] * inv)));
-                word |= (uint32_t)((int)qf + 128) << (8 * q);
-                const float p = qf * sc;
-                const float pe = fmaf(qf, sc, -p);  // q s = p + pe exactly
-                const float z = ((vals[q] - p) - pe) * winv;
-                e = fmaf(z, z, e);
+                for (int q = 0; q < 4; q++) {
+                    const float qf = fminf(127.f, fmaxf(-127.f, rintf(vals[q] * inv)));
+                    const int qi = (int)qf;
+                    word |= (uint32_t)(qi & 0xff) << (8 * q);
+                    qq += qi * qi;
+                    const float p = qf * sc;
+                    const float pe = fmaf(qf, sc, -p);  // q s = p + pe exactly
+                    const float z = ((vals[q] - p) - pe) * winv;
+                    e = fmaf(z, z, e);
+                }
             }
-            // row-major: word col; lane-major (d4 = 32 nv): the word of vector col = l + 32 v goes to l nv + v
-            const int nv = d4 >> 5;
-            Cq[(int64_t)r * d4 + (lane_major ? (col & 31) * nv + (col >> 5) : col)] = word;
+            Cq[(int64_t)r * words + col] = word;
         }
         for (int o = 16; o > 0; o >>= 1)
             e += __shfl_xor_sync(FULL_MASK, e, o);
+        qq = __reduce_add_sync(FULL_MASK, qq);
         if (lane == 0) {
-            delta[r] = sqrtf(e * (1.f + (float)(d + 24) * 1.2e-7f)) * 1.00001f * wu + sqrtf((float)d) * 4e-15f * mx +
-                       1e-30f;
-            scale[r] = sc;
+            const float delta = sqrtf(e * (1.f + (float)(d + 24) * 1.2e-7f)) * 1.00001f * wu +
+                                sqrtf((float)d) * 4e-15f * mx + 1e-30f;
+            meta[r] = finite ? make_float4(sc, sc * sc * (float)qq, delta, 0.f)
+                             : make_float4(0.f, 0.f, __int_as_float(0x7f800000), 0.f);
         }
     }
+}
+
+// Four signed bytes by four, added to c.
+__device__ __forceinline__ int dot4(uint32_t a, uint32_t b, int c) { return __dp4a((int)a, (int)b, c); }
+
+// k_assign_rows with the candidates screened against the int8 shadow in integer arithmetic.  The sample is coded in 15
+// bits, x_t = s_x (128 h_t + l_t) + error with s_x = max|x| / 16256 and signed bytes h, l, so that a candidate's
+// product with it is exact in two __dp4a per four coordinates, where widening the codes to FP32 took ten instructions
+// (and bounded this pass: 75 warp instructions a candidate at d = 512, about 20 now).  A row of the shadow is 16 * LPR *
+// NW bytes (the smallest that hold d): LPR lanes read one candidate's row, 16 bytes each, NW times, so a warp takes 32 /
+// LPR candidates at once.  With X2 = |x~|^2 and C2 = |c~|^2 of the coded vectors,
+//   D~ = X2 + C2 - 2 s_x s_r dot,
+// the true distance's root is within delta = delta_r + 0.51 s_x sqrt(d) of the coded one's; to
+// E = delta (2 sqrt(D~ + er) + delta) come er = 64 2^-24 (X2 + C2) for the FP32 evaluation of D~ (X2 summed over at most
+// 32 terms a lane and 5 steps) and the rounding gam of the canonical sum.  Pass 2 recomputes every candidate whose lower
+// value does not exceed the smallest upper value, as the BF16 form does, with the same bits.  A sample that is not
+// finite, or with at most Q8_FEW candidates, goes to pass 2 whole.
+constexpr int Q8_FEW = 3;
+
+template <int LPR, int NW, int NV, typename XT, bool LISTS>
+__global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k_assign_rows_scr(
+    const XT *__restrict__ X, int64_t n, int d, int64_t ld, const int32_t *__restrict__ G, int kappa,
+    const float *__restrict__ C, const uint4 *__restrict__ Cq, const float4 *__restrict__ meta, int k,
+    const int32_t *__restrict__ Lin, int32_t *__restrict__ Lout, float *__restrict__ best_out, DevStatus *st,
+    const Track trk, const int32_t *__restrict__ todo)
+{
+    __shared__ __align__(16) int s_q[AS_WARPS][AS_QROW];
+    __shared__ __align__(16) int s_h[AS_WARPS][AS_HASH];
+    __shared__ float s_lo[AS_WARPS][AS_QROW];
+    const int w = threadIdx.x >> 5, lane = lane_id();
+    int *qlist = s_q[w];
+    int *tab = s_h[w];
+    float *lov = s_lo[w];
+    constexpr int G4 = 32 / LPR;                  // candidates side by side
+    constexpr int U = LPR == 32 ? 4 : LPR == 16 ? 2 : 1;  // such groups in flight (LPR = 32: a transposed reduction)
+    const int sub = lane % LPR, grp = lane / LPR;
+    const int d4 = d >> 2;
+    const float4 *C4 = reinterpret_cast<const float4 *>(C);
+    const float gam = (float)(d + 8) * 5.9604645e-8f;  // FP32 rounding of a d-term sum, relative
+    const float rootd = 0.51f * sqrtf((float)d);
+
+    each_sample<LISTS>((int64_t)blockIdx.x * AS_WARPS + w, (int64_t)gridDim.x * AS_WARPS, n, trk, todo,
+                       [&](int64_t i, auto part_list) {
+        constexpr bool PART = decltype(part_list)::value;
+        const XT *xrow = X + i * ld;
+        // this lane's 16 coordinates of every 16 * LPR
+        float4 v[NW * 4];
+#pragma unroll
+        for (int q = 0; q < NW * 4; q++) {
+            const int col = ((q >> 2) * LPR + sub) * 4 + (q & 3);
+            v[q] = col < d4 ? ldx4<XT>(xrow + 4 * col) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        const int own = Lin[i];
+        int u = collect_labels(i, own, G, kappa, n, k, Lin, qlist, tab, st);
+        float bd = __int_as_float(0x7f800000);
+        int br = 0x7fffffff;
+        if constexpr (PART) {
+            u = track_filter(trk, qlist, u);
+            bd = best_out[i];
+            br = own;
+        }
+        unsigned mb = 0;
+#pragma unroll
+        for (int q = 0; q < NW * 4; q++) {
+            mb = max(max(mb, __float_as_uint(fabsf(v[q].x))), __float_as_uint(fabsf(v[q].y)));
+            mb = max(max(mb, __float_as_uint(fabsf(v[q].z))), __float_as_uint(fabsf(v[q].w)));
+        }
+        mb = __reduce_max_sync(FULL_MASK, mb);
+        const bool screen = u > Q8_FEW && mb < 0x7f800000u;
+        float best_up = bd;  // the known distance, or infinity
+        if (screen) {
+            if (lane < G4 * U)
+                qlist[u + lane] = qlist[0];
+            __syncwarp();
+            const float mx = fmaxf(__uint_as_float(mb), 1e-30f);
+            const float sx = mx / 16256.f, inv = 16256.f / mx;
+            uint32_t hx[NW * 4], lx[NW * 4];
+            float x2 = 0.f;
+#pragma unroll
+            for (int q = 0; q < NW * 4; q++) {
+                const float vals[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+                uint32_t hw = 0, lw = 0;
+#pragma unroll
+                for (int z = 0; z < 4; z++) {
+                    // rint(x / s_x) in the low bits of a float (magnitude below 2^22)
+                    const float t = fmaf(vals[z], inv, 12582912.f);
+                    const int c = __float_as_int(t) - 0x4b400000, h = (c + 64) >> 7;
+                    const float f = t - 12582912.f;
+                    x2 = fmaf(f, f, x2);
+                    hw |= (uint32_t)(h & 0xff) << (8 * z);
+                    lw |= (uint32_t)((c - (h << 7)) & 0xff) << (8 * z);
+                }
+                hx[q] = hw;
+                lx[q] = lw;
+            }
+#pragma unroll
+            for (int o = LPR / 2; o > 0; o >>= 1)
+                x2 += __shfl_xor_sync(FULL_MASK, x2, o);
+            const float X2 = x2 * sx * sx, dx = rootd * sx;
+            // candidate c's lower and upper values, from its dot product with the sample
+            auto bounds = [&](int c, int dot, bool first) {
+                const float4 mt = __ldg(meta + qlist[c]);
+                const float n2 = X2 + mt.y;
+                const float dt = fmaf(-2.f * sx * mt.x, (float)dot, n2);
+                const float er = 3.8146973e-6f * n2, dl = mt.z + dx;
+                const float dp = fmaxf(dt, 0.f) + er;
+                const float sq = dl * (2.f * sqrtf(dp) + dl);
+                const float e = 1.01f * (sq + er + gam * (2.f * dp + sq));
+                float lo = dt - e, up = dt + e;
+                if (!(fabsf(dt) < 1e37f) || !(e < 1e37f))
+                    lo = -__int_as_float(0x7f800000), up = __int_as_float(0x7f800000);
+                if (first)
+                    lov[c] = lo;
+                best_up = fminf(best_up, up);
+            };
+            for (int c0 = 0; c0 < u; c0 += G4 * U) {
+                int part[U];
+#pragma unroll
+                for (int z = 0; z < U; z++) {
+                    const uint4 *row = Cq + (int64_t)qlist[c0 + z * G4 + grp] * (LPR * NW) + sub;
+                    int hh = 0, ll = 0;
+#pragma unroll
+                    for (int q = 0; q < NW; q++) {
+                        const uint4 cw = __ldg(row + q * LPR);
+                        hh = dot4(cw.x, hx[4 * q], hh);
+                        hh = dot4(cw.y, hx[4 * q + 1], hh);
+                        hh = dot4(cw.z, hx[4 * q + 2], hh);
+                        hh = dot4(cw.w, hx[4 * q + 3], hh);
+                        ll = dot4(cw.x, lx[4 * q], ll);
+                        ll = dot4(cw.y, lx[4 * q + 1], ll);
+                        ll = dot4(cw.z, lx[4 * q + 2], ll);
+                        ll = dot4(cw.w, lx[4 * q + 3], ll);
+                    }
+                    part[z] = (hh << 7) + ll;  // |sum over d <= 1024| < 2^31
+                }
+                if constexpr (LPR == 32) {
+                    // four sums at once: lane l ends with candidate l / 8
+                    const bool up = (lane & 16) != 0, up2 = (lane & 8) != 0;
+                    int a = (up ? part[2] : part[0]) + __shfl_xor_sync(FULL_MASK, up ? part[0] : part[2], 16);
+                    const int b = (up ? part[3] : part[1]) + __shfl_xor_sync(FULL_MASK, up ? part[1] : part[3], 16);
+                    a = (up2 ? b : a) + __shfl_xor_sync(FULL_MASK, up2 ? a : b, 8);
+#pragma unroll
+                    for (int o = 4; o > 0; o >>= 1)
+                        a += __shfl_xor_sync(FULL_MASK, a, o);
+                    bounds(c0 + (lane >> 3), a, (lane & 7) == 0);
+                } else {
+#pragma unroll
+                    for (int z = 0; z < U; z++) {
+#pragma unroll
+                        for (int o = LPR / 2; o > 0; o >>= 1)
+                            part[z] += __shfl_xor_sync(FULL_MASK, part[z], o);
+                        bounds(c0 + z * G4 + grp, part[z], sub == 0);
+                    }
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                best_up = fminf(best_up, __shfl_xor_sync(FULL_MASK, best_up, o));
+        }
+        __syncwarp();
+        // pass 2: exact FP32 distances of the candidates that may be the minimum
+        float4 xv[NV];
+#pragma unroll
+        for (int q = 0; q < NV; q++) {
+            const int col = lane + 32 * q;
+            xv[q] = col < d4 ? ldx4<XT>(xrow + 4 * col) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        for (int g0 = 0; g0 < u; g0 += 32) {
+            const int cnt = min(32, u - g0);
+            unsigned sel = __ballot_sync(FULL_MASK, lane < cnt && (!screen || lov[g0 + lane] <= best_up));
+            while (sel) {
+                const int c = __ffs(sel) - 1;
+                sel &= sel - 1;
+                const int r = qlist[g0 + c];
+                const float4 *row = C4 + (int64_t)r * d4;
+                const float tot = warp_total(lane_partial<NV>(xv, d4, [&](int col) { return __ldg(row + col); }));
+                if (key_less(tot, r, bd, br)) {
+                    bd = tot;
+                    br = r;
+                }
+            }
+        }
+        write_winner(i, own, k, bd, br, Lout, best_out, trk);
+        __syncwarp();
+    });
 }
 
 // k_assign_rows with the candidate distances first taken against the BF16
@@ -895,12 +1072,22 @@ static size_t al256(size_t b) { return (b + 255) & ~size_t(255); }
 size_t assign_scratch_bytes(int64_t n, int32_t k, int64_t d)
 {
     const size_t part = al256((size_t)AS_BLOCKS * (sizeof(double) + sizeof(unsigned long long)) + sizeof(unsigned));
-    const size_t shadow = al256((size_t)k * (size_t)d * 2) + 2 * al256((size_t)k * 4);
+    const size_t shadow = al256((size_t)k * (size_t)d * 2) + 2 * al256((size_t)k * 4) + al256((size_t)k * 16);
     const size_t best = al256((size_t)n * 4);
     const size_t tiles = al256((size_t)((n + AS_TILE - 1) / AS_TILE) * 4);
     const size_t sel = al256((size_t)n * 8 * 4) + al256((size_t)n * 4);
     return part + shadow + best + tiles + sel;
 }
+
+// Narrowest rows the int8 screening takes (a row of the shadow has at least 64 bytes, in the place of 2 d).
+constexpr int Q8_MIN_D = 32;
+
+// Where precision 0 and 1 take the int8 screening: rows of more than Q8_PAYS_D values, in sample sets large enough for
+// its extra launch.  FP32 rows against screening, us an assignment: 200k x 256 230 / 300 (539 / 607 at kappa = 50),
+// 200k x 300 290 / 280, 100k x 384 259 / 215, 300k x 512 BF16 1317 / 801, 100k x 960 960 / 366; at 300k x 128 401 / 516.
+constexpr int Q8_PAYS_D = 320;
+
+static bool assign_q8_pays(int64_t n, int64_t d) { return d > Q8_PAYS_D && n * d >= ((int64_t)1 << 22); }
 
 template <typename XT>
 static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *g_idx, int32_t kappa,
@@ -919,6 +1106,8 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     sp += al256((size_t)k * 4);
     float *cnorm = reinterpret_cast<float *>(sp);
     sp += al256((size_t)k * 4);
+    float4 *meta = reinterpret_cast<float4 *>(sp);
+    sp += al256((size_t)k * 16);
     float *best = best_d2 ? best_d2 : reinterpret_cast<float *>(sp);
     sp += al256((size_t)n * 4);
     int32_t *tile_flag = reinterpret_cast<int32_t *>(sp);
@@ -947,61 +1136,55 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
         else
             k_assign_select<4><<<sgrid, SL_WARPS * 32, 0, s>>>(n, g_idx, kappa, k, labels_in, labels_out, trk, sel_lab);
     }
-    if ((precision == 2 || precision == 4) && vec4 && d4 <= 32 * 8) {
-        // the shadow: BF16 (2) or int8 with a per-row scale (4); the int8 codes take the BF16 shadow's space
+    // The int8 screening at precision 4, and at 0 and 1 where it is faster than the FP32 rows (assign_q8_pays): the
+    // results are the same.
+    const bool q8 = vec4 && d >= Q8_MIN_D && d4 <= 32 * 8 &&
+                    (precision == 4 || (precision <= 1 && assign_q8_pays(n, d)));
+    if (q8) {
+        const int units = d <= 64 ? 4 : d <= 128 ? 8 : d <= 256 ? 16 : d <= 512 ? 32 : 64;  // 16 bytes each
         const int sgrid = (k + 7) / 8 < 152 * 16 ? (k + 7) / 8 : 152 * 16;
-        // int8 rows lane-major where a screening kernel has whole vectors in every lane (d = 128, 256, 512, 1024: the
-        // kernels' d4 == 32 NV below): one load per lane and row
-        const bool lane_major = precision == 4 && (d4 == 32 || d4 == 64 || d4 == 128 || d4 == 256);
-        if (precision == 2)
-            k_shadow_bf16<<<sgrid, 256, 0, s>>>(C, k, (int)d, Cb, delta, cnorm, trk.dirty);
-        else
-            k_shadow_i8<<<sgrid, 256, 0, s>>>(C, k, (int)d, lane_major, reinterpret_cast<uint32_t *>(Cb), delta,
-                                              cnorm, trk.dirty);
-#define GK_ASB8F(NV, GS, F)                                                                                      \
-    do {                                                                                                         \
-        if (trk.dirty)                                                                                           \
-            GK_ASB8T(NV, GS, F, true);                                                                           \
-        else                                                                                                     \
-            GK_ASB8T(NV, GS, F, false);                                                                          \
-    } while (0)
-#define GK_ASB8T(NV, GS, F, T)                                                                                   \
-    do {                                                                                                         \
-        if ((e = resident_grid(reinterpret_cast<const void *>(k_assign_rows_scr<NV, XT, GS, F, T>),              \
-                               AS_WARPS * 32, 0, &grid)) != cudaSuccess)                                         \
-            return e;                                                                                            \
-        k_assign_rows_scr<NV, XT, GS, F, T><<<grid, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, Cb,  \
-                                                                           delta, cnorm, k, labels_in, labels_out, \
-                                                                           best, st, trk, sel_lab);                       \
-    } while (0)
-#define GK_ASB8G(NV, GS)                                                                                         \
-    do {                                                                                                         \
-        if (precision == 2)                                                                                      \
-            GK_ASB8F(NV, GS, 0);                                                                                 \
-        else if (lane_major && d4 == 32 * NV)                                                                    \
-            GK_ASB8F(NV, GS, 2);                                                                                 \
-        else                                                                                                     \
-            GK_ASB8F(NV, GS, 1);                                                                                 \
-    } while (0)
-#define GK_ASB8(NV)                                                                                              \
-    do {                                                                                                         \
-        if (NV >= 8 || gw == 4)                                                                                  \
-            GK_ASB8G(NV, 4);                                                                                     \
-        else                                                                                                     \
-            GK_ASB8G(NV, 8);                                                                                     \
-    } while (0)
+        k_shadow_i8<<<sgrid, 256, 0, s>>>(C, k, (int)d, units, reinterpret_cast<uint32_t *>(Cb), meta, trk.dirty);
+        auto launch = [&](auto kernel) -> cudaError_t {
+            cudaError_t le = resident_grid(reinterpret_cast<const void *>(kernel), AS_WARPS * 32, 0, &grid);
+            if (le == cudaSuccess)
+                kernel<<<grid, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, reinterpret_cast<const uint4 *>(Cb),
+                                                      meta, k, labels_in, labels_out, best, st, trk, sel_lab);
+            return le;
+        };
+#define GK_ASQ8(LPR, NW, NV) \
+    (trk.dirty ? launch(k_assign_rows_scr<LPR, NW, NV, XT, true>) : launch(k_assign_rows_scr<LPR, NW, NV, XT, false>))
+        e = d <= 64    ? GK_ASQ8(4, 1, 1)
+            : d <= 128 ? GK_ASQ8(8, 1, 1)
+            : d <= 256 ? GK_ASQ8(16, 1, 2)
+            : d <= 512 ? GK_ASQ8(32, 1, 4)
+                       : GK_ASQ8(32, 2, 8);
+#undef GK_ASQ8
+        if (e != cudaSuccess)
+            return e;
+        done = true;
+    } else if (precision == 2 && vec4 && d4 <= 32 * 8) {
+        const int sgrid = (k + 7) / 8 < 152 * 16 ? (k + 7) / 8 : 152 * 16;
+        k_shadow_bf16<<<sgrid, 256, 0, s>>>(C, k, (int)d, Cb, delta, cnorm, trk.dirty);
+        auto launch = [&](auto kernel) -> cudaError_t {
+            cudaError_t le = resident_grid(reinterpret_cast<const void *>(kernel), AS_WARPS * 32, 0, &grid);
+            if (le == cudaSuccess)
+                kernel<<<grid, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, Cb, delta, k, labels_in, labels_out,
+                                                      best, st, trk, sel_lab);
+            return le;
+        };
+#define GK_ASBF(NV, GS) \
+    (trk.dirty ? launch(k_assign_rows_scr<NV, XT, GS, true>) : launch(k_assign_rows_scr<NV, XT, GS, false>))
         if (d4 <= 32)
-            GK_ASB8(1);
+            e = gw == 4 ? GK_ASBF(1, 4) : GK_ASBF(1, 8);
         else if (d4 <= 64)
-            GK_ASB8(2);
+            e = gw == 4 ? GK_ASBF(2, 4) : GK_ASBF(2, 8);
         else if (d4 <= 128)
-            GK_ASB8(4);
+            e = gw == 4 ? GK_ASBF(4, 4) : GK_ASBF(4, 8);
         else
-            GK_ASB8(8);
-#undef GK_ASB8
-#undef GK_ASB8G
-#undef GK_ASB8F
-#undef GK_ASB8T
+            e = GK_ASBF(8, 4);
+#undef GK_ASBF
+        if (e != cudaSuccess)
+            return e;
         done = true;
     }
     if constexpr (std::is_same_v<XT, float>) {  // tensor-core screening: FP32 samples only
