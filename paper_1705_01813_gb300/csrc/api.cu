@@ -111,6 +111,7 @@ struct Layout {
     uint8_t *dirty[2];     // FIT, BUILD: clusters changed by the last two assignments
     uint8_t *row_changed;  // BUILD: graph rows changed since the last assignment
     int32_t *todo_n;       // FIT, BUILD: Track's counters
+    uint8_t *mark;         // FIT, BUILD: samples in clusters changed by the last assignment
     size_t bytes;
 };
 
@@ -141,6 +142,7 @@ Layout carve(void *ws, int op, int64_t n, int64_t d, int32_t k)
         L.todo_n = cv.take<int32_t>(64);  // 256 bytes, followed by dirty[0]: one memset clears both
         L.dirty[0] = cv.take<uint8_t>((size_t)k);
         L.dirty[1] = cv.take<uint8_t>((size_t)k);
+        L.mark = cv.take<uint8_t>((size_t)n);
     }
     if (op == GK_OP_BUILD) {
         L.labels_a = cv.take<int32_t>((size_t)n);
@@ -167,7 +169,7 @@ Track track_of(const Layout &L, int t, int64_t n, int64_t d, int32_t precision, 
 {
     if ((precision & 0xff) == 3 || n * d < TRACK_MIN_VALUES)
         return Track{};
-    return Track{t > 0 ? L.dirty[(t + 1) & 1] : nullptr, L.dirty[t & 1], rows ? L.row_changed : nullptr,
+    return Track{t > 0 ? L.dirty[(t + 1) & 1] : nullptr, L.mark, L.dirty[t & 1], rows ? L.row_changed : nullptr,
                  L.dirty[(t + 1) & 1], L.todo_n};
 }
 

@@ -102,7 +102,9 @@ __device__ __forceinline__ int collect_labels(int64_t i, int own, const int32_t 
 // a sample whose own centroid or graph row changed goes to the front list (all candidates).  The assignment kernels
 // then walk the lists.  Doing the test inside them cost registers that the evaluation needs: 30 -> 32 ms for the
 // 1M x 128 graph construction, where almost no sample is done early (this kernel: 13 us of 1 ms there).  The lists' order varies from call to call and
-// decides nothing but which warp takes a sample.  Against evaluating everything: a fit of 2M x 512 BF16 (k = 200,000)
+// decides nothing but which warp takes a sample.  A neighbour costs one byte gather, of the mark that k_assign_reduce
+// left for its cluster (its label and then the cluster's byte, 0.52 ms at 2M x 40: the L1's one lookup a cycle).
+// Against evaluating everything: a fit of 2M x 512 BF16 (k = 200,000)
 // takes 1.0 ms an assignment instead of 9.0 once its labels have settled.
 constexpr int SL_WARPS = 8;
 
@@ -122,7 +124,7 @@ __global__ void __launch_bounds__(SL_WARPS * 32) k_assign_select(int64_t n, cons
         bool known = false;
         if (i < n) {
             own = Lin[i];
-            known = (unsigned)own < (unsigned)k && trk.dirty[own] == 0;
+            known = trk.mark[i] == 0;  // a label out of range is marked
             if (trk.row_changed && trk.row_changed[i]) {
                 trk.row_changed[i] = 0;
                 known = false;
@@ -148,14 +150,13 @@ __global__ void __launch_bounds__(SL_WARPS * 32) k_assign_select(int64_t n, cons
 #pragma unroll
                 for (int u = 0; u < S; u++)
                     if (nb[q][u] != -2)
-                        nb[q][u] = (unsigned)nb[q][u] < (unsigned)n ? Lin[nb[q][u]] : -1;
+                        nb[q][u] = (unsigned)nb[q][u] < (unsigned)n ? trk.mark[nb[q][u]] : 1;
 #pragma unroll
             for (int q = 0; q < B; q++) {
                 bool any = false;
 #pragma unroll
                 for (int u = 0; u < S; u++)
-                    if (nb[q][u] != -2)
-                        any |= (unsigned)nb[q][u] >= (unsigned)k || trk.dirty[nb[q][u]] != 0;
+                    any |= nb[q][u] > 0;
                 if (__any_sync(FULL_MASK, any) && src[q] >= 0)
                     touched |= 1u << src[q];
             }
@@ -1014,6 +1015,11 @@ __global__ void __launch_bounds__(256) k_assign_reduce(const float *__restrict__
                                                        int64_t *__restrict__ n_changed)
 {
     static_assert(AS_BLOCKS > 1024 && AS_BLOCKS <= 2048, "two blocks per chain at most");
+    if (trk.dirty_out)  // for the next assignment's k_assign_select
+        for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
+            const int r = Lout[i];
+            trk.mark[i] = (unsigned)r < (unsigned)k ? trk.dirty_out[r] : 1;
+        }
     if (trk.clear) {  // Track's clears, here to save a launch
         for (int64_t r = (int64_t)blockIdx.x * 256 + threadIdx.x; r < k; r += (int64_t)gridDim.x * 256)
             trk.clear[r] = 0;
@@ -1269,13 +1275,9 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
         if (e != cudaSuccess)
             return e;
     }
-    if (sum_d2 || n_changed) {
+    if (sum_d2 || n_changed || trk.dirty_out) {
         k_assign_reduce<<<AS_BLOCKS, 256, 0, s>>>(best, labels_in, labels_out, n, blk_sum, blk_chg, trk, k, sum_d2,
                                                   n_changed);
-    } else if (trk.clear) {
-        if ((e = cudaMemsetAsync(trk.clear, 0, (size_t)k, s)) != cudaSuccess ||
-            (e = cudaMemsetAsync(trk.todo_n, 0, 2 * sizeof(int32_t), s)) != cudaSuccess)
-            return e;
     }
     return cudaGetLastError();
 }

@@ -291,6 +291,7 @@ unsigned *update_ticket(void *scratch, int32_t k);
 // leaves its centroid's bits as they are, so distances to it need not be taken again (assign.cu).
 struct Track {
     const uint8_t *dirty;      // k: the cluster gained or lost members in the previous assignment (NULL: the first)
+    uint8_t *mark;             // n: the sample's cluster is such a one (written after the previous assignment)
     uint8_t *dirty_out;        // k, zeroed: the clusters this assignment changes (NULL: not kept)
     uint8_t *row_changed;      // n: the graph row changed since the previous assignment, read and cleared (NULL: none)
     uint8_t *clear;            // k: zeroed after this assignment (the next one's dirty_out; may be `dirty`)
