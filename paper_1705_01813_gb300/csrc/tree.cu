@@ -26,6 +26,7 @@
 // fused multiply-add per step, the decisions' precision.  Clusters are
 // numbered left to right at the end.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -35,10 +36,11 @@ namespace {
 constexpr uint64_t TAG_TREE = 0x5452454500000000ull;  // "TREE"
 constexpr int TR_THREADS = 128;                       // pass kernel: one member per thread at a time
 constexpr int TR_STAGE = 64;                          // coordinates staged per round
-constexpr int TR_PITCH = TR_STAGE + 1;                // padded row of the stage (conflict-free column reads)
+constexpr int TR_VP = TR_STAGE + 4;                   // pitch of a staged row: 16-byte reads of neighbouring rows and
+                                                      // 4-byte reads along a row hit distinct banks
 constexpr int64_t TR_CHUNK = 512;                     // members per chunk block; larger clusters take several
 constexpr int SEL_THREADS = 256;
-static_assert(TR_THREADS == 2 * TR_STAGE, "the sums give each thread one coordinate of one half");
+static_assert(TR_THREADS == 2 * TR_STAGE, "the sums give each coordinate two threads");
 
 // Range of cluster j of depth L: the bits of j from the most significant, 0 = u (the left ceil(m/2)).
 __device__ __forceinline__ void seg_geom(int64_t n, int L, int64_t j, int64_t &off, int64_t &m)
@@ -255,47 +257,130 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_seed_final(const XT *__rest
     }
 }
 
-// The coordinates t0 .. t0 + tw - 1 of the block's TR_THREADS member rows into the stage: warp w loads rows
-// w, w + 4, ..., one coalesced load per 32 coordinates.
+// Largest magnitude of every column, as the bits of its float (infinities and NaN above every number): colmax[d], zeroed.
 template <typename XT>
-__device__ __forceinline__ void stage_rows(const XT *__restrict__ X, int64_t ld, const int *sid, int t0, int tw,
-                                           float *stage, int warp, int lane)
+__global__ void __launch_bounds__(256) k_tree_colmax(const XT *__restrict__ X, int64_t n, int d, int64_t ld, bool vec,
+                                                     unsigned *__restrict__ colmax)
 {
-    for (int r = warp; r < TR_THREADS; r += TR_THREADS / 32) {
-        const XT *row = X + (int64_t)sid[r] * ld + t0;
-        for (int q = lane; q < tw; q += 32)
-            stage[r * TR_PITCH + q] = ldx(row + q);
+    __shared__ unsigned s_mx[128];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, col = blockIdx.y * 128 + lane * 4;
+    if (threadIdx.x < 128)
+        s_mx[threadIdx.x] = 0u;
+    __syncthreads();
+    unsigned mx[4] = {0u, 0u, 0u, 0u};
+    if (col < d) {
+#pragma unroll 4
+        for (int64_t i = (int64_t)blockIdx.x * 8 + warp; i < n; i += (int64_t)gridDim.x * 8) {
+            const XT *p = X + i * ld + col;
+            if (vec) {
+                const float4 v = ldx4<XT>(p);
+                mx[0] = max(mx[0], __float_as_uint(fabsf(v.x)));
+                mx[1] = max(mx[1], __float_as_uint(fabsf(v.y)));
+                mx[2] = max(mx[2], __float_as_uint(fabsf(v.z)));
+                mx[3] = max(mx[3], __float_as_uint(fabsf(v.w)));
+            } else {
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    if (col + q < d)
+                        mx[q] = max(mx[q], __float_as_uint(fabsf(ldx(p + q))));
+            }
+        }
     }
+#pragma unroll
+    for (int q = 0; q < 4; q++)
+        atomicMax(&s_mx[lane * 4 + q], mx[q]);
+    __syncthreads();
+    const int t = blockIdx.y * 128 + threadIdx.x;
+    if (threadIdx.x < 128 && t < d)
+        atomicMax(colmax + t, s_mx[threadIdx.x]);
 }
 
-// Dynamic shared memory of the pass kernel: FP64 sums of both halves, both centres, the staged rows, the block's
-// member ids and halves.
+// ---------------------------------------------------------------------------
+// The centres.  A centre is defined as the FP32 rounding of an FP64 mean whose sum runs over the members in ascending id
+// (chunk by chunk, the chunks' sums in order), and the FP64 pipe would bound the tree: one addition per member and
+// coordinate, 0.5 a cycle and SM, was 70% of it.  The sums are taken in integers instead, which no order changes.  With
+// column t's largest magnitude below 2^(e + 1), y = x 2^(20 - e) is below 2^21 and split exactly as
+//   y = h0 + h1 2^-22 + h2 2^-44 + error,  |error| <= 2^-45,
+// h0, h1, h2 integers of at most 2^21 (the sum of y 2^22 and 1.5 2^23 rounds to an integer in the float's low bits).
+// Where every h1 is zero, or every h2 and at most 1024 members are summed (and y itself is exact: no scaling down),
+// all partial sums are multiples of one unit that FP64 holds exactly, so the ordered FP64 sum is this sum.  Otherwise
+// the two means differ by at most (chunk + chunks) 2^-53 mean|x| plus the split's remainder, and their FP32 roundings
+// are the same unless the mean lies that close to the midpoint of two floats: a few centre coordinates in 10^6.  Those
+// get the code REDO and k_tree_redo sums them in the defined order.  So every centre has the bits of the definition.
+// ---------------------------------------------------------------------------
+constexpr unsigned REDO = 0x7fb0dead;  // a NaN no mean takes
+constexpr float SPLIT_M = 12582912.f;  // 1.5 2^23
+
+// 2^(20 - e) for a column whose largest magnitude has the given bits; 0 when it is not finite.
+__device__ __forceinline__ float col_scale(unsigned mx)
+{
+    const int e = max((int)(mx >> 23) - 127, -106);  // 2^126 at most
+    return mx >= 0x7f800000u ? 0.f : __uint_as_float((unsigned)(20 - e + 127) << 23);
+}
+
+// The centre coordinate of cnt > 0 members from their limb sums, or REDO.  any: bit 0 a second limb, bit 1 a third limb
+// or remainder occurred; mass: the sum of |y|, added in any order.
+__device__ __forceinline__ unsigned centre_bits(int64_t h0, int64_t h1, int64_t h2, unsigned any, float mass,
+                                                int64_t cnt, unsigned mx, int64_t chunks)
+{
+    const float sc = col_scale(mx);
+    if (sc == 0.f)
+        return REDO;
+    const double y = (double)h0 + ((double)h1 * 0x1p-22 + (double)h2 * 0x1p-44);
+    const double q = y / (double)sc / (double)cnt;  // the scaling is exact
+    const unsigned f = __float_as_uint((float)q);
+    if (sc >= 1.f && (any == 0 || (any == 1 && cnt <= 1024)))
+        return f;
+    const uint64_t bits = (uint64_t)__double_as_longlong(q);
+    const int e = (int)((bits >> 52) & 0x7ff) - 1023;
+    if (e < -126 || e >= 127)  // outside FP32's normal range, or zero
+        return REDO;
+    // distance of q from the midpoint of its two floats, and the bound, in units of q's last place, 2^(e - 52)
+    const int64_t frac = (int64_t)(bits & 0x1fffffffull) - 0x10000000ll;
+    const double rel = ((double)(TR_CHUNK + 8) + (double)chunks) * (1.02 + (double)chunks * 0x1p-23) * 0x1p-53;
+    const double tol = ((double)mass * rel / (double)cnt + 0x1p-44) / (double)sc;
+    const double units = tol * __longlong_as_double((long long)(52 - e + 1023) << 52) + 4.0;
+    return (double)llabs(frac) <= units ? REDO : f;
+}
+
+// Dynamic shared memory of the pass kernel: limb sums, masses and flags of both halves, both centres, the staged rows,
+// the block's member ids and counts, the rows by half.
 __host__ __device__ constexpr size_t pass_smem(int d)
 {
-    return (size_t)16 * d + (size_t)8 * d + sizeof(float) * TR_THREADS * TR_PITCH + 2 * sizeof(int) * TR_THREADS;
+    return (size_t)44 * d + sizeof(float) * TR_THREADS * TR_VP + 2 * sizeof(int) * TR_THREADS + TR_THREADS + 64;
 }
 
 // One pass over the members of every splitting cluster of depth L, C chunks per cluster (grid S x C).  Each thread
 // takes one member at a time: the rows of the block's 128 members are staged 64 coordinates at a time and each
-// thread sums its member's two distances in the canonical FP32 order.
-//   KEYS = false (a Lloyd iteration): the member joins u when d_u <= d_v and its row is added, in FP64 and in
-//     member order, to its half's sums (a second staging of the group's rows; one thread per coordinate and
-//     half keeps each sum); with one chunk the block writes the new centres, otherwise its sums and counts go
-//     to part (2d + 2 doubles per chunk) for k_tree_reduce.
+// thread sums its member's two distances in the canonical FP32 order (both at once in packed FP32x2).
+//   KEYS = false (a Lloyd iteration): the member joins u when d_u <= d_v and its row is added to its half's limb sums
+//     (the stages again, the last one first as it is still there; threads share out coordinates and rows); with one chunk
+//     the block writes the new centres, otherwise its sums and counts are added to acc, mass, flg and cnts, for
+//     k_tree_centres.  halves[p] is the half, for k_tree_redo.
 //   KEYS = true: keys[p] = (order(d_u - d_v) << 32) | id.
+// Bound by the reads of the rows: 1M x 128 FP32 (512 MB) takes 84 us with KEYS, 6.1 TB/s, and 159 us without (all but
+// the last stage are read again, mostly from the L2, and the sums).  With loads through registers, four in flight, it
+// was 229 and 332 us; before the packed distances and the integer sums 421 and 879 us, the FP64 additions' time.  Two
+// stage buffers, the next stage in flight during the distances, leave 3 blocks of an SM instead of 5: 91 and 174 us.
 template <typename XT, bool KEYS>
 __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__ X, int64_t n, int d, int64_t ld,
-                                                          int L, int64_t C, const int32_t *__restrict__ perm,
+                                                          bool vec, int L, int64_t C, const int32_t *__restrict__ perm,
                                                           const int32_t *__restrict__ spl, float *__restrict__ cen,
-                                                          double *__restrict__ part, uint64_t *__restrict__ keys,
-                                                          DevStatus *st)
+                                                          const unsigned *__restrict__ colmax,
+                                                          unsigned long long *__restrict__ acc,
+                                                          unsigned *__restrict__ flg, float *__restrict__ mass,
+                                                          unsigned *__restrict__ cnts, uint8_t *__restrict__ halves,
+                                                          uint64_t *__restrict__ keys, DevStatus *st)
 {
     extern __shared__ __align__(16) unsigned char tr_smem[];
-    double *acc = reinterpret_cast<double *>(tr_smem);              // [2][d]
-    float *cuv = reinterpret_cast<float *>(acc + 2 * (size_t)d);    // [2][d]
-    float *stage = cuv + 2 * (size_t)d;                             // [TR_THREADS][TR_PITCH]
-    int *sid = reinterpret_cast<int *>(stage + TR_THREADS * TR_PITCH);
-    int *shalf = sid + TR_THREADS;
+    float *stage = reinterpret_cast<float *>(tr_smem);                       // [TR_THREADS][TR_VP]
+    int *sid = reinterpret_cast<int *>(stage + TR_THREADS * TR_VP);
+    int *s_n = sid + TR_THREADS;                                             // members of u, of u and v in the group
+    unsigned char *order = reinterpret_cast<unsigned char *>(s_n + TR_THREADS);  // rows of u, then of v
+    float2 *cuv = reinterpret_cast<float2 *>(order + TR_THREADS);            // [d]: (c_u, c_v)
+    int *lsum = reinterpret_cast<int *>(cuv + d);                            // [2][3][d]
+    float *lmass = reinterpret_cast<float *>(lsum + 6 * (size_t)d);          // [2][d]
+    unsigned *lany = reinterpret_cast<unsigned *>(lmass + 2 * (size_t)d);    // [d], two bits per half
     const int64_t j = blockIdx.x / C, c = blockIdx.x % C;
     if (spl && !spl[j])
         return;
@@ -304,11 +389,36 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
     chunk_range(off, m, C, c, b, e);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float *cj = cen + j * 2 * (int64_t)d;
-    for (int t = tid; t < 2 * d; t += TR_THREADS) {
-        cuv[t] = cj[t];
-        if (!KEYS)
-            acc[t] = 0.0;
-    }
+    for (int t = tid; t < d; t += TR_THREADS)
+        cuv[t] = make_float2(cj[t], cj[d + t]);
+    if (!KEYS)
+        for (int t = tid; t < 9 * d; t += TR_THREADS)  // the masses and flags too
+            lsum[t] = 0;
+    const int nst = (d + TR_STAGE - 1) / TR_STAGE;
+    // the 64 coordinates of stage s of the block's rows (zeros past d), all in flight at once: 16 lanes per row, or a
+    // lane per coordinate
+    auto stage_rows = [&](int s) {
+        const int t0 = s * TR_STAGE;
+        if (vec) {
+            const int t = t0 + (tid & 15) * 4;
+            float *to = stage + (tid & 15) * 4;
+#pragma unroll 8
+            for (int r = tid >> 4; r < TR_THREADS; r += TR_THREADS / 16) {
+                float *q = to + r * TR_VP;
+                if (t >= d)
+                    *reinterpret_cast<float4 *>(q) = make_float4(0.f, 0.f, 0.f, 0.f);
+                else if constexpr (std::is_same_v<XT, float>)
+                    cp_async16(q, X + (int64_t)sid[r] * ld + t);
+                else
+                    *reinterpret_cast<float4 *>(q) = ldx4<XT>(X + (int64_t)sid[r] * ld + t);
+            }
+        } else {
+            for (int r = warp; r < TR_THREADS; r += TR_THREADS / 32)
+                for (int q = lane; q < TR_STAGE; q += 32)
+                    stage[r * TR_VP + q] = t0 + q < d ? ldx(X + (int64_t)sid[r] * ld + t0 + q) : 0.f;
+        }
+        cp_async_wait_all();
+    };
     __syncthreads();
     int64_t cnt_u = 0, cnt_v = 0;
     for (int64_t g = b; g < e; g += TR_THREADS) {
@@ -320,98 +430,208 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
             id = 0;
         }
         sid[tid] = id;
-        float du = 0.f, dv = 0.f;
-        for (int t0 = 0; t0 < d; t0 += TR_STAGE) {
-            const int tw = min(TR_STAGE, d - t0);
-            __syncthreads();  // sid written; the previous round's stage consumed
-            stage_rows(X, ld, sid, t0, tw, stage, warp, lane);
+        float2 duv = make_float2(0.f, 0.f);
+        const float2 m1 = make_float2(-1.f, -1.f);
+        for (int s = 0; s < nst; s++) {
+            __syncthreads();  // sid written; the previous stage consumed
+            stage_rows(s);
             __syncthreads();
-            const float *xs = stage + tid * TR_PITCH;
-            for (int tt = 0; tt < tw; tt++) {
-                const float x = xs[tt];
-                const float eu = __fsub_rn(x, cuv[t0 + tt]);
-                const float ev = __fsub_rn(x, cuv[d + t0 + tt]);
-                du = __fmaf_rn(eu, eu, du);
-                dv = __fmaf_rn(ev, ev, dv);
+            const float *xs = stage + tid * TR_VP;
+            const float2 *cs = cuv + s * TR_STAGE;
+            const int tw = min(TR_STAGE, d - s * TR_STAGE);
+            auto add = [&](float x, float2 cc) {
+                const float2 ee = __ffma2_rn(cc, m1, make_float2(x, x));  // x - c, rounded once
+                duv = __ffma2_rn(ee, ee, duv);
+            };
+            int tt = 0;
+#pragma unroll 4
+            for (; tt + 4 <= tw; tt += 4) {
+                const float4 x = *reinterpret_cast<const float4 *>(xs + tt);
+                const float4 a = *reinterpret_cast<const float4 *>(cs + tt), h = *reinterpret_cast<const float4 *>(cs + tt + 2);
+                add(x.x, make_float2(a.x, a.y));
+                add(x.y, make_float2(a.z, a.w));
+                add(x.z, make_float2(h.x, h.y));
+                add(x.w, make_float2(h.z, h.w));
             }
+            for (; tt < tw; tt++)
+                add(xs[tt], cs[tt]);
         }
         if (KEYS) {
             if (valid) {
-                const float dk = __fsub_rn(du, dv);
+                const float dk = __fsub_rn(duv.x, duv.y);
                 if (!isfinite(dk))
                     flag_error(st, GK_ERR_NUMERIC, (unsigned)id);
                 keys[p] = ((uint64_t)f32_order(dk) << 32) | (uint32_t)id;
             }
         } else {
-            // the group's rows are staged again, 64 coordinates at a time; thread (c, h) adds coordinate c of the
-            // members of half h in member order (ascending id within the cluster)
-            shalf[tid] = valid ? (du <= dv ? 0 : 1) : 2;
-            const int gn = (int)min((int64_t)TR_THREADS, e - g);
-            for (int t0 = 0; t0 < d; t0 += TR_STAGE) {
-                const int tw = min(TR_STAGE, d - t0);
-                __syncthreads();  // shalf written; the previous round's stage consumed
-                stage_rows(X, ld, sid, t0, tw, stage, warp, lane);
-                __syncthreads();
-                const int hh = tid / TR_STAGE, cc = tid % TR_STAGE;  // warps 0-1: half u, 2-3: half v
-                if (cc < tw) {
-                    double sum = acc[(size_t)hh * d + t0 + cc];
-                    for (int r = 0; r < gn; r++)
-                        if (shalf[r] == hh)
-                            sum += widen(stage[r * TR_PITCH + cc]);
-                    acc[(size_t)hh * d + t0 + cc] = sum;
+            // the group's rows by half
+            const int half = duv.x <= duv.y ? 0 : 1;
+            if (valid)
+                halves[p] = (uint8_t)half;
+            const unsigned bu = __ballot_sync(FULL_MASK, valid && half == 0), bv = __ballot_sync(FULL_MASK, valid && half == 1);
+            if (lane == 0) {
+                s_n[warp] = __popc(bu);
+                s_n[4 + warp] = __popc(bv);
+            }
+            __syncthreads();
+            int nu = 0, nv = 0, au = 0, av = 0;
+            for (int w = 0; w < TR_THREADS / 32; w++) {
+                au += w < warp ? s_n[w] : 0;
+                av += w < warp ? s_n[4 + w] : 0;
+                nu += s_n[w];
+                nv += s_n[4 + w];
+            }
+            if (valid)
+                order[half == 0 ? au + __popc(bu & lanemask_lt()) : nu + av + __popc(bv & lanemask_lt())] = (unsigned char)tid;
+            cnt_u += nu;
+            cnt_v += nv;
+            __syncthreads();
+            const int cc = tid % TR_STAGE, gg = tid / TR_STAGE;  // coordinate of the stage, rows gg, gg + 2, ...
+            for (int s = nst - 1; s >= 0; s--) {
+                if (s < nst - 1) {
+                    __syncthreads();  // the stage before is consumed
+                    stage_rows(s);
+                    __syncthreads();
+                }
+                const int t = s * TR_STAGE + cc;
+                const float sc = t < d ? col_scale(colmax[t]) : 0.f;
+                if (sc != 0.f) {
+                    auto half_sum = [&](int lo, int hi, int h) {
+                        int s0 = 0, s1 = 0, s2 = 0;
+                        float ms = 0.f;
+                        unsigned a1 = 0, a2 = 0;
+                        constexpr int MB = 0x4b400000;  // the bits of SPLIT_M
+#pragma unroll 4
+                        for (int r = lo + gg; r < hi; r += 2) {
+                            const float y = stage[order[r] * TR_VP + cc] * sc;
+                            const float t0 = __fadd_rn(y, SPLIT_M), r0 = __fsub_rn(y, __fsub_rn(t0, SPLIT_M));
+                            const float t1 = __fmaf_rn(r0, 4194304.f, SPLIT_M);
+                            const float r1 = __fmaf_rn(__fsub_rn(t1, SPLIT_M), -0x1p-22f, r0);
+                            const float t2 = __fmaf_rn(r1, 0x1p44f, SPLIT_M);
+                            ms += fabsf(y);
+                            s0 += __float_as_int(t0) - MB;
+                            s1 += __float_as_int(t1) - MB;
+                            s2 += __float_as_int(t2) - MB;
+                            a1 |= __float_as_uint(r0) << 1;  // without the sign of a zero
+                            a2 |= __float_as_uint(r1) << 1;
+                        }
+                        atomicAdd(&lsum[(3 * h) * d + t], s0);
+                        atomicAdd(&lmass[h * d + t], ms);
+                        if (a1) {
+                            atomicAdd(&lsum[(3 * h + 1) * d + t], s1);
+                            atomicAdd(&lsum[(3 * h + 2) * d + t], s2);
+                            atomicOr(&lany[t], (a2 ? 3u : 1u) << (2 * h));
+                        }
+                    };
+                    half_sum(0, nu, 0);
+                    half_sum(nu, nu + nv, 1);
                 }
             }
-            for (int r = 0; r < gn; r++) {
-                cnt_u += shalf[r] == 0;
-                cnt_v += shalf[r] == 1;
-            }
         }
-        __syncthreads();  // sid and shalf are rewritten by the next group
+        __syncthreads();  // sid and order are rewritten by the next group
     }
     if (KEYS)
         return;
     if (C == 1) {
-        for (int t = tid; t < d; t += TR_THREADS) {
-            if (cnt_u)
-                cj[t] = (float)(acc[t] / (double)cnt_u);
-            if (cnt_v)
-                cj[d + t] = (float)(acc[d + t] / (double)cnt_v);
+        for (int t = tid; t < 2 * d; t += TR_THREADS) {
+            const int h = t >= d ? 1 : 0, tc = t - h * d;
+            const int64_t cnt = h ? cnt_v : cnt_u;
+            if (cnt)
+                cj[t] = __uint_as_float(centre_bits(lsum[3 * h * d + tc], lsum[(3 * h + 1) * d + tc],
+                                                    lsum[(3 * h + 2) * d + tc], (lany[tc] >> (2 * h)) & 3u, lmass[t], cnt,
+                                                    colmax[tc], 1));
         }
     } else {
-        double *pc = part + blockIdx.x * (2 * (int64_t)d + 2);
-        for (int t = tid; t < 2 * d; t += TR_THREADS)
-            pc[t] = acc[t];
+        for (int t = tid; t < 6 * d; t += TR_THREADS)
+            if (lsum[t])
+                atomicAdd(acc + j * 6 * (int64_t)d + t, (unsigned long long)(long long)lsum[t]);
+        for (int t = tid; t < 2 * d; t += TR_THREADS) {
+            const int h = t >= d ? 1 : 0;
+            const unsigned any = (lany[t - h * d] >> (2 * h)) & 3u;
+            atomicAdd(mass + j * 2 * (int64_t)d + t, lmass[t]);
+            if (any)
+                atomicOr(flg + j * 2 * (int64_t)d + t, any);
+        }
         if (tid == 0) {
-            pc[2 * d] = (double)cnt_u;
-            pc[2 * d + 1] = (double)cnt_v;
+            atomicAdd(cnts + 2 * j, (unsigned)cnt_u);
+            atomicAdd(cnts + 2 * j + 1, (unsigned)cnt_v);
         }
     }
 }
 
-// Centres of the clusters split over several chunks: the chunks' FP64 sums added in chunk order.
-__global__ void __launch_bounds__(TR_THREADS) k_tree_reduce(int d, int64_t C, const int32_t *__restrict__ spl,
-                                                            float *__restrict__ cen, const double *__restrict__ part)
+// Centres of the clusters of several chunks from their limb sums; acc, mass and flg are left zeroed for the next
+// pass; k_tree_redo, which follows, clears cnts.
+__global__ void __launch_bounds__(256) k_tree_centres(int64_t S, int d, int64_t C, const int32_t *__restrict__ spl,
+                                                      float *__restrict__ cen, const unsigned *__restrict__ colmax,
+                                                      unsigned long long *__restrict__ acc, unsigned *__restrict__ flg,
+                                                      float *__restrict__ mass, const unsigned *__restrict__ cnts)
 {
-    const int64_t j = blockIdx.x;
-    if (spl && !spl[j])
-        return;
-    const double *p0 = part + j * C * (2 * (int64_t)d + 2);
-    double nu = 0.0, nv = 0.0;
-    for (int64_t c = 0; c < C; c++) {
-        nu += p0[c * (2 * (int64_t)d + 2) + 2 * d];
-        nv += p0[c * (2 * (int64_t)d + 2) + 2 * d + 1];
+    for (int64_t q = blockIdx.x * (int64_t)256 + threadIdx.x; q < S * 2 * d; q += (int64_t)gridDim.x * 256) {
+        const int64_t j = q / (2 * d);
+        if (spl && !spl[j])
+            continue;
+        const int t = (int)(q - j * 2 * d), h = t >= d ? 1 : 0, tc = t - h * d;
+        unsigned long long *a = acc + j * 6 * (int64_t)d + 3 * h * (int64_t)d + tc;
+        const int64_t cnt = cnts[2 * j + h];
+        if (cnt)
+            cen[q] = __uint_as_float(
+                centre_bits((int64_t)a[0], (int64_t)a[d], (int64_t)a[2 * (int64_t)d], flg[q], mass[q], cnt, colmax[tc], C));
+        a[0] = a[d] = a[2 * (int64_t)d] = 0ull;
+        flg[q] = 0u;
+        mass[q] = 0.f;
     }
-    float *cj = cen + j * 2 * (int64_t)d;
-    for (int t = threadIdx.x; t < d; t += blockDim.x) {
-        double su = 0.0, sv = 0.0;
-        for (int64_t c = 0; c < C; c++) {
-            su += p0[c * (2 * (int64_t)d + 2) + t];
-            sv += p0[c * (2 * (int64_t)d + 2) + d + t];
+}
+
+// The centre coordinates coded REDO, in the defined order: a warp per coordinate, a lane per chunk (chunk by chunk in
+// ascending id, the chunks' sums added in order).  cnts (of several chunks) is cleared for the next pass.
+template <typename XT>
+__global__ void __launch_bounds__(256) k_tree_redo(const XT *__restrict__ X, int64_t n, int d, int64_t ld, int L,
+                                                   int64_t S, int64_t C, const int32_t *__restrict__ perm,
+                                                   const int32_t *__restrict__ spl, const uint8_t *__restrict__ halves,
+                                                   float *__restrict__ cen, unsigned *__restrict__ cnts)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t total = S * 2 * d, step = (int64_t)gridDim.x * 256;
+    if (C > 1)
+        for (int64_t q = blockIdx.x * (int64_t)256 + threadIdx.x; q < 2 * S; q += step)
+            cnts[q] = 0u;
+    for (int64_t q0 = blockIdx.x * (int64_t)256 + (threadIdx.x & ~31); q0 < total; q0 += step) {
+        const int64_t q = q0 + lane;
+        unsigned left = __ballot_sync(FULL_MASK, q < total && __float_as_uint(cen[q]) == REDO);
+        while (left) {
+            const int64_t z = q0 + __ffs(left) - 1;
+            left &= left - 1;
+            const int64_t j = z / (2 * d);
+            const int t = (int)(z - j * 2 * d), h = t >= d ? 1 : 0, tc = t - h * d;
+            int64_t off, m;
+            seg_geom(n, L, j, off, m);
+            double total_sum = 0.0;
+            long long cnt = 0;
+            for (int64_t c0 = 0; c0 < C; c0 += 32) {
+                double sum = 0.0;
+                int nc = 0;
+                if (c0 + lane < C) {
+                    int64_t b, e;
+                    chunk_range(off, m, C, c0 + lane, b, e);
+#pragma unroll 4
+                    for (int64_t p = b; p < e; p++) {
+                        const int id = perm[p];
+                        const double x = (unsigned)id < (unsigned)n ? widen(ldx(X + (int64_t)id * ld + tc)) : widen(ldx(X + tc));
+                        if (halves[p] == h) {
+                            sum += x;
+                            nc++;
+                        }
+                    }
+                }
+                for (int s = 0; s < 32 && c0 + s < C; s++) {
+                    const double v = __shfl_sync(FULL_MASK, sum, s);
+                    total_sum = C > 1 ? total_sum + v : v;
+                    cnt += __shfl_sync(FULL_MASK, nc, s);
+                }
+            }
+            if (lane == 0)
+                cen[z] = (float)(total_sum / (double)cnt);
         }
-        if (nu > 0.0)
-            cj[t] = (float)(su / nu);
-        if (nv > 0.0)
-            cj[d + t] = (float)(sv / nv);
     }
 }
 
@@ -682,8 +902,11 @@ struct TreeBufs {
     unsigned *ghist;
     Top2 *seeds;
     float *cen;
-    double *part;
-    size_t bytes;
+    unsigned long long *acc;  // limb sums of the clusters of several chunks [2][3][d]; flags, masses [2][d]; counts [2]
+    unsigned *flg, *cnts, *colmax;
+    float *mass;
+    uint8_t *halves;
+    size_t zero_off, zero_bytes, bytes;
 };
 
 TreeBufs tree_carve(void *scratch, int64_t n, int64_t d, int32_t k)
@@ -691,14 +914,12 @@ TreeBufs tree_carve(void *scratch, int64_t n, int64_t d, int32_t k)
     Carver cv{static_cast<char *>(scratch), 0, 0};
     const int Lf = tree_depth(k);
     const int64_t S = (int64_t)1 << Lf;
-    int64_t part = 1, chunks = 1, multi = 1;  // doubles of partial sums; chunk blocks; clusters of several chunks
+    int64_t chunks = 1, multi = 1;  // chunk blocks; clusters of several chunks
     for (int L = 0; L <= Lf; L++) {
         const int64_t C = tree_chunks(n, L);
         chunks = std::max(chunks, ((int64_t)1 << L) * C);
-        if (C > 1) {
-            part = std::max(part, ((int64_t)1 << L) * C * (2 * d + 2));
+        if (C > 1)
             multi = std::max(multi, (int64_t)1 << L);
-        }
     }
     TreeBufs B{};
     B.perm_a = cv.take<int32_t>((size_t)n);
@@ -713,23 +934,36 @@ TreeBufs tree_carve(void *scratch, int64_t n, int64_t d, int32_t k)
     B.ccount = cv.take<int32_t>((size_t)chunks);
     B.cbase = cv.take<int32_t>((size_t)chunks);
     B.ghist = cv.take<unsigned>((size_t)multi * 256);
-    B.part = cv.take<double>((size_t)part);
+    B.halves = cv.take<uint8_t>((size_t)n);
+    B.zero_off = cv.off;  // from here on zero before the first pass
+    B.colmax = cv.take<unsigned>((size_t)d);
+    B.acc = cv.take<unsigned long long>((size_t)multi * 6 * (size_t)d);
+    B.flg = cv.take<unsigned>((size_t)multi * 2 * (size_t)d);
+    B.mass = cv.take<float>((size_t)multi * 2 * (size_t)d);
+    B.cnts = cv.take<unsigned>((size_t)multi * 2);
+    B.zero_bytes = cv.off - B.zero_off;
     B.bytes = cv.off;
     return B;
 }
 
 // Per depth L (S clusters, C chunk blocks per cluster; spl = NULL when every cluster splits):
-//   seeds (2 launches), iters x {pass, reduce if C > 1}, keys pass, select (1 launch, or 17 when C > 1),
+//   seeds (2 launches), iters x {pass, centres if C > 1, redo}, keys pass, select (1 launch, or 17 when C > 1),
 //   split (1 launch, or 3 when C > 1).
 template <typename XT>
 cudaError_t tree_run(const XT *X, int64_t n, int d, int64_t ld, int32_t k, int32_t iters, uint64_t seed,
-                     int32_t *labels, const TreeBufs &B, DevStatus *st, cudaStream_t s)
+                     int32_t *labels, void *scratch, const TreeBufs &B, DevStatus *st, cudaStream_t s)
 {
     cudaError_t e;
     if ((e = set_max_smem((const void *)k_tree_pass<XT, false>, (int)pass_smem(MAX_D))) != cudaSuccess ||
         (e = set_max_smem((const void *)k_tree_pass<XT, true>, (int)pass_smem(MAX_D))) != cudaSuccess)
         return e;
     const size_t smem = pass_smem(d);
+    const bool vec = x_vec4(X, d, ld);
+    if ((e = cudaMemsetAsync(static_cast<char *>(scratch) + B.zero_off, 0, B.zero_bytes, s)) != cudaSuccess)
+        return e;
+    if (iters > 0)
+        k_tree_colmax<XT><<<dim3((unsigned)std::min<int64_t>((n + 63) / 64, 152 * 8), (unsigned)((d + 127) / 128)), 256, 0,
+                            s>>>(X, n, d, ld, vec, B.colmax);
     k_tree_iota<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, s>>>(B.perm_a, n);
     const int Lf = tree_depth(k);
     const int64_t r = (int64_t)k - ((int64_t)1 << Lf);
@@ -748,12 +982,15 @@ cudaError_t tree_run(const XT *X, int64_t n, int d, int64_t ld, int32_t k, int32
         k_tree_seed_part<<<SC, SEL_THREADS, 0, s>>>(n, L, C, cur, spl, seed, B.seeds);
         k_tree_seed_final<XT><<<(unsigned)S, TR_THREADS, 0, s>>>(X, n, d, ld, C, spl, B.seeds, B.cen, st);
         for (int it = 0; it < iters; it++) {
-            k_tree_pass<XT, false><<<SC, TR_THREADS, smem, s>>>(X, n, d, ld, L, C, cur, spl, B.cen, B.part, B.keys,
-                                                                st);
+            k_tree_pass<XT, false><<<SC, TR_THREADS, smem, s>>>(X, n, d, ld, vec, L, C, cur, spl, B.cen, B.colmax, B.acc,
+                                                                B.flg, B.mass, B.cnts, B.halves, B.keys, st);
+            const unsigned cb = (unsigned)std::min<int64_t>((S * 2 * d + 255) / 256, 152 * 8);
             if (C > 1)
-                k_tree_reduce<<<(unsigned)S, TR_THREADS, 0, s>>>(d, C, spl, B.cen, B.part);
+                k_tree_centres<<<cb, 256, 0, s>>>(S, d, C, spl, B.cen, B.colmax, B.acc, B.flg, B.mass, B.cnts);
+            k_tree_redo<XT><<<cb, 256, 0, s>>>(X, n, d, ld, L, S, C, cur, spl, B.halves, B.cen, B.cnts);
         }
-        k_tree_pass<XT, true><<<SC, TR_THREADS, smem, s>>>(X, n, d, ld, L, C, cur, spl, B.cen, B.part, B.keys, st);
+        k_tree_pass<XT, true><<<SC, TR_THREADS, smem, s>>>(X, n, d, ld, vec, L, C, cur, spl, B.cen, B.colmax, B.acc, B.flg,
+                                                           B.mass, B.cnts, B.halves, B.keys, st);
         if (C == 1) {
             k_tree_select<<<(unsigned)S, SEL_THREADS, 0, s>>>(n, L, spl, B.keys, B.thr);
             k_tree_split<<<SC, SEL_THREADS, 0, s>>>(n, L, C, spl, B.keys, B.thr, nullptr, cur, nxt, st);
@@ -784,8 +1021,8 @@ cudaError_t launch_tree(const void *X, bool bf16, int64_t n, int64_t d, int64_t 
 {
     const TreeBufs B = tree_carve(scratch, n, d, k);
     if (bf16)
-        return tree_run(static_cast<const __nv_bfloat16 *>(X), n, (int)d, ld, k, iters, seed, labels, B, st, s);
-    return tree_run(static_cast<const float *>(X), n, (int)d, ld, k, iters, seed, labels, B, st, s);
+        return tree_run(static_cast<const __nv_bfloat16 *>(X), n, (int)d, ld, k, iters, seed, labels, scratch, B, st, s);
+    return tree_run(static_cast<const float *>(X), n, (int)d, ld, k, iters, seed, labels, scratch, B, st, s);
 }
 
 }  // namespace gkm

@@ -108,3 +108,29 @@ def test_tree_full_size(G):
     outer = np.searchsorted(bounds, starts, side="right")  # the depth-2 cluster holding each of the k clusters
     want = O.two_means_tree(X.cpu().numpy(), 4, iters=2, seed=3)
     assert np.array_equal(outer[L1.cpu().numpy()], want)
+
+
+@pytest.mark.parametrize("kind", ["tiny", "huge", "outlier", "subnormal", "zeros", "ties"])
+@pytest.mark.parametrize("n,d,k", [(511, 9, 20), (512, 65, 8), (1025, 64, 16), (6001, 132, 24)])
+def test_tree_centres_of_any_scale(G, kind, n, d, k):
+    # the centres' sums are split into integers by column scale: columns far from 1, of a range beyond the split's,
+    # below FP32's normal range, mostly zero, and means half way between two floats
+    g = np.random.default_rng(n + d)
+    X = datagen.gauss_mixture(n, d, 12, seed=n)
+    if kind == "tiny":
+        X = X * np.float32(1e-17)  # squares stay normal
+    elif kind == "huge":
+        X = X * np.float32(1e16)
+    elif kind == "outlier":
+        X[g.integers(0, n, 3)] *= np.float32(1e9)
+        X[:, 1] *= np.float32(1e-9)
+    elif kind == "subnormal":
+        X[:, ::2] = (g.integers(-9, 10, X[:, ::2].shape) * np.float32(1.4e-45)).astype(np.float32)
+        X[g.integers(0, n, 2), 0] = np.float32(3e9)  # that column scales its subnormal values away
+    elif kind == "zeros":
+        X[g.random(X.shape) < 0.9] = 0
+    else:
+        X = (1 + g.integers(0, 2, X.shape) * 2.0 ** -23).astype(np.float32) + np.float32(2.0 ** -20) * g.integers(
+            0, 8, (n, 1)).astype(np.float32)
+    X = np.ascontiguousarray(X, np.float32)
+    assert np.array_equal(_run(G, X, k, 3, 5), O.two_means_tree(X, k, iters=3, seed=5))
