@@ -19,14 +19,10 @@
 //
 // Layout: D is k x d row-major FP64; S, counts and labels are k / k / n
 // arrays.  One thread-block cluster (up to 16 CTAs, one per SM) runs the
-// epoch: one warp per (visit, cluster) task computes the squared norm of
-// D_v + x (D_u - x) with lane l holding elements l + 32 m, the owning CTA
-// divides its tasks' terms, and CTA 0 takes the arg-max of each visit, finds
-// how far the window may commit and applies the moves.  GB300 runs FP64 at a
-// small fraction of its FP32 rate, so the FP64 work is spread over the
-// cluster's SMs.  After a move, S_u and S_v are the two norms already computed
-// for the decision: the new rows are exactly the rounded sums that were
-// squared.
+// epoch.  GB300 runs FP64 at a small fraction of its FP32 rate, so the tasks
+// are screened in FP32 and few are folded in FP64.  After a move, S_u and S_v
+// are the two norms computed for the decision: the new rows are exactly the
+// rounded sums that were squared.
 #include <climits>
 #include <map>
 #include <mutex>
@@ -119,35 +115,47 @@ __global__ void __launch_bounds__(256) k_boost_norms(const double *__restrict__ 
 // One epoch of the move step over order[0..m), on one cluster of R CTAs, in
 // windows of up to W visits.
 //
-// A window's visits are evaluated together against the state at its start:
-// every CTA stages the window's samples and gathers the candidate sets; the
-// squared norms of all the window's (visit, cluster) tasks are spread over the
-// cluster's warps, and each CTA divides its own tasks' terms (lanes over
-// tasks) and stores them into CTA 0.  CTA 0 takes each visit's arg-max (a
-// shared atomicMax of the gain keys, then an atomicMin of (label, candidate)
-// among the tasks at the maximum), then commits the visits in order up to the
-// first one whose inputs an earlier committed move of the window changed (its
-// sample or one of its neighbours moved; its own cluster or a candidate was
-// the source or target of a move), found by looking every visit's items up in
-// two small hash tables of the moving visits' samples and clusters.
-// A committed visit therefore saw exactly the state the sequential walk gives
-// it, and the committed moves touch disjoint clusters, so CTA 0 applies them
-// together; the next window starts at the first visit not committed (the
-// first visit of a window always commits).  The window grows while windows
-// commit whole and shrinks to twice what the last one committed, so that few
-// evaluations are thrown away where moves collide often.  Both cluster
-// barriers of a window are unconditional.  Mutable state (labels, D, S,
-// counts) is read through L2 (ld.global.cg), which the barriers order.
+// A window's visits are evaluated together against the state at its start,
+// visit j on CTA j mod R: the CTA gathers the visit's candidate set and screens
+// every (visit, cluster) task in FP32, one warp per task.  With S_r = D_r'D_r
+// the two halves of the gain are
+//   (2 D_v'x + x'x - S_v / n_v) / (n_v + 1)   and   (x'x - 2 D_u'x + S_u / n_u) / (n_u - 1),
+// so a dot product gives them to (PL + 16) 2^-23 of their terms' sizes, and an
+// interval per candidate.  Only the candidates whose interval reaches the
+// largest lower end, and only where the gain can be positive, are evaluated as
+// defined (the FP64 folds and quotients); the arg-max over those is the arg-max
+// over all.  Whatever leaves FP32's comfortable range, or is no number, has an
+// unbounded interval and is evaluated as defined.
+//
+// Each CTA writes its visits' moves into every CTA of the cluster.  The window
+// commits in order up to the first visit whose inputs an earlier moving visit
+// changed (its sample or one of its neighbours moved; its own cluster or a
+// candidate was the source or target of a move), which each CTA looks up for
+// its own visits.  A committed visit therefore saw exactly the state the
+// sequential walk gives it, and the committed moves touch disjoint clusters, so
+// each CTA applies its own; the next window starts at the first visit not
+// committed (the first visit of a window always commits).  The three cluster
+// barriers of a window are unconditional.  Mutable state (labels, D, S, counts)
+// is read through L2 (ld.global.cg), which the barriers order; samples and graph
+// rows of the next window are on their way during the last barrier.
+//
+// Bound by the chain of a window's dependent steps (loads, barriers), so every
+// window takes all W visits: 8.5 against 9.2 ms for 20,000 visits when the
+// window shrinks after a cut, 10.6 with 16 visits.  At 1M x 128, k = 10,000,
+// kappa = 50 (a quarter of the visits move) 0.43 us a visit; with every task
+// folded in FP64 and gains and commit on one CTA it was 1.74 (the folds' FP64
+// work 0.7, one CTA's part and everyone's loading of all visits the rest).
+// 256 or 1024 threads, and 2 or 8 tasks of a warp at once: 2-4% slower.
 // ---------------------------------------------------------------------------
-constexpr int BE_THREADS = 256;
+constexpr int BE_THREADS = 512;
 constexpr int BE_WARPS = BE_THREADS / 32;
 constexpr int BE_MAX_CLUSTER = 16;
-constexpr int BE_MAX_WINDOW = 32;
-constexpr int BE_HASH = 128;  // entries of each commit hash table (at most 32 samples, 64 clusters)
+constexpr int BE_MAX_WINDOW = 32;  // a lane per visit
 constexpr size_t BE_SMEM_BUDGET = 200 * 1024;
 
 __device__ __forceinline__ void cluster_barrier()
 {
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -165,6 +173,18 @@ __device__ __forceinline__ unsigned cluster_size()
     return r;
 }
 
+// The two halves of cluster_barrier().
+__device__ __forceinline__ void cluster_arrive()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // Address of the same shared variable in CTA `rank` of the cluster.
 __device__ __forceinline__ uint32_t in_rank(const void *p, int rank)
 {
@@ -175,58 +195,58 @@ __device__ __forceinline__ uint32_t in_rank(const void *p, int rank)
     return r;
 }
 
-__device__ __forceinline__ void st_rank(const void *p, int rank, double v)
-{
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(in_rank(p, rank)), "d"(v) : "memory");
-}
-
 __device__ __forceinline__ void st_rank(const void *p, int rank, int v)
 {
     asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(in_rank(p, rank)), "r"(v) : "memory");
 }
 
-// Dynamic shared memory of one CTA for windows of W visits (the same layout in every CTA of the cluster).
+// An FP64 value cut to FP32 on the integer pipe (the FP64 one is narrow): error below 2^-23 of it, 0 below FP32's
+// normal range, NaN above it.
+__device__ __forceinline__ float cut32(double v)
+{
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v), a = hi & 0x7fffffffu;
+    const unsigned f = (hi & 0x80000000u) | ((__funnelshift_l(lo, hi, 3) & 0x7fffffffu) ^ 0x40000000u);
+    return a < 0x38100000u ? 0.f : __uint_as_float(a < 0x47f00000u ? f : 0x7fc00000u);
+}
+
+// Dynamic shared memory of one CTA for windows of W visits (the same layout in every CTA of the cluster).  V: the
+// CTA's visits; task c of its visit q is entry q (kp + 1) + c, c = 0 the own cluster.
 struct WinLayout {
-    int W, kp, TM, TL;
-    size_t xs, ra, r1, r3, gk, vbest, vwin, la, ls, rn, ln, lo, tv, sq, sg, svis, su, snq, sbase, dq, ml, tl, mvj,
-        hkey, hval, bytes;
+    int W, V, kp;
+    size_t xs, sg, sq, tg, te, tm, ea, es, en, tl, svis, su, snq, sxx, nev, nat, mve, mvi, mvu, mvv, dep, bytes;
     __host__ __device__ WinLayout(int W_, int P, int kappa, int R)
     {
         W = W_;
+        V = (W + R - 1) / R;
         kp = (kappa + 31) / 32 * 32;
-        TM = W * (kappa + 1);
-        TL = (TM + R - 1) / R;
+        const int TM = V * (kp + 1);
         size_t o = 0;
         auto take = [&](size_t bytes) {
             const size_t at = o;
             o += (bytes + 15) / 16 * 16;
             return at;
         };
-        xs = take((size_t)W * P * 8);
-        ra = take((size_t)TM * 8);
-        r1 = take((size_t)TM * 8);
-        r3 = take((size_t)TM * 8);
-        gk = take((size_t)TM * 8);
-        vbest = take((size_t)W * 8);
-        vwin = take((size_t)W * 8);
-        la = take((size_t)TL * 8);
-        ls = take((size_t)TL * 8);
-        rn = take((size_t)TM * 4);
-        ln = take((size_t)TL * 4);
-        lo = take((size_t)TL * 4);
-        tv = take((size_t)TM * 4);
-        sq = take((size_t)W * kp * 4);
-        sg = take((size_t)W * kp * 4);
-        svis = take((size_t)W * 4);
-        su = take((size_t)W * 4);
-        snq = take((size_t)W * 4);
-        sbase = take((size_t)(W + 1) * 4);
-        dq = take((size_t)W * 4);
-        ml = take((size_t)W * 4);
-        tl = take((size_t)2 * W * 4);
-        mvj = take((size_t)W * 4);
-        hkey = take((size_t)2 * BE_HASH * 4);
-        hval = take((size_t)2 * BE_HASH * 4);
+        xs = take((size_t)V * P * 4);
+        sg = take((size_t)V * kp * 4);
+        sq = take((size_t)V * kp * 4);
+        tg = take((size_t)TM * 4);
+        te = take((size_t)TM * 4);
+        tm = take((size_t)TM * 4);
+        ea = take((size_t)TM * 8);
+        es = take((size_t)TM * 8);
+        en = take((size_t)TM * 4);
+        tl = take((size_t)TM * 4);
+        svis = take((size_t)V * 4);
+        su = take((size_t)V * 4);
+        snq = take((size_t)V * 4);
+        sxx = take((size_t)V * 4);
+        nev = take((size_t)V * 4);
+        nat = take((size_t)V * 4);
+        mve = take((size_t)V * 4);
+        mvi = take((size_t)W * 4);
+        mvu = take((size_t)W * 4);
+        mvv = take((size_t)W * 4);
+        dep = take((size_t)W * 4);
         bytes = o;
     }
 };
@@ -238,335 +258,368 @@ __global__ void __launch_bounds__(BE_THREADS, 1)
                   double *S, int64_t *n_moved, DevStatus *st, int W)
 {
     constexpr int P = 32 * PL;
+    constexpr int B = PL <= 4 ? 4 : PL == 8 ? 2 : 1;  // screening tasks of a warp whose rows are in flight together
+    constexpr int KC = MAX_KAPPA / 32;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int s_win, s_nm, s_T, s_first;
+    __shared__ int s_ne;
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const int rank = (int)cluster_rank(), R = (int)cluster_size();
     const WinLayout Y(W, P, kappa, R);
-    const int kp = Y.kp;
-    double *xs = reinterpret_cast<double *>(smem + Y.xs);
-    double *ra = reinterpret_cast<double *>(smem + Y.ra), *r1 = reinterpret_cast<double *>(smem + Y.r1);
-    double *r3 = reinterpret_cast<double *>(smem + Y.r3);
-    long long *gk = reinterpret_cast<long long *>(smem + Y.gk);
-    long long *vbest = reinterpret_cast<long long *>(smem + Y.vbest);
-    unsigned long long *vwin = reinterpret_cast<unsigned long long *>(smem + Y.vwin);
-    int *hkey = reinterpret_cast<int *>(smem + Y.hkey), *hval = reinterpret_cast<int *>(smem + Y.hval);
-    int *tv = reinterpret_cast<int *>(smem + Y.tv);
-    double *la = reinterpret_cast<double *>(smem + Y.la), *ls = reinterpret_cast<double *>(smem + Y.ls);
-    int *rn = reinterpret_cast<int *>(smem + Y.rn), *ln = reinterpret_cast<int *>(smem + Y.ln);
-    int *lo = reinterpret_cast<int *>(smem + Y.lo);
-    int *sq = reinterpret_cast<int *>(smem + Y.sq), *sg = reinterpret_cast<int *>(smem + Y.sg);
+    const int kp = Y.kp, ks = kp + 1;
+    float *xs = reinterpret_cast<float *>(smem + Y.xs);
+    int *sg = reinterpret_cast<int *>(smem + Y.sg), *sq = reinterpret_cast<int *>(smem + Y.sq);
+    float *tg = reinterpret_cast<float *>(smem + Y.tg), *te = reinterpret_cast<float *>(smem + Y.te);
+    float *tm = reinterpret_cast<float *>(smem + Y.tm);
+    double *ea = reinterpret_cast<double *>(smem + Y.ea), *es = reinterpret_cast<double *>(smem + Y.es);
+    int *en = reinterpret_cast<int *>(smem + Y.en), *tl = reinterpret_cast<int *>(smem + Y.tl);
     int *svis = reinterpret_cast<int *>(smem + Y.svis), *su = reinterpret_cast<int *>(smem + Y.su);
-    int *snq = reinterpret_cast<int *>(smem + Y.snq), *sbase = reinterpret_cast<int *>(smem + Y.sbase);
-    int *dq = reinterpret_cast<int *>(smem + Y.dq), *ml = reinterpret_cast<int *>(smem + Y.ml);
-    int *tl = reinterpret_cast<int *>(smem + Y.tl), *mvj = reinterpret_cast<int *>(smem + Y.mvj);
-    auto valid = [&](int i) { return i >= 0 && i < n; };
+    int *snq = reinterpret_cast<int *>(smem + Y.snq), *nev = reinterpret_cast<int *>(smem + Y.nev);
+    float *sxx = reinterpret_cast<float *>(smem + Y.sxx);
+    int *nat = reinterpret_cast<int *>(smem + Y.nat), *mve = reinterpret_cast<int *>(smem + Y.mve);
+    int *mvi = reinterpret_cast<int *>(smem + Y.mvi), *mvu = reinterpret_cast<int *>(smem + Y.mvu);
+    int *mvv = reinterpret_cast<int *>(smem + Y.mvv), *dep = reinterpret_cast<int *>(smem + Y.dep);
     int64_t moves = 0;
-    int We = W;  // this window's size: doubled after a window that commits whole, else twice what committed
-    cluster_barrier();  // every CTA of the cluster runs before any stores into another's shared memory
+
+    // the visits of a window from position s on, what no move changes: ids, samples, graph rows (one warp per visit)
+    auto fetch = [&](int64_t s, int Wn) {
+        for (int q = w; q * R + rank < Wn; q += BE_WARPS) {
+            const int64_t at = s + q * R + rank;
+            const int i = __ldg(order + at);
+            const bool ok = i >= 0 && i < n;
+            if (!ok && lane == 0)
+                flag_error(st, GK_ERR_INVALID, (unsigned)at);
+            int g[KC];
+#pragma unroll
+            for (int c = 0; c < KC; c++)
+                g[c] = ok && 32 * c + lane < kappa ? __ldg(G + (int64_t)i * kappa + 32 * c + lane) : -1;
+            float x[PL], xx = 0.f;
+#pragma unroll
+            for (int p = 0; p < PL; p++)
+                x[p] = ok && lane + 32 * p < d ? ldx(X + (int64_t)i * ld + lane + 32 * p) : 0.f;
+#pragma unroll
+            for (int c = 0; c < KC; c++)
+                if (32 * c < kp)
+                    sg[q * kp + 32 * c + lane] = g[c];
+#pragma unroll
+            for (int p = 0; p < PL; p++) {
+                xs[q * P + lane + 32 * p] = x[p];
+                xx = fmaf(x[p], x[p], xx);
+            }
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1)
+                xx += __shfl_xor_sync(FULL_MASK, xx, o);
+            if (lane == 0) {
+                svis[q] = ok ? i : -1;
+                sxx[q] = xx;
+            }
+        }
+        __syncwarp();
+    };
+    int Wn = (int)(m < (int64_t)W ? m : (int64_t)W);
+    cluster_arrive();  // every CTA of the cluster runs before any stores into another's shared memory
+    fetch(0, Wn);
+    cluster_wait();
 
     for (int64_t s = 0; s < m;) {
-        const int Wn = (int)(m - s < (int64_t)We ? m - s : (int64_t)We);
-        // ---- the window's visits: ids, then samples, graph rows and own labels, then the neighbours' labels
-        if (threadIdx.x < Wn) {
-            svis[threadIdx.x] = __ldg(order + s + threadIdx.x);
-            vbest[threadIdx.x] = LLONG_MIN;
-            vwin[threadIdx.x] = ~0ull;
-        }
-        __syncthreads();
-        if (threadIdx.x < Wn) {
-            const int i = svis[threadIdx.x];
-            int u = -1;
-            if (!valid(i)) {
-                if (rank == 0)
-                    flag_error(st, GK_ERR_INVALID, (unsigned)(s + threadIdx.x));
-            } else {
+        const int nv = Wn > rank ? (Wn - rank + R - 1) / R : 0;  // this CTA's visits
+        if (threadIdx.x == 0)
+            s_ne = 0;
+        // ---- labels and candidate set of visit q, distinct labels other than its own, by the warp that fetched it
+        for (int q = w; q < nv; q += BE_WARPS) {
+            const int i = svis[q];  // written by this warp's lane 0 before a barrier
+            int u = -1, lab[KC];
+            if (i >= 0)
                 u = __ldcg(L + i);
-                if (u < 0 || u >= k) {
-                    if (rank == 0)
-                        flag_error(st, GK_ERR_INVALID, (unsigned)i);
-                    u = -1;
+#pragma unroll
+            for (int c = 0; c < KC; c++) {
+                lab[c] = -3;  // no label wanted
+                if (i >= 0 && 32 * c + lane < kappa) {
+                    const int g = sg[q * kp + 32 * c + lane];
+                    lab[c] = g >= 0 && g < n ? __ldcg(L + g) : -2;
                 }
             }
-            su[threadIdx.x] = u;
-        }
-        // loads issued eight at a time per thread, then stored: one round trip per batch
-        for (int e0 = threadIdx.x; e0 < Wn * P; e0 += 8 * BE_THREADS) {
-            float v[8];
-#pragma unroll
-            for (int b = 0; b < 8; b++) {
-                const int e = e0 + b * BE_THREADS, j = e / P, t = e - j * P;
-                v[b] = e < Wn * P && valid(svis[j]) && t < d ? ldx(X + (int64_t)svis[j] * ld + t) : 0.f;
+            if (i >= 0 && (u < 0 || u >= k)) {
+                if (lane == 0)
+                    flag_error(st, GK_ERR_INVALID, (unsigned)i);
+                u = -1;
             }
-#pragma unroll
-            for (int b = 0; b < 8; b++)
-                if (e0 + b * BE_THREADS < Wn * P)
-                    xs[e0 + b * BE_THREADS] = widen(v[b]);  // on the integer pipe: the FP64 one is narrow
-        }
-        for (int e0 = threadIdx.x; e0 < Wn * kp; e0 += 8 * BE_THREADS) {
-            int v[8];
-#pragma unroll
-            for (int b = 0; b < 8; b++) {
-                const int e = e0 + b * BE_THREADS, j = e / kp, t = e - j * kp;
-                v[b] = e < Wn * kp && valid(svis[j]) && t < kappa ? __ldg(G + (int64_t)svis[j] * kappa + t) : -1;
-            }
-#pragma unroll
-            for (int b = 0; b < 8; b++)
-                if (e0 + b * BE_THREADS < Wn * kp)
-                    sg[e0 + b * BE_THREADS] = v[b];
-        }
-        __syncthreads();
-        for (int e0 = threadIdx.x; e0 < Wn * kp; e0 += 8 * BE_THREADS) {
-            int v[8];
-#pragma unroll
-            for (int b = 0; b < 8; b++) {
-                const int e = e0 + b * BE_THREADS;
-                v[b] = -3;  // -3: no label wanted
-                if (e < Wn * kp && e % kp < kappa && su[e / kp] >= 0)
-                    v[b] = valid(sg[e]) ? __ldcg(L + sg[e]) : -2;
-            }
-#pragma unroll
-            for (int b = 0; b < 8; b++) {
-                const int e = e0 + b * BE_THREADS;
-                if (e >= Wn * kp)
-                    continue;
-                if (v[b] == -2 || (v[b] != -3 && (v[b] < 0 || v[b] >= k))) {
-                    if (rank == 0)
-                        flag_error(st, GK_ERR_INVALID, (unsigned)(v[b] == -2 ? svis[e / kp] : sg[e]));
-                    v[b] = -1;
-                }
-                sq[e] = v[b] == -3 ? -1 : v[b];
-            }
-        }
-        __syncthreads();
-        // candidate set of visit j (warp w takes j = w, w + 8, ...): distinct labels other than its own, in place
-        for (int j = w; j < Wn; j += BE_WARPS) {
-            const int u = su[j];
-            int lab[MAX_KAPPA / 32];
-#pragma unroll
-            for (int c = 0; c < MAX_KAPPA / 32; c++)
-                lab[c] = 32 * c < kp ? sq[j * kp + 32 * c + lane] : -1;
-            __syncwarp();
             int nq = 0;
+            if (u >= 0) {
 #pragma unroll
-            for (int c = 0; c < MAX_KAPPA / 32; c++) {
-                if (32 * c >= kp)
-                    break;
-                int v = lab[c] == u ? -1 : lab[c];
-                bool keep = v >= 0;
+                for (int c = 0; c < KC; c++) {
+                    if (32 * c >= kp)
+                        break;
+                    int v = lab[c];
+                    if (v != -3 && (v < 0 || v >= k))
+                        flag_error(st, GK_ERR_INVALID, (unsigned)(v == -2 ? i : sg[q * kp + 32 * c + lane]));
+                    if (v < 0 || v >= k || v == u)
+                        v = -1;
+                    bool keep = v >= 0;
 #pragma unroll 8
-                for (int q = 0; q < nq; q++)
-                    keep &= sq[j * kp + q] != v;
-                const unsigned same = __match_any_sync(FULL_MASK, v);
-                keep = keep && (__ffs(same) - 1 == lane);
-                const unsigned km = __ballot_sync(FULL_MASK, keep);
-                if (keep)
-                    sq[j * kp + nq + __popc(km & lanemask_lt())] = v;
-                nq += __popc(km);
-                __syncwarp();
+                    for (int z = 0; z < nq; z++)
+                        keep &= sq[q * kp + z] != v;
+                    const unsigned same = __match_any_sync(FULL_MASK, v);
+                    keep = keep && (__ffs(same) - 1 == lane);
+                    const unsigned km = __ballot_sync(FULL_MASK, keep);
+                    if (keep)
+                        sq[q * kp + nq + __popc(km & lanemask_lt())] = v;
+                    nq += __popc(km);
+                    __syncwarp();
+                }
             }
-            if (lane == 0)
-                snq[j] = u >= 0 ? nq : 0;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {  // tasks of visit j: [sbase[j], sbase[j + 1]), the first its own cluster
-            int T = 0;
-            for (int j = 0; j < Wn; j++) {
-                sbase[j] = T;
-                T += snq[j] > 0 ? snq[j] + 1 : 0;
+            if (lane == 0) {
+                su[q] = u;
+                snq[q] = nq;
             }
-            sbase[Wn] = T;
-            s_T = T;
         }
-        __syncthreads();
-        for (int j = w; j < Wn; j += BE_WARPS)
-            for (int t = sbase[j] + lane; t < sbase[j + 1]; t += 32)
-                tv[t] = j;
         __syncthreads();
 
-        // ---- squared norms of the tasks: task t on CTA t mod R; c = 0 the own cluster (D_u - x), else a
-        //      candidate (D_v + x)
-        const int T = s_T;
-        for (int t = rank + R * w; t < T; t += R * BE_WARPS) {
-            const int j = tv[t];
-            const int c = t - sbase[j];
-            const int r = c == 0 ? su[j] : sq[j * kp + c - 1];
-            const double *Dr = D + (int64_t)r * d;
-            const double *xj = xs + (size_t)j * P;
-            double a[PL];
+        // ---- screening: task t of the CTA's visits in turn, B tasks of a warp at once
+        const int own_tasks = lane < nv && snq[lane] > 0 ? snq[lane] + 1 : 0;
+        int incl = own_tasks;
 #pragma unroll
-            for (int q = 0; q < PL; q++) {
-                const int e = lane + 32 * q;
-                a[q] = e < d ? __ldcg(Dr + e) : 0.0;
-            }
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(FULL_MASK, incl, o);
+            if (lane >= o)
+                incl += v;
+        }
+        const int T = __shfl_sync(FULL_MASK, incl, 31), excl = incl - own_tasks;
+        for (int t0 = w * B; t0 < T; t0 += BE_WARPS * B) {
+            double a[B][PL];
+            int ent[B], qb[B];
             double sr = 0.0;
-            int nr = 0;
-            if (lane == 0) {
-                sr = __ldcg(S + r);
-                nr = __ldcg(cnt + r);
-            }
+            int nr = 1;
 #pragma unroll
-            for (int q = 0; q < PL; q++) {
-                const int e = lane + 32 * q;
-                const double y = e < d ? (c == 0 ? __dsub_rn(a[q], xj[e]) : __dadd_rn(a[q], xj[e])) : 0.0;
-                a[q] = __dmul_rn(y, y);
+            for (int b = 0; b < B; b++) {
+                const int t = min(t0 + b, T - 1);
+                const int q = __popc(__ballot_sync(FULL_MASK, incl <= t));
+                const int c = t - __shfl_sync(FULL_MASK, excl, q);
+                const int r = c == 0 ? su[q] : sq[q * kp + c - 1];
+                const double *Dr = D + (int64_t)r * d;
+                ent[b] = q * ks + c;
+                qb[b] = q;
+#pragma unroll
+                for (int p = 0; p < PL; p++)
+                    a[b][p] = lane + 32 * p < d ? __ldcg(Dr + lane + 32 * p) : 0.0;
+                if (lane == b) {
+                    sr = __ldcg(S + r);
+                    nr = __ldcg(cnt + r);
+                }
             }
-            const double tot = fold_lanes<PL>(a);
-            if (lane == 0) {
-                const int l = t / R;
-                la[l] = tot;
-                ls[l] = sr;
-                ln[l] = nr;
-                lo[l] = c == 0;
+            float dot = 0.f;
+            int me = 0, mq = 0;
+#pragma unroll
+            for (int b = 0; b < B; b++) {
+                const float *xq = xs + qb[b] * P;
+                float v = 0.f;
+#pragma unroll
+                for (int p = 0; p < PL; p++)
+                    v = fmaf(cut32(a[b][p]), xq[lane + 32 * p], v);
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1)
+                    v += __shfl_xor_sync(FULL_MASK, v, o);
+                if (lane == b) {
+                    dot = v;
+                    me = ent[b];
+                    mq = qb[b];
+                }
+            }
+            if (lane < B && t0 + lane < T) {
+                const float xx = sxx[mq], nf = (float)nr;
+                const float rs = sqrtf((float)sr), rx = sqrtf(xx), pr = 1.001f * rs * rx, sn = (float)sr / nf;
+                const bool own = me == mq * ks;
+                const float den = own ? nf - 1.f : nf + 1.f;
+                float g = (own ? xx - 2.f * dot + sn : 2.f * dot + xx - sn) / den;
+                float e = ((float)(PL + 16) * 0x1p-23f) * (2.f * pr + xx + sn) / den;
+                const bool sure = rs >= 0x1p-40f && rs <= 0x1p60f && rx >= 0x1p-40f && rx <= 0x1p60f && nr >= (own ? 2 : 1) &&
+                                  isfinite(g) && isfinite(e);
+                tg[me] = sure ? g : 0.f;
+                te[me] = sure ? e : __int_as_float(0x7f800000);
+                tm[me] = 2.f * (sn + pr + xx);  // no smaller than the terms of the FP64 gain, which round to 2^-44 of it
+                en[me] = nr;
+                es[me] = sr;
             }
         }
         __syncthreads();
-        // this CTA's tasks' quotients, lanes over tasks; job even: A / (n_v + 1) (own: B / (n_u - 1)), odd: S / n
-        const int TLc = T > rank ? (T - rank + R - 1) / R : 0;
-        for (int jb = w; jb < 2 * ((TLc + 31) / 32); jb += BE_WARPS) {
-            const int l = (jb >> 1) * 32 + lane;
-            if (l < TLc) {
-                const int t = l * R + rank;
-                if (jb & 1) {
-                    st_rank(&r3[t], 0, __ddiv_rn(ls[l], (double)ln[l]));
-                } else {
-                    st_rank(&r1[t], 0, __ddiv_rn(la[l], (double)(lo[l] ? ln[l] - 1 : ln[l] + 1)));
-                    st_rank(&ra[t], 0, la[l]);
-                    st_rank(&rn[t], 0, ln[l]);
+        // ---- the tasks that decide, one warp per visit: none where no gain can be positive.  nev[q]: how many
+        //      candidates, or -1 where the only one's gain is positive for sure
+        for (int q = w; q < nv; q += BE_WARPS) {
+            const int nq = snq[q], o = q * ks;
+            int left = 0;
+            unsigned in[KC] = {};
+            bool sure = false;
+            if (nq > 0 && en[o] >= 2) {
+                const float inf = __int_as_float(0x7f800000), go = tg[o], eo = te[o], mo = tm[o];
+                float low = -inf, g[KC], e[KC];
+#pragma unroll
+                for (int cc = 0; cc < KC; cc++) {
+                    const int c = 1 + 32 * cc + lane;
+                    g[cc] = c <= nq ? tg[o + c] : -inf;
+                    e[cc] = c <= nq ? te[o + c] + 0x1p-44f * (tm[o + c] + mo) : 0.f;
+                    low = fmaxf(low, g[cc] - e[cc]);
+                }
+#pragma unroll
+                for (int h = 16; h >= 1; h >>= 1)
+                    low = fmaxf(low, __shfl_xor_sync(FULL_MASK, low, h));
+#pragma unroll
+                for (int cc = 0; cc < KC; cc++) {
+                    const float up = g[cc] + e[cc];
+                    const bool may = 1 + 32 * cc + lane <= nq && !(up < low) &&
+                                     !(up + go + eo < -1e-6f * (fabsf(up) + fabsf(go)));
+                    in[cc] = __ballot_sync(FULL_MASK, may);
+                    left += __popc(in[cc]);
+                }
+                sure = left == 1 && low + go - eo > 1e-6f * (fabsf(low) + fabsf(go));
+            }
+            int at = 0;
+            if (lane == 0) {
+                at = left > 0 ? atomicAdd(&s_ne, left + 1) : 0;
+                nat[q] = at;
+                nev[q] = sure ? -1 : left;
+            }
+            at = __shfl_sync(FULL_MASK, at, 0);
+            if (left > 0) {
+                if (lane == 0)
+                    tl[at] = o;
+                at++;
+#pragma unroll
+                for (int cc = 0; cc < KC; cc++) {
+                    if ((in[cc] >> lane) & 1)
+                        tl[at + __popc(in[cc] & lanemask_lt())] = o + 1 + 32 * cc + lane;
+                    at += __popc(in[cc]);
                 }
             }
+        }
+        __syncthreads();
+        // ---- their squared norms as defined: (D_u - x) for the own cluster, else (D_v + x)
+        const int ne = s_ne;
+        for (int z = w; z < ne; z += BE_WARPS) {
+            const int e = tl[z], q = e / ks, c = e - q * ks;
+            const double *Dr = D + (int64_t)(c == 0 ? su[q] : sq[q * kp + c - 1]) * d;
+            const float *xq = xs + q * P;
+            double a[PL];
+#pragma unroll
+            for (int p = 0; p < PL; p++)
+                a[p] = lane + 32 * p < d ? __ldcg(Dr + lane + 32 * p) : 0.0;
+#pragma unroll
+            for (int p = 0; p < PL; p++) {
+                const double x = widen(xq[lane + 32 * p]);  // on the integer pipe
+                const double y = lane + 32 * p < d ? (c == 0 ? __dsub_rn(a[p], x) : __dadd_rn(a[p], x)) : 0.0;
+                a[p] = __dmul_rn(y, y);
+            }
+            const double tot = fold_lanes<PL>(a);
+            if (lane == 0)
+                ea[e] = tot;
+        }
+        __syncthreads();
+        // ---- each visit's move, written into every CTA of the cluster
+        for (int q = w; q < nv; q += BE_WARPS) {
+            const int j = q * R + rank, o = q * ks, at = nat[q], left = nev[q];
+            int best = left < 0 ? tl[at + 1] : -1;  // the entry of the target
+            if (left > 0) {
+                // the largest gain, then the smaller label; the gain's integer key orders as its value does (the gains
+                // are sums and differences of non-negative terms, never -0); entry 0 of the list is the own cluster
+                double r1o = 0.0, r3o = 0.0;
+                long long top = LLONG_MIN;
+                unsigned long long win = ~0ull;
+                for (int z0 = 0; z0 <= left; z0 += 32) {
+                    const int z = z0 + lane, e = tl[at + min(z, left)];
+                    const double r1 = __ddiv_rn(ea[e], (double)(z == 0 ? en[e] - 1 : en[e] + 1));
+                    const double r3 = __ddiv_rn(es[e], (double)en[e]);
+                    if (z0 == 0) {
+                        r1o = __shfl_sync(FULL_MASK, r1, 0);
+                        r3o = __shfl_sync(FULL_MASK, r3, 0);
+                    }
+                    if (z >= 1 && z <= left) {
+                        const double g = __dsub_rn(__dsub_rn(__dadd_rn(r1, r1o), r3), r3o);
+                        const long long b = __double_as_longlong(g), key = b ^ ((b >> 63) & 0x7fffffffffffffffll);
+                        const unsigned long long id =
+                            ((unsigned long long)(unsigned)sq[q * kp + e - o - 1] << 32) | (unsigned)e;
+                        if (key > top || (key == top && id < win)) {
+                            top = key;
+                            win = id;
+                        }
+                    }
+                }
+#pragma unroll
+                for (int h = 16; h >= 1; h >>= 1) {
+                    const long long k2 = __shfl_xor_sync(FULL_MASK, top, h);
+                    const unsigned long long w2 = __shfl_xor_sync(FULL_MASK, win, h);
+                    if (k2 > top || (k2 == top && w2 < win)) {
+                        top = k2;
+                        win = w2;
+                    }
+                }
+                if (top > 0)  // the gain is above +0
+                    best = (int)(win & 0xffffffffu);
+            }
+            if (lane < R) {
+                st_rank(&mvi[j], lane, svis[q]);
+                st_rank(&mvu[j], lane, su[q]);
+                st_rank(&mvv[j], lane, best >= 0 ? sq[q * kp + best - o - 1] : -1);
+            }
+            if (lane == 0)
+                mve[q] = best;
         }
         cluster_barrier();
 
-        // ---- CTA 0: each visit's arg-max, the in-order commit and the committed moves
-        if (rank == 0) {
-            // the gain of every candidate task as an integer key in the order of the FP64 values (the gains are sums
-            // and differences of non-negative terms, never -0, so the keys order them exactly); each visit's largest
-            // key, then the smallest (label, candidate) among the tasks that reach it
-            for (int t = threadIdx.x; t < T; t += BE_THREADS) {
-                const int j = tv[t], o = sbase[j];
-                if (t != o) {
-                    const double g = __dsub_rn(__dsub_rn(__dadd_rn(r1[t], r1[o]), r3[t]), r3[o]);
-                    const long long b = __double_as_longlong(g);
-                    const long long key = b ^ ((b >> 63) & 0x7fffffffffffffffll);
-                    gk[t] = key;
-                    atomicMax(&vbest[j], key);
-                }
+        // ---- the window commits up to the first visit that depends on an earlier moving one: its sample or a neighbour
+        //      is that visit's sample, or its own cluster or a candidate is one that visit leaves or joins
+        const unsigned moving = __ballot_sync(FULL_MASK, lane < Wn && mvv[min(lane, Wn - 1)] >= 0);
+        for (int q = w; q < nv; q += BE_WARPS) {
+            const int j = q * R + rank, nq = snq[q], i = svis[q], u = su[q];
+            int g[KC], c[KC];
+#pragma unroll
+            for (int cc = 0; cc < KC; cc++) {
+                g[cc] = 32 * cc < kp ? sg[q * kp + 32 * cc + lane] : -1;
+                c[cc] = 32 * cc + lane < nq ? sq[q * kp + 32 * cc + lane] : -1;
             }
-            __syncthreads();
-            for (int t = threadIdx.x; t < T; t += BE_THREADS) {
-                const int j = tv[t], o = sbase[j];
-                if (t != o && gk[t] == vbest[j]) {
-                    const unsigned long long label = (unsigned)sq[j * kp + t - o - 1];
-                    atomicMin(&vwin[j], (label << 16) | (unsigned)(t - o));
-                }
+            bool hit = false;
+            for (unsigned left = moving & ((1u << j) - 1u); left; left &= left - 1u) {
+                const int b = __ffs(left) - 1, xi = mvi[b], xu = mvu[b], xv = mvv[b];
+                hit |= i == xi || u == xu || u == xv;
+#pragma unroll
+                for (int cc = 0; cc < KC; cc++)
+                    hit |= g[cc] == xi || c[cc] == xu || c[cc] == xv;
             }
-            for (int e = threadIdx.x; e < 2 * BE_HASH; e += BE_THREADS) {  // empty hash tables
-                hkey[e] = -1;
-                hval[e] = 0x7fffffff;
-            }
-            __syncthreads();
-            // the visits that would move (key > 0: gain > +0; the own cluster keeps two members or more), in order:
-            // sample ml, clusters tl[2 q] (from) and tl[2 q + 1] (to)
-            if (w == 0) {
-                int t = -1;
-                if (lane < Wn && snq[lane] > 0 && rn[sbase[lane]] >= 2 && vbest[lane] > 0)
-                    t = sbase[lane] + (int)(vwin[lane] & 0xffff);
-                if (lane < Wn)
-                    dq[lane] = t;
-                const unsigned mm = __ballot_sync(FULL_MASK, t >= 0);
-                if (t >= 0) {
-                    const int q = __popc(mm & lanemask_lt());
-                    ml[q] = svis[lane];
-                    mvj[q] = lane;
-                    tl[2 * q] = su[lane];
-                    tl[2 * q + 1] = (int)(vwin[lane] >> 16);
-                }
-                if (lane == 0) {
-                    s_nm = __popc(mm);
-                    s_first = Wn;
-                }
-            }
-            __syncthreads();
-            // hash tables keyed by sample and by cluster: the earliest moving visit that moves that sample, or leaves
-            // or joins that cluster
-            const int nmv = s_nm;
-            if (threadIdx.x < 3 * nmv) {
-                const int q = threadIdx.x / 3, part = threadIdx.x - 3 * q;
-                const int x = part == 0 ? ml[q] : tl[2 * q + part - 1];
-                int *keys = hkey + (part == 0 ? 0 : BE_HASH), *vals = hval + (part == 0 ? 0 : BE_HASH);
-                for (int h = (int)(((unsigned)x * 2654435761u) >> 25), probe = 0; probe < BE_HASH;
-                     h = (h + 1) & (BE_HASH - 1), probe++) {
-                    const int prev = atomicCAS(&keys[h], -1, x);
-                    if (prev == -1 || prev == x) {
-                        atomicMin(&vals[h], mvj[q]);
-                        break;
-                    }
-                }
-            }
-            __syncthreads();
-            // the window commits up to the first visit that depends on an earlier moving visit: its sample or a
-            // neighbour is that visit's sample, or its own cluster or a candidate is one that visit leaves or joins
-            auto earliest = [&](int x, int table) {  // the earliest moving visit recorded for x, or Wn
-                const int *keys = hkey + table * BE_HASH, *vals = hval + table * BE_HASH;
-                for (int h = (int)(((unsigned)x * 2654435761u) >> 25), probe = 0; probe < BE_HASH;
-                     h = (h + 1) & (BE_HASH - 1), probe++) {
-                    const int kx = keys[h];
-                    if (kx == x)
-                        return vals[h];
-                    if (kx == -1)
-                        break;
-                }
-                return 0x7fffffff;
-            };
-            if (nmv > 0) {
-                for (int j = mvj[0] + 1 + w; j < Wn; j += BE_WARPS) {
-                    bool hit = false;
-                    for (int c = lane; c <= kappa; c += 32) {  // the sample (c = 0) and its neighbours
-                        const int x = c == 0 ? svis[j] : sg[j * kp + c - 1];
-                        hit |= x >= 0 && earliest(x, 0) < j;
-                    }
-                    if (su[j] >= 0)
-                        for (int c = lane; c <= snq[j]; c += 32) {  // the own cluster (c = 0) and the candidates
-                            const int x = c == 0 ? su[j] : sq[j * kp + c - 1];
-                            hit |= earliest(x, 1) < j;
-                        }
-                    if (__any_sync(FULL_MASK, hit) && lane == 0)
-                        atomicMin(&s_first, j);
-                }
-            }
-            __syncthreads();
-            const int done = s_first;
-            if (w == 0) {
-                if (lane < R)
-                    st_rank(&s_win, lane, done);
-            }
-            int nm = 0;  // the committed moves: the moving visits before `done`
-            while (nm < nmv && mvj[nm] < done)
-                nm++;
-            // the committed moves touch disjoint clusters: x leaves S_u for S_v in each
-            for (int e = threadIdx.x; e < nm * d; e += BE_THREADS) {
-                const int q = e / d, t = e - q * d, j = mvj[q];
-                const int u = su[j], v = tl[2 * q + 1];
-                const double x = xs[(size_t)j * P + t];
-                D[(int64_t)u * d + t] = __dsub_rn(__ldcg(D + (int64_t)u * d + t), x);
-                D[(int64_t)v * d + t] = __dadd_rn(__ldcg(D + (int64_t)v * d + t), x);
-            }
-            if (threadIdx.x < nm) {
-                const int j = mvj[threadIdx.x], o = sbase[j], t = dq[j];
-                const int u = su[j], v = tl[2 * threadIdx.x + 1];
-                cnt[u] = rn[o] - 1;
-                cnt[v] = rn[t] + 1;
-                S[u] = ra[o];
-                S[v] = ra[t];
-                L[svis[j]] = v;
-            }
-            moves += nm;
+            hit = __any_sync(FULL_MASK, hit);
+            if (lane < R)
+                st_rank(&dep[j], lane, hit ? j : Wn);
         }
-        cluster_barrier();  // the window's moves before the next window reads labels and rows
-        const int got = s_win;  // the same in every CTA
-        We = got == Wn ? (2 * We < W ? 2 * We : W) : (2 * got < W ? (2 * got > 2 ? 2 * got : 2) : W);
-        s += got;
+        cluster_barrier();
+
+        // ---- the committed moves touch disjoint clusters: x leaves D_u for D_v in each, by the CTA that evaluated it
+        const int done = (int)__reduce_min_sync(FULL_MASK, (unsigned)(lane < Wn ? dep[lane] : Wn));
+        const unsigned commit = moving & (done >= 32 ? ~0u : (1u << done) - 1u);
+        moves += __popc(commit);
+        for (int z = threadIdx.x; z < nv * d; z += BE_THREADS) {
+            const int q = z / d, t = z - q * d, j = q * R + rank;
+            if ((commit >> j) & 1u) {
+                const double x = widen(xs[q * P + t]);
+                double *Du = D + (int64_t)su[q] * d + t, *Dv = D + (int64_t)mvv[j] * d + t;
+                const double a = __ldcg(Du), b = __ldcg(Dv);
+                *Du = __dsub_rn(a, x);
+                *Dv = __dadd_rn(b, x);
+            }
+        }
+        if (threadIdx.x < nv) {
+            const int q = threadIdx.x, j = q * R + rank;
+            if ((commit >> j) & 1u) {
+                const int u = su[q], v = mvv[j], o = q * ks, e = mve[q];
+                cnt[u] = en[o] - 1;
+                cnt[v] = en[e] + 1;
+                S[u] = ea[o];
+                S[v] = ea[e];
+                L[svis[q]] = v;
+            }
+        }
+        __syncthreads();  // the window's samples are read
+        s += done;
+        Wn = (int)(m - s < (int64_t)W ? m - s : (int64_t)W);
+        cluster_arrive();  // the window's moves before the next window reads labels and rows
+        if (s < m)
+            fetch(s, Wn);
+        cluster_wait();
     }
     if (rank == 0 && threadIdx.x == 0 && n_moved)
         *n_moved = moves;

@@ -183,3 +183,29 @@ def test_boost_sift_full_size_prefix_and_properties(G):
     assert torch.allclose(D, D2, rtol=1e-12, atol=1e-6) and torch.allclose(S, S2, rtol=1e-12)
     ne = cnt > 0
     assert float((S[ne] / cnt[ne]).sum()) > I0
+
+
+@pytest.mark.parametrize("d", [3, 32, 65, 200, 260, 700])
+@pytest.mark.parametrize("kind", ["ties", "tiny", "huge", "mixed", "zeros", "large_mean"])
+def test_boost_screening_decides_as_defined(G, kind, d):
+    # candidates are screened in FP32 before they are evaluated: equal gains, rows outside the screening's range, rows
+    # of very different length, zero rows, and gains far below the terms they are differences of
+    g = np.random.default_rng(d)
+    n, k, kappa = 700, 60, 33
+    X = datagen.gauss_mixture(n, d, 25, seed=d)
+    if kind == "ties":
+        X = np.repeat(g.integers(-2, 3, (n // 10, d)), 10, axis=0).astype(np.float32)
+    elif kind == "tiny":
+        X = X * np.float32(1e-16)
+    elif kind == "huge":
+        X = X * np.float32(1e17)
+    elif kind == "mixed":
+        X = X * (10.0 ** g.integers(-14, 15, (n, 1))).astype(np.float32)
+    elif kind == "zeros":
+        X[g.random(n) < 0.6] = 0
+    else:
+        X = X + np.float32(3e4)
+    X = np.ascontiguousarray(X, np.float32)
+    gi = _graph(X, kappa, seed=d)
+    L0 = O.default().init_labels(n, k, 3)
+    _run_both(G, X, gi, L0, k, [g.permutation(n), g.permutation(n)])
