@@ -42,15 +42,20 @@ static_assert(AS_HASH > AS_QCAP, "the label set must never fill up");
 // The distinct candidate labels of sample i in list order (the own label first, then the neighbours'), written to
 // qlist; returns their number.  Repeats are dropped with __match_any_sync inside each batch of 32 and, across batches,
 // with a per-warp open-addressing set in shared memory (one atomicCAS per new label).
+// SHORT: lists of one batch are expected and spared the set (a test of it costs the wider rows 2%).
+template <bool SHORT = false>
 __device__ __forceinline__ int collect_labels(int64_t i, int own, const int32_t *__restrict__ G, int kappa, int64_t n,
                                               int k, const int32_t *__restrict__ Lin, int *qlist, int *tab,
                                               DevStatus *st)
 {
     const int lane = lane_id(), ncand = kappa + 1;
+    const bool several = !SHORT || ncand > 32;
+    if (several) {
 #pragma unroll
-    for (int q = lane * 4; q < AS_HASH; q += 128)
-        *reinterpret_cast<int4 *>(tab + q) = make_int4(-1, -1, -1, -1);
-    __syncwarp();
+        for (int q = lane * 4; q < AS_HASH; q += 128)
+            *reinterpret_cast<int4 *>(tab + q) = make_int4(-1, -1, -1, -1);
+        __syncwarp();
+    }
     int u = 0;
     for (int c0 = 0; c0 < ncand; c0 += 32) {
         int c = c0 + lane;
@@ -69,8 +74,9 @@ __device__ __forceinline__ int collect_labels(int64_t i, int own, const int32_t 
             lab = -1;
         }
         const unsigned peers = __match_any_sync(FULL_MASK, lab);
-        bool fresh = false;
-        if (lab >= 0 && (peers & lanemask_lt()) == 0u) {
+        bool fresh = lab >= 0 && (peers & lanemask_lt()) == 0u;
+        if (fresh && several) {
+            fresh = false;
             unsigned h = ((unsigned)lab * 0x9E3779B1u) >> 24;  // 8-bit multiplicative hash
             for (int probe = 0; probe < AS_HASH; probe++) {    // the set is never full: ends early
                 const int old = atomicCAS(tab + h, -1, lab);
@@ -359,13 +365,14 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign(const XT *__restrict__
 }
 
 // Coalesced variant for 16-byte rows (d % 4 == 0, d <= 32 * 4 * NV): the warp
-// keeps x_i in registers (lane l owns vectors l, l + 32, ...).  Distances are taken AS_G candidates at a
+// keeps x_i in registers (lane l owns vectors l, l + 32, ...; with LPR < 32 each
+// set of LPR lanes holds the whole row and takes candidates of its own).  Distances are taken AS_G candidates at a
 // time (AS_G / 2 for rows over 512 floats): each lane loads one 16-byte vector
 // of every centroid of the group, and transpose_reduce completes the group's
 // sums together.  The candidate list is padded to a multiple of the group with
 // its first entry, whose second evaluation
 // cannot change the (distance, label) minimum.
-template <int NV, typename XT, int GS, bool LISTS>
+template <int NV, typename XT, int GS, bool LISTS, int LPR = 32>
 __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k_assign_rows(const XT *__restrict__ X, int64_t n, int d,
                                                                int64_t ld, const int32_t *__restrict__ G, int kappa,
                                                                const float *__restrict__ C, int k,
@@ -374,12 +381,15 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
                                                                float *__restrict__ best_out, DevStatus *st,
                                                                const Track trk, const int32_t *__restrict__ todo)
 {
-    __shared__ __align__(16) int s_q[AS_WARPS][AS_QROW];
+    __shared__ __align__(16) int s_q[AS_WARPS][AS_QROW + (LPR < 32 ? GS * 32 / LPR : 0)];
     __shared__ __align__(16) int s_h[AS_WARPS][AS_HASH];
     const int w = threadIdx.x >> 5, lane = lane_id();
     int *qlist = s_q[w];
     int *tab = s_h[w];
-    static_assert(GS == 4 || GS == 8, "candidates per group: 4 or 8");
+    static_assert(GS == 4 || GS == 8, "candidates per lane set and group: 4 or 8");
+    static_assert(LPR == 32 || (NV == 1 && LPR >= GS), "lane sets hold whole rows");
+    constexpr int SETS = 32 / LPR;
+    const int set = lane / LPR, sl = lane % LPR;
     const int d4 = d >> 2;
     const float4 *C4 = reinterpret_cast<const float4 *>(C);
 
@@ -390,11 +400,11 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
         float4 xv[NV];
 #pragma unroll
         for (int v = 0; v < NV; v++) {
-            int col = lane + 32 * v;
+            int col = sl + 32 * v;
             xv[v] = col < d4 ? ldx4<XT, true>(xrow + 4 * col) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         const int own = Lin[i];
-        int u = collect_labels(i, own, G, kappa, n, k, Lin, qlist, tab, st);
+        int u = collect_labels<(LPR < 32)>(i, own, G, kappa, n, k, Lin, qlist, tab, st);
         float bd = __int_as_float(0x7f800000);
         int br = 0x7fffffff;
         if constexpr (PART) {
@@ -402,15 +412,16 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
             bd = best_out[i];
             br = own;
         }
-        if (u > 0 && lane < GS)
+        if (u > 0 && lane < GS * SETS)
             qlist[u + lane] = qlist[0];
         __syncwarp();
 
-        for (int g0 = 0; g0 < u; g0 += GS) {
+        for (int g0 = 0; g0 < u; g0 += GS * SETS) {
+            const int *ql = qlist + g0 + set * GS;
             int lab[GS];
 #pragma unroll
             for (int c = 0; c < GS; c += 4) {
-                const int4 q4 = *reinterpret_cast<const int4 *>(qlist + g0 + c);
+                const int4 q4 = *reinterpret_cast<const int4 *>(ql + c);
                 lab[c] = q4.x;
                 lab[c + 1] = q4.y;
                 lab[c + 2] = q4.z;
@@ -420,18 +431,18 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
 #pragma unroll
             for (int c = 0; c < GS; c++) {
                 const float4 *row = C4 + (int64_t)lab[c] * d4;
-                part[c] = lane_partial<NV>(xv, d4, [&](int col) { return __ldg(row + col); });
+                part[c] = lane_partial<NV, LPR>(xv, d4, [&](int col) { return __ldg(row + col); });
             }
-            const float tot = transpose_reduce<GS>(part);
-            const int r = qlist[g0 + lane / (32 / GS)];
+            const float tot = transpose_reduce<GS, LPR>(part);
+            const int r = ql[sl / (LPR / GS)];
             if (key_less(tot, r, bd, br)) {
                 bd = tot;
                 br = r;
             }
         }
-        // lanes that share bits 4 .. log2(32 / GS) hold the same candidates
+        // lanes that share bits 4 .. log2(LPR / GS) hold the same candidates
 #pragma unroll
-        for (int o = 16; o >= 32 / GS; o >>= 1) {
+        for (int o = 16; o >= LPR / GS; o >>= 1) {
             float od = __shfl_xor_sync(FULL_MASK, bd, o);
             int orr = __shfl_xor_sync(FULL_MASK, br, o);
             if (key_less(od, orr, bd, br)) {
@@ -1126,7 +1137,9 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     const int d4 = (int)(d / 4);
     // candidates per group of the row kernels (a tile shape: every width gives the same bits, transpose_reduce
     // forms each total with warp_total's tree): 8 by default, 4 for rows of more than 512 values, where 8 would
-    // not keep the loads in registers; a caller (the autotuner) may ask for 4 or 8
+    // not keep the loads in registers; a caller (the autotuner) may ask for 4 or 8.  Rows of at most 64 (32) values
+    // of precision 0 and 1 take two (four) candidates to a load, four loads a group: 1.3M x 64, kappa = 20 329 us
+    // an assignment instead of 422 (eight loads a group 392); 20k x 32 9.1 us instead of 11.6 (eight 11.0)
     const int gw = (precision >> 8) & 0xff;
     precision &= 0xff;
     cudaError_t e;
@@ -1224,29 +1237,34 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     }
     if (done) {
     } else if (vec4 && d4 <= 32 * 8) {
-#define GK_ASGG(NV, GS)                                                                                          \
+#define GK_ASGG(NV, GS, LPR)                                                                                          \
     do {                                                                                                         \
         if (trk.dirty)                                                                                           \
-            GK_ASGT(NV, GS, true);                                                                               \
+            GK_ASGT(NV, GS, true, LPR);                                                                               \
         else                                                                                                     \
-            GK_ASGT(NV, GS, false);                                                                              \
+            GK_ASGT(NV, GS, false, LPR);                                                                              \
     } while (0)
-#define GK_ASGT(NV, GS, T)                                                                                       \
+#define GK_ASGT(NV, GS, T, LPR)                                                                                  \
     do {                                                                                                         \
-        if ((e = resident_grid(reinterpret_cast<const void *>(k_assign_rows<NV, XT, GS, T>), AS_WARPS * 32, 0,   \
-                               &grid)) != cudaSuccess)                                                           \
+        if ((e = resident_grid(reinterpret_cast<const void *>(k_assign_rows<NV, XT, GS, T, LPR>), AS_WARPS * 32, \
+                               0, &grid)) != cudaSuccess)                                                        \
             return e;                                                                                            \
-        k_assign_rows<NV, XT, GS, T><<<grid, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, k, labels_in, \
-                                                                    labels_out, best, st, trk, sel_lab);                  \
+        k_assign_rows<NV, XT, GS, T, LPR><<<grid, AS_WARPS * 32, 0, s>>>(X, n, (int)d, ld, g_idx, kappa, C, k,   \
+                                                                         labels_in, labels_out, best, st, trk,   \
+                                                                         sel_lab);                               \
     } while (0)
 #define GK_ASG(NV)                                                                                               \
     do {                                                                                                         \
         if (NV >= 8 || gw == 4)                                                                                  \
-            GK_ASGG(NV, 4);                                                                                      \
+            GK_ASGG(NV, 4, 32);                                                                                  \
         else                                                                                                     \
-            GK_ASGG(NV, 8);                                                                                      \
+            GK_ASGG(NV, 8, 32);                                                                                  \
     } while (0)
-        if (d4 <= 32)
+        if (d4 <= 8)
+            GK_ASGG(1, 4, 8);
+        else if (d4 <= 16)
+            GK_ASGG(1, 4, 16);
+        else if (d4 <= 32)
             GK_ASG(1);
         else if (d4 <= 64)
             GK_ASG(2);

@@ -15,13 +15,17 @@ namespace gkm {
 // plain xor butterfly.  Every candidate's total is thus formed with the tree
 // of warp_total (bit 4 first, then 3, 2, 1, 0), so all three give the same
 // bits.  Afterwards lane l holds the total of candidate l / (32 / G).
-template <int G>
+// With LPR = 8 or 16 the lanes of each LPR have their own G candidates: rows
+// of at most LPR vectors leave the lanes from LPR on at +0 in warp_total's
+// tree, which adds nothing, so the totals are that tree's here too (lane l of
+// the LPR holds candidate l / (LPR / G)).
+template <int G, int LPR = 32>
 __device__ __forceinline__ float transpose_reduce(float (&v)[G])
 {
-    static_assert(G >= 2 && G <= 32 && (G & (G - 1)) == 0, "G must be a power of two in [2, 32]");
+    static_assert(G >= 2 && G <= LPR && (G & (G - 1)) == 0, "G must be a power of two in [2, LPR]");
     const int lane = lane_id();
 #pragma unroll
-    for (int h = G / 2, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    for (int h = G / 2, o = LPR / 2; h >= 1; h >>= 1, o >>= 1) {
         const bool upper = (lane & o) != 0;
 #pragma unroll
         for (int j = 0; j < h; j++) {
@@ -32,7 +36,7 @@ __device__ __forceinline__ float transpose_reduce(float (&v)[G])
     }
     float t = v[0];
 #pragma unroll
-    for (int o = 16 / G; o >= 1; o >>= 1)
+    for (int o = LPR / 2 / G; o >= 1; o >>= 1)
         t += __shfl_xor_sync(FULL_MASK, t, o);
     return t;
 }
@@ -45,10 +49,10 @@ __device__ __forceinline__ float transpose_reduce32(float (&v)[32]) { return tra
 // each a round-to-nearest FMA, and a0 + a1 at the end.  The packed FP32x2 FMA
 // of sm_100+ performs each pair at once with the same roundings; e = x - c is
 // formed as fma(c, -1, x), which is x - c rounded once.
-template <int NV, typename RowLoad>
+template <int NV, int LPR = 32, typename RowLoad>
 __device__ __forceinline__ float lane_partial(const float4 (&xv)[NV], int d4, RowLoad load)
 {
-    const int lane = lane_id();
+    const int lane = lane_id() & (LPR - 1);
     const float2 m1 = make_float2(-1.f, -1.f);
     float2 a = make_float2(0.f, 0.f);
 #pragma unroll

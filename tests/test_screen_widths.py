@@ -32,3 +32,29 @@ def test_screened_labels_equal_fp32(d, dtype):
         assert torch.equal(got, want), p
         assert torch.equal(b.view(torch.int32), best.view(torch.int32)), p
         assert float(s2) == float(s)
+
+
+@pytest.mark.parametrize("kappa", [1, 20, 31, 32, 50, 128])
+@pytest.mark.parametrize("d", [4, 12, 28, 32, 36, 56, 64])
+def test_narrow_rows_equal_zero_padded_rows(d, kappa):
+    # rows of at most 64 values take several candidates to a load; zero columns up to 68 values change no distance's bits
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1705_01813_gb300 import gkm
+    n, k = 5003, 150
+    g = np.random.default_rng(d * 131 + kappa)
+    gi = torch.from_numpy(g.integers(0, n, (n, kappa)).astype(np.int32)).cuda()
+    L = torch.from_numpy(g.integers(0, k, n).astype(np.int32)).cuda()
+    for bf16 in (False, True):
+        X = torch.from_numpy(g.standard_normal((n, d)).astype(np.float32)).cuda()
+        C = torch.from_numpy(g.standard_normal((k, d)).astype(np.float32)).cuda()
+        C[5] = C[6]  # equal distances
+        Xw, Cw = torch.zeros((n, 68), device="cuda"), torch.zeros((k, 68), device="cuda")
+        Xw[:, :d], Cw[:, :d] = X, C
+        if bf16:
+            X, Xw = X.to(torch.bfloat16), Xw.to(torch.bfloat16)
+        got, b, s, _ = gkm.assign_step(X, gi, C, L, precision=1)
+        want, bw, sw, _ = gkm.assign_step(Xw, gi, Cw, L, precision=1)
+        assert torch.equal(got, want)
+        assert torch.equal(b.view(torch.int32), bw.view(torch.int32))
+        assert float(s) == float(sw)
