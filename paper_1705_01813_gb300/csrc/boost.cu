@@ -153,53 +153,6 @@ constexpr int BE_MAX_CLUSTER = 16;
 constexpr int BE_MAX_WINDOW = 32;  // a lane per visit
 constexpr size_t BE_SMEM_BUDGET = 200 * 1024;
 
-__device__ __forceinline__ void cluster_barrier()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ unsigned cluster_rank()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-
-__device__ __forceinline__ unsigned cluster_size()
-{
-    unsigned r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-
-// The two halves of cluster_barrier().
-__device__ __forceinline__ void cluster_arrive()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait()
-{
-    __syncwarp();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// Address of the same shared variable in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t in_rank(const void *p, int rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
-                 : "=r"(r)
-                 : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
-    return r;
-}
-
-__device__ __forceinline__ void st_rank(const void *p, int rank, int v)
-{
-    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(in_rank(p, rank)), "r"(v) : "memory");
-}
-
 // An FP64 value cut to FP32 on the integer pipe (the FP64 one is narrow): error below 2^-23 of it, 0 below FP32's
 // normal range, NaN above it.
 __device__ __forceinline__ float cut32(double v)

@@ -227,6 +227,62 @@ struct Carver {
     }
 };
 
+// Thread-block clusters: the barrier of all their threads (and its two halves), the CTA's rank, and stores into the
+// shared memory of another CTA of the cluster.
+__device__ __forceinline__ void cluster_barrier()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ unsigned cluster_rank()
+{
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ unsigned cluster_size()
+{
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+
+// The two halves of cluster_barrier().
+__device__ __forceinline__ void cluster_arrive()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Address of the same shared variable in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t in_rank(const void *p, int rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(r)
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+
+__device__ __forceinline__ void st_rank(const void *p, int rank, float4 v)
+{
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(in_rank(p, rank)), "f"(v.x), "f"(v.y), "f"(v.z),
+                 "f"(v.w)
+                 : "memory");
+}
+
+__device__ __forceinline__ void st_rank(const void *p, int rank, int v)
+{
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(in_rank(p, rank)), "r"(v) : "memory");
+}
+
 // cudaFuncSetAttribute(kernel, MaxDynamicSharedMemorySize, bytes) on the current
 // device, the first time only (thread-safe); `bytes` must be the same on every call.
 cudaError_t set_max_smem(const void *kernel, int bytes);
