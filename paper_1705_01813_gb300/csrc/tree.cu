@@ -305,11 +305,31 @@ __global__ void __launch_bounds__(256) k_tree_colmax(const XT *__restrict__ X, i
 // Where every h1 is zero, or every h2 and at most 1024 members are summed (and y itself is exact: no scaling down),
 // all partial sums are multiples of one unit that FP64 holds exactly, so the ordered FP64 sum is this sum.  Otherwise
 // the two means differ by at most (chunk + chunks) 2^-53 mean|x| plus the split's remainder, and their FP32 roundings
-// are the same unless the mean lies that close to the midpoint of two floats: a few centre coordinates in 10^6.  Those
-// get the code REDO and k_tree_redo sums them in the defined order.  So every centre has the bits of the definition.
+// are the same unless the mean lies that close to the midpoint of two floats: a few centre coordinates in 10^6, more
+// where a mean is small beside its members.  Those get the code REDO and k_tree_redo sums them in the defined order.
+// So every centre has the bits of the definition.
 // ---------------------------------------------------------------------------
 constexpr unsigned REDO = 0x7fb0dead;  // a NaN no mean takes
 constexpr float SPLIT_M = 12582912.f;  // 1.5 2^23
+constexpr int REDO_CAP = 1 << 16;      // listed coordinates, at most
+
+// The coordinates coded REDO in the current pass: their number, which may exceed the list's room (cap entries).
+struct RedoList {
+    unsigned *n;
+    int64_t *at;
+    int cap;
+};
+
+// Writes a centre coordinate and lists it when it is to be summed again.
+__device__ __forceinline__ void put_centre(float *cen, int64_t z, unsigned bits, const RedoList &redo)
+{
+    cen[z] = __uint_as_float(bits);
+    if (bits == REDO) {
+        const unsigned i = atomicAdd(redo.n, 1u);
+        if (i < (unsigned)redo.cap)
+            redo.at[i] = z;
+    }
+}
 
 // 2^(20 - e) for a column whose largest magnitude has the given bits; 0 when it is not finite.
 __device__ __forceinline__ float col_scale(unsigned mx)
@@ -370,7 +390,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
                                                           unsigned long long *__restrict__ acc,
                                                           unsigned *__restrict__ flg, float *__restrict__ mass,
                                                           unsigned *__restrict__ cnts, uint8_t *__restrict__ halves,
-                                                          uint64_t *__restrict__ keys, DevStatus *st)
+                                                          uint64_t *__restrict__ keys, const RedoList redo, DevStatus *st)
 {
     extern __shared__ __align__(16) unsigned char tr_smem[];
     float *stage = reinterpret_cast<float *>(tr_smem);                       // [TR_THREADS][TR_VP]
@@ -395,15 +415,16 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
         for (int t = tid; t < 9 * d; t += TR_THREADS)  // the masses and flags too
             lsum[t] = 0;
     const int nst = (d + TR_STAGE - 1) / TR_STAGE;
-    // the 64 coordinates of stage s of the block's rows (zeros past d), all in flight at once: 16 lanes per row, or a
+    // the 64 coordinates of stage s of the block's gn rows (zeros past d), all in flight at once: 16 lanes per row, or a
     // lane per coordinate
+    int gn = 0;
     auto stage_rows = [&](int s) {
         const int t0 = s * TR_STAGE;
         if (vec) {
             const int t = t0 + (tid & 15) * 4;
             float *to = stage + (tid & 15) * 4;
 #pragma unroll 8
-            for (int r = tid >> 4; r < TR_THREADS; r += TR_THREADS / 16) {
+            for (int r = tid >> 4; r < gn; r += TR_THREADS / 16) {
                 float *q = to + r * TR_VP;
                 if (t >= d)
                     *reinterpret_cast<float4 *>(q) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -413,7 +434,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
                     *reinterpret_cast<float4 *>(q) = ldx4<XT>(X + (int64_t)sid[r] * ld + t);
             }
         } else {
-            for (int r = warp; r < TR_THREADS; r += TR_THREADS / 32)
+            for (int r = warp; r < gn; r += TR_THREADS / 32)
                 for (int q = lane; q < TR_STAGE; q += 32)
                     stage[r * TR_VP + q] = t0 + q < d ? ldx(X + (int64_t)sid[r] * ld + t0 + q) : 0.f;
         }
@@ -424,6 +445,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
     for (int64_t g = b; g < e; g += TR_THREADS) {
         const int64_t p = g + tid;
         const bool valid = p < e;
+        gn = (int)min((int64_t)TR_THREADS, e - g);
         int id = perm[valid ? p : b];
         if ((unsigned)id >= (unsigned)n) {
             flag_error(st, GK_ERR_INVALID, (unsigned)j);
@@ -436,6 +458,8 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
             __syncthreads();  // sid written; the previous stage consumed
             stage_rows(s);
             __syncthreads();
+            if (!valid)
+                continue;
             const float *xs = stage + tid * TR_VP;
             const float2 *cs = cuv + s * TR_STAGE;
             const int tw = min(TR_STAGE, d - s * TR_STAGE);
@@ -537,9 +561,10 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
             const int h = t >= d ? 1 : 0, tc = t - h * d;
             const int64_t cnt = h ? cnt_v : cnt_u;
             if (cnt)
-                cj[t] = __uint_as_float(centre_bits(lsum[3 * h * d + tc], lsum[(3 * h + 1) * d + tc],
-                                                    lsum[(3 * h + 2) * d + tc], (lany[tc] >> (2 * h)) & 3u, lmass[t], cnt,
-                                                    colmax[tc], 1));
+                put_centre(cen, j * 2 * (int64_t)d + t,
+                           centre_bits(lsum[3 * h * d + tc], lsum[(3 * h + 1) * d + tc], lsum[(3 * h + 2) * d + tc],
+                                       (lany[tc] >> (2 * h)) & 3u, lmass[t], cnt, colmax[tc], 1),
+                           redo);
         }
     } else {
         for (int t = tid; t < 6 * d; t += TR_THREADS)
@@ -564,7 +589,8 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
 __global__ void __launch_bounds__(256) k_tree_centres(int64_t S, int d, int64_t C, const int32_t *__restrict__ spl,
                                                       float *__restrict__ cen, const unsigned *__restrict__ colmax,
                                                       unsigned long long *__restrict__ acc, unsigned *__restrict__ flg,
-                                                      float *__restrict__ mass, const unsigned *__restrict__ cnts)
+                                                      float *__restrict__ mass, const unsigned *__restrict__ cnts,
+                                                      const RedoList redo)
 {
     for (int64_t q = blockIdx.x * (int64_t)256 + threadIdx.x; q < S * 2 * d; q += (int64_t)gridDim.x * 256) {
         const int64_t j = q / (2 * d);
@@ -574,67 +600,127 @@ __global__ void __launch_bounds__(256) k_tree_centres(int64_t S, int d, int64_t 
         unsigned long long *a = acc + j * 6 * (int64_t)d + 3 * h * (int64_t)d + tc;
         const int64_t cnt = cnts[2 * j + h];
         if (cnt)
-            cen[q] = __uint_as_float(
-                centre_bits((int64_t)a[0], (int64_t)a[d], (int64_t)a[2 * (int64_t)d], flg[q], mass[q], cnt, colmax[tc], C));
+            put_centre(cen, q,
+                       centre_bits((int64_t)a[0], (int64_t)a[d], (int64_t)a[2 * (int64_t)d], flg[q], mass[q], cnt,
+                                   colmax[tc], C),
+                       redo);
         a[0] = a[d] = a[2 * (int64_t)d] = 0ull;
         flg[q] = 0u;
         mass[q] = 0.f;
     }
 }
 
-// The centre coordinates coded REDO, in the defined order: a warp per coordinate, a lane per chunk (chunk by chunk in
-// ascending id, the chunks' sums added in order).  cnts (of several chunks) is cleared for the next pass.
+// The centre coordinates coded REDO, in the defined order (chunk by chunk in ascending id, the chunks' sums added in
+// order): a warp per listed coordinate and chunk, which loads 32 members at a time; with several chunks their sums go
+// to part (cap C <= n doubles, the keys' place) and the last block to finish adds them up.  The last block also clears
+// the list and cnts (of several chunks) for the next pass.  When the list overflowed, all coordinates are looked
+// through instead, a warp per coordinate and a lane per chunk.  (That form for every coordinate took up to 32 ms for
+// one of the root of 1M members: one warp; this one 0.1.)
 template <typename XT>
 __global__ void __launch_bounds__(256) k_tree_redo(const XT *__restrict__ X, int64_t n, int d, int64_t ld, int L,
                                                    int64_t S, int64_t C, const int32_t *__restrict__ perm,
-                                                   const int32_t *__restrict__ spl, const uint8_t *__restrict__ halves,
-                                                   float *__restrict__ cen, unsigned *__restrict__ cnts)
+                                                   const uint8_t *__restrict__ halves, float *__restrict__ cen,
+                                                   unsigned *__restrict__ cnts, double *__restrict__ part,
+                                                   const RedoList redo, unsigned *__restrict__ ticket)
 {
     const int lane = threadIdx.x & 31;
     const int64_t total = S * 2 * d, step = (int64_t)gridDim.x * 256;
-    if (C > 1)
-        for (int64_t q = blockIdx.x * (int64_t)256 + threadIdx.x; q < 2 * S; q += step)
-            cnts[q] = 0u;
-    for (int64_t q0 = blockIdx.x * (int64_t)256 + (threadIdx.x & ~31); q0 < total; q0 += step) {
-        const int64_t q = q0 + lane;
-        unsigned left = __ballot_sync(FULL_MASK, q < total && __float_as_uint(cen[q]) == REDO);
-        while (left) {
-            const int64_t z = q0 + __ffs(left) - 1;
-            left &= left - 1;
-            const int64_t j = z / (2 * d);
+    const unsigned listed = *redo.n;
+    const bool all = listed > (unsigned)redo.cap;
+    auto member = [&](int64_t p, int tc) {
+        const int id = perm[p];
+        return ldx(X + ((unsigned)id < (unsigned)n ? (int64_t)id * ld : 0) + tc);
+    };
+    if (!all) {
+        const int64_t items = (int64_t)listed * C;
+        for (int64_t it = (blockIdx.x * (int64_t)256 + threadIdx.x) >> 5; it < items; it += step >> 5) {
+            const int64_t z = redo.at[it / C], c = it % C, j = z / (2 * d);
             const int t = (int)(z - j * 2 * d), h = t >= d ? 1 : 0, tc = t - h * d;
-            int64_t off, m;
+            int64_t off, m, b, e;
             seg_geom(n, L, j, off, m);
-            double total_sum = 0.0;
-            long long cnt = 0;
-            for (int64_t c0 = 0; c0 < C; c0 += 32) {
-                double sum = 0.0;
-                int nc = 0;
-                if (c0 + lane < C) {
-                    int64_t b, e;
-                    chunk_range(off, m, C, c0 + lane, b, e);
-#pragma unroll 4
-                    for (int64_t p = b; p < e; p++) {
-                        const int id = perm[p];
-                        const double x = (unsigned)id < (unsigned)n ? widen(ldx(X + (int64_t)id * ld + tc)) : widen(ldx(X + tc));
-                        if (halves[p] == h) {
-                            sum += x;
-                            nc++;
-                        }
-                    }
-                }
-                for (int s = 0; s < 32 && c0 + s < C; s++) {
-                    const double v = __shfl_sync(FULL_MASK, sum, s);
-                    total_sum = C > 1 ? total_sum + v : v;
-                    cnt += __shfl_sync(FULL_MASK, nc, s);
+            chunk_range(off, m, C, c, b, e);
+            double sum = 0.0;
+            int cnt = 0;
+            float x = b + lane < e ? member(b + lane, tc) : 0.f;
+            int hl = b + lane < e ? halves[b + lane] : 2;
+            for (int64_t p = b; p < e; p += 32) {
+                const float x0 = x;
+                unsigned mine = __ballot_sync(FULL_MASK, hl == h);
+                const int64_t q = p + 32 + lane;
+                x = q < e ? member(q, tc) : 0.f;
+                hl = q < e ? halves[q] : 2;
+                cnt += __popc(mine);
+                while (mine) {
+                    sum = __dadd_rn(sum, widen(__shfl_sync(FULL_MASK, x0, __ffs(mine) - 1)));
+                    mine &= mine - 1;
                 }
             }
-            if (lane == 0)
-                cen[z] = (float)(total_sum / (double)cnt);
+            if (lane == 0) {
+                if (C == 1)
+                    cen[z] = (float)(sum / (double)cnt);
+                else
+                    part[it] = sum;
+            }
+        }
+    } else {
+        for (int64_t q0 = blockIdx.x * (int64_t)256 + (threadIdx.x & ~31); q0 < total; q0 += step) {
+            const int64_t q = q0 + lane;
+            unsigned left = __ballot_sync(FULL_MASK, q < total && __float_as_uint(cen[q]) == REDO);
+            while (left) {
+                const int64_t z = q0 + __ffs(left) - 1;
+                left &= left - 1;
+                const int64_t j = z / (2 * d);
+                const int t = (int)(z - j * 2 * d), h = t >= d ? 1 : 0, tc = t - h * d;
+                int64_t off, m;
+                seg_geom(n, L, j, off, m);
+                double total_sum = 0.0;
+                long long cnt = 0;
+                for (int64_t c0 = 0; c0 < C; c0 += 32) {
+                    double sum = 0.0;
+                    int nc = 0;
+                    if (c0 + lane < C) {
+                        int64_t b, e;
+                        chunk_range(off, m, C, c0 + lane, b, e);
+#pragma unroll 8
+                        for (int64_t p = b; p < e; p++) {
+                            const float x = member(p, tc);
+                            if (halves[p] == h) {
+                                sum = __dadd_rn(sum, widen(x));
+                                nc++;
+                            }
+                        }
+                    }
+                    for (int s = 0; s < 32 && c0 + s < C; s++) {
+                        total_sum = __dadd_rn(total_sum, __shfl_sync(FULL_MASK, sum, s));
+                        cnt += __shfl_sync(FULL_MASK, nc, s);
+                    }
+                }
+                if (lane == 0)
+                    cen[z] = (float)(total_sum / (double)cnt);
+            }
         }
     }
+    if (!last_block(ticket))
+        return;
+    if (C > 1) {
+        if (!all)
+            for (int64_t i = threadIdx.x; i < listed; i += 256) {
+                const int64_t z = redo.at[i], j = z / (2 * d);
+                double sum = 0.0;
+#pragma unroll 8
+                for (int64_t c = 0; c < C; c++)
+                    sum = __dadd_rn(sum, __ldcg(part + i * C + c));
+                cen[z] = (float)(sum / (double)cnts[2 * j + (z - j * 2 * d >= d ? 1 : 0)]);
+            }
+        __syncthreads();  // the counts are read
+        for (int64_t q = threadIdx.x; q < 2 * S; q += 256)
+            cnts[q] = 0u;
+    }
+    if (threadIdx.x == 0) {
+        *redo.n = 0u;
+        *ticket = 0u;
+    }
 }
-
 
 // The ceil(m/2)-th smallest key of every splitting cluster (keys are distinct: they end in the member's id), by
 // radix selection over 8-bit digits from the most significant.  Clusters of one chunk: one block each.
@@ -903,7 +989,8 @@ struct TreeBufs {
     Top2 *seeds;
     float *cen;
     unsigned long long *acc;  // limb sums of the clusters of several chunks [2][3][d]; flags, masses [2][d]; counts [2]
-    unsigned *flg, *cnts, *colmax;
+    unsigned *flg, *cnts, *colmax, *redo_n, *ticket;
+    int64_t *redo_at;
     float *mass;
     uint8_t *halves;
     size_t zero_off, zero_bytes, bytes;
@@ -935,7 +1022,10 @@ TreeBufs tree_carve(void *scratch, int64_t n, int64_t d, int32_t k)
     B.cbase = cv.take<int32_t>((size_t)chunks);
     B.ghist = cv.take<unsigned>((size_t)multi * 256);
     B.halves = cv.take<uint8_t>((size_t)n);
+    B.redo_at = cv.take<int64_t>(REDO_CAP);
     B.zero_off = cv.off;  // from here on zero before the first pass
+    B.redo_n = cv.take<unsigned>(1);
+    B.ticket = cv.take<unsigned>(1);
     B.colmax = cv.take<unsigned>((size_t)d);
     B.acc = cv.take<unsigned long long>((size_t)multi * 6 * (size_t)d);
     B.flg = cv.take<unsigned>((size_t)multi * 2 * (size_t)d);
@@ -982,15 +1072,17 @@ cudaError_t tree_run(const XT *X, int64_t n, int d, int64_t ld, int32_t k, int32
         k_tree_seed_part<<<SC, SEL_THREADS, 0, s>>>(n, L, C, cur, spl, seed, B.seeds);
         k_tree_seed_final<XT><<<(unsigned)S, TR_THREADS, 0, s>>>(X, n, d, ld, C, spl, B.seeds, B.cen, st);
         for (int it = 0; it < iters; it++) {
+            const RedoList redo{B.redo_n, B.redo_at, (int)std::min<int64_t>(REDO_CAP, C > 1 ? n / C : REDO_CAP)};
             k_tree_pass<XT, false><<<SC, TR_THREADS, smem, s>>>(X, n, d, ld, vec, L, C, cur, spl, B.cen, B.colmax, B.acc,
-                                                                B.flg, B.mass, B.cnts, B.halves, B.keys, st);
+                                                                B.flg, B.mass, B.cnts, B.halves, B.keys, redo, st);
             const unsigned cb = (unsigned)std::min<int64_t>((S * 2 * d + 255) / 256, 152 * 8);
             if (C > 1)
-                k_tree_centres<<<cb, 256, 0, s>>>(S, d, C, spl, B.cen, B.colmax, B.acc, B.flg, B.mass, B.cnts);
-            k_tree_redo<XT><<<cb, 256, 0, s>>>(X, n, d, ld, L, S, C, cur, spl, B.halves, B.cen, B.cnts);
+                k_tree_centres<<<cb, 256, 0, s>>>(S, d, C, spl, B.cen, B.colmax, B.acc, B.flg, B.mass, B.cnts, redo);
+            k_tree_redo<XT><<<std::max(152u, cb), 256, 0, s>>>(X, n, d, ld, L, S, C, cur, B.halves, B.cen, B.cnts,
+                                                               reinterpret_cast<double *>(B.keys), redo, B.ticket);
         }
         k_tree_pass<XT, true><<<SC, TR_THREADS, smem, s>>>(X, n, d, ld, vec, L, C, cur, spl, B.cen, B.colmax, B.acc, B.flg,
-                                                           B.mass, B.cnts, B.halves, B.keys, st);
+                                                           B.mass, B.cnts, B.halves, B.keys, RedoList{}, st);
         if (C == 1) {
             k_tree_select<<<(unsigned)S, SEL_THREADS, 0, s>>>(n, L, spl, B.keys, B.thr);
             k_tree_split<<<SC, SEL_THREADS, 0, s>>>(n, L, C, spl, B.keys, B.thr, nullptr, cur, nxt, st);

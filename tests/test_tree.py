@@ -134,3 +134,13 @@ def test_tree_centres_of_any_scale(G, kind, n, d, k):
             0, 8, (n, 1)).astype(np.float32)
     X = np.ascontiguousarray(X, np.float32)
     assert np.array_equal(_run(G, X, k, 3, 5), O.two_means_tree(X, k, iters=3, seed=5))
+
+
+@pytest.mark.parametrize("n,d,k", [(2000, 300, 8), (400, 40, 30), (5000, 33, 700)])
+def test_tree_where_no_integer_sum_decides(G, n, d, k):
+    # one far sample sets every column's scale, so that every other centre is summed in order: more coordinates than the
+    # list of those takes (the first shape), clusters of one chunk and of several
+    X = datagen.gauss_mixture(n, d, 12, seed=n) * np.float32(1e-9)
+    X[n // 3] = np.float32(3e9)
+    X = np.ascontiguousarray(X, np.float32)
+    assert np.array_equal(_run(G, X, k, 3, 5), O.two_means_tree(X, k, iters=3, seed=5))
