@@ -36,8 +36,10 @@ namespace {
 constexpr uint64_t TAG_TREE = 0x5452454500000000ull;  // "TREE"
 constexpr int TR_THREADS = 128;                       // pass kernel: one member per thread at a time
 constexpr int TR_STAGE = 64;                          // coordinates staged per round
-constexpr int TR_VP = TR_STAGE + 4;                   // pitch of a staged row: 16-byte reads of neighbouring rows and
-                                                      // 4-byte reads along a row hit distinct banks
+// Pitch of a staged row in elements (16 bytes more than its values): reads of four values of neighbouring rows, and of
+// one value along a row, hit distinct banks (two-way for BF16's four).
+template <typename XT>
+constexpr int TR_VP = TR_STAGE + 16 / (int)sizeof(XT);
 constexpr int64_t TR_CHUNK = 512;                     // members per chunk block; larger clusters take several
 constexpr int SEL_THREADS = 256;
 static_assert(TR_THREADS == 2 * TR_STAGE, "the sums give each coordinate two threads");
@@ -365,9 +367,17 @@ __device__ __forceinline__ unsigned centre_bits(int64_t h0, int64_t h1, int64_t 
 
 // Dynamic shared memory of the pass kernel: limb sums, masses and flags of both halves, both centres, the staged rows,
 // the block's member ids and counts, the rows by half.
+template <typename XT>
 __host__ __device__ constexpr size_t pass_smem(int d)
 {
-    return (size_t)44 * d + sizeof(float) * TR_THREADS * TR_VP + 2 * sizeof(int) * TR_THREADS + TR_THREADS + 64;
+    return (size_t)44 * d + sizeof(XT) * TR_THREADS * TR_VP<XT> + 2 * sizeof(int) * TR_THREADS + TR_THREADS + 64;
+}
+
+// Four staged values, widened exactly.
+__device__ __forceinline__ float4 staged4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 staged4(const __nv_bfloat16 *p)
+{
+    return bf16x4_to_float4(*reinterpret_cast<const uint2 *>(p));
 }
 
 // One pass over the members of every splitting cluster of depth L, C chunks per cluster (grid S x C).  Each thread
@@ -380,7 +390,7 @@ __host__ __device__ constexpr size_t pass_smem(int d)
 //   KEYS = true: keys[p] = (order(d_u - d_v) << 32) | id.
 // Bound by the reads of the rows: 1M x 128 FP32 (512 MB) takes 84 us with KEYS, 6.1 TB/s, and 159 us without (all but
 // the last stage are read again, mostly from the L2, and the sums).  With loads through registers, four in flight, it
-// was 229 and 332 us; before the packed distances and the integer sums 421 and 879 us, the FP64 additions' time.  Two
+// was 229 and 332 us (BF16 225 and 337, now 64 and 150); before the packed distances and the integer sums 421 and 879 us, the FP64 additions' time.  Two
 // stage buffers, the next stage in flight during the distances, leave 3 blocks of an SM instead of 5: 91 and 174 us.
 template <typename XT, bool KEYS>
 __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__ X, int64_t n, int d, int64_t ld,
@@ -393,8 +403,9 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
                                                           uint64_t *__restrict__ keys, const RedoList redo, DevStatus *st)
 {
     extern __shared__ __align__(16) unsigned char tr_smem[];
-    float *stage = reinterpret_cast<float *>(tr_smem);                       // [TR_THREADS][TR_VP]
-    int *sid = reinterpret_cast<int *>(stage + TR_THREADS * TR_VP);
+    constexpr int VP = TR_VP<XT>;
+    XT *stage = reinterpret_cast<XT *>(tr_smem);                       // [TR_THREADS][TR_VP]
+    int *sid = reinterpret_cast<int *>(stage + TR_THREADS * VP);
     int *s_n = sid + TR_THREADS;                                             // members of u, of u and v in the group
     unsigned char *order = reinterpret_cast<unsigned char *>(s_n + TR_THREADS);  // rows of u, then of v
     float2 *cuv = reinterpret_cast<float2 *>(order + TR_THREADS);            // [d]: (c_u, c_v)
@@ -422,21 +433,27 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
         const int t0 = s * TR_STAGE;
         if (vec) {
             const int t = t0 + (tid & 15) * 4;
-            float *to = stage + (tid & 15) * 4;
+            XT *to = stage + (tid & 15) * 4;
 #pragma unroll 8
             for (int r = tid >> 4; r < gn; r += TR_THREADS / 16) {
-                float *q = to + r * TR_VP;
-                if (t >= d)
-                    *reinterpret_cast<float4 *>(q) = make_float4(0.f, 0.f, 0.f, 0.f);
-                else if constexpr (std::is_same_v<XT, float>)
-                    cp_async16(q, X + (int64_t)sid[r] * ld + t);
-                else
-                    *reinterpret_cast<float4 *>(q) = ldx4<XT>(X + (int64_t)sid[r] * ld + t);
+                XT *q = to + r * VP;
+                const XT *x = X + (int64_t)sid[r] * ld + t;
+                if constexpr (std::is_same_v<XT, float>) {
+                    if (t < d)
+                        cp_async16(q, x);
+                    else
+                        *reinterpret_cast<uint4 *>(q) = make_uint4(0u, 0u, 0u, 0u);
+                } else {
+                    if (t < d)
+                        cp_async8(q, x);
+                    else
+                        *reinterpret_cast<uint2 *>(q) = make_uint2(0u, 0u);
+                }
             }
         } else {
             for (int r = warp; r < gn; r += TR_THREADS / 32)
                 for (int q = lane; q < TR_STAGE; q += 32)
-                    stage[r * TR_VP + q] = t0 + q < d ? ldx(X + (int64_t)sid[r] * ld + t0 + q) : 0.f;
+                    stage[r * VP + q] = t0 + q < d ? X[(int64_t)sid[r] * ld + t0 + q] : XT(0.f);
         }
         cp_async_wait_all();
     };
@@ -460,7 +477,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
             __syncthreads();
             if (!valid)
                 continue;
-            const float *xs = stage + tid * TR_VP;
+            const XT *xs = stage + tid * VP;
             const float2 *cs = cuv + s * TR_STAGE;
             const int tw = min(TR_STAGE, d - s * TR_STAGE);
             auto add = [&](float x, float2 cc) {
@@ -470,7 +487,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
             int tt = 0;
 #pragma unroll 4
             for (; tt + 4 <= tw; tt += 4) {
-                const float4 x = *reinterpret_cast<const float4 *>(xs + tt);
+                const float4 x = staged4(xs + tt);
                 const float4 a = *reinterpret_cast<const float4 *>(cs + tt), h = *reinterpret_cast<const float4 *>(cs + tt + 2);
                 add(x.x, make_float2(a.x, a.y));
                 add(x.y, make_float2(a.z, a.w));
@@ -478,7 +495,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
                 add(x.w, make_float2(h.z, h.w));
             }
             for (; tt < tw; tt++)
-                add(xs[tt], cs[tt]);
+                add((float)xs[tt], cs[tt]);
         }
         if (KEYS) {
             if (valid) {
@@ -527,7 +544,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
                         constexpr int MB = 0x4b400000;  // the bits of SPLIT_M
 #pragma unroll 4
                         for (int r = lo + gg; r < hi; r += 2) {
-                            const float y = stage[order[r] * TR_VP + cc] * sc;
+                            const float y = (float)stage[order[r] * VP + cc] * sc;
                             const float t0 = __fadd_rn(y, SPLIT_M), r0 = __fsub_rn(y, __fsub_rn(t0, SPLIT_M));
                             const float t1 = __fmaf_rn(r0, 4194304.f, SPLIT_M);
                             const float r1 = __fmaf_rn(__fsub_rn(t1, SPLIT_M), -0x1p-22f, r0);
@@ -1044,10 +1061,10 @@ cudaError_t tree_run(const XT *X, int64_t n, int d, int64_t ld, int32_t k, int32
                      int32_t *labels, void *scratch, const TreeBufs &B, DevStatus *st, cudaStream_t s)
 {
     cudaError_t e;
-    if ((e = set_max_smem((const void *)k_tree_pass<XT, false>, (int)pass_smem(MAX_D))) != cudaSuccess ||
-        (e = set_max_smem((const void *)k_tree_pass<XT, true>, (int)pass_smem(MAX_D))) != cudaSuccess)
+    if ((e = set_max_smem((const void *)k_tree_pass<XT, false>, (int)pass_smem<XT>(MAX_D))) != cudaSuccess ||
+        (e = set_max_smem((const void *)k_tree_pass<XT, true>, (int)pass_smem<XT>(MAX_D))) != cudaSuccess)
         return e;
-    const size_t smem = pass_smem(d);
+    const size_t smem = pass_smem<XT>(d);
     const bool vec = x_vec4(X, d, ld);
     if ((e = cudaMemsetAsync(static_cast<char *>(scratch) + B.zero_off, 0, B.zero_bytes, s)) != cudaSuccess)
         return e;
