@@ -26,8 +26,9 @@ cudaError_t launch_assign_tc(const float *X, int64_t n, int64_t d, int64_t ld, c
 
 constexpr int AS_WARPS = 8;
 constexpr int AS_BLOCKS = 152 * 8;  // fixed grid: the FP64 partial sums have a fixed order
-// The row kernels for d <= 256 fit six blocks per SM (at most 40 registers a thread: more warps in flight
-// for the latency-bound centroid gathers).  Every row kernel runs on a grid of the blocks resident at once
+// The row kernels for d <= 128 fit six blocks per SM (at most 40 registers a thread: more warps in flight
+// for the latency-bound centroid gathers), those for d <= 256 five (the FP32 one spills at 40: 400k x 256 1003 us at
+// six, 895 at five).  Every row kernel runs on a grid of the blocks resident at once
 // (resident_grid), one wave; the distortion sums do not depend on it: k_assign_reduce forms them on its
 // own fixed grid.
 constexpr int AS_ROWS_PER_SM = 6;
@@ -95,6 +96,44 @@ __device__ __forceinline__ int collect_labels(int64_t i, int own, const int32_t 
         u += __popc(fr);
     }
     __syncwarp();
+    return u;
+}
+
+// The same without a set: repeats across batches are looked for in the list.  For k_assign, whose lanes walk centroid
+// rows of their own and live on L1, of which the sets would take 8 KB a block (300k x 130 2500 us an assignment with
+// them, 2240 without).
+__device__ __forceinline__ int collect_labels_plain(int64_t i, int own, const int32_t *__restrict__ G, int kappa,
+                                                    int64_t n, int k, const int32_t *__restrict__ Lin, int *qlist,
+                                                    DevStatus *st)
+{
+    const int lane = lane_id(), ncand = kappa + 1;
+    int u = 0;
+    for (int c0 = 0; c0 < ncand; c0 += 32) {
+        const int c = c0 + lane;
+        int lab = -1;
+        if (c == 0) {
+            lab = own;
+        } else if (c < ncand) {
+            const int nb = __ldcs(G + i * kappa + (c - 1));
+            if ((unsigned)nb < (unsigned)n)
+                lab = Lin[nb];
+            else
+                flag_error(st, GK_ERR_INVALID, (unsigned)i);
+        }
+        if (c < ncand && (unsigned)lab >= (unsigned)k) {
+            flag_error(st, GK_ERR_INVALID, (unsigned)i);
+            lab = -1;
+        }
+        const unsigned peers = __match_any_sync(FULL_MASK, lab);
+        bool fresh = lab >= 0 && (peers & lanemask_lt()) == 0u;
+        for (int q = 0; q < u && fresh; q++)
+            fresh = qlist[q] != lab;
+        const unsigned fr = __ballot_sync(FULL_MASK, fresh);
+        if (fresh)
+            qlist[u + __popc(fr & lanemask_lt())] = lab;
+        u += __popc(fr);
+        __syncwarp();
+    }
     return u;
 }
 
@@ -204,7 +243,7 @@ __device__ __forceinline__ void each_sample(int64_t first, int64_t step, int64_t
     if (blockIdx.x == 0 && threadIdx.x == 0)
         *trk.ticket = 0u;  // for k_assign_reduce
     if constexpr (!LISTS) {
-        for (int64_t i = first; i < n; i += step)
+        for (int64_t i = first; i < n; i += (int64_t)gridDim.x * (blockDim.x >> 5))  // `step`, not kept in registers
             f(i, std::false_type{});
     } else {
         const int nf = trk.todo_n[0], np = trk.todo_n[1];
@@ -240,11 +279,14 @@ __device__ __forceinline__ int track_filter(const Track &trk, int *qlist, int u)
 
 // The winner (bd, br) of sample i, written by lane 0.  Without a valid candidate (br still INT_MAX) the input label
 // stays, with distance 0, and its cluster counts as changed, so that the next assignment looks again.
-__device__ __forceinline__ void write_winner(int64_t i, int own, int k, float bd, int br, int32_t *__restrict__ Lout,
-                                             float *__restrict__ best, const Track &trk)
+__device__ __forceinline__ void write_winner(int64_t i, const int32_t *__restrict__ Lin, int k, float bd, int br,
+                                             int32_t *__restrict__ Lout, float *__restrict__ best, const Track &trk)
 {
     if (lane_id() != 0)
         return;
+    int own = br;
+    if (trk.dirty_out || br == 0x7fffffff)
+        own = Lin[i];  // read again: kept in a register it cost the wide rows spills
     bool changed = br != own;
     if (br == 0x7fffffff) {
         br = own, bd = 0.f;
@@ -314,14 +356,22 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign(const XT *__restrict__
     const int w = threadIdx.x >> 5, lane = lane_id();
     const int dpad = (d + 3) & ~3;
     float *xs = smem + w * dpad;
-    int *tab = reinterpret_cast<int *>(smem + AS_WARPS * dpad) + w * (AS_HASH + AS_QROW);
-    int *qlist = tab + AS_HASH;
+    int *qlist = reinterpret_cast<int *>(smem + AS_WARPS * dpad) + w * AS_QCAP;
 
     each_sample<LISTS>((int64_t)blockIdx.x * AS_WARPS + w, (int64_t)gridDim.x * AS_WARPS, n, trk, todo,
                        [&](int64_t i, auto part) {
         constexpr bool PART = decltype(part)::value;
+        // stage x_i
+        const XT *xi = X + i * ld;
+        if (VEC == 4) {
+            for (int t = lane; t < (d >> 2); t += 32)
+                reinterpret_cast<float4 *>(xs)[t] = ldx4<XT>(xi + 4 * t);
+        } else {
+            for (int t = lane; t < d; t += 32)
+                xs[t] = ldx(xi + t);
+        }
         const int own = Lin[i];
-        int u = collect_labels(i, own, G, kappa, n, k, Lin, qlist, tab, st);
+        int u = collect_labels_plain(i, own, G, kappa, n, k, Lin, qlist, st);
         float bd = __int_as_float(0x7f800000);
         int br = 0x7fffffff;
         if constexpr (PART) {
@@ -329,18 +379,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign(const XT *__restrict__
             bd = best_out[i];
             br = own;
         }
-        if (u > 0) {
-            // stage x_i
-            const XT *xi = X + i * ld;
-            if (VEC == 4) {
-                for (int t = lane; t < (d >> 2); t += 32)
-                    reinterpret_cast<float4 *>(xs)[t] = ldx4<XT>(xi + 4 * t);
-            } else {
-                for (int t = lane; t < d; t += 32)
-                    xs[t] = ldx(xi + t);
-            }
-            __syncwarp();
-        }
+        __syncwarp();
         // distances to the kept centroids, lane-parallel over candidates
         for (int q = lane; q < u; q += 32) {
             int r = qlist[q];
@@ -359,7 +398,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign(const XT *__restrict__
                 br = orr;
             }
         }
-        write_winner(i, own, k, bd, br, Lout, best_out, trk);
+        write_winner(i, Lin, k, bd, br, Lout, best_out, trk);
         __syncwarp();
     });
 }
@@ -373,7 +412,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign(const XT *__restrict__
 // its first entry, whose second evaluation
 // cannot change the (distance, label) minimum.
 template <int NV, typename XT, int GS, bool LISTS, int LPR = 32>
-__global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k_assign_rows(const XT *__restrict__ X, int64_t n, int d,
+__global__ void __launch_bounds__(AS_WARPS * 32, NV == 1 ? AS_ROWS_PER_SM : NV == 2 ? 5 : 4) k_assign_rows(const XT *__restrict__ X, int64_t n, int d,
                                                                int64_t ld, const int32_t *__restrict__ G, int kappa,
                                                                const float *__restrict__ C, int k,
                                                                const int32_t *__restrict__ Lin,
@@ -389,7 +428,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
     static_assert(GS == 4 || GS == 8, "candidates per lane set and group: 4 or 8");
     static_assert(LPR == 32 || (NV == 1 && LPR >= GS), "lane sets hold whole rows");
     constexpr int SETS = 32 / LPR;
-    const int set = lane / LPR, sl = lane % LPR;
+    const int set = LPR == 32 ? 0 : lane / LPR, sl = LPR == 32 ? lane : lane % LPR;
     const int d4 = d >> 2;
     const float4 *C4 = reinterpret_cast<const float4 *>(C);
 
@@ -450,7 +489,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
                 br = orr;
             }
         }
-        write_winner(i, own, k, bd, br, Lout, best_out, trk);
+        write_winner(i, Lin, k, bd, br, Lout, best_out, trk);
         __syncwarp();
     });
 }
@@ -556,7 +595,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV 
                 }
             }
         }
-        write_winner(i, own, k, bd, br, Lout, best_out, trk);
+        write_winner(i, Lin, k, bd, br, Lout, best_out, trk);
         __syncwarp();
     });
 }
@@ -838,7 +877,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
                 }
             }
         }
-        write_winner(i, own, k, bd, br, Lout, best_out, trk);
+        write_winner(i, Lin, k, bd, br, Lout, best_out, trk);
         __syncwarp();
     });
 }
@@ -1102,7 +1141,7 @@ constexpr int Q8_MIN_D = 32;
 // Where precision 0 and 1 take the int8 screening: rows of more than Q8_PAYS_D values, in sample sets large enough for
 // its extra launch.  FP32 rows against screening, us an assignment: 200k x 256 230 / 300 (539 / 607 at kappa = 50),
 // 200k x 300 290 / 280, 100k x 384 259 / 215, 300k x 512 BF16 1317 / 801, 100k x 960 960 / 366; at 300k x 128 401 / 516.
-constexpr int Q8_PAYS_D = 320;
+constexpr int Q8_PAYS_D = 288;
 
 static bool assign_q8_pays(int64_t n, int64_t d) { return d > Q8_PAYS_D && n * d >= ((int64_t)1 << 22); }
 
@@ -1277,8 +1316,8 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
 #undef GK_ASGT
     } else {
         int dpad = (int)((d + 3) & ~3);
-        size_t shm = sizeof(float) * (size_t)AS_WARPS * dpad + sizeof(int) * AS_WARPS * (AS_HASH + AS_QROW);
-        const int shm_max = (int)(sizeof(float) * (size_t)AS_WARPS * MAX_D + sizeof(int) * AS_WARPS * (AS_HASH + AS_QROW));
+        size_t shm = sizeof(float) * (size_t)AS_WARPS * dpad + sizeof(int) * AS_WARPS * AS_QCAP;
+        const int shm_max = (int)(sizeof(float) * (size_t)AS_WARPS * MAX_D + sizeof(int) * AS_WARPS * AS_QCAP);
         auto launch = [&](auto kernel) -> cudaError_t {
             cudaError_t le = set_max_smem(reinterpret_cast<const void *>(kernel), shm_max);
             if (le == cudaSuccess)

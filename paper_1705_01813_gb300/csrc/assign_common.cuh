@@ -52,7 +52,7 @@ __device__ __forceinline__ float transpose_reduce32(float (&v)[32]) { return tra
 template <int NV, int LPR = 32, typename RowLoad>
 __device__ __forceinline__ float lane_partial(const float4 (&xv)[NV], int d4, RowLoad load)
 {
-    const int lane = lane_id() & (LPR - 1);
+    const int lane = LPR == 32 ? lane_id() : lane_id() & (LPR - 1);
     const float2 m1 = make_float2(-1.f, -1.f);
     float2 a = make_float2(0.f, 0.f);
 #pragma unroll
