@@ -208,6 +208,10 @@ __device__ __forceinline__ bool merge_many(uint64_t (&ck)[NC], bool (&ok)[NC], b
             mb.bk[m + __popc(bal & lanemask_lt())] = ck[v];
         m += __popc(bal);
     }
+    if (m == 0) {  // every candidate is in the row
+        __syncwarp();
+        return false;
+    }
     if ((m & 1) && lane == 0)
         mb.bk[m] = ~0ull;  // the ranking loop reads pairs
     __syncwarp();

@@ -186,17 +186,22 @@ __device__ __forceinline__ void load_members(const int32_t *__restrict__ S, int 
 }
 
 // Listed runs blockIdx.x, + gridDim.x, ... (LONG: the list from the back of the array), T-wide tiles.
-template <int T, typename XT, bool VEC>
+// STEP: no previous refinement and a graph of any caller's (prev NULL, canon unset), compiled apart: what only the
+// other calls need costs this form registers it spilled (1M x 128, k = 20,000 2336 us a call with one kernel for both,
+// 2269 with two).
+template <int T, typename XT, bool VEC, bool STEP>
 __global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT *__restrict__ X, int64_t n, int d,
                                                                         int64_t ld, const int32_t *__restrict__ mem,
                                                                         const int2 *__restrict__ runs,
                                                                         int64_t runs_cap,
                                                                         const RunCounts *__restrict__ cnt, bool longs,
-                                                                        const int32_t *__restrict__ prev, bool canon,
+                                                                        const int32_t *__restrict__ prev_in, bool canon_in,
                                                                         uint8_t *__restrict__ row_changed, int kappa,
                                                                         int32_t *__restrict__ g_idx,
                                                                         float *__restrict__ g_dist, DevStatus *st)
 {
+    const int32_t *__restrict__ prev = STEP ? nullptr : prev_in;
+    const bool canon = STEP ? false : canon_in;
     using TL = RefineTile<T>;
     constexpr int DS = TL::DS, NC = T / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -226,7 +231,7 @@ __global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT
                 const int rn = row + RF_WARPS;
                 if (rn < nr && rid[rn] >= 0)  // next row's list in flight during this merge
                     load_row(nxt, g_idx + (int64_t)rid[rn] * kappa, g_dist + (int64_t)rid[rn] * kappa, kappa);
-                if (i >= 0 && merge_row<NC>(i, rpr[row], canon, ci, cp, si, sm, dt + row * DS, ncl, kappa, cur,
+                if (i >= 0 && merge_row<NC>(i, STEP ? -1 : rpr[row], canon, ci, cp, si, sm, dt + row * DS, ncl, kappa, cur,
                                             g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mb) &&
                     row_changed && lane_id() == 0)
                     row_changed[i] = 1;
@@ -236,12 +241,19 @@ __global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT
         __syncthreads();  // the previous run's merges are done
         if (sz <= T) {
             load_members<T>(S, sz, n, prev, rid, rpr, sid, smap, spr, tid, first, st, sync);
-            const int nlive = live_blocks<T, RF_THREADS>(sz, prev ? rpr : nullptr, list, wcnt, tid, sync);
             // the arithmetic goes to the block's warps rot, rot + 1, ... (rot = blockIdx.x % 4): each warp of an SM
             // issues on scheduler (its index % 4), so blocks that share an SM spread their few busy warps over all
             // four schedulers instead of all starting at scheduler 0
             const int t = (tid - (int)(blockIdx.x & 3) * 32) & (RF_THREADS - 1);
-            const int code = t < nlive ? list[t] : 0;
+            int nlive, code;
+            if (prev) {
+                nlive = live_blocks<T, RF_THREADS>(sz, rpr, list, wcnt, tid, sync);
+                code = t < nlive ? list[t] : 0;
+            } else {
+                const int nb = (sz + TL::Q - 1) / TL::Q;
+                nlive = nb * (nb + 1) / 2;
+                code = t < nlive ? triangle_block(nb, t) : 0;
+            }
             tile_distances<T, true, VEC>(X, d, ld, rid, rid, code >> 8, code & 255, t < nlive, xr, dt);
             __syncthreads();
             merge_rows(sz, sz, rid, rpr, sid, prev ? smap : nullptr);
@@ -335,9 +347,17 @@ __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restric
             int *rid = rids + (j & 1) * T, *rpr = rprs + (j & 1) * T;
             load_members<T>(mem + rec.x, rec.y, n, prev, rid, rpr, sids + (j & 1) * T, smaps + (j & 1) * T, spr, ct, rec.x,
                             st, sync);
-            const int nlive = live_blocks<T, WS_NC>(rec.y, prev ? rpr : nullptr, list, wcnt, ct, sync);
+            int nlive, code;
+            if (prev) {
+                nlive = live_blocks<T, WS_NC>(rec.y, rpr, list, wcnt, ct, sync);
+                code = ct < nlive ? list[ct] : 0;
+            } else {
+                const int nb = (rec.y + Q - 1) / Q;
+                nlive = nb * (nb + 1) / 2;
+                code = ct < nlive ? triangle_block(nb, ct) : 0;
+            }
             const bool live = ct < nlive;
-            const int code = live ? list[ct] : 0, by = code >> 8, bx = code & 255;
+            const int by = code >> 8, bx = code & 255;
             float2 acc[Q][Q / 2];
             tile_distances_group<WS_NC, VEC>(X, d, ld, rid, by, bx, live, stage, ct, WS_BAR_C, acc);
             bar_sync(WS_BAR_EMPTY, WS_THREADS);  // the merge warps no longer read the distance tile
@@ -431,15 +451,17 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
     // an upper bound of the number of runs: sum over clusters of (m / cap + 1)
     const int64_t bound = (int64_t)k + n / max_cluster + 1;
     auto blocks = [&](int resident) { return (unsigned)(bound < resident ? bound : resident); };
-    int grid = 0;
+    // a block per run, handed out as blocks finish (a wave of blocks walking the list was 4% slower)
+    const bool step = !prev_in && !canon;
     // runs of more than `split` members (FP32 tiles of 128; longer runs in several tiles)
     if (max_cluster > split) {
         constexpr size_t shm = refine_smem_bytes<128>();
-        const void *f = reinterpret_cast<const void *>(k_refine<128, XT, VEC>);
-        if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, RF_THREADS, shm, &grid)) != cudaSuccess)
+        auto kernel = step ? k_refine<128, XT, VEC, true> : k_refine<128, XT, VEC, false>;
+        const void *f = reinterpret_cast<const void *>(kernel);
+        if ((e = set_max_smem(f, (int)shm)) != cudaSuccess)
             return e;
-        k_refine<128, XT, VEC><<<blocks(grid), RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, true,
-                                                                     prev_in, canon, row_changed, kappa, g_idx, g_dist, st);
+        kernel<<<(unsigned)bound, RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, true, prev_in, canon,
+                                                    row_changed, kappa, g_idx, g_dist, st);
     }
     if (tensor) {
         // tensor-core Gram for runs of <= 128 members
@@ -453,6 +475,7 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
     // where five warps' share of the element loads made the specialised form slower (1M x 960 FP32: 7.6
     // against 7.7 ms; 1M x 128 FP32: 3.7 against 3.9 ms)
     if constexpr (VEC) {
+        int grid = 0;
         constexpr size_t shm = refine_ws_smem_bytes();
         const void *f = reinterpret_cast<const void *>(k_refine_ws<XT, VEC>);
         if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, WS_THREADS, shm, &grid)) != cudaSuccess)
@@ -461,11 +484,12 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
                                                                    g_idx, g_dist, st);
     } else {
         constexpr size_t shm = refine_smem_bytes<64>();
-        const void *f = reinterpret_cast<const void *>(k_refine<64, XT, VEC>);
-        if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, RF_THREADS, shm, &grid)) != cudaSuccess)
+        auto kernel = step ? k_refine<64, XT, VEC, true> : k_refine<64, XT, VEC, false>;
+        const void *f = reinterpret_cast<const void *>(kernel);
+        if ((e = set_max_smem(f, (int)shm)) != cudaSuccess)
             return e;
-        k_refine<64, XT, VEC><<<blocks(grid), RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, false,
-                                                                    prev_in, canon, row_changed, kappa, g_idx, g_dist, st);
+        kernel<<<(unsigned)bound, RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, false, prev_in, canon,
+                                                    row_changed, kappa, g_idx, g_dist, st);
     }
     return cudaGetLastError();
 }

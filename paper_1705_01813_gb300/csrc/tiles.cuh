@@ -57,11 +57,24 @@ __host__ __device__ inline bool tile_vec16(const XT *X, int d, int64_t ld)
     return d % E == 0 && ld % E == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
 }
 
+// Block t of the nb (nb + 1) / 2 blocks on and above the diagonal, row by row, as a code by << 8 | bx (past the last: by
+// = nb).
+__device__ __forceinline__ int triangle_block(int nb, int t)
+{
+    int bx = t, by = 0;
+    while (by < nb && bx >= nb - by) {
+        bx -= nb - by;
+        by++;
+    }
+    return by << 8 | (bx + by);
+}
+
 // The Q x Q blocks of a run's own tile (rows = columns = the run's nr members) that have to be computed, as codes
 // by << 8 | bx in list[].  The tile is symmetric, d(i, j) = d(j, i) bit for bit (the difference only changes sign),
 // so only blocks with by <= bx < nb = ceil(nr / Q) count (a run of 50 has 91 at Q = 4); and with prun, the run each
 // member belonged to in the previous refinement (members sorted by it, -1: none), a block whose rows and columns all
-// come from one such run holds only pairs that were compared then, and is left out.  Called by NT threads with index
+// come from one such run holds only pairs that were compared then, and is left out.  (Without a previous refinement
+// all of them count, and the callers take triangle_block: two barriers less, 5% of a refinement of narrow runs.)  Called by NT threads with index
 // t in [0, NT), NT a multiple of 32 and >= NBLK; sync() is their barrier, wcnt has NT / 32 entries.  Returns the
 // number of blocks (the list is valid after the call).
 template <int T, int NT, typename Sync>
@@ -70,14 +83,9 @@ __device__ __forceinline__ int live_blocks(int nr, const int *prun, unsigned sho
     constexpr int Q = RefineTile<T>::Q;
     static_assert(NT >= RefineTile<T>::NBLK && NT % 32 == 0, "one thread per block");
     const int nb = (nr + Q - 1) / Q;
-    int bx = t, by = 0;
-    while (by < nb && bx >= nb - by) {
-        bx -= nb - by;
-        by++;
-    }
-    bx += by;
+    const int by = triangle_block(nb, t) >> 8, bx = triangle_block(nb, t) & 255;
     bool live = by < nb;
-    if (live && prun)
+    if (live)
         live = prun[Q * by] < 0 || prun[Q * by] != prun[min(Q * bx + Q, nr) - 1];
     const unsigned bal = __ballot_sync(FULL_MASK, live);
     if ((t & 31) == 0)
