@@ -281,12 +281,14 @@ def launches_per_step(w, precision):
     # update: the warp-per-cluster kernel for clusters of at most 32 members (16-byte rows of at most 512 values),
     # the block kernel for the others, the FP64 sum (chains and tree: the step's groupings come from their own call)
     upd = 4 if (w.d % 4 == 0 and w.d <= 512) else 3
+    if w.d % 4 == 0 and w.d > 512 and w.n > 512:
+        upd += 1  # the column blocks of large clusters
 
     def asg(k):
         # (then the reduction): kernel (0, 1; wide rows of large sets take the int8 screening); shadow copy + screening
         # kernel (2, 4); BF16 copy, tensor-core tiles, SIMT leftovers (3)
         if precision < 2:
-            return 3 if w.d % 4 == 0 and 320 < w.d <= 1024 and w.n * w.d >= 1 << 22 else 2
+            return 3 if w.d % 4 == 0 and 288 < w.d <= 1024 and w.n * w.d >= 1 << 22 else 2
         return 3 if precision in (2, 4) or w.d > 128 else 4
     # refine: the run lists, then cluster-sorted copy + Gram + exact recompute + merge (tensor cores) or the two FP32
     # tile widths (runs of max_cluster = 128 members at most)
@@ -317,10 +319,15 @@ def tc_refine(precision, d, storage="f32"):
     return precision >= 1 and 64 <= d <= 128
 
 
+def int8_rows(precision, d):
+    """The library's dispatch of the assignment to int8 screening (its rule at the workloads' sizes)."""
+    return precision == 4 or (precision <= 1 and d % 4 == 0 and 288 < d <= 1024)
+
+
 def kernel_of(tag, precision=1, d=128, storage="f32"):
     if tag == "refine" and tc_refine(precision, d, storage):
         return "k_refine_gram"
-    if tag == "assign" and precision in (2, 4):
+    if tag == "assign" and (precision in (2, 4) or int8_rows(precision, d)):
         return "k_assign_rows_scr"
     if tag == "assign" and precision == 3:
         return "k_assign_tc"
@@ -619,7 +626,8 @@ def run_gpu(args):
                       3: "1 plus bf16 tcgen05 screening of assignment candidates with exact fp32 recompute",
                       4: "1 plus int8 (per-row scale) screening of assignment candidates (simt) with exact fp32 "
                          "recompute"}
-                     [lvl],
+                     [lvl] + ("; int8 screening of assignment candidates with exact fp32 recompute (rows of more than "
+                              "288 values)" if lvl <= 1 and int8_rows(lvl, w.d) else ""),
         "assign_group_width": (args.precision >> 8) & 0xff or None,
         "plain_fp32_ms_per_step": fp32_ms,
         "assign_samples_per_s": w.n / statistics.mean(assign_times) if assign_times else None,
@@ -644,19 +652,19 @@ def run_gpu(args):
         "e2e": e2e,
     }
     # roofline of every call type, for context
-    # The assignment gathers one centroid row per candidate: n u d (BF16 rows at precision >= 2, FP32 rows
-    # otherwise) bytes per call beyond the algorithmic ones, u the measured mean candidate count of the phase
+    # The assignment gathers one centroid row per candidate: n u d (int8 rows where it screens with them, BF16 rows
+    # at precision 2 and 3, FP32 rows otherwise) bytes per call beyond the algorithmic ones, u the measured mean candidate count of the phase
     # (graph rounds at k0, fit iterations at k).  They come from L2 while the centroid table fits it and from
     # HBM otherwise; the probe kernels measure both gather ceilings on this GPU.
     if dom == "assign" and u:
-        row_b = {2: 2, 3: 2, 4: 1}.get(lvl, 4)
+        row_b = 1 if int8_rows(lvl, w.d) else {2: 2, 3: 2}.get(lvl, 4)
         per = [(w.k0, u.get("build"), w.tau), (w.k, u.get("fit"), w.iters)]
         g_l2 = sum(w.n * uu * w.d * row_b * c for kk, uu, c in per if uu and kk * w.d * 4 <= L2_BYTES)
         g_hbm = sum(w.n * uu * w.d * row_b * c for kk, uu, c in per if uu and kk * w.d * 4 > L2_BYTES)
         g_l2, g_hbm = g_l2 / (w.tau + w.iters), g_hbm / (w.tau + w.iters)
         gath = {"bytes_per_launch": int(g_l2 + g_hbm), "from_l2": int(g_l2), "from_hbm": int(g_hbm),
                 "achieved_gbs": (g_l2 + g_hbm) / avg / 1e9,
-                "note": "candidate centroid rows, one per candidate (exact second-pass rows at precision 2 not "
+                "note": "candidate centroid rows, one per candidate (exact second-pass rows of a screening not "
                         "counted)"}
         if ceilings:
             # time the gathers would take at the measured ceilings, against the call's time

@@ -14,14 +14,16 @@
 
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 namespace gkm {
 
 constexpr int UP_WARPS = 4;
 constexpr int UP_MCHUNK = 1024;  // member ids staged in shared memory at a time
-constexpr int UP_RV = 8;         // member rows per group and pipeline stage (PIPE kernels): 16-byte vectors per lane
-constexpr int UP_SPLIT = 8;      // CTAs of a row's column blocks, at most
+constexpr int UP_SPLIT = 8;      // blocks of a large cluster's column blocks, at most
+constexpr int UP_LARGE = 512;    // members of a cluster whose column blocks get blocks of their own
+constexpr int UP_RV = 8;         // 16-byte vectors per lane and pipeline stage (PIPE kernels): 8 / CPL rows
 
 __device__ __forceinline__ void kahan_add(float &s, float &c, float x)
 {
@@ -152,24 +154,17 @@ __device__ __forceinline__ DF chains_sum(float2 qs, float2 qc)
     return df_add(fast_two_sum(qs.x, -qc.x), fast_two_sum(qs.y, -qc.y));
 }
 
-// One block of UP_WARPS warps per cluster and column block of 32 row vectors, the
-// blocks of a cluster a thread-block cluster of up to UP_SPLIT (the rule depends on
-// the row width only, so BF16 samples and their FP32 widening sum alike).  A
-// cluster's time is that of its longest chain, the compensated sum of squares, and
-// one block walking all columns of every member made a launch wait for its largest
-// cluster: 200k x 960, k = 2000 494 us with one block, 286 split; 300k x 200,
-// k = 3000 uneven 78 and 67 us (six loads in flight per warp instead of two: 523, 79).  Each warp is split into G groups
+// One block of UP_WARPS warps per cluster.  Each warp is split into G groups
 // of L lanes; the W * G groups of the block take members g, g + W G, ... of
 // the cluster (UNR of them in flight per group), and lane s of a group owns
-// row vector s of the column block.  Group sums are
+// row vectors s, s + L, ... (CPL of them per column block).  Group sums are
 // combined (double-float) across the groups of a warp by shuffles and across
 // the warps through shared memory in a fixed order (reproducible bits).
 // PIPE (16-byte vectors): the member rows are streamed into a two-stage
-// shared-memory ring with cp.async, UP_RV rows per group and stage, so the
+// shared-memory ring with cp.async, UP_RV / CPL rows per group and stage, so the
 // next stage's loads are in flight while the current one is summed; the
 // summation order is the same.  The ring shares its memory with the partial
-// sums of the epilogue, which run after it.  The blocks' parts of the distortion
-// term meet in the first one's shared memory.
+// sums of the epilogue, which run after it.
 // One VEC-wide vector of a sample row as floats (BF16 samples are widened).
 template <int VEC, typename XT>
 __device__ __forceinline__ typename VecT<VEC>::T load_vec(const XT *p)
@@ -180,15 +175,209 @@ __device__ __forceinline__ typename VecT<VEC>::T load_vec(const XT *p)
         return ldx(p);
 }
 
-template <int VEC, bool PIPE, bool WALK, typename XT>
-__global__ void __launch_bounds__(UP_WARPS * 32, PIPE ? 6 : 8) k_update(const XT *__restrict__ X, int d, int64_t ld,
+template <int VEC, int CPL, bool PIPE, typename XT>
+__global__ void __launch_bounds__(UP_WARPS * 32) k_update(const XT *__restrict__ X, int d, int64_t ld,
                                                           const int32_t *__restrict__ off,
-                                                          const int32_t *__restrict__ mem, int k, int small_max, int nb, int chunk,
+                                                          const int32_t *__restrict__ mem, int k, int small_max, int large,
                                                           float *__restrict__ C, int32_t *__restrict__ counts,
                                                           double *__restrict__ contrib,
                                                           const uint8_t *__restrict__ dirty, DevStatus *st)
 {
     using V = typename VecT<VEC>::T;
+    static_assert(!PIPE || std::is_same_v<XT, float>, "the cp.async ring moves FP32 rows");
+    constexpr int UNR = CPL >= 8 ? 1 : (CPL >= 4 ? 2 : (CPL >= 2 ? 4 : 4));  // member rows in flight per group
+    constexpr int R = PIPE ? UP_RV / CPL : 1;  // rows per group and stage
+    constexpr size_t PART_BYTES = sizeof(float2) * UP_WARPS * 32 * CPL * VEC;
+    constexpr size_t RING_BYTES = PIPE ? sizeof(float4) * UP_WARPS * 2 * R * 32 * CPL : 0;
+    __shared__ __align__(16) unsigned char s_buf[PART_BYTES > RING_BYTES ? PART_BYTES : RING_BYTES];
+    auto s_part = reinterpret_cast<float2 (*)[32 * CPL * VEC]>(s_buf);
+    __shared__ float2 s_sq[UP_WARPS], s_dd[UP_WARPS];
+    __shared__ int s_mem[UP_MCHUNK];
+    static_assert(!PIPE || (VEC == 4 && UP_RV % CPL == 0), "the pipelined variant moves 16-byte vectors");
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const int nv = d / VEC;  // vectors per row
+    int L = 1;
+    while (L < 32 && L < nv)
+        L <<= 1;
+    const int G = 32 / L;
+    const int g = lane / L, sub = lane % L;
+    const int gstride = UP_WARPS * G, gidx = w * G + g;
+    const int64_t ldv = ld / VEC;
+    const V *Xv = reinterpret_cast<const V *>(X);
+
+    // clusters r = blockIdx.x, + gridDim.x, ...; those of at most small_max members are k_update_small's,
+    // those of more than large k_update_wide's
+    for (int r = blockIdx.x; r < k; r += gridDim.x) {
+    const int beg = off[r], m = off[r + 1] - beg;
+    if (m <= small_max || m > large || (dirty && dirty[r] == 0))
+        continue;
+    if (counts && threadIdx.x == 0)
+        counts[r] = m;
+    if (m == 0) {
+        if (threadIdx.x == 0)
+            contrib[r] = 0.0;
+        continue;
+    }
+    const float mf = (float)m, inv_m = 1.0f / mf;
+    DF sq_lane = {0.f, 0.f}, dd_lane = {0.f, 0.f};
+    for (int cb = 0; cb < nv; cb += L * CPL) {
+        float s[CPL][VEC], c[CPL][VEC];
+        float2 qs = make_float2(0.f, 0.f), qc = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int u = 0; u < CPL; u++)
+#pragma unroll
+            for (int q = 0; q < VEC; q++)
+                s[u][q] = c[u][q] = 0.f;
+        // the member ids of a chunk are staged in shared memory first, so each row
+        // load waits for one memory round trip instead of two
+        for (int mb = 0; mb < m; mb += UP_MCHUNK) {
+            const int mc = min(UP_MCHUNK, m - mb);
+            __syncthreads();  // the previous chunk's ids are no longer read
+            for (int q = threadIdx.x; q < mc; q += UP_WARPS * 32)
+                s_mem[q] = __ldg(mem + beg + mb + q);
+            __syncthreads();
+            if constexpr (PIPE) {
+                float4 *ring = reinterpret_cast<float4 *>(s_buf) + w * (2 * R * 32 * CPL);  // [stage][row][u][lane]
+                const int wlead = w * G;                       // the warp's first group has the most rows
+                const int njw = mc > wlead ? (mc - wlead + gstride - 1) / gstride : 0;
+                const int nst = (njw + R - 1) / R;
+                auto issue = [&](int t) {
+                    float4 *buf = ring + (t & 1) * (R * 32 * CPL);
+#pragma unroll
+                    for (int z = 0; z < R; z++) {
+                        const int p = gidx + gstride * (t * R + z);
+                        if (p < mc) {
+                            const V *row = Xv + (int64_t)s_mem[p] * ldv;
+#pragma unroll
+                            for (int u = 0; u < CPL; u++) {
+                                const int col = cb + sub + u * L;
+                                if (col < nv)
+                                    cp_async16(buf + (z * CPL + u) * 32 + lane, row + col);
+                            }
+                        }
+                    }
+                    cp_async_commit();
+                };
+                if (nst > 0)
+                    issue(0);
+                for (int t = 0; t < nst; t++) {
+                    if (t + 1 < nst)
+                        issue(t + 1);
+                    else
+                        cp_async_commit();  // empty group: the wait below always leaves one
+                    cp_async_wait<1>();
+                    __syncwarp();
+                    const float4 *buf = ring + (t & 1) * (R * 32 * CPL);
+#pragma unroll
+                    for (int z = 0; z < R; z++) {
+                        if (gidx + gstride * (t * R + z) < mc) {
+                            V vz[CPL];
+#pragma unroll
+                            for (int u = 0; u < CPL; u++)
+                                vz[u] = buf[(z * CPL + u) * 32 + lane];
+                            accumulate<VEC, CPL, std::is_same_v<XT, __nv_bfloat16>>(vz, s, c, qs, qc, cb, sub, L, nv);
+                        }
+                    }
+                    __syncwarp();  // stage t & 1 is refilled by issue(t + 2)
+                }
+            } else {
+                for (int p0 = gidx; p0 < mc; p0 += UNR * gstride) {
+                    V v[UNR][CPL];
+#pragma unroll
+                    for (int z = 0; z < UNR; z++) {
+                        const int p = p0 + z * gstride;
+                        if (p < mc) {
+                            const XT *rowx = X + (int64_t)s_mem[p] * ld;
+#pragma unroll
+                            for (int u = 0; u < CPL; u++) {
+                                const int col = cb + sub + u * L;
+                                if (col < nv)
+                                    v[z][u] = load_vec<VEC>(rowx + (int64_t)col * VEC);
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int z = 0; z < UNR; z++)
+                        if (p0 + z * gstride < mc)
+                            accumulate<VEC, CPL, std::is_same_v<XT, __nv_bfloat16>>(v[z], s, c, qs, qc, cb, sub, L, nv);
+                }
+            }
+        }
+        if constexpr (PIPE)
+            __syncthreads();  // every warp is done with the ring before the partial sums overwrite it
+        sq_lane = df_add(sq_lane, chains_sum(qs, qc));
+        // combine the G groups of the warp, then the warps of the block, in a fixed order
+#pragma unroll
+        for (int u = 0; u < CPL; u++) {
+#pragma unroll
+            for (int q = 0; q < VEC; q++) {
+                DF S = fast_two_sum(s[u][q], -c[u][q]);  // the Kahan sum s - c, exactly
+                for (int o = L; o < 32; o <<= 1)
+                    S = df_add(S, df_shfl_xor(S, o));
+                if (g == 0)
+                    s_part[w][(u * L + sub) * VEC + q] = make_float2(S.hi, S.lo);
+            }
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < L * CPL * VEC; e += UP_WARPS * 32) {
+            // entry e = (u * L + sb) * VEC + q holds column vector cb + sb + u * L, component q
+            const int u = (e / VEC) / L, sb = (e / VEC) % L;
+            const int colv = cb + sb + u * L;
+            if (colv < nv) {
+                DF S = {s_part[0][e].x, s_part[0][e].y};
+                for (int ww = 1; ww < UP_WARPS; ww++)
+                    S = df_add(S, DF{s_part[ww][e].x, s_part[ww][e].y});
+                C[(int64_t)r * d + (int64_t)colv * VEC + (e % VEC)] = df_div(S, mf, inv_m);
+                dd_lane = df_add(dd_lane, df_sqr(S));
+            }
+        }
+        __syncthreads();
+    }
+    // sum of ||x||^2 over all lanes, sum of D_t^2 over the threads that wrote means
+    for (int o = 1; o < 32; o <<= 1) {
+        sq_lane = df_add(sq_lane, df_shfl_xor(sq_lane, o));
+        dd_lane = df_add(dd_lane, df_shfl_xor(dd_lane, o));
+    }
+    if (lane == 0) {
+        s_sq[w] = make_float2(sq_lane.hi, sq_lane.lo);
+        s_dd[w] = make_float2(dd_lane.hi, dd_lane.lo);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        DF sq = {s_sq[0].x, s_sq[0].y}, dd = {s_dd[0].x, s_dd[0].y};
+        for (int ww = 1; ww < UP_WARPS; ww++) {
+            sq = df_add(sq, DF{s_sq[ww].x, s_sq[ww].y});
+            dd = df_add(dd, DF{s_dd[ww].x, s_dd[ww].y});
+        }
+        const double cr = df_to_double(sq) - df_to_double(dd) / (double)m;
+        contrib[r] = cr;
+        if (!isfinite(cr))  // a non-finite sample in the cluster (Inf or NaN spreads into its sums)
+            flag_error(st, GK_ERR_NUMERIC, (unsigned)r);
+    }
+    __syncthreads();  // s_sq / s_dd are read above before the next cluster writes them
+    }
+}
+
+// The clusters of more than `large` members, where rows have several column blocks of L vectors: a block of UP_WARPS
+// warps per column block, the blocks of a cluster a thread-block cluster of up to UP_SPLIT.  A cluster's time is that of
+// its longest chain, the compensated sum of squares, and one block walking all columns of every member made a launch
+// wait for its largest cluster.  Rows of up to four column blocks take this kernel for every cluster that is not
+// k_update_small's: 300k x 100, k = 3001 (uneven) 78 us a call with k_update, 67 with this.  Wider rows take it for clusters
+// of more than UP_LARGE members: 200k x 960, k = 2000 (uneven) 494 us with k_update alone, 265 with both; for every cluster
+// it would be slower there (1M x 960, k = 20,000 1297 against 739 us: eight blocks' set-up for 50 members).  Member
+// groups, lanes and the order of the sums are k_update's; the blocks' parts of the distortion term meet in the first
+// one's shared memory.  The rule depends on the cluster's size and the row width only, so BF16 samples and their FP32
+// widening, and a job alone and in a batch, sum alike.
+template <bool PIPE, typename XT>
+__global__ void __launch_bounds__(UP_WARPS * 32, PIPE ? 6 : 8) k_update_wide(const XT *__restrict__ X, int d, int64_t ld,
+                                                          const int32_t *__restrict__ off,
+                                                          const int32_t *__restrict__ mem, int k, int large, int nb, int chunk,
+                                                          float *__restrict__ C, int32_t *__restrict__ counts,
+                                                          double *__restrict__ contrib,
+                                                          const uint8_t *__restrict__ dirty, DevStatus *st)
+{
+    constexpr int VEC = 4;
+    using V = float4;
     static_assert(!PIPE || std::is_same_v<XT, float>, "the cp.async ring moves FP32 rows");
     constexpr int UNR = 4;                // member rows in flight per group
     constexpr int R = PIPE ? UP_RV : 1;   // rows per group and stage
@@ -199,7 +388,6 @@ __global__ void __launch_bounds__(UP_WARPS * 32, PIPE ? 6 : 8) k_update(const XT
     __shared__ float2 s_sq[UP_WARPS], s_dd[UP_WARPS];
     __shared__ int s_mem[UP_MCHUNK];
     __shared__ float4 s_terms[2][UP_SPLIT];  // of the first block: the blocks' sums of squares and of D_t^2
-    static_assert(!PIPE || VEC == 4, "the pipelined variant moves 16-byte vectors");
     const int lane = lane_id(), w = threadIdx.x >> 5;
     const int nv = d / VEC;  // vectors per row
     int L = 1;
@@ -215,11 +403,9 @@ __global__ void __launch_bounds__(UP_WARPS * 32, PIPE ? 6 : 8) k_update(const XT
     int turn = 0;
     if (nb > 1)
         cluster_barrier();  // every block of the thread-block cluster runs before any stores into the first one's memory
-    // one cluster r, by all threads; those of at most small_max members are k_update_small's
+    // one cluster r, by all threads
     auto cluster = [&](const int r) {
     const int beg = off[r], m = off[r + 1] - beg;
-    if (m <= small_max || (dirty && dirty[r] == 0))
-        return;
     if (counts && threadIdx.x == 0 && rank == 0)
         counts[r] = m;
     if (m == 0) {
@@ -357,32 +543,29 @@ __global__ void __launch_bounds__(UP_WARPS * 32, PIPE ? 6 : 8) k_update(const XT
     turn ^= 1;
     __syncthreads();  // s_sq / s_dd are read above before the next cluster writes them
     };
-    if constexpr (!WALK) {
-        cluster(blockIdx.x / nb);
-    } else {
-        // chunk by chunk, a thread per cluster finding the large ones (looking at the clusters one by one took 0.3 ms for
-        // 200,000 small ones at nb = 4)
-        __shared__ int s_list[UP_WARPS * 32], s_found[UP_WARPS];
-        for (int64_t base = (int64_t)(blockIdx.x / nb) * chunk; base < k; base += (int64_t)(gridDim.x / nb) * chunk) {
-            const int64_t r = base + threadIdx.x;
-            const bool mine =
-                threadIdx.x < chunk && r < k && off[r + 1] - off[r] > small_max && !(dirty && dirty[r] == 0);
-            const unsigned bal = __ballot_sync(FULL_MASK, mine);
-            __syncthreads();  // the previous chunk's list is no longer read
-            if (lane == 0)
-                s_found[w] = __popc(bal);
-            __syncthreads();
-            int before = 0, found = 0;
-            for (int ww = 0; ww < UP_WARPS; ww++) {
-                before += ww < w ? s_found[ww] : 0;
-                found += s_found[ww];
-            }
-            if (mine)
-                s_list[before + __popc(bal & lanemask_lt())] = (int)r;
-            __syncthreads();
-            for (int z = 0; z < found; z++)
-                cluster(s_list[z]);
+    // a thread per cluster finds the large ones, `chunk` of this block's clusters c, c + stride, ... at a time (large ones
+    // often follow one another: 300k x 200 took 195 us with neighbouring clusters on one block)
+    __shared__ int s_list[UP_WARPS * 32], s_found[UP_WARPS];
+    const int64_t stride = gridDim.x / nb;
+    for (int64_t base = blockIdx.x / nb; base < k; base += stride * chunk) {
+        const int64_t r = base + threadIdx.x * stride;
+        const bool mine =
+            threadIdx.x < chunk && r < k && off[r + 1] - off[r] > large && !(dirty && dirty[r] == 0);
+        const unsigned bal = __ballot_sync(FULL_MASK, mine);
+        __syncthreads();  // the previous chunk's list is no longer read
+        if (lane == 0)
+            s_found[w] = __popc(bal);
+        __syncthreads();
+        int before = 0, found = 0;
+        for (int ww = 0; ww < UP_WARPS; ww++) {
+            before += ww < w ? s_found[ww] : 0;
+            found += s_found[ww];
         }
+        if (mine)
+            s_list[before + __popc(bal & lanemask_lt())] = (int)r;
+        __syncthreads();
+        for (int z = 0; z < found; z++)
+            cluster(s_list[z]);
     }
 }
 
@@ -567,7 +750,7 @@ static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     const bool vec4 = x_vec4(X, d, ld);
     const int nv = vec4 ? (int)(d / 4) : (int)d;
     const int L = nv >= 32 ? 32 : (nv >= 16 ? 16 : nv >= 8 ? 8 : nv >= 4 ? 4 : nv >= 2 ? 2 : 1);
-    const int need = (nv + L - 1) / L;  // column blocks of a row
+    const int need = (nv + L - 1) / L;  // vectors per lane to cover a row in one column block
     const int dd = (int)d;
     constexpr bool PIPE = std::is_same_v<XT, float>;  // FP32 rows stream through the cp.async ring
     // clusters of at most small_max members go to the warp-per-cluster kernel where rows are 16-byte vectors of
@@ -594,23 +777,42 @@ static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
             GK_UPS(4);
 #undef GK_UPS
     }
-    // nb blocks per cluster while the clusters are mostly the block kernel's (the hardware then hands clusters
-    // of uneven sizes to SMs as blocks finish); where most clusters are small, a one-wave grid looks for the few large
-    // ones in chunks of up to a cluster per thread instead of launching blocks per cluster that would return at once.  Which block sums a
+    // the block kernel walks the clusters grid-stride on a one-wave grid (at most k blocks)
+    int bg = 0;
+    if ((e = resident_grid(reinterpret_cast<const void *>(vec4 ? (need <= 1 ? (const void *)k_update<4, 1, PIPE, XT>
+                                                                                         : (const void *)k_update<4, 8, PIPE, XT>)
+                                                                 : (need <= 1 ? (const void *)k_update<1, 1, false, XT>
+                                                                             : need <= 2 ? (const void *)k_update<1, 2, false, XT>
+                                                                             : need <= 4 ? (const void *)k_update<1, 4, false, XT>
+                                                                                         : (const void *)k_update<1, 8, false, XT>)),
+                           UP_WARPS * 32, 0, &bg)) != cudaSuccess)
+        return e;
+    // one block per cluster while the clusters are mostly the block kernel's (the hardware then hands clusters
+    // of uneven sizes to SMs as blocks finish); where most clusters are small, a one-wave grid walks the few
+    // large ones instead of launching a block per cluster that would return at once.  Which block sums a
     // cluster changes none of its bits.
     const bool mostly_small = small && n <= (int64_t)k * small_max;
-    const int nb = need < UP_SPLIT ? need : UP_SPLIT;
-    auto launch = [&](auto kernel, auto walker) -> cudaError_t {
-        int bg = 0;
-        cudaError_t le = resident_grid(reinterpret_cast<const void *>(walker), UP_WARPS * 32, 0, &bg);
-        if (le != cudaSuccess)
-            return le;
-        const int wave = bg / nb > 0 ? bg / nb : 1;
-        const bool walk = mostly_small && wave < k;
-        const int each = (k + wave - 1) / wave;
-        const int chunk = walk ? (each < UP_WARPS * 32 ? each : UP_WARPS * 32) : 1;
+    const unsigned grid = (unsigned)(mostly_small ? (k < bg ? k : bg) : k);
+    // rows of several column blocks: k_update_wide for every cluster (need <= 4), or for the large ones (before the
+    // block kernel, whose blocks then fill the rest of the chip)
+    const bool wide = vec4 && need > 1, wide_only = wide && need <= 4;
+    const int large = wide_only ? small_max : wide ? UP_LARGE : 0x7fffffff;
+    if (wide && (wide_only || n > UP_LARGE)) {
+        const int nb = need < UP_SPLIT ? need : UP_SPLIT;
+        auto kernel = k_update_wide<PIPE, XT>;
+        int wg = 0;
+        if ((e = resident_grid(reinterpret_cast<const void *>(kernel), UP_WARPS * 32, 0, &wg)) != cudaSuccess)
+            return e;
+        // thread-block clusters: one per cluster where most are this kernel's, else a wave that looks for them
+        int64_t wave = wg / nb > 0 ? wg / nb : 1;
+        if (!wide_only)
+            wave = std::min(wave, n / (UP_LARGE + 1));  // there are no more of them
+        wave = std::min<int64_t>(wave, k);
+        if (wide_only ? !mostly_small : n / k >= UP_LARGE / 4)
+            wave = k;
+        const int64_t each = (k + wave - 1) / wave;
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(walk ? wave : k) * (unsigned)nb);
+        cfg.gridDim = dim3((unsigned)(wave * nb));
         cfg.blockDim = dim3(UP_WARPS * 32);
         cfg.stream = s;
         cudaLaunchAttribute at[1];
@@ -619,14 +821,32 @@ static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
         at[0].val.clusterDim.y = 1;
         at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
-        cfg.numAttrs = nb > 1 ? 1 : 0;
-        return cudaLaunchKernelEx(&cfg, walk ? walker : kernel, X, dd, ld, offsets, members, (int)k, small_max, nb, chunk, C, counts, contrib,
-                                  dirty, st);
-    };
-    e = vec4 ? launch(k_update<4, PIPE, false, XT>, k_update<4, PIPE, true, XT>)
-             : launch(k_update<1, false, false, XT>, k_update<1, false, true, XT>);
-    if (e != cudaSuccess)
-        return e;
+        cfg.numAttrs = 1;
+        if ((e = cudaLaunchKernelEx(&cfg, kernel, X, dd, ld, offsets, members, (int)k, large, nb,
+                                    (int)std::min<int64_t>(each, UP_WARPS * 32), C, counts, contrib, dirty, st)) !=
+            cudaSuccess)
+            return e;
+    }
+#define GK_UPD(VEC, CPL, P) \
+    k_update<VEC, CPL, P, XT><<<grid, UP_WARPS * 32, 0, s>>>(X, dd, ld, offsets, members, k, small_max, large, C, counts, \
+                                                             contrib, dirty, st)
+    if (wide_only) {
+    } else if (vec4) {
+        if (need <= 1)
+            GK_UPD(4, 1, PIPE);
+        else
+            GK_UPD(4, 8, PIPE);
+    } else {
+        if (need <= 1)
+            GK_UPD(1, 1, false);
+        else if (need <= 2)
+            GK_UPD(1, 2, false);
+        else if (need <= 4)
+            GK_UPD(1, 4, false);
+        else
+            GK_UPD(1, 8, false);
+    }
+#undef GK_UPD
     if (sum_d2) {
         double *part = reinterpret_cast<double *>(static_cast<char *>(scratch) + contrib_bytes(k));
         k_sum_f64<<<SUM_BLOCKS, 32, 0, s>>>(contrib, k, part, ticket, sum_d2);
