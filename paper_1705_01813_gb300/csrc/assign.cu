@@ -243,7 +243,7 @@ __device__ __forceinline__ void each_sample(int64_t first, int64_t step, int64_t
     if (blockIdx.x == 0 && threadIdx.x == 0)
         *trk.ticket = 0u;  // for k_assign_reduce
     if constexpr (!LISTS) {
-        for (int64_t i = first; i < n; i += (int64_t)gridDim.x * (blockDim.x >> 5))  // `step`, not kept in registers
+        for (int64_t i = first; i < n; i += step)
             f(i, std::false_type{});
     } else {
         const int nf = trk.todo_n[0], np = trk.todo_n[1];
@@ -284,9 +284,7 @@ __device__ __forceinline__ void write_winner(int64_t i, const int32_t *__restric
 {
     if (lane_id() != 0)
         return;
-    int own = br;
-    if (trk.dirty_out || br == 0x7fffffff)
-        own = Lin[i];  // read again: kept in a register it cost the wide rows spills
+    const int own = Lin[i];
     bool changed = br != own;
     if (br == 0x7fffffff) {
         br = own, bd = 0.f;
