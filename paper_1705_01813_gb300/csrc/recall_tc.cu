@@ -22,8 +22,9 @@
 // list.  The queries' operand stays in shared memory where it fits (d <= 128)
 // and is staged beside the samples' otherwise.
 //
-// Bounds.  With x', y' the centred rows, u = 2^-9 the BF16 rounding (0 for a
-// row that rounding left unchanged) and G the tensor cores' product,
+// Bounds.  With x', y' the centred rows, u = 2^-8 the BF16 rounding (8
+// significant bits: half a unit in the last place; 0 for a row that rounding
+// left unchanged) and G the tensor cores' product,
 // D = |x'|^2 + |y'|^2 - 2 G is within
 //   E = 1.02 [|x'| |y'| (2 (u_x + u_y + u_x u_y) + 8 (d + 2) 2^-24)
 //             + (2 d + 16) 2^-23 (|x'|^2 + |y'|^2)]
@@ -66,7 +67,7 @@ constexpr int RC_CAP = 2048;               // list entries per query
 constexpr uint32_t RC_WAIT_ITERS = 1u << 20;
 constexpr uint32_t RC_TMEM = 512;          // two buffers x two query tiles x 128 columns
 
-constexpr float RC_U = 1.f / 512.f;
+constexpr float RC_U = 1.f / 256.f;  // BF16 rounding (8 significant bits), relative
 
 struct RcBars {
     uint64_t full[RC_STAGES], empty[RC_STAGES], acc_full[2], acc_empty[2], nrm_full[2], fin;
