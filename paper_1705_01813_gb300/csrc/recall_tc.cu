@@ -35,6 +35,9 @@
 // 1e-25, where the bound's relative terms end), whose list overflows or stays
 // empty goes to the FP32 tile kernel instead.
 //
+// More than RC_BATCH queries are screened in batches that reuse the buffers: a
+// list takes 8 KB, and all samples of a million as queries would need 8.4 GB.
+//
 // What bounds it: instruction issue, in the epilogue (two packed FMAs and a
 // minimum for two pairs) and the loaders' conversion about alike.  1,000
 // queries against 1M x 128 FP32 take 0.71 ms in all; the FP32 tiles took 16.1 ms, bound
@@ -48,6 +51,7 @@
 
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 namespace gkm {
@@ -64,6 +68,7 @@ constexpr int RC_RESIDENT = 2;             // K-blocks up to which the queries s
 constexpr int RC_STAGES = 3, RC_STAGES_A = 2;  // operand stages: samples only, samples and queries
 constexpr int RC_AHEAD = 3;                // steps of raw rows in flight
 constexpr int RC_CAP = 2048;               // list entries per query
+constexpr int RC_BATCH = 38 * RC_Q;        // queries screened at once, at most (four slices each fill the chip): 80 MB of lists
 constexpr uint32_t RC_WAIT_ITERS = 1u << 20;
 constexpr uint32_t RC_TMEM = 512;          // two buffers x two query tiles x 128 columns
 
@@ -554,21 +559,21 @@ __global__ void __launch_bounds__(RC_THREADS, 1) k_rc_screen(const XT *__restric
         tc::tmem_dealloc(taddr, RC_TMEM);
 }
 
-// One block per query: the canonical distances of its list, the smallest key; a query without a usable list goes to
-// `left` (counted in *nleft), for the FP32 tiles.
+// One block per query of a batch that begins at query q0 of the call: the canonical distances of its list, the smallest
+// key; a query without a usable list goes to `left` (by its place in the call, counted in *nleft), for the FP32 tiles.
 template <typename XT>
 __global__ void __launch_bounds__(128) k_rc_exact(const XT *__restrict__ X, int64_t n, int d, int64_t ld, bool vec,
                                                   const int32_t *__restrict__ queries, int m,
                                                   const float2 *__restrict__ info, const int32_t *__restrict__ list,
                                                   const int32_t *__restrict__ cnt, uint64_t *__restrict__ best,
-                                                  int32_t *__restrict__ left, int32_t *__restrict__ nleft)
+                                                  int q0, int32_t *__restrict__ left, int32_t *__restrict__ nleft)
 {
     __shared__ uint64_t s_best[4];
     const int q = blockIdx.x;
     const int c = cnt[q], i = queries[q];
     if (info[q].y < 0.f || c <= 0 || c > RC_CAP) {
         if (threadIdx.x == 0)
-            left[atomicAdd(nleft, 1)] = q;
+            left[atomicAdd(nleft, 1)] = q0 + q;
         return;
     }
     uint64_t k = ~0ull;
@@ -587,29 +592,39 @@ __global__ void __launch_bounds__(128) k_rc_exact(const XT *__restrict__ X, int6
 }
 
 struct RcBufs {
-    int *flags;  // lossy, rounded, nleft; then the list counters
+    int *nleft;  // of the call; then, of the batch: lossy, rounded and the list counters
+    int *flags;
     int32_t *cnt, *left, *list;
     float *centre;
     float2 *info;
     unsigned *bound;
     __nv_bfloat16 *Aq;
-    size_t zero_bytes, bytes;
+    size_t bytes;
 };
 
+// Queries per batch: the call's, shared out evenly over as few batches as hold them.
+int32_t rc_batch(int32_t m)
+{
+    const int32_t nb = (int32_t)(((int64_t)m + RC_BATCH - 1) / RC_BATCH);
+    return (int32_t)((((int64_t)m + nb - 1) / nb + RC_Q - 1) / RC_Q * RC_Q);
+}
+
+// Everything but `left` is of one batch, whatever m.
 RcBufs rc_carve(void *scratch, int64_t d, int32_t m)
 {
     Carver cv{static_cast<char *>(scratch), 0, 0};
-    const int64_t cols = (d + RC_KB - 1) / RC_KB * RC_KB, mp = ((int64_t)m + RC_Q - 1) / RC_Q * RC_Q;
+    const int64_t cols = (d + RC_KB - 1) / RC_KB * RC_KB;
+    const size_t mb = (size_t)std::min(m, RC_BATCH), mp = (mb + RC_Q - 1) / RC_Q * RC_Q;
     RcBufs B{};
+    B.nleft = cv.take<int>(64);
     B.flags = cv.take<int>(64);
-    B.cnt = cv.take<int32_t>((size_t)m);
-    B.zero_bytes = cv.off;
+    B.cnt = cv.take<int32_t>(mb);
     B.left = cv.take<int32_t>((size_t)m);
-    B.list = cv.take<int32_t>((size_t)m * RC_CAP);
+    B.list = cv.take<int32_t>(mb * RC_CAP);
     B.centre = cv.take<float>((size_t)cols);
-    B.info = cv.take<float2>((size_t)m);
-    B.bound = cv.take<unsigned>((size_t)m);
-    B.Aq = cv.take<__nv_bfloat16>((size_t)mp * (size_t)cols);
+    B.info = cv.take<float2>(mb);
+    B.bound = cv.take<unsigned>(mb);
+    B.Aq = cv.take<__nv_bfloat16>(mp * (size_t)cols);
     B.bytes = cv.off;
     return B;
 }
@@ -621,27 +636,31 @@ cudaError_t screen_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_
 {
     const RcBufs B = rc_carve(scratch, d, m);
     const int nkb = (int)((d + RC_KB - 1) / RC_KB), cols = nkb * RC_KB;
-    const int qb = (m + RC_Q - 1) / RC_Q;
     const int64_t tiles = (n + RC_N - 1) / RC_N;
-    int64_t slices = 152 / qb > 1 ? 152 / qb : 1;
-    if (slices > tiles)
-        slices = tiles;
+    const int32_t batch = rc_batch(m);
+    const bool vec = x_vec4(X, d, ld);
     cudaError_t e;
-    if ((e = set_max_smem(reinterpret_cast<const void *>(k_rc_screen<XT>), 227 * 1024)) != cudaSuccess ||
-        (e = cudaMemsetAsync(B.flags, 0, B.zero_bytes, s)) != cudaSuccess)
+    if ((e = set_max_smem(reinterpret_cast<const void *>(k_rc_screen<XT>), 227 * 1024)) != cudaSuccess)
         return e;
-    if (std::is_same_v<XT, float>)  // BF16 samples are not rounded
-        k_rc_lossy<XT><<<(m + 7) / 8, 256, 0, s>>>(X, n, (int)d, ld, queries, m, B.flags);
-    k_rc_centre<XT><<<(cols + 127) / 128, 128, 0, s>>>(X, n, (int)d, ld, queries, m, B.flags, B.centre, cols);
-    k_rc_queries<XT><<<qb * RC_Q / 8, 256, 0, s>>>(X, n, (int)d, ld, queries, m, g_idx, kappa, B.centre, cols,
-                                                   x_vec4(X, d, ld), B.Aq,
-                                                   B.info, B.bound, B.flags + 1);
-    k_rc_screen<XT><<<dim3((unsigned)qb, (unsigned)slices), RC_THREADS, rc_smem(nkb), s>>>(
-        X, n, (int)d, ld, x_vec4(X, d, ld), queries, m, B.Aq, B.info, B.centre, B.flags + 1, nkb, B.bound, B.list, B.cnt, st);
-    k_rc_exact<XT><<<(unsigned)m, 128, 0, s>>>(X, n, (int)d, ld, x_vec4(X, d, ld), queries, m, B.info, B.list, B.cnt, best, B.left,
-                                               B.flags + 2);
+    for (int64_t q0 = 0; q0 < m; q0 += batch) {
+        const int32_t *qs = queries + q0;
+        const int mb = (int)std::min<int64_t>(batch, m - q0), qb = (mb + RC_Q - 1) / RC_Q;
+        const int64_t slices = std::min<int64_t>(std::max(1, 152 / qb), tiles);
+        char *zero = reinterpret_cast<char *>(q0 == 0 ? B.nleft : B.flags);
+        if ((e = cudaMemsetAsync(zero, 0, reinterpret_cast<char *>(B.cnt + mb) - zero, s)) != cudaSuccess)
+            return e;
+        if (std::is_same_v<XT, float>)  // BF16 samples are not rounded
+            k_rc_lossy<XT><<<(mb + 7) / 8, 256, 0, s>>>(X, n, (int)d, ld, qs, mb, B.flags);
+        k_rc_centre<XT><<<(cols + 127) / 128, 128, 0, s>>>(X, n, (int)d, ld, qs, mb, B.flags, B.centre, cols);
+        k_rc_queries<XT><<<qb * RC_Q / 8, 256, 0, s>>>(X, n, (int)d, ld, qs, mb, g_idx, kappa, B.centre, cols, vec, B.Aq,
+                                                       B.info, B.bound, B.flags + 1);
+        k_rc_screen<XT><<<dim3((unsigned)qb, (unsigned)slices), RC_THREADS, rc_smem(nkb), s>>>(
+            X, n, (int)d, ld, vec, qs, mb, B.Aq, B.info, B.centre, B.flags + 1, nkb, B.bound, B.list, B.cnt, st);
+        k_rc_exact<XT><<<(unsigned)mb, 128, 0, s>>>(X, n, (int)d, ld, vec, qs, mb, B.info, B.list, B.cnt, best + q0,
+                                                    (int)q0, B.left, B.nleft);
+    }
     *left = B.left;
-    *nleft = B.flags + 2;
+    *nleft = B.nleft;
     return cudaGetLastError();
 }
 
