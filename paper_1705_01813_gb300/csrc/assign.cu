@@ -706,10 +706,11 @@ __device__ __forceinline__ int dot4(uint32_t a, uint32_t b, int c) { return __dp
 // LPR candidates at once.  With X2 = |x~|^2 and C2 = |c~|^2 of the coded vectors,
 //   D~ = X2 + C2 - 2 s_x s_r dot,
 // the true distance's root is within delta = delta_r + 0.51 s_x sqrt(d) of the coded one's; to
-// E = delta (2 sqrt(D~ + er) + delta) come er = 64 2^-24 (X2 + C2) for the FP32 evaluation of D~ (X2 summed over at most
-// 32 terms a lane and 5 steps) and the rounding gam of the canonical sum.  Pass 2 recomputes every candidate whose lower
-// value does not exceed the smallest upper value, as the BF16 form does, with the same bits.  A sample that is not
-// finite, or with at most Q8_FEW candidates, goes to pass 2 whole.
+// E = delta (2 sqrt(D~ + er) + delta) come er = 64 2^-24 (X2 + C2) + 2^-117 for the FP32 evaluation of D~ (X2 summed over
+// at most 32 terms a lane and 5 steps; below FP32's normal range s_x s_r is off by up to 2^-150, times |dot| < 2^31, and
+// the other products and the canonical sum by less) and the rounding gam of the canonical sum.  Pass 2 recomputes every
+// candidate whose lower value does not exceed the smallest upper value, as the BF16 form does, with the same bits.  A
+// sample that is not finite, or with at most Q8_FEW candidates, goes to pass 2 whole.
 constexpr int Q8_FEW = 3;
 
 template <int LPR, int NW, int NV, typename XT, bool LISTS>
@@ -797,7 +798,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : 4) k
                 const float4 mt = __ldg(meta + qlist[c]);
                 const float n2 = X2 + mt.y;
                 const float dt = fmaf(-2.f * sx * mt.x, (float)dot, n2);
-                const float er = 3.8146973e-6f * n2, dl = mt.z + dx;
+                const float er = fmaf(3.8146973e-6f, n2, 6.0e-36f), dl = mt.z + dx;
                 const float dp = fmaxf(dt, 0.f) + er;
                 const float sq = dl * (2.f * sqrtf(dp) + dl);
                 const float e = 1.01f * (sq + er + gam * (2.f * dp + sq));

@@ -1,0 +1,33 @@
+"""Int8 screening of samples and centroids of small magnitude, where products of the two rows' scales leave FP32's range:
+labels and distances are those of the FP32 rows at every power of two."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d", [32, 64, 128, 256, 512, 1024])
+@pytest.mark.parametrize("exp", [0, -40, -56, -62, -64, -66, -68, -70])
+def test_scaled_rows_keep_their_labels(d, exp):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1705_01813_gb300 import gkm
+    n, k, kappa = 3001, 150, 24
+    g = np.random.default_rng(d)
+    X = g.uniform(-3, 3, (50, d))[g.integers(0, 50, n)] + g.standard_normal((n, d))
+    X = torch.from_numpy(X.astype(np.float32)).cuda() * 2.0 ** exp
+    X[11] = 0.0
+    gi = torch.from_numpy(g.integers(0, n, (n, kappa)).astype(np.int32)).cuda()
+    L = gkm.init_labels(n, k, 1)
+    C = torch.zeros((k, d), device="cuda")
+    gkm.update_step(X, L, k, C)
+    C[:40] = X[:40]
+    C[7], C[9] = C[8], 0.0
+    for x in (X, X.to(torch.bfloat16)):
+        want, best, s, _ = gkm.assign_step(x, gi, C, L, precision=0)
+        got, b, s2, _ = gkm.assign_step(x, gi, C, L, precision=4)
+        assert torch.equal(got, want), int((got != want).sum())
+        assert torch.equal(b.view(torch.int32), best.view(torch.int32))
+        assert float(s) == float(s2)
