@@ -390,13 +390,13 @@ GK_API int gk_kmeans_fit_bf16(const uint16_t *X, int64_t n, int64_t d, int64_t l
  *                  nearest neighbour and its distance (-1 / +inf if none)
  *   hits           device int64[1]: number of hits (overwritten)
  *   ws             gk_workspace_size(GK_OP_RECALL, n, d, m, kappa) bytes
- * Cost: m n d pair terms.  From 10^9 on they are screened on the tensor cores
- * (BF16 operands, a rigorous error bound), batches of up to 9,728 queries at a
- * time, and the few pairs that may be the nearest are recomputed in FP32;
- * fewer, and queries that keep too many, take FP32 tiles of 64 queries x 64
- * samples on the SIMT cores.  The results are the same.  The workspace of a
- * screened call is 12 bytes a query beside about 8.3 KB + 2 d for each of up
- * to 9,728.
+ * Cost: m n d pair terms.  From 10^9 of them on, at d >= 4, they are screened
+ * on the tensor cores (BF16 operands, a rigorous error bound), batches of up to
+ * 9,728 queries at a time, and the few pairs that may be the nearest are
+ * recomputed in FP32; fewer, and queries that keep too many, take FP32 tiles of
+ * 64 queries x 64 samples on the SIMT cores.  The results are the same.  The
+ * workspace of a screened call is 12 bytes a query beside about 8.3 KB + 2 d
+ * for each of up to 9,728.
  */
 GK_API int gk_graph_recall(const float *X, int64_t n, int64_t d, int64_t ld, const int32_t *g_idx, int32_t kappa,
                            const int32_t *queries, int32_t m, int32_t *nn_idx, float *nn_dist, int64_t *hits,

@@ -44,8 +44,17 @@ int recall_slices(int64_t n, int32_t m)
 // 1M x 32, 40 queries 203 against 243, 8,000 x 960, 200 queries 221 against 250; at 6.4e8 (10,000 x 64, 1,000 queries)
 // the tiles take 110 us, the screening's seven launches and 256 queries at a time about as much.
 constexpr double RECALL_SCREEN_MIN = 1.0e9;
+// Nor does it for rows of fewer values: BF16's rounding is then as large as the distances to thousands of samples, and
+// the lists overflow.  FP32 tiles against screening, us, graph rows with the true neighbour: Gaussian 400k x 2, 1,300
+// queries 1,769 / 3,153, 1M x 1, 1,000 queries 3,425 / 5,081, 4M x 3, 300 queries 4,608 / 5,263; 400k x 4, 1,000 queries
+// 1,495 / 435.  (Wider rows whose norm lies in one column lose as well: 400k x 32 2,216 / 3,006, 400k x 128, 500 queries
+// 2,657 / 3,435, 1M x 128 16,154 / 14,802.)
+constexpr int64_t RECALL_SCREEN_MIN_D = 4;
 
-static bool recall_screened(int64_t n, int64_t d, int32_t m) { return (double)n * (double)d * (double)m >= RECALL_SCREEN_MIN; }
+static bool recall_screened(int64_t n, int64_t d, int32_t m)
+{
+    return d >= RECALL_SCREEN_MIN_D && (double)n * (double)d * (double)m >= RECALL_SCREEN_MIN;
+}
 
 static size_t best_bytes(int32_t m) { return ((size_t)m * sizeof(uint64_t) + 255) & ~size_t(255); }
 
