@@ -285,11 +285,11 @@ def launches_per_step(w, precision):
         upd += 1  # the column blocks of large clusters
 
     def asg(k):
-        # (then the reduction): kernel (0, 1; wide rows of large sets take the int8 screening); shadow copy + screening
-        # kernel (2, 4); BF16 copy, tensor-core tiles, SIMT leftovers (3)
-        if precision < 2:
-            return 3 if w.d % 4 == 0 and 288 < w.d <= 1024 and w.n * w.d >= 1 << 22 else 2
-        return 3 if precision in (2, 4) or w.d > 128 else 4
+        # (then the reduction): kernel; shadow copy + screening kernel (2, int8); BF16 copy, tensor-core tiles, SIMT
+        # leftovers (3)
+        if int8_rows(precision, w, k):
+            return 3
+        return 2 if precision in (0, 1, 4) else 3 if precision == 2 or w.d > 128 else 4
     # refine: the run lists, then cluster-sorted copy + Gram + exact recompute + merge (tensor cores) or the two FP32
     # tile widths (runs of max_cluster = 128 members at most)
     ref = 1 + (4 if tc_refine(precision, w.d, w.storage) else 2)
@@ -319,15 +319,26 @@ def tc_refine(precision, d, storage="f32"):
     return precision >= 1 and 64 <= d <= 128
 
 
-def int8_rows(precision, d):
-    """The library's dispatch of the assignment to int8 screening (its rule at the workloads' sizes)."""
-    return precision == 4 or (precision <= 1 and d % 4 == 0 and 288 < d <= 1024)
+def int8_row_bytes(d):
+    """Bytes of a row of the library's int8 copy of the centroids."""
+    return next(b for b in (64, 128, 256, 512, 1024) if d <= b)
 
 
-def kernel_of(tag, precision=1, d=128, storage="f32"):
+def int8_rows(precision, w, k):
+    """The library's dispatch of the assignment to int8 screening at k clusters."""
+    n, d = w.n, w.d
+    if d % 4 or not 32 <= d <= 1024 or precision not in (1, 4):
+        return False
+    if precision == 4:
+        return True
+    return (d > 288 and n * d >= 1 << 22 and k >= 100 and
+            min(w.kappa, k) * (4 * d - int8_row_bytes(d)) >= 12000 + 3000 * k // n + 8000 * (1 << 22) // (n * d))
+
+
+def kernel_of(tag, precision=1, d=128, storage="f32", int8=False):
     if tag == "refine" and tc_refine(precision, d, storage):
         return "k_refine_gram"
-    if tag == "assign" and (precision in (2, 4) or int8_rows(precision, d)):
+    if tag == "assign" and (precision in (2, 4) or int8):
         return "k_assign_rows_scr"
     if tag == "assign" and precision == 3:
         return "k_assign_tc"
@@ -347,8 +358,8 @@ def file_sha(f):
         return hashlib.sha256(fh.read()).hexdigest()[:16]
 
 
-def source_sha(tag, precision=1, d=128, storage="f32"):
-    return file_sha(KERNEL_SOURCE[kernel_of(tag, precision, d, storage)])
+def source_sha(tag, precision=1, d=128, storage="f32", int8=False):
+    return file_sha(KERNEL_SOURCE[kernel_of(tag, precision, d, storage, int8)])
 
 
 def write_traffic(csv_path, workload):
@@ -393,15 +404,15 @@ def write_traffic(csv_path, workload):
     print(json.dumps({k: v["dram_bytes_per_launch"] for k, v in j.items() if not k.startswith("_")}, indent=1))
 
 
-def ncu_traffic(tag, workload, precision=1, d=128, storage="f32"):
+def ncu_traffic(tag, workload, precision=1, d=128, storage="f32", int8=False):
     """DRAM bytes per launch from the committed ncu summary, if it is for the current source."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
         return None
     with open(p) as f:
         j = json.load(f)
-    e = j.get(f"{kernel_of(tag, precision, d, storage)}:{workload}")
-    if not e or e.get("source_sha") != source_sha(tag, precision, d, storage):
+    e = j.get(f"{kernel_of(tag, precision, d, storage, int8)}:{workload}")
+    if not e or e.get("source_sha") != source_sha(tag, precision, d, storage, int8):
         return None
     return e.get("dram_bytes_per_launch")
 
@@ -492,6 +503,7 @@ def run_gpu(args):
     # the plain FP32 path (SIMT pair distances) on the same workload, for comparison
     fp32_ms = None
     lvl = args.precision & 0xff  # the level; bits 8-15 carry the assignment's candidates per group
+    int8 = int8_rows(lvl, w, w.k)
     if lvl != 0 and not args.no_fp32_compare:
         path.precision = 0
         path.step()
@@ -626,17 +638,18 @@ def run_gpu(args):
                       3: "1 plus bf16 tcgen05 screening of assignment candidates with exact fp32 recompute",
                       4: "1 plus int8 (per-row scale) screening of assignment candidates (simt) with exact fp32 "
                          "recompute"}
-                     [lvl] + ("; int8 screening of assignment candidates with exact fp32 recompute (rows of more than "
-                              "288 values)" if lvl <= 1 and int8_rows(lvl, w.d) else ""),
+                     [lvl] + ("; int8 screening of assignment candidates (simt) with exact fp32 recompute"
+                              if lvl == 1 and int8 else ""),
         "assign_group_width": (args.precision >> 8) & 0xff or None,
         "plain_fp32_ms_per_step": fp32_ms,
         "assign_samples_per_s": w.n / statistics.mean(assign_times) if assign_times else None,
         "per_call_ms": {t: round(1e3 * statistics.mean(v), 4) for t, v in per_tag.items()},
         "per_step_share": {t: round(v / sum(totals.values()), 4) for t, v in totals.items()},
-        "roofline": {"kernel": kernel_of(dom, lvl, w.d, w.storage), "bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
+        "roofline": {"kernel": kernel_of(dom, lvl, w.d, w.storage, int8), "bound": "hbm", "achieved": achieved,
+                     "peak": hbm, "unit": "GB/s",
                      "frac": achieved / hbm, "peak_source": peak_src,
                      "algorithmic_bytes_per_launch": int(alg),
-                     "traffic": ncu_traffic(dom, w.name, lvl, w.d, w.storage)},
+                     "traffic": ncu_traffic(dom, w.name, lvl, w.d, w.storage, int8)},
         "gpu_launches": launches_per_step(w, lvl) * args.steps,
         "measured_ceilings": ceilings,
         "precision_tuning": tuning,
@@ -652,15 +665,16 @@ def run_gpu(args):
         "e2e": e2e,
     }
     # roofline of every call type, for context
-    # The assignment gathers one centroid row per candidate: n u d (int8 rows where it screens with them, BF16 rows
-    # at precision 2 and 3, FP32 rows otherwise) bytes per call beyond the algorithmic ones, u the measured mean candidate count of the phase
-    # (graph rounds at k0, fit iterations at k).  They come from L2 while the centroid table fits it and from
-    # HBM otherwise; the probe kernels measure both gather ceilings on this GPU.
+    # The assignment gathers one centroid row per candidate (an int8 row, padded, where it screens with them, a BF16
+    # row at precision 2 and 3, an FP32 row otherwise) beyond the algorithmic bytes of a call, for each of the u
+    # candidates measured in the phase (graph rounds at k0, fit iterations at k).  They come from L2 while the table of
+    # rows fits it and from HBM otherwise; the probe kernels measure both gather ceilings on this GPU.
     if dom == "assign" and u:
-        row_b = 1 if int8_rows(lvl, w.d) else {2: 2, 3: 2}.get(lvl, 4)
+        row = lambda kk: (int8_row_bytes(w.d) if int8_rows(lvl, w, kk) else  # noqa: E731
+                          w.d * {2: 2, 3: 2}.get(lvl, 4))
         per = [(w.k0, u.get("build"), w.tau), (w.k, u.get("fit"), w.iters)]
-        g_l2 = sum(w.n * uu * w.d * row_b * c for kk, uu, c in per if uu and kk * w.d * 4 <= L2_BYTES)
-        g_hbm = sum(w.n * uu * w.d * row_b * c for kk, uu, c in per if uu and kk * w.d * 4 > L2_BYTES)
+        g_l2 = sum(w.n * uu * row(kk) * c for kk, uu, c in per if uu and kk * row(kk) <= L2_BYTES)
+        g_hbm = sum(w.n * uu * row(kk) * c for kk, uu, c in per if uu and kk * row(kk) > L2_BYTES)
         g_l2, g_hbm = g_l2 / (w.tau + w.iters), g_hbm / (w.tau + w.iters)
         gath = {"bytes_per_launch": int(g_l2 + g_hbm), "from_l2": int(g_l2), "from_hbm": int(g_hbm),
                 "achieved_gbs": (g_l2 + g_hbm) / avg / 1e9,

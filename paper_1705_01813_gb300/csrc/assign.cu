@@ -14,6 +14,7 @@
 
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <type_traits>
 
 namespace gkm {
@@ -1137,12 +1138,29 @@ size_t assign_scratch_bytes(int64_t n, int32_t k, int64_t d)
 // Narrowest rows the int8 screening takes (a row of the shadow has at least 64 bytes, in the place of 2 d).
 constexpr int Q8_MIN_D = 32;
 
-// Where precision 0 and 1 take the int8 screening: rows of more than Q8_PAYS_D values, in sample sets large enough for
-// its extra launch.  FP32 rows against screening, us an assignment: 200k x 256 230 / 300 (539 / 607 at kappa = 50),
-// 200k x 300 290 / 280, 100k x 384 259 / 215, 300k x 512 BF16 1317 / 801, 100k x 960 960 / 366; at 300k x 128 401 / 516.
-constexpr int Q8_PAYS_D = 288;
+// 16-byte vectors of a row of the int8 shadow.
+static int q8_units(int64_t d) { return d <= 64 ? 4 : d <= 128 ? 8 : d <= 256 ? 16 : d <= 512 ? 32 : 64; }
 
-static bool assign_q8_pays(int64_t n, int64_t d) { return d > Q8_PAYS_D && n * d >= ((int64_t)1 << 22); }
+// Where precision 1 takes the int8 screening (0 never does): rows of more than Q8_PAYS_D values, where the bytes that a
+// sample's candidates spare, min(kappa, k) times a row's, outweigh what the screening costs a sample (its bounds, the
+// shadow's k / n rows, its launch); not for few clusters, whose samples have few distinct candidates.  FP32 rows against
+// screening, us an assignment in the middle of a fit:
+//   200k x 256, k = 2k, kappa = 20  230 / 300     300k x 128, k = 3k, kappa = 20 401 / 516    (Q8_PAYS_D)
+//   100k x 300, k = 2k, kappa = 20  200 / 183     kappa = 10  151 / 154     k = n, kappa = 20 239 / 255
+//   200k x 512 BF16, k = 4k, kappa = 20  457 / 349     kappa = 10  306 / 280     kappa = 4  206 / 241
+//   100k x 960, k = 2k, kappa = 10  390 / 258     k = n, kappa = 50  2947 / 702     k = 10, kappa = 50  263 / 305
+//   15k x 300, k = 300, kappa = 20  62 / 63       9k x 512, k = 900, kappa = 10  52 / 57     (2^22 values or few more)
+constexpr int Q8_PAYS_D = 288;
+constexpr int Q8_PAYS_K = 100;
+
+static bool assign_q8_pays(int64_t n, int64_t d, int32_t k, int32_t kappa)
+{
+    const int64_t large = (int64_t)1 << 22;
+    if (d <= Q8_PAYS_D || n * d < large || k < Q8_PAYS_K)
+        return false;
+    const int64_t spared = std::min(kappa, k) * (4 * d - 16 * q8_units(d));
+    return spared >= 12000 + 3000 * (int64_t)k / n + 8000 * large / (n * d);
+}
 
 template <typename XT>
 static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *g_idx, int32_t kappa,
@@ -1193,14 +1211,13 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
         else
             k_assign_select<4><<<sgrid, SL_WARPS * 32, 0, s>>>(n, g_idx, kappa, k, labels_in, labels_out, trk, sel_lab);
     }
-    // The int8 screening at precision 4, and at 0 and 1 where it is faster than the FP32 rows (assign_q8_pays): the
-    // results are the same.
+    // The int8 screening at precision 4, and at 1 where it is faster than the FP32 rows (assign_q8_pays): the results
+    // are the same.
     const bool q8 = vec4 && d >= Q8_MIN_D && d4 <= 32 * 8 &&
-                    (precision == 4 || (precision <= 1 && assign_q8_pays(n, d)));
+                    (precision == 4 || (precision == 1 && assign_q8_pays(n, d, k, kappa)));
     if (q8) {
-        const int units = d <= 64 ? 4 : d <= 128 ? 8 : d <= 256 ? 16 : d <= 512 ? 32 : 64;  // 16 bytes each
         const int sgrid = (k + 7) / 8 < 152 * 16 ? (k + 7) / 8 : 152 * 16;
-        k_shadow_i8<<<sgrid, 256, 0, s>>>(C, k, (int)d, units, reinterpret_cast<uint32_t *>(Cb), meta, trk.dirty);
+        k_shadow_i8<<<sgrid, 256, 0, s>>>(C, k, (int)d, q8_units(d), reinterpret_cast<uint32_t *>(Cb), meta, trk.dirty);
         auto launch = [&](auto kernel) -> cudaError_t {
             cudaError_t le = resident_grid(reinterpret_cast<const void *>(kernel), AS_WARPS * 32, 0, &grid);
             if (le == cudaSuccess)
@@ -1293,7 +1310,9 @@ static cudaError_t assign_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     } while (0)
 #define GK_ASG(NV)                                                                                               \
     do {                                                                                                         \
-        if (NV >= 8 || gw == 4)                                                                                  \
+        if constexpr (NV >= 8)                                                                                   \
+            GK_ASGG(NV, 4, 32);                                                                                  \
+        else if (gw == 4)                                                                                        \
             GK_ASGG(NV, 4, 32);                                                                                  \
         else                                                                                                     \
             GK_ASGG(NV, 8, 32);                                                                                  \

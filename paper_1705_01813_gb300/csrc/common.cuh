@@ -361,7 +361,7 @@ struct Track {
     unsigned *ticket;          // set by launch_assign: block counter of the distance sum, cleared by the row kernels
 };
 size_t assign_scratch_bytes(int64_t n, int32_t k, int64_t d);
-// precision 0 and 1: FP32 candidate rows; 2: BF16 screening on the SIMT cores; 3: on the tensor cores over
+// precision 0: FP32 candidate rows; 1: those, or 4 where it is faster; 2: BF16 screening on the SIMT cores; 3: on the tensor cores over
 // 128-sample tiles when members, the grouping of labels_in, is given and d <= 128; 4: int8 screening (per-row
 // scale) on the SIMT cores; all with the exact FP32 recompute (same results).  3 takes FP32 samples only.
 // Bits 8-15 of precision: candidates per group of the row kernels (0: default, 4 or 8).
