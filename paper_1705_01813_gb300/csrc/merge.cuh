@@ -3,6 +3,8 @@
 // refinement kernels.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace gkm {
@@ -27,22 +29,23 @@ __device__ __forceinline__ float key_dist(uint64_t key)
 
 __device__ __forceinline__ int key_id(uint64_t key) { return (int)(uint32_t)key; }
 
-// A graph row's kappa keys held in registers (lane l owns entries l, l + 32,
-// l + 64, l + 96), so that the next row's list can be loaded while the
-// current row is merged.
+// A graph row's kappa keys held in registers (lane l owns entries l, l + 32, ..., NU slots: 32 NU >= kappa), so that the
+// next row's list can be loaded while the current row is merged.
+template <int NU>
 struct RowRegs {
-    int id[4];
-    float dv[4];
+    int id[NU];
+    float dv[NU];
     int thi;  // the kappa-th key, in every lane
     float thd;
 };
 
-__device__ __forceinline__ void load_row(RowRegs &r, const int32_t *__restrict__ gi, const float *__restrict__ gd,
+template <int NU>
+__device__ __forceinline__ void load_row(RowRegs<NU> &r, const int32_t *__restrict__ gi, const float *__restrict__ gd,
                                          int kappa)
 {
     const int lane = lane_id();
 #pragma unroll
-    for (int u = 0; u < 4; u++) {
+    for (int u = 0; u < NU; u++) {
         const int q = lane + 32 * u;
         if (q < kappa) {
             r.id[u] = __ldcg(gi + q);
@@ -51,6 +54,15 @@ __device__ __forceinline__ void load_row(RowRegs &r, const int32_t *__restrict__
     }
     r.thi = __ldcg(gi + kappa - 1);
     r.thd = __ldcg(gd + kappa - 1);
+}
+
+// The kernels that merge are compiled for each number of row slots: f(std::integral_constant<int, NU>) for this kappa.
+template <typename F>
+auto with_row_slots(int32_t kappa, F f)
+{
+    return kappa <= 32   ? f(std::integral_constant<int, 1>{})
+           : kappa <= 64 ? f(std::integral_constant<int, 2>{})
+                         : f(std::integral_constant<int, MAX_KAPPA / 32>{});
 }
 
 // Merging candidates into a graph row, warp-cooperative.  Lane l holds candidates l, l + 32, ... (NC slots) as packed
@@ -69,10 +81,10 @@ __device__ __forceinline__ void load_row(RowRegs &r, const int32_t *__restrict__
 // key is found at its place; otherwise the row ids are looked up among the candidates' ids (ascending, in shared
 // memory).
 //
-// Only the entries that move are written; the result says whether a candidate entered the row.  Instruction issue bounds the merge: ranking, then binary searches for
-// every candidate and row entry, took 1,400 warp instructions a row with 50 candidates and 830 with 15; with these
-// forms the merge of a 1M x 128 graph construction (kappa = 50) takes 0.64 ms a round instead of 0.94, the pairs left
-// out included.
+// Only the entries that move are written; the result says whether a candidate entered the row.  Instruction issue bounds
+// the merge: ranking, then binary searches for every candidate and row entry, took 1,400 warp instructions a row with 50
+// candidates and 830 with 15; with these forms the merge of a 1M x 128 graph construction (kappa = 50) takes 0.64 ms a
+// round instead of 0.94, the pairs left out included.
 constexpr int MERGE_FEW = 4;
 
 // Shared memory of one warp: the row's keys, the candidates' keys, repeat flags.
@@ -83,7 +95,7 @@ struct alignas(16) MergeBuf {
 };
 
 template <int NU, int NC>
-__device__ __forceinline__ bool merge_few(uint64_t (&ck)[NC], bool (&ok)[NC], int kappa, const RowRegs &cur,
+__device__ __forceinline__ bool merge_few(uint64_t (&ck)[NC], bool (&ok)[NC], int kappa, const RowRegs<NU> &cur,
                                           int32_t *__restrict__ gi, float *__restrict__ gd)
 {
     const int lane = lane_id();
@@ -168,7 +180,7 @@ __device__ __forceinline__ int lower_rank(const uint64_t *k, uint64_t key)
 template <int NU, int NC>
 __device__ __forceinline__ bool merge_many(uint64_t (&ck)[NC], bool (&ok)[NC], bool canon, const int *__restrict__ sid,
                                            const unsigned char *__restrict__ smap, int ns, int kappa,
-                                           const RowRegs &cur, int32_t *__restrict__ gi, float *__restrict__ gd,
+                                           const RowRegs<NU> &cur, int32_t *__restrict__ gi, float *__restrict__ gd,
                                            MergeBuf<NC> &mb)
 {
     const int lane = lane_id();
@@ -278,12 +290,12 @@ __device__ __forceinline__ bool merge_many(uint64_t (&ck)[NC], bool (&ok)[NC], b
     return below > 0;
 }
 
-// The form and the number of row slots that the flagged candidates and kappa ask for.
-template <int NC>
-__device__ __forceinline__ bool merge_slots(uint64_t (&ck)[NC], bool (&ok)[NC], bool canon,
-                                            const int *__restrict__ sid, const unsigned char *__restrict__ smap, int ns,
-                                            int kappa, const RowRegs &cur, int32_t *__restrict__ gi,
-                                            float *__restrict__ gd, MergeBuf<NC> &mb)
+// The form that the number of flagged candidates asks for.
+template <int NU, int NC>
+__device__ __forceinline__ bool merge_keys(uint64_t (&ck)[NC], bool (&ok)[NC], bool canon, const int *__restrict__ sid,
+                                           const unsigned char *__restrict__ smap, int ns, int kappa,
+                                           const RowRegs<NU> &cur, int32_t *__restrict__ gi, float *__restrict__ gd,
+                                           MergeBuf<NC> &mb)
 {
     int m = 0;
 #pragma unroll
@@ -292,12 +304,8 @@ __device__ __forceinline__ bool merge_slots(uint64_t (&ck)[NC], bool (&ok)[NC], 
     if (m == 0)
         return false;
     if (m <= MERGE_FEW)
-        return kappa <= 32   ? merge_few<1, NC>(ck, ok, kappa, cur, gi, gd)
-               : kappa <= 64 ? merge_few<2, NC>(ck, ok, kappa, cur, gi, gd)
-                             : merge_few<4, NC>(ck, ok, kappa, cur, gi, gd);
-    return kappa <= 32   ? merge_many<1, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb)
-           : kappa <= 64 ? merge_many<2, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb)
-                         : merge_many<4, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb);
+        return merge_few<NU, NC>(ck, ok, kappa, cur, gi, gd);
+    return merge_many<NU, NC>(ck, ok, canon, sid, smap, ns, kappa, cur, gi, gd, mb);
 }
 
 // Merge a run's pair distances drow[0 .. ncol) (ncol <= 32 NC) to the members cid[] into graph row i of that run.
@@ -305,11 +313,11 @@ __device__ __forceinline__ bool merge_slots(uint64_t (&ck)[NC], bool (&ok)[NC], 
 // that shared a run then has been offered to this row already, when it entered the row or lost to its kappa-th key,
 // which has only decreased since, so it is left out here (its distance need not have been computed).  canon, sid, smap: see
 // merge_many (the members in ascending id and the columns they have).
-template <int NC>
+template <int NU, int NC>
 __device__ __forceinline__ bool merge_row(int i, int irun, bool canon, const int *__restrict__ cid,
                                           const int *__restrict__ crun,
                                           const int *__restrict__ sid, const unsigned char *__restrict__ smap,
-                                          const float *__restrict__ drow, int ncol, int kappa, const RowRegs &cur,
+                                          const float *__restrict__ drow, int ncol, int kappa, const RowRegs<NU> &cur,
                                           int32_t *__restrict__ gi, float *__restrict__ gd, MergeBuf<NC> &mb)
 {
     const int lane = lane_id();
@@ -329,7 +337,7 @@ __device__ __forceinline__ bool merge_row(int i, int irun, bool canon, const int
             }
         }
     }
-    return merge_slots<NC>(ck, ok, canon, sid, smap, ncol, kappa, cur, gi, gd, mb);
+    return merge_keys<NU, NC>(ck, ok, canon, sid, smap, ncol, kappa, cur, gi, gd, mb);
 }
 
 }  // namespace gkm

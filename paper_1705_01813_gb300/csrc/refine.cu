@@ -11,9 +11,9 @@
 // only decreases, so it can neither be missing nor enter again (after the first
 // round 1-67% of the pairs are new on the workloads' data; the refinements of a
 // graph construction at 2M x 512 BF16 go from 62.1 to 16.4 ms, at 200k x 960
-// FP32 from 16.3 to 12.9, at 1.3M x 64 in 16 jobs from 20.0 to 13.0).  Blocks walk the
-// lists grid-stride: a 64-wide tile for runs of at most 64 members (the common
-// case, several blocks per SM) and a 128-wide tile for longer ones.
+// FP32 from 16.3 to 12.9, at 1.3M x 64 in 16 jobs from 20.0 to 13.0).  A block
+// takes a run: in a 64-wide tile where it has at most 64 members (the common
+// case, several blocks per SM), in 128-wide tiles where it is longer.
 // A run is covered by T x T tiles (rows x columns of the run); for each tile
 // the block stages 32 coordinates of the row and column samples at a time in
 // shared memory (the row samples twice over, as broadcast pairs) and every
@@ -185,23 +185,23 @@ __device__ __forceinline__ void load_members(const int32_t *__restrict__ S, int 
     sync();
 }
 
-// Listed runs blockIdx.x, + gridDim.x, ... (LONG: the list from the back of the array), T-wide tiles.
-// STEP: no previous refinement and a graph of any caller's (prev NULL, canon unset), compiled apart: what only the
-// other calls need costs this form registers it spilled (1M x 128, k = 20,000 2336 us a call with one kernel for both,
-// 2269 with two).
-template <int T, typename XT, bool VEC, bool STEP>
+// Listed run blockIdx.x (longs: of the list from the back of the array) in T-wide tiles; the 64-wide instance gets runs of
+// one tile only.  Registers bound it (the tile's accumulators, two rows' keys): compiled for the number of row slots
+// NU, with the merge in one place and a run per block, it spills 28 bytes a thread (T = 64), 144 (T = 128) or none (T =
+// 128, 16-byte loads).  With a choice of three NU inside and the merge inlined for runs of one tile and of several it
+// spilled 208, 416 and 188: a refinement call of 1M x 960, k = 10,000 11.05 ms, now 9.36; 500k x 768 BF16, k = 5,000 4.56
+// and 3.92; 1M x 128 at level 0 2.18 and 1.65 (kappa = 40; repeated calls 9.83 and 8.16, 3.94 and 3.30, 1.69 and 1.23).
+template <int T, int NU, typename XT, bool VEC>
 __global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT *__restrict__ X, int64_t n, int d,
                                                                         int64_t ld, const int32_t *__restrict__ mem,
                                                                         const int2 *__restrict__ runs,
                                                                         int64_t runs_cap,
                                                                         const RunCounts *__restrict__ cnt, bool longs,
-                                                                        const int32_t *__restrict__ prev_in, bool canon_in,
+                                                                        const int32_t *__restrict__ prev, bool canon,
                                                                         uint8_t *__restrict__ row_changed, int kappa,
                                                                         int32_t *__restrict__ g_idx,
                                                                         float *__restrict__ g_dist, DevStatus *st)
 {
-    const int32_t *__restrict__ prev = STEP ? nullptr : prev_in;
-    const bool canon = STEP ? false : canon_in;
     using TL = RefineTile<T>;
     constexpr int DS = TL::DS, NC = T / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -216,54 +216,20 @@ __global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT
     unsigned char *smap = reinterpret_cast<unsigned char *>(reinterpret_cast<MergeBuf<NC> *>(wcnt + RF_WARPS) + RF_WARPS);
     unsigned short *list = reinterpret_cast<unsigned short *>(smap + T);
     auto sync = [] { __syncthreads(); };
-    const int nrun = longs ? cnt->b : cnt->a;
-    for (int run = blockIdx.x; run < nrun; run += gridDim.x) {
-        const int2 rec = longs ? runs[runs_cap - 1 - run] : runs[run];
-        const int first = rec.x, sz = rec.y;
-        const int32_t *S = mem + first;
-        // the merges of the rows of one tile
-        auto merge_rows = [&](int nr, int ncl, const int *ci, const int *cp, const int *si, const unsigned char *sm) {
-            RowRegs cur, nxt;
-            if (w < nr && rid[w] >= 0)
-                load_row(cur, g_idx + (int64_t)rid[w] * kappa, g_dist + (int64_t)rid[w] * kappa, kappa);
-            for (int row = w; row < nr; row += RF_WARPS) {
-                const int i = rid[row];
-                const int rn = row + RF_WARPS;
-                if (rn < nr && rid[rn] >= 0)  // next row's list in flight during this merge
-                    load_row(nxt, g_idx + (int64_t)rid[rn] * kappa, g_dist + (int64_t)rid[rn] * kappa, kappa);
-                if (i >= 0 && merge_row<NC>(i, STEP ? -1 : rpr[row], canon, ci, cp, si, sm, dt + row * DS, ncl, kappa, cur,
-                                            g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mb) &&
-                    row_changed && lane_id() == 0)
-                    row_changed[i] = 1;
-                cur = nxt;
-            }
-        };
-        __syncthreads();  // the previous run's merges are done
-        if (sz <= T) {
-            load_members<T>(S, sz, n, prev, rid, rpr, sid, smap, spr, tid, first, st, sync);
-            // the arithmetic goes to the block's warps rot, rot + 1, ... (rot = blockIdx.x % 4): each warp of an SM
-            // issues on scheduler (its index % 4), so blocks that share an SM spread their few busy warps over all
-            // four schedulers instead of all starting at scheduler 0
-            const int t = (tid - (int)(blockIdx.x & 3) * 32) & (RF_THREADS - 1);
-            int nlive, code;
-            if (prev) {
-                nlive = live_blocks<T, RF_THREADS>(sz, rpr, list, wcnt, tid, sync);
-                code = t < nlive ? list[t] : 0;
+    if ((int)blockIdx.x >= (longs ? cnt->b : cnt->a))
+        return;
+    const int2 rec = longs ? runs[runs_cap - 1 - blockIdx.x] : runs[blockIdx.x];
+    const int first = rec.x, sz = rec.y;
+    const int32_t *S = mem + first;
+    const bool one = T == 64 || sz <= T;  // one tile, whose members are sorted by their previous runs
+    for (int rb = 0; rb < sz; rb += T) {
+        const int nr = min(T, sz - rb);
+        for (int cb = 0; cb < sz; cb += T) {
+            const int ncl = min(T, sz - cb);
+            __syncthreads();  // the previous tile's merges are done
+            if (one) {
+                load_members<T>(S, sz, n, prev, rid, rpr, sid, smap, spr, tid, first, st, sync);
             } else {
-                const int nb = (sz + TL::Q - 1) / TL::Q;
-                nlive = nb * (nb + 1) / 2;
-                code = t < nlive ? triangle_block(nb, t) : 0;
-            }
-            tile_distances<T, true, VEC>(X, d, ld, rid, rid, code >> 8, code & 255, t < nlive, xr, dt);
-            __syncthreads();
-            merge_rows(sz, sz, rid, rpr, sid, prev ? smap : nullptr);
-            continue;
-        }
-        for (int rb = 0; rb < sz; rb += T) {
-            const int nr = min(T, sz - rb);
-            for (int cb = 0; cb < sz; cb += T) {
-                const int ncl = min(T, sz - cb);
-                __syncthreads();
                 for (int q = tid; q < T; q += RF_THREADS) {
                     int a = q < nr ? S[rb + q] : -1;
                     int b = q < ncl ? S[cb + q] : -1;
@@ -278,9 +244,41 @@ __global__ void __launch_bounds__(RF_THREADS, T == 64 ? 3 : 2) k_refine(const XT
                     cpr[q] = prev && b >= 0 ? prev[b] : -1;
                 }
                 __syncthreads();
+            }
+            if (rb == cb) {
+                // the arithmetic goes to the block's warps rot, rot + 1, ... (rot = blockIdx.x % 4): each warp of an SM
+                // issues on scheduler (its index % 4), so blocks that share an SM spread their few busy warps over all
+                // four schedulers instead of all starting at scheduler 0
+                const int t = (tid - (int)(blockIdx.x & 3) * 32) & (RF_THREADS - 1);
+                int nlive, code;
+                if (prev && one) {
+                    nlive = live_blocks<T, RF_THREADS>(sz, rpr, list, wcnt, tid, sync);
+                    code = t < nlive ? list[t] : 0;
+                } else {
+                    const int nb = (nr + TL::Q - 1) / TL::Q;
+                    nlive = nb * (nb + 1) / 2;
+                    code = t < nlive ? triangle_block(nb, t) : 0;
+                }
+                tile_distances<T, true, VEC>(X, d, ld, rid, rid, code >> 8, code & 255, t < nlive, xr, dt);
+            } else {
                 tile_distances<T, false, VEC>(X, d, ld, rid, cid, tid >> 4, tid & 15, TL::Q * (tid >> 4) < nr, xr, dt);
-                __syncthreads();
-                merge_rows(nr, ncl, cid, cpr, cid, nullptr);
+            }
+            __syncthreads();
+            const int *ci = one ? rid : cid, *cp = one ? rpr : cpr, *si = one ? sid : cid;
+            const unsigned char *sm = one && prev ? smap : nullptr;
+            RowRegs<NU> cur, nxt;
+            if (w < nr && rid[w] >= 0)
+                load_row(cur, g_idx + (int64_t)rid[w] * kappa, g_dist + (int64_t)rid[w] * kappa, kappa);
+            for (int row = w; row < nr; row += RF_WARPS) {
+                const int i = rid[row];
+                const int rn = row + RF_WARPS;
+                if (rn < nr && rid[rn] >= 0)  // next row's list in flight during this merge
+                    load_row(nxt, g_idx + (int64_t)rid[rn] * kappa, g_dist + (int64_t)rid[rn] * kappa, kappa);
+                if (i >= 0 && merge_row<NU, NC>(i, rpr[row], canon, ci, cp, si, sm, dt + row * DS, ncl, kappa, cur,
+                                                g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mb) &&
+                    row_changed && lane_id() == 0)
+                    row_changed[i] = 1;
+                cur = nxt;
             }
         }
     }
@@ -309,7 +307,7 @@ __host__ __device__ constexpr size_t refine_ws_smem_bytes()
            sizeof(int) * 8 + sizeof(MergeBuf<2>) * WS_NM + sizeof(unsigned short) * ((TL::NBLK + 3) & ~3);
 }
 
-template <typename XT, bool VEC>
+template <int NU, typename XT, bool VEC>
 __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restrict__ X, int64_t n, int d, int64_t ld,
                                                              const int32_t *__restrict__ mem,
                                                              const int2 *__restrict__ runs,
@@ -390,7 +388,7 @@ __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restric
             const int *sid = sids + (j & 1) * T;
             const unsigned char *smap = prev ? smaps + (j & 1) * T : nullptr;
             bar_sync(WS_BAR_FULL, WS_THREADS);  // run j's ids and distances
-            RowRegs cur, nxt;
+            RowRegs<NU> cur, nxt;
             if (mw < sz && rid[mw] >= 0)
                 load_row(cur, g_idx + (int64_t)rid[mw] * kappa, g_dist + (int64_t)rid[mw] * kappa, kappa);
             for (int row = mw; row < sz; row += WS_NM) {
@@ -398,7 +396,7 @@ __global__ void __launch_bounds__(WS_THREADS, 3) k_refine_ws(const XT *__restric
                 const int rn = row + WS_NM;
                 if (rn < sz && rid[rn] >= 0)  // next row's list in flight during this merge
                     load_row(nxt, g_idx + (int64_t)rid[rn] * kappa, g_dist + (int64_t)rid[rn] * kappa, kappa);
-                if (i >= 0 && merge_row<T / 32>(i, rpr[row], canon, rid, rpr, sid, smap, dt + row * DS, sz, kappa, cur,
+                if (i >= 0 && merge_row<NU, T / 32>(i, rpr[row], canon, rid, rpr, sid, smap, dt + row * DS, sz, kappa, cur,
                                                 g_idx + (int64_t)i * kappa, g_dist + (int64_t)i * kappa, mbufs[mw]) &&
                     row_changed && lane == 0)
                     row_changed[i] = 1;
@@ -452,11 +450,10 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
     const int64_t bound = (int64_t)k + n / max_cluster + 1;
     auto blocks = [&](int resident) { return (unsigned)(bound < resident ? bound : resident); };
     // a block per run, handed out as blocks finish (a wave of blocks walking the list was 4% slower)
-    const bool step = !prev_in && !canon;
     // runs of more than `split` members (FP32 tiles of 128; longer runs in several tiles)
     if (max_cluster > split) {
         constexpr size_t shm = refine_smem_bytes<128>();
-        auto kernel = step ? k_refine<128, XT, VEC, true> : k_refine<128, XT, VEC, false>;
+        auto kernel = with_row_slots(kappa, [](auto nu) { return k_refine<128, decltype(nu)::value, XT, VEC>; });
         const void *f = reinterpret_cast<const void *>(kernel);
         if ((e = set_max_smem(f, (int)shm)) != cudaSuccess)
             return e;
@@ -477,14 +474,15 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
     if constexpr (VEC) {
         int grid = 0;
         constexpr size_t shm = refine_ws_smem_bytes();
-        const void *f = reinterpret_cast<const void *>(k_refine_ws<XT, VEC>);
+        auto kernel = with_row_slots(kappa, [](auto nu) { return k_refine_ws<decltype(nu)::value, XT, VEC>; });
+        const void *f = reinterpret_cast<const void *>(kernel);
         if ((e = set_max_smem(f, (int)shm)) != cudaSuccess || (e = resident_grid(f, WS_THREADS, shm, &grid)) != cudaSuccess)
             return e;
-        k_refine_ws<XT, VEC><<<blocks(grid), WS_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, cnt, prev_in, canon, row_changed, kappa,
-                                                                   g_idx, g_dist, st);
+        kernel<<<blocks(grid), WS_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, cnt, prev_in, canon, row_changed,
+                                                     kappa, g_idx, g_dist, st);
     } else {
         constexpr size_t shm = refine_smem_bytes<64>();
-        auto kernel = step ? k_refine<64, XT, VEC, true> : k_refine<64, XT, VEC, false>;
+        auto kernel = with_row_slots(kappa, [](auto nu) { return k_refine<64, decltype(nu)::value, XT, VEC>; });
         const void *f = reinterpret_cast<const void *>(kernel);
         if ((e = set_max_smem(f, (int)shm)) != cudaSuccess)
             return e;
@@ -502,9 +500,10 @@ static cudaError_t refine_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
                             float *g_dist, void *scratch, DevStatus *st, cudaStream_t s, int precision,
                             const int32_t *prev_in, int32_t *prev_out, bool canon, uint8_t *row_changed)
 {
-    if (std::is_same_v<XT, __nv_bfloat16> && tile_vec16(X, (int)d, ld))
-        return refine_tv<XT, true>(X, n, d, ld, offsets, members, k, kappa, max_cluster, g_idx, g_dist, scratch, st, s,
-                                   precision, prev_in, prev_out, canon, row_changed);
+    if constexpr (std::is_same_v<XT, __nv_bfloat16>)
+        if (tile_vec16(X, (int)d, ld))
+            return refine_tv<XT, true>(X, n, d, ld, offsets, members, k, kappa, max_cluster, g_idx, g_dist, scratch, st,
+                                       s, precision, prev_in, prev_out, canon, row_changed);
     return refine_tv<XT, false>(X, n, d, ld, offsets, members, k, kappa, max_cluster, g_idx, g_dist, scratch, st, s,
                                 precision, prev_in, prev_out, canon, row_changed);
 }

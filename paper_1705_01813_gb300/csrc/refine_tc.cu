@@ -480,6 +480,7 @@ __global__ void __launch_bounds__(EX_THREADS) k_refine_exact(const XT *__restric
 // merge of the FP32 path.  Candidate ids arrive in ascending order.
 constexpr int MG_WARPS = 8;
 
+template <int NU>
 __global__ void __launch_bounds__(MG_WARPS * 32) k_refine_merge(int64_t n, int kappa, bool canon,
                                                                 uint8_t *__restrict__ row_changed,
                                                                 const int32_t *__restrict__ cand_id,
@@ -494,7 +495,7 @@ __global__ void __launch_bounds__(MG_WARPS * 32) k_refine_merge(int64_t n, int k
     const int w = threadIdx.x >> 5, lane = lane_id();
     int *cid = s_cid[w];
     // all lanes take part: nc slots of candidates
-    auto merge = [&](auto slots, int64_t i, int cnt, const RowRegs &cur) {
+    auto merge = [&](auto slots, int64_t i, int cnt, const RowRegs<NU> &cur) {
         constexpr int S = decltype(slots)::value;
         uint64_t ck[S];
         bool ok[S];
@@ -511,7 +512,7 @@ __global__ void __launch_bounds__(MG_WARPS * 32) k_refine_merge(int64_t n, int k
             ok[v] = ck[v] < th;  // a recomputed pair may miss the row after all (~0 for no candidate)
         }
         __syncwarp();
-        if (merge_slots<S>(ck, ok, canon, cid, nullptr, cnt, kappa, cur, g_idx + i * kappa, g_dist + i * kappa,
+        if (merge_keys<NU, S>(ck, ok, canon, cid, nullptr, cnt, kappa, cur, g_idx + i * kappa, g_dist + i * kappa,
                            reinterpret_cast<MergeBuf<S> &>(mbuf[w])) &&
             row_changed && lane == 0)
             row_changed[i] = 1;
@@ -521,7 +522,7 @@ __global__ void __launch_bounds__(MG_WARPS * 32) k_refine_merge(int64_t n, int k
         const int cnt = cand_n[i];
         if (cnt == 0)
             continue;
-        RowRegs cur;
+        RowRegs<NU> cur;
         load_row(cur, g_idx + i * kappa, g_dist + i * kappa, kappa);
         if (cnt <= 64)
             merge(std::integral_constant<int, 2>{}, i, cnt, cur);
@@ -626,7 +627,9 @@ static cudaError_t refine_tc_t(const XT *X, int64_t n, int64_t d, int64_t ld, co
     int64_t mblocks = (n + MG_WARPS - 1) / MG_WARPS;
     if (mblocks > 152 * 64)
         mblocks = 152 * 64;
-    k_refine_merge<<<(unsigned)mblocks, MG_WARPS * 32, 0, s>>>(n, kappa, canon, row_changed, cand_id, cand_d, cand_n, g_idx, g_dist);
+    auto merge = with_row_slots(kappa, [](auto nu) { return k_refine_merge<decltype(nu)::value>; });
+    merge<<<(unsigned)mblocks, MG_WARPS * 32, 0, s>>>(n, kappa, canon, row_changed, cand_id, cand_d, cand_n, g_idx,
+                                                      g_dist);
     return cudaGetLastError();
 }
 
