@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(RF_THREADS) k_nn_tiles(const XT *__restrict__ 
                                                         const int32_t *__restrict__ queries, int m, int slices,
                                                         const int32_t *__restrict__ left,
                                                         const int32_t *__restrict__ nleft,
-                                                        uint64_t *__restrict__ bestq, DevStatus *st)
+                                                        uint64_t *__restrict__ bestq,
+                                                        unsigned long long *__restrict__ hits, DevStatus *st)
 {
     using TL = RefineTile<NN_T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -79,6 +80,8 @@ __global__ void __launch_bounds__(RF_THREADS) k_nn_tiles(const XT *__restrict__ 
     int *cid = rid + NN_T;
     uint64_t *best = reinterpret_cast<uint64_t *>(cid + NN_T);
     const int tid = threadIdx.x, w = tid >> 5, lane = lane_id();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0)
+        *hits = 0ull;  // k_nn_finish counts; a clear of its own was a launch more (5,000 x 24, 100 queries 34 us, 32 so)
     // left (may be NULL): the queries to take, *nleft of them, instead of all m
     const int q0 = blockIdx.x * NN_T, nr = min(NN_T, (left ? *nleft : m) - q0);
     if (nr <= 0)
@@ -153,9 +156,8 @@ static cudaError_t recall_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     cudaError_t e = set_max_smem(reinterpret_cast<const void *>(k_nn_tiles<XT>), (int)NN_SMEM);
     if (e != cudaSuccess)
         return e;
-    if ((e = cudaMemsetAsync(hits, 0, sizeof(int64_t), s)) != cudaSuccess)
-        return e;
     const int slices = recall_slices(n, m);
+    auto *count = reinterpret_cast<unsigned long long *>(hits);
     uint64_t *best = static_cast<uint64_t *>(scratch);
     if ((e = cudaMemsetAsync(best, 0xff, sizeof(uint64_t) * (size_t)m, s)) != cudaSuccess)
         return e;
@@ -165,9 +167,8 @@ static cudaError_t recall_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
                                   static_cast<char *>(scratch) + best_bytes(m), &left, &nleft, st, s)) != cudaSuccess)
         return e;
     const dim3 grid((unsigned)nn_qblocks(m), (unsigned)slices);
-    k_nn_tiles<XT><<<grid, RF_THREADS, NN_SMEM, s>>>(X, n, d, ld, queries, m, slices, left, nleft, best, st);
-    k_nn_finish<<<(m + 255) / 256, 256, 0, s>>>(best, m, queries, n, g_idx, kappa, nn_idx, nn_dist,
-                                                reinterpret_cast<unsigned long long *>(hits));
+    k_nn_tiles<XT><<<grid, RF_THREADS, NN_SMEM, s>>>(X, n, d, ld, queries, m, slices, left, nleft, best, count, st);
+    k_nn_finish<<<(m + 255) / 256, 256, 0, s>>>(best, m, queries, n, g_idx, kappa, nn_idx, nn_dist, count);
     return cudaGetLastError();
 }
 
