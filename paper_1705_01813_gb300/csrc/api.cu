@@ -893,8 +893,8 @@ static int batch_fit_impl(const void *X, bool bf16, int64_t d, int64_t ld, int32
             GK_CUDA(launch_update(X, bf16, N, d, ld, L.grp.offsets, L.grp.members, bd.K0, L.cent, L.grp.counts,
                                   nullptr, L.upd_scratch, L.st, s, trk.dirty_out));
             GK_CUDA(launch_refine(X, bf16, N, d, ld, L.grp.offsets, L.grp.members, bd.K0, p->kappa, p->max_cluster,
-                                  g_idx, g_dist, L.ref_scratch, L.st, s, p->precision & 0xff, t > 0 ? L.prev[(t + 1) & 1] : nullptr,
-                                  L.prev[t & 1], true, trk.row_changed));
+                                  g_idx, g_dist, L.ref_scratch, L.st, s, p->precision & 0xff,
+                                  t > 0 ? L.prev[(t + 1) & 1] : nullptr, L.prev[t & 1], true, trk.row_changed));
             int32_t *tmp = cur;
             cur = nxt;
             nxt = tmp;

@@ -144,14 +144,14 @@ __device__ __forceinline__ int collect_labels_plain(int64_t i, int own, const in
 // clusters can win now.  The result, and every bit of best[], is that of the whole evaluation.
 //
 // k_assign_select sorts the samples by what they need: none of a known sample's neighbours is in a changed cluster:
-// its label is written and it is done; otherwise it goes to the back list (candidates of changed clusters only), and
-// a sample whose own centroid or graph row changed goes to the front list (all candidates).  The assignment kernels
-// then walk the lists.  Doing the test inside them cost registers that the evaluation needs: 30 -> 32 ms for the
-// 1M x 128 graph construction, where almost no sample is done early (this kernel: 13 us of 1 ms there).  The lists' order varies from call to call and
-// decides nothing but which warp takes a sample.  A neighbour costs one byte gather, of the mark that k_assign_reduce
-// left for its cluster (its label and then the cluster's byte, 0.52 ms at 2M x 40: the L1's one lookup a cycle).
-// Against evaluating everything: a fit of 2M x 512 BF16 (k = 200,000)
-// takes 1.0 ms an assignment instead of 9.0 once its labels have settled.
+// its label is written and it is done; otherwise it goes to the back list (candidates of changed clusters only), and a
+// sample whose own centroid or graph row changed goes to the front list (all candidates).  The assignment kernels then
+// walk the lists.  Doing the test inside them cost registers that the evaluation needs: 30 -> 32 ms for the 1M x 128
+// graph construction, where almost no sample is done early (this kernel: 13 us of 1 ms there).  The lists' order
+// varies from call to call and decides nothing but which warp takes a sample.  A neighbour costs one byte gather, of
+// the mark that k_assign_reduce left for its cluster (its label and then the cluster's byte, 0.52 ms at 2M x 40: the
+// L1's one lookup a cycle). Against evaluating everything: a fit of 2M x 512 BF16 (k = 200,000) takes 1.0 ms an
+// assignment instead of 9.0 once its labels have settled.
 constexpr int SL_WARPS = 8;
 
 template <int S>
@@ -411,13 +411,10 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign(const XT *__restrict__
 // its first entry, whose second evaluation
 // cannot change the (distance, label) minimum.
 template <int NV, typename XT, int GS, bool LISTS, int LPR = 32>
-__global__ void __launch_bounds__(AS_WARPS * 32, NV == 1 ? AS_ROWS_PER_SM : NV == 2 ? 5 : 4) k_assign_rows(const XT *__restrict__ X, int64_t n, int d,
-                                                               int64_t ld, const int32_t *__restrict__ G, int kappa,
-                                                               const float *__restrict__ C, int k,
-                                                               const int32_t *__restrict__ Lin,
-                                                               int32_t *__restrict__ Lout,
-                                                               float *__restrict__ best_out, DevStatus *st,
-                                                               const Track trk, const int32_t *__restrict__ todo)
+__global__ void __launch_bounds__(AS_WARPS * 32, NV == 1 ? AS_ROWS_PER_SM : NV == 2 ? 5 : 4) k_assign_rows(
+    const XT *__restrict__ X, int64_t n, int d, int64_t ld, const int32_t *__restrict__ G, int kappa,
+    const float *__restrict__ C, int k, const int32_t *__restrict__ Lin, int32_t *__restrict__ Lout,
+    float *__restrict__ best_out, DevStatus *st, const Track trk, const int32_t *__restrict__ todo)
 {
     __shared__ __align__(16) int s_q[AS_WARPS][AS_QROW + (LPR < 32 ? GS * 32 / LPR : 0)];
     __shared__ __align__(16) int s_h[AS_WARPS][AS_HASH];
@@ -508,8 +505,8 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV == 1 ? AS_ROWS_PER_SM : NV =
 template <int NV, typename XT, int GS, bool LISTS>
 __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV == 4 ? 4 : 3)) k_assign_rows_scr(
     const XT *__restrict__ X, int64_t n, int d, int64_t ld, const int32_t *__restrict__ G, int kappa,
-    const float *__restrict__ C, const void *__restrict__ Cs, const float *__restrict__ delta, int k, const int32_t *__restrict__ Lin, int32_t *__restrict__ Lout,
-    float *__restrict__ best_out, DevStatus *st, const Track trk, const int32_t *__restrict__ todo)
+    const float *__restrict__ C, const void *__restrict__ Cs, const float *__restrict__ delta, int k,
+    const int32_t *__restrict__ Lin, int32_t *__restrict__ Lout, float *__restrict__ best_out, DevStatus *st, const Track trk, const int32_t *__restrict__ todo)
 {
     __shared__ __align__(16) int s_q[AS_WARPS][AS_QROW];
     __shared__ __align__(16) int s_h[AS_WARPS][AS_HASH];
@@ -899,10 +896,11 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign_rows_bf(const float *_
                                                                   const int32_t *__restrict__ Lin,
                                                                   int32_t *__restrict__ Lout,
                                                                   float *__restrict__ best_out,
-                                                                  const int32_t *__restrict__ tmem_members, const int32_t *__restrict__ tile_flag,
-                                                               const int32_t *__restrict__ sel_lab,
-                                                               const int32_t *__restrict__ sel_n, DevStatus *st,
-                                                               unsigned *__restrict__ ticket)
+                                                                  const int32_t *__restrict__ tmem_members,
+                                                                  const int32_t *__restrict__ tile_flag,
+                                                                  const int32_t *__restrict__ sel_lab,
+                                                                  const int32_t *__restrict__ sel_n, DevStatus *st,
+                                                                  unsigned *__restrict__ ticket)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0)
         *ticket = 0u;  // for k_assign_reduce

@@ -384,8 +384,8 @@ __global__ void __launch_bounds__(BE_THREADS, 1)
                 const float den = own ? nf - 1.f : nf + 1.f;
                 float g = (own ? xx - 2.f * dot + sn : 2.f * dot + xx - sn) / den;
                 float e = ((float)(PL + 16) * 0x1p-23f) * (2.f * pr + xx + sn) / den;
-                const bool sure = rs >= 0x1p-40f && rs <= 0x1p60f && rx >= 0x1p-40f && rx <= 0x1p60f && nr >= (own ? 2 : 1) &&
-                                  isfinite(g) && isfinite(e);
+                const bool sure = rs >= 0x1p-40f && rs <= 0x1p60f && rx >= 0x1p-40f && rx <= 0x1p60f &&
+                                  nr >= (own ? 2 : 1) && isfinite(g) && isfinite(e);
                 tg[me] = sure ? g : 0.f;
                 te[me] = sure ? e : __int_as_float(0x7f800000);
                 tm[me] = 2.f * (sn + pr + xx);  // no smaller than the terms of the FP64 gain, which round to 2^-44 of it

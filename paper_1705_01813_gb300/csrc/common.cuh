@@ -197,7 +197,8 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
 
 __device__ __forceinline__ void cp_async8(void *smem_dst, const void *gmem_src)
 {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gmem_src)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gmem_src)
                  : "memory");
 }
 
@@ -361,9 +362,9 @@ struct Track {
     unsigned *ticket;          // set by launch_assign: block counter of the distance sum, cleared by the row kernels
 };
 size_t assign_scratch_bytes(int64_t n, int32_t k, int64_t d);
-// precision 0: FP32 candidate rows; 1: those, or 4 where it is faster; 2: BF16 screening on the SIMT cores; 3: on the tensor cores over
-// 128-sample tiles when members, the grouping of labels_in, is given and d <= 128; 4: int8 screening (per-row
-// scale) on the SIMT cores; all with the exact FP32 recompute (same results).  3 takes FP32 samples only.
+// precision 0: FP32 candidate rows; 1: those, or 4 where it is faster; 2: BF16 screening on the SIMT cores; 3: on the
+// tensor cores over 128-sample tiles when members, the grouping of labels_in, is given and d <= 128; 4: int8 screening
+// (per-row scale) on the SIMT cores; all with the exact FP32 recompute (same results).  3 takes FP32 samples only.
 // Bits 8-15 of precision: candidates per group of the row kernels (0: default, 4 or 8).
 cudaError_t launch_assign(const void *X, bool bf16, int64_t n, int64_t d, int64_t ld, const int32_t *g_idx,
                           int32_t kappa, const float *C, int32_t k, const int32_t *labels_in, int32_t *labels_out,

@@ -71,7 +71,7 @@ constexpr int RC_RESIDENT = 2;             // K-blocks up to which the queries s
 constexpr int RC_STAGES = 3, RC_STAGES_A = 2;  // operand stages: samples only, samples and queries
 constexpr int RC_AHEAD = 3;                // steps of raw rows in flight
 constexpr int RC_CAP = 2048;               // list entries per query
-constexpr int RC_BATCH = 38 * RC_Q;        // queries screened at once, at most (four slices each fill the chip): 80 MB of lists
+constexpr int RC_BATCH = 38 * RC_Q;        // queries screened at once, at most (four slices fill the chip): 80 MB of lists
 constexpr uint32_t RC_WAIT_ITERS = 1u << 20;
 constexpr uint32_t RC_TMEM = 512;          // two buffers x two query tiles x 128 columns
 

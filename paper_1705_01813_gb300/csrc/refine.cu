@@ -457,14 +457,14 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
         const void *f = reinterpret_cast<const void *>(kernel);
         if ((e = set_max_smem(f, (int)shm)) != cudaSuccess)
             return e;
-        kernel<<<(unsigned)bound, RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, true, prev_in, canon,
-                                                    row_changed, kappa, g_idx, g_dist, st);
+        kernel<<<(unsigned)bound, RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, true, prev_in,
+                                                        canon, row_changed, kappa, g_idx, g_dist, st);
     }
     if (tensor) {
         // tensor-core Gram for runs of <= 128 members
         constexpr bool bf16 = std::is_same_v<XT, __nv_bfloat16>;
-        return launch_refine_tc(X, bf16, n, d, ld, members, runs, cnt, bound, k, kappa, prev_in, canon, row_changed, g_idx, g_dist, tc_scratch,
-                                st, s);
+        return launch_refine_tc(X, bf16, n, d, ld, members, runs, cnt, bound, k, kappa, prev_in, canon, row_changed, g_idx,
+                                g_dist, tc_scratch, st, s);
     }
     // runs of <= 64 members.  Rows staged by
     // 16-byte loads take the persistent warp-specialised kernel (one wave of blocks; 10M x 512 BF16: 32.0 ->
@@ -486,8 +486,8 @@ static cudaError_t refine_tv(const XT *X, int64_t n, int64_t d, int64_t ld, cons
         const void *f = reinterpret_cast<const void *>(kernel);
         if ((e = set_max_smem(f, (int)shm)) != cudaSuccess)
             return e;
-        kernel<<<(unsigned)bound, RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, false, prev_in, canon,
-                                                    row_changed, kappa, g_idx, g_dist, st);
+        kernel<<<(unsigned)bound, RF_THREADS, shm, s>>>(X, n, (int)d, ld, members, runs, runs_cap, cnt, false, prev_in,
+                                                        canon, row_changed, kappa, g_idx, g_dist, st);
     }
     return cudaGetLastError();
 }

@@ -387,92 +387,93 @@ __global__ void __launch_bounds__(EX_THREADS) k_refine_exact(const XT *__restric
     __shared__ int rid[TC_M], pre[TC_M + 1], wsum[EX_THREADS / 32];
     const int nrun = cnt->x;
     for (int q = blockIdx.x; q < nrun; q += gridDim.x) {
-    const int2 rec = runs[inexact_runs[q]];
-    const int p0 = rec.x, sz = rec.y;
-    const int tid = threadIdx.x, w = tid >> 5, lane = lane_id();
-    const int ds = vec ? d + 4 : d + 1;
-    int cnt = 0;
-    if (tid < sz) {
-        const int a = mem[p0 + tid];
-        rid[tid] = (a >= 0 && a < n) ? a : -1;
-        cnt = rid[tid] >= 0 ? cand_n[rid[tid]] : 0;
-    }
-    // exclusive prefix of the rows' candidate counts
-    int incl = cnt;
+        const int2 rec = runs[inexact_runs[q]];
+        const int p0 = rec.x, sz = rec.y;
+        const int tid = threadIdx.x, w = tid >> 5, lane = lane_id();
+        const int ds = vec ? d + 4 : d + 1;
+        int cnt = 0;
+        if (tid < sz) {
+            const int a = mem[p0 + tid];
+            rid[tid] = (a >= 0 && a < n) ? a : -1;
+            cnt = rid[tid] >= 0 ? cand_n[rid[tid]] : 0;
+        }
+        // exclusive prefix of the rows' candidate counts
+        int incl = cnt;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(FULL_MASK, incl, o);
-        if (lane >= o)
-            incl += v;
-    }
-    if (lane == 31)
-        wsum[w] = incl;
-    __syncthreads();
-    int base = 0;
-    for (int q = 0; q < w; q++)
-        base += wsum[q];
-    pre[tid] = base + incl - cnt;
-    if (tid == EX_THREADS - 1)
-        pre[EX_THREADS] = base + incl;
-    if (vec) {
-        const int d4 = d >> 2;
-#pragma unroll 4
-        for (int e = tid; e < sz * d4; e += EX_THREADS) {
-            const int row = e / d4, t = 4 * (e - row * d4), a = rid[row];
-            *reinterpret_cast<float4 *>(xs + row * ds + t) =
-                a >= 0 ? ldx4<XT>(X + (int64_t)a * ld + t) : make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(FULL_MASK, incl, o);
+            if (lane >= o)
+                incl += v;
         }
-    } else {
-#pragma unroll 4
-        for (int row = w; row < sz; row += EX_THREADS / 32) {
-            const int a = rid[row];
-            for (int t = lane; t < d; t += 32)
-                xs[row * ds + t] = a >= 0 ? ldx(X + (int64_t)a * ld + t) : 0.f;
-        }
-    }
-    __syncthreads();  // the staged rows and the prefix pre[] (pre[EX_THREADS]: the run's pair count)
-    const int total = pre[EX_THREADS];
-    for (int p = tid; p < total; p += EX_THREADS) {
-        int lo = 0, hi = sz;  // the row of pair p: last row with pre[row] <= p
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (pre[mid] <= p)
-                lo = mid;
-            else
-                hi = mid;
-        }
-        const int row = lo, q = p - pre[row];
-        const int64_t slot = (int64_t)rid[row] * TC_CAP + q;
-        const unsigned raw = (unsigned)cand_id[slot];
-        if (!(raw & TC_RERANK))
-            continue;
-        const int col = (int)(raw & ~TC_RERANK);
-        if (col >= sz || rid[col] < 0) {
-            flag_error(st, GK_ERR_INVALID, (unsigned)p0);
-            continue;
-        }
-        const float *xa = xs + row * ds, *xb = xs + col * ds;
-        float acc = 0.f;
+        if (lane == 31)
+            wsum[w] = incl;
+        __syncthreads();
+        int base = 0;
+        for (int q = 0; q < w; q++)
+            base += wsum[q];
+        pre[tid] = base + incl - cnt;
+        if (tid == EX_THREADS - 1)
+            pre[EX_THREADS] = base + incl;
         if (vec) {
+            const int d4 = d >> 2;
 #pragma unroll 4
-            for (int t = 0; t < d; t += 4) {
-                const float4 x = *reinterpret_cast<const float4 *>(xa + t), y = *reinterpret_cast<const float4 *>(xb + t);
-                const float e0 = x.x - y.x, e1 = x.y - y.y, e2 = x.z - y.z, e3 = x.w - y.w;
-                acc = fmaf(e0, e0, acc);
-                acc = fmaf(e1, e1, acc);
-                acc = fmaf(e2, e2, acc);
-                acc = fmaf(e3, e3, acc);
+            for (int e = tid; e < sz * d4; e += EX_THREADS) {
+                const int row = e / d4, t = 4 * (e - row * d4), a = rid[row];
+                *reinterpret_cast<float4 *>(xs + row * ds + t) =
+                    a >= 0 ? ldx4<XT>(X + (int64_t)a * ld + t) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         } else {
-            for (int t = 0; t < d; t++) {
-                const float e = xa[t] - xb[t];
-                acc = fmaf(e, e, acc);
+#pragma unroll 4
+            for (int row = w; row < sz; row += EX_THREADS / 32) {
+                const int a = rid[row];
+                for (int t = lane; t < d; t += 32)
+                    xs[row * ds + t] = a >= 0 ? ldx(X + (int64_t)a * ld + t) : 0.f;
             }
         }
-        cand_d[slot] = acc;
-        cand_id[slot] = rid[col];
-    }
-    __syncthreads();  // the next run rewrites the staged rows and ids
+        __syncthreads();  // the staged rows and the prefix pre[] (pre[EX_THREADS]: the run's pair count)
+        const int total = pre[EX_THREADS];
+        for (int p = tid; p < total; p += EX_THREADS) {
+            int lo = 0, hi = sz;  // the row of pair p: last row with pre[row] <= p
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (pre[mid] <= p)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            const int row = lo, q = p - pre[row];
+            const int64_t slot = (int64_t)rid[row] * TC_CAP + q;
+            const unsigned raw = (unsigned)cand_id[slot];
+            if (!(raw & TC_RERANK))
+                continue;
+            const int col = (int)(raw & ~TC_RERANK);
+            if (col >= sz || rid[col] < 0) {
+                flag_error(st, GK_ERR_INVALID, (unsigned)p0);
+                continue;
+            }
+            const float *xa = xs + row * ds, *xb = xs + col * ds;
+            float acc = 0.f;
+            if (vec) {
+#pragma unroll 4
+                for (int t = 0; t < d; t += 4) {
+                    const float4 x = *reinterpret_cast<const float4 *>(xa + t);
+                    const float4 y = *reinterpret_cast<const float4 *>(xb + t);
+                    const float e0 = x.x - y.x, e1 = x.y - y.y, e2 = x.z - y.z, e3 = x.w - y.w;
+                    acc = fmaf(e0, e0, acc);
+                    acc = fmaf(e1, e1, acc);
+                    acc = fmaf(e2, e2, acc);
+                    acc = fmaf(e3, e3, acc);
+                }
+            } else {
+                for (int t = 0; t < d; t++) {
+                    const float e = xa[t] - xb[t];
+                    acc = fmaf(e, e, acc);
+                }
+            }
+            cand_d[slot] = acc;
+            cand_id[slot] = rid[col];
+        }
+        __syncthreads();  // the next run rewrites the staged rows and ids
     }
 }
 
@@ -591,7 +592,8 @@ static cudaError_t perm_tensor_map(CUtensorMap *tm, const __nv_bfloat16 *Xp, int
 template <typename XT>
 static cudaError_t refine_tc_t(const XT *X, int64_t n, int64_t d, int64_t ld, const int32_t *members, const int2 *runs,
                                RunCounts *cnt, int64_t bound, int32_t k, int32_t kappa, const int32_t *prev, bool canon,
-                               uint8_t *row_changed, int32_t *g_idx, float *g_dist, void *scratch, DevStatus *st, cudaStream_t s)
+                               uint8_t *row_changed, int32_t *g_idx, float *g_dist, void *scratch, DevStatus *st,
+                               cudaStream_t s)
 {
     const size_t a = al256((size_t)n * TC_CAP * sizeof(int32_t));
     const size_t t = al256((size_t)(k + n / 2 + 1) * sizeof(int32_t));
@@ -622,8 +624,8 @@ static cudaError_t refine_tc_t(const XT *X, int64_t n, int64_t d, int64_t ld, co
                                                                g_dist, pnrm, run_flags, cand_id, cand_d, cand_n, st);
     // the inexact runs are listed: three blocks per SM fit at d = 128, more at smaller d
     const int64_t ex_blocks = bound < 152 * 6 ? bound : 152 * 6;
-    k_refine_exact<XT><<<(unsigned)ex_blocks, EX_THREADS, shm_exact, s>>>(X, n, (int)d, ld, x_vec4(X, d, ld), members, runs, cnt,
-                                                                          inexact_runs, cand_id, cand_d, cand_n, st);
+    k_refine_exact<XT><<<(unsigned)ex_blocks, EX_THREADS, shm_exact, s>>>(
+        X, n, (int)d, ld, x_vec4(X, d, ld), members, runs, cnt, inexact_runs, cand_id, cand_d, cand_n, st);
     int64_t mblocks = (n + MG_WARPS - 1) / MG_WARPS;
     if (mblocks > 152 * 64)
         mblocks = 152 * 64;

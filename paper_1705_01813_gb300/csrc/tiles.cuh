@@ -74,9 +74,9 @@ __device__ __forceinline__ int triangle_block(int nb, int t)
 // so only blocks with by <= bx < nb = ceil(nr / Q) count (a run of 50 has 91 at Q = 4); and with prun, the run each
 // member belonged to in the previous refinement (members sorted by it, -1: none), a block whose rows and columns all
 // come from one such run holds only pairs that were compared then, and is left out.  (Without a previous refinement
-// all of them count, and the callers take triangle_block: two barriers less, 5% of a refinement of narrow runs.)  Called by NT threads with index
-// t in [0, NT), NT a multiple of 32 and >= NBLK; sync() is their barrier, wcnt has NT / 32 entries.  Returns the
-// number of blocks (the list is valid after the call).
+// all of them count, and the callers take triangle_block: two barriers less, 5% of a refinement of narrow runs.)
+// Called by NT threads with index t in [0, NT), NT a multiple of 32 and >= NBLK; sync() is their barrier, wcnt has NT /
+// 32 entries.  Returns the number of blocks (the list is valid after the call).
 template <int T, int NT, typename Sync>
 __device__ __forceinline__ int live_blocks(int nr, const int *prun, unsigned short *list, int *wcnt, int t, Sync sync)
 {

@@ -390,8 +390,9 @@ __device__ __forceinline__ float4 staged4(const __nv_bfloat16 *p)
 //   KEYS = true: keys[p] = (order(d_u - d_v) << 32) | id.
 // Bound by the reads of the rows: 1M x 128 FP32 (512 MB) takes 84 us with KEYS, 6.1 TB/s, and 159 us without (all but
 // the last stage are read again, mostly from the L2, and the sums).  With loads through registers, four in flight, it
-// was 229 and 332 us (BF16 225 and 337, now 64 and 150); before the packed distances and the integer sums 421 and 879 us, the FP64 additions' time.  Two
-// stage buffers, the next stage in flight during the distances, leave 3 blocks of an SM instead of 5: 91 and 174 us.
+// was 229 and 332 us (BF16 225 and 337, now 64 and 150); before the packed distances and the integer sums 421 and 879
+// us, the FP64 additions' time.  Two stage buffers, the next stage in flight during the distances, leave 3 blocks of an
+// SM instead of 5: 91 and 174 us.
 template <typename XT, bool KEYS>
 __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__ X, int64_t n, int d, int64_t ld,
                                                           bool vec, int L, int64_t C, const int32_t *__restrict__ perm,
@@ -488,7 +489,8 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
 #pragma unroll 4
             for (; tt + 4 <= tw; tt += 4) {
                 const float4 x = staged4(xs + tt);
-                const float4 a = *reinterpret_cast<const float4 *>(cs + tt), h = *reinterpret_cast<const float4 *>(cs + tt + 2);
+                const float4 a = *reinterpret_cast<const float4 *>(cs + tt);
+                const float4 h = *reinterpret_cast<const float4 *>(cs + tt + 2);
                 add(x.x, make_float2(a.x, a.y));
                 add(x.y, make_float2(a.z, a.w));
                 add(x.z, make_float2(h.x, h.y));
@@ -509,7 +511,8 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
             const int half = duv.x <= duv.y ? 0 : 1;
             if (valid)
                 halves[p] = (uint8_t)half;
-            const unsigned bu = __ballot_sync(FULL_MASK, valid && half == 0), bv = __ballot_sync(FULL_MASK, valid && half == 1);
+            const unsigned bu = __ballot_sync(FULL_MASK, valid && half == 0);
+            const unsigned bv = __ballot_sync(FULL_MASK, valid && half == 1);
             if (lane == 0) {
                 s_n[warp] = __popc(bu);
                 s_n[4 + warp] = __popc(bv);
@@ -523,7 +526,8 @@ __global__ void __launch_bounds__(TR_THREADS) k_tree_pass(const XT *__restrict__
                 nv += s_n[4 + w];
             }
             if (valid)
-                order[half == 0 ? au + __popc(bu & lanemask_lt()) : nu + av + __popc(bv & lanemask_lt())] = (unsigned char)tid;
+                order[half == 0 ? au + __popc(bu & lanemask_lt()) : nu + av + __popc(bv & lanemask_lt())] =
+                    (unsigned char)tid;
             cnt_u += nu;
             cnt_v += nv;
             __syncthreads();

@@ -208,153 +208,153 @@ __global__ void __launch_bounds__(UP_WARPS * 32) k_update(const XT *__restrict__
     // clusters r = blockIdx.x, + gridDim.x, ...; those of at most small_max members are k_update_small's,
     // those of more than large k_update_wide's
     for (int r = blockIdx.x; r < k; r += gridDim.x) {
-    const int beg = off[r], m = off[r + 1] - beg;
-    if (m <= small_max || m > large || (dirty && dirty[r] == 0))
-        continue;
-    if (counts && threadIdx.x == 0)
-        counts[r] = m;
-    if (m == 0) {
-        if (threadIdx.x == 0)
-            contrib[r] = 0.0;
-        continue;
-    }
-    const float mf = (float)m, inv_m = 1.0f / mf;
-    DF sq_lane = {0.f, 0.f}, dd_lane = {0.f, 0.f};
-    for (int cb = 0; cb < nv; cb += L * CPL) {
-        float s[CPL][VEC], c[CPL][VEC];
-        float2 qs = make_float2(0.f, 0.f), qc = make_float2(0.f, 0.f);
+        const int beg = off[r], m = off[r + 1] - beg;
+        if (m <= small_max || m > large || (dirty && dirty[r] == 0))
+            continue;
+        if (counts && threadIdx.x == 0)
+            counts[r] = m;
+        if (m == 0) {
+            if (threadIdx.x == 0)
+                contrib[r] = 0.0;
+            continue;
+        }
+        const float mf = (float)m, inv_m = 1.0f / mf;
+        DF sq_lane = {0.f, 0.f}, dd_lane = {0.f, 0.f};
+        for (int cb = 0; cb < nv; cb += L * CPL) {
+            float s[CPL][VEC], c[CPL][VEC];
+            float2 qs = make_float2(0.f, 0.f), qc = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int u = 0; u < CPL; u++)
+            for (int u = 0; u < CPL; u++)
 #pragma unroll
-            for (int q = 0; q < VEC; q++)
-                s[u][q] = c[u][q] = 0.f;
-        // the member ids of a chunk are staged in shared memory first, so each row
-        // load waits for one memory round trip instead of two
-        for (int mb = 0; mb < m; mb += UP_MCHUNK) {
-            const int mc = min(UP_MCHUNK, m - mb);
-            __syncthreads();  // the previous chunk's ids are no longer read
-            for (int q = threadIdx.x; q < mc; q += UP_WARPS * 32)
-                s_mem[q] = __ldg(mem + beg + mb + q);
+                for (int q = 0; q < VEC; q++)
+                    s[u][q] = c[u][q] = 0.f;
+            // the member ids of a chunk are staged in shared memory first, so each row
+            // load waits for one memory round trip instead of two
+            for (int mb = 0; mb < m; mb += UP_MCHUNK) {
+                const int mc = min(UP_MCHUNK, m - mb);
+                __syncthreads();  // the previous chunk's ids are no longer read
+                for (int q = threadIdx.x; q < mc; q += UP_WARPS * 32)
+                    s_mem[q] = __ldg(mem + beg + mb + q);
+                __syncthreads();
+                if constexpr (PIPE) {
+                    float4 *ring = reinterpret_cast<float4 *>(s_buf) + w * (2 * R * 32 * CPL);  // [stage][row][u][lane]
+                    const int wlead = w * G;                       // the warp's first group has the most rows
+                    const int njw = mc > wlead ? (mc - wlead + gstride - 1) / gstride : 0;
+                    const int nst = (njw + R - 1) / R;
+                    auto issue = [&](int t) {
+                        float4 *buf = ring + (t & 1) * (R * 32 * CPL);
+#pragma unroll
+                        for (int z = 0; z < R; z++) {
+                            const int p = gidx + gstride * (t * R + z);
+                            if (p < mc) {
+                                const V *row = Xv + (int64_t)s_mem[p] * ldv;
+#pragma unroll
+                                for (int u = 0; u < CPL; u++) {
+                                    const int col = cb + sub + u * L;
+                                    if (col < nv)
+                                        cp_async16(buf + (z * CPL + u) * 32 + lane, row + col);
+                                }
+                            }
+                        }
+                        cp_async_commit();
+                    };
+                    if (nst > 0)
+                        issue(0);
+                    for (int t = 0; t < nst; t++) {
+                        if (t + 1 < nst)
+                            issue(t + 1);
+                        else
+                            cp_async_commit();  // empty group: the wait below always leaves one
+                        cp_async_wait<1>();
+                        __syncwarp();
+                        const float4 *buf = ring + (t & 1) * (R * 32 * CPL);
+#pragma unroll
+                        for (int z = 0; z < R; z++) {
+                            if (gidx + gstride * (t * R + z) < mc) {
+                                V vz[CPL];
+#pragma unroll
+                                for (int u = 0; u < CPL; u++)
+                                    vz[u] = buf[(z * CPL + u) * 32 + lane];
+                                accumulate<VEC, CPL, std::is_same_v<XT, __nv_bfloat16>>(vz, s, c, qs, qc, cb, sub, L, nv);
+                            }
+                        }
+                        __syncwarp();  // stage t & 1 is refilled by issue(t + 2)
+                    }
+                } else {
+                    for (int p0 = gidx; p0 < mc; p0 += UNR * gstride) {
+                        V v[UNR][CPL];
+#pragma unroll
+                        for (int z = 0; z < UNR; z++) {
+                            const int p = p0 + z * gstride;
+                            if (p < mc) {
+                                const XT *rowx = X + (int64_t)s_mem[p] * ld;
+#pragma unroll
+                                for (int u = 0; u < CPL; u++) {
+                                    const int col = cb + sub + u * L;
+                                    if (col < nv)
+                                        v[z][u] = load_vec<VEC>(rowx + (int64_t)col * VEC);
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int z = 0; z < UNR; z++)
+                            if (p0 + z * gstride < mc)
+                                accumulate<VEC, CPL, std::is_same_v<XT, __nv_bfloat16>>(v[z], s, c, qs, qc, cb, sub, L, nv);
+                    }
+                }
+            }
+            if constexpr (PIPE)
+                __syncthreads();  // every warp is done with the ring before the partial sums overwrite it
+            sq_lane = df_add(sq_lane, chains_sum(qs, qc));
+            // combine the G groups of the warp, then the warps of the block, in a fixed order
+#pragma unroll
+            for (int u = 0; u < CPL; u++) {
+#pragma unroll
+                for (int q = 0; q < VEC; q++) {
+                    DF S = fast_two_sum(s[u][q], -c[u][q]);  // the Kahan sum s - c, exactly
+                    for (int o = L; o < 32; o <<= 1)
+                        S = df_add(S, df_shfl_xor(S, o));
+                    if (g == 0)
+                        s_part[w][(u * L + sub) * VEC + q] = make_float2(S.hi, S.lo);
+                }
+            }
             __syncthreads();
-            if constexpr (PIPE) {
-                float4 *ring = reinterpret_cast<float4 *>(s_buf) + w * (2 * R * 32 * CPL);  // [stage][row][u][lane]
-                const int wlead = w * G;                       // the warp's first group has the most rows
-                const int njw = mc > wlead ? (mc - wlead + gstride - 1) / gstride : 0;
-                const int nst = (njw + R - 1) / R;
-                auto issue = [&](int t) {
-                    float4 *buf = ring + (t & 1) * (R * 32 * CPL);
-#pragma unroll
-                    for (int z = 0; z < R; z++) {
-                        const int p = gidx + gstride * (t * R + z);
-                        if (p < mc) {
-                            const V *row = Xv + (int64_t)s_mem[p] * ldv;
-#pragma unroll
-                            for (int u = 0; u < CPL; u++) {
-                                const int col = cb + sub + u * L;
-                                if (col < nv)
-                                    cp_async16(buf + (z * CPL + u) * 32 + lane, row + col);
-                            }
-                        }
-                    }
-                    cp_async_commit();
-                };
-                if (nst > 0)
-                    issue(0);
-                for (int t = 0; t < nst; t++) {
-                    if (t + 1 < nst)
-                        issue(t + 1);
-                    else
-                        cp_async_commit();  // empty group: the wait below always leaves one
-                    cp_async_wait<1>();
-                    __syncwarp();
-                    const float4 *buf = ring + (t & 1) * (R * 32 * CPL);
-#pragma unroll
-                    for (int z = 0; z < R; z++) {
-                        if (gidx + gstride * (t * R + z) < mc) {
-                            V vz[CPL];
-#pragma unroll
-                            for (int u = 0; u < CPL; u++)
-                                vz[u] = buf[(z * CPL + u) * 32 + lane];
-                            accumulate<VEC, CPL, std::is_same_v<XT, __nv_bfloat16>>(vz, s, c, qs, qc, cb, sub, L, nv);
-                        }
-                    }
-                    __syncwarp();  // stage t & 1 is refilled by issue(t + 2)
-                }
-            } else {
-                for (int p0 = gidx; p0 < mc; p0 += UNR * gstride) {
-                    V v[UNR][CPL];
-#pragma unroll
-                    for (int z = 0; z < UNR; z++) {
-                        const int p = p0 + z * gstride;
-                        if (p < mc) {
-                            const XT *rowx = X + (int64_t)s_mem[p] * ld;
-#pragma unroll
-                            for (int u = 0; u < CPL; u++) {
-                                const int col = cb + sub + u * L;
-                                if (col < nv)
-                                    v[z][u] = load_vec<VEC>(rowx + (int64_t)col * VEC);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int z = 0; z < UNR; z++)
-                        if (p0 + z * gstride < mc)
-                            accumulate<VEC, CPL, std::is_same_v<XT, __nv_bfloat16>>(v[z], s, c, qs, qc, cb, sub, L, nv);
+            for (int e = threadIdx.x; e < L * CPL * VEC; e += UP_WARPS * 32) {
+                // entry e = (u * L + sb) * VEC + q holds column vector cb + sb + u * L, component q
+                const int u = (e / VEC) / L, sb = (e / VEC) % L;
+                const int colv = cb + sb + u * L;
+                if (colv < nv) {
+                    DF S = {s_part[0][e].x, s_part[0][e].y};
+                    for (int ww = 1; ww < UP_WARPS; ww++)
+                        S = df_add(S, DF{s_part[ww][e].x, s_part[ww][e].y});
+                    C[(int64_t)r * d + (int64_t)colv * VEC + (e % VEC)] = df_div(S, mf, inv_m);
+                    dd_lane = df_add(dd_lane, df_sqr(S));
                 }
             }
+            __syncthreads();
         }
-        if constexpr (PIPE)
-            __syncthreads();  // every warp is done with the ring before the partial sums overwrite it
-        sq_lane = df_add(sq_lane, chains_sum(qs, qc));
-        // combine the G groups of the warp, then the warps of the block, in a fixed order
-#pragma unroll
-        for (int u = 0; u < CPL; u++) {
-#pragma unroll
-            for (int q = 0; q < VEC; q++) {
-                DF S = fast_two_sum(s[u][q], -c[u][q]);  // the Kahan sum s - c, exactly
-                for (int o = L; o < 32; o <<= 1)
-                    S = df_add(S, df_shfl_xor(S, o));
-                if (g == 0)
-                    s_part[w][(u * L + sub) * VEC + q] = make_float2(S.hi, S.lo);
-            }
+        // sum of ||x||^2 over all lanes, sum of D_t^2 over the threads that wrote means
+        for (int o = 1; o < 32; o <<= 1) {
+            sq_lane = df_add(sq_lane, df_shfl_xor(sq_lane, o));
+            dd_lane = df_add(dd_lane, df_shfl_xor(dd_lane, o));
+        }
+        if (lane == 0) {
+            s_sq[w] = make_float2(sq_lane.hi, sq_lane.lo);
+            s_dd[w] = make_float2(dd_lane.hi, dd_lane.lo);
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < L * CPL * VEC; e += UP_WARPS * 32) {
-            // entry e = (u * L + sb) * VEC + q holds column vector cb + sb + u * L, component q
-            const int u = (e / VEC) / L, sb = (e / VEC) % L;
-            const int colv = cb + sb + u * L;
-            if (colv < nv) {
-                DF S = {s_part[0][e].x, s_part[0][e].y};
-                for (int ww = 1; ww < UP_WARPS; ww++)
-                    S = df_add(S, DF{s_part[ww][e].x, s_part[ww][e].y});
-                C[(int64_t)r * d + (int64_t)colv * VEC + (e % VEC)] = df_div(S, mf, inv_m);
-                dd_lane = df_add(dd_lane, df_sqr(S));
+        if (threadIdx.x == 0) {
+            DF sq = {s_sq[0].x, s_sq[0].y}, dd = {s_dd[0].x, s_dd[0].y};
+            for (int ww = 1; ww < UP_WARPS; ww++) {
+                sq = df_add(sq, DF{s_sq[ww].x, s_sq[ww].y});
+                dd = df_add(dd, DF{s_dd[ww].x, s_dd[ww].y});
             }
+            const double cr = df_to_double(sq) - df_to_double(dd) / (double)m;
+            contrib[r] = cr;
+            if (!isfinite(cr))  // a non-finite sample in the cluster (Inf or NaN spreads into its sums)
+                flag_error(st, GK_ERR_NUMERIC, (unsigned)r);
         }
-        __syncthreads();
-    }
-    // sum of ||x||^2 over all lanes, sum of D_t^2 over the threads that wrote means
-    for (int o = 1; o < 32; o <<= 1) {
-        sq_lane = df_add(sq_lane, df_shfl_xor(sq_lane, o));
-        dd_lane = df_add(dd_lane, df_shfl_xor(dd_lane, o));
-    }
-    if (lane == 0) {
-        s_sq[w] = make_float2(sq_lane.hi, sq_lane.lo);
-        s_dd[w] = make_float2(dd_lane.hi, dd_lane.lo);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        DF sq = {s_sq[0].x, s_sq[0].y}, dd = {s_dd[0].x, s_dd[0].y};
-        for (int ww = 1; ww < UP_WARPS; ww++) {
-            sq = df_add(sq, DF{s_sq[ww].x, s_sq[ww].y});
-            dd = df_add(dd, DF{s_dd[ww].x, s_dd[ww].y});
-        }
-        const double cr = df_to_double(sq) - df_to_double(dd) / (double)m;
-        contrib[r] = cr;
-        if (!isfinite(cr))  // a non-finite sample in the cluster (Inf or NaN spreads into its sums)
-            flag_error(st, GK_ERR_NUMERIC, (unsigned)r);
-    }
-    __syncthreads();  // s_sq / s_dd are read above before the next cluster writes them
+        __syncthreads();  // s_sq / s_dd are read above before the next cluster writes them
     }
 }
 
@@ -371,7 +371,8 @@ __global__ void __launch_bounds__(UP_WARPS * 32) k_update(const XT *__restrict__
 template <bool PIPE, typename XT>
 __global__ void __launch_bounds__(UP_WARPS * 32, PIPE ? 6 : 8) k_update_wide(const XT *__restrict__ X, int d, int64_t ld,
                                                           const int32_t *__restrict__ off,
-                                                          const int32_t *__restrict__ mem, int k, int large, int nb, int chunk,
+                                                          const int32_t *__restrict__ mem, int k, int large, int nb,
+                                                          int chunk,
                                                           float *__restrict__ C, int32_t *__restrict__ counts,
                                                           double *__restrict__ contrib,
                                                           const uint8_t *__restrict__ dirty, DevStatus *st)
@@ -405,143 +406,143 @@ __global__ void __launch_bounds__(UP_WARPS * 32, PIPE ? 6 : 8) k_update_wide(con
         cluster_barrier();  // every block of the thread-block cluster runs before any stores into the first one's memory
     // one cluster r, by all threads
     auto cluster = [&](const int r) {
-    const int beg = off[r], m = off[r + 1] - beg;
-    if (counts && threadIdx.x == 0 && rank == 0)
-        counts[r] = m;
-    if (m == 0) {
-        if (threadIdx.x == 0 && rank == 0)
-            contrib[r] = 0.0;
-        return;
-    }
-    const float mf = (float)m, inv_m = 1.0f / mf;
-    DF sq_lane = {0.f, 0.f}, dd_lane = {0.f, 0.f};
-    for (int cb = rank * L; cb < nv; cb += nb * L) {
-        const int col = cb + sub;  // this lane's vector
-        float s[1][VEC], c[1][VEC];
-        float2 qs = make_float2(0.f, 0.f), qc = make_float2(0.f, 0.f);
+        const int beg = off[r], m = off[r + 1] - beg;
+        if (counts && threadIdx.x == 0 && rank == 0)
+            counts[r] = m;
+        if (m == 0) {
+            if (threadIdx.x == 0 && rank == 0)
+                contrib[r] = 0.0;
+            return;
+        }
+        const float mf = (float)m, inv_m = 1.0f / mf;
+        DF sq_lane = {0.f, 0.f}, dd_lane = {0.f, 0.f};
+        for (int cb = rank * L; cb < nv; cb += nb * L) {
+            const int col = cb + sub;  // this lane's vector
+            float s[1][VEC], c[1][VEC];
+            float2 qs = make_float2(0.f, 0.f), qc = make_float2(0.f, 0.f);
 #pragma unroll
-        for (int q = 0; q < VEC; q++)
-            s[0][q] = c[0][q] = 0.f;
-        // the member ids of a chunk are staged in shared memory first, so each row
-        // load waits for one memory round trip instead of two
-        for (int mb = 0; mb < m; mb += UP_MCHUNK) {
-            const int mc = min(UP_MCHUNK, m - mb);
-            __syncthreads();  // the previous chunk's ids are no longer read
-            for (int q = threadIdx.x; q < mc; q += UP_WARPS * 32)
-                s_mem[q] = __ldg(mem + beg + mb + q);
-            __syncthreads();
-            if constexpr (PIPE) {
-                float4 *ring = reinterpret_cast<float4 *>(s_buf) + w * (2 * R * 32);  // [stage][row][lane]
-                const int wlead = w * G;                       // the warp's first group has the most rows
-                const int njw = mc > wlead ? (mc - wlead + gstride - 1) / gstride : 0;
-                const int nst = (njw + R - 1) / R;
-                auto issue = [&](int t) {
-                    float4 *buf = ring + (t & 1) * (R * 32);
+            for (int q = 0; q < VEC; q++)
+                s[0][q] = c[0][q] = 0.f;
+            // the member ids of a chunk are staged in shared memory first, so each row
+            // load waits for one memory round trip instead of two
+            for (int mb = 0; mb < m; mb += UP_MCHUNK) {
+                const int mc = min(UP_MCHUNK, m - mb);
+                __syncthreads();  // the previous chunk's ids are no longer read
+                for (int q = threadIdx.x; q < mc; q += UP_WARPS * 32)
+                    s_mem[q] = __ldg(mem + beg + mb + q);
+                __syncthreads();
+                if constexpr (PIPE) {
+                    float4 *ring = reinterpret_cast<float4 *>(s_buf) + w * (2 * R * 32);  // [stage][row][lane]
+                    const int wlead = w * G;                       // the warp's first group has the most rows
+                    const int njw = mc > wlead ? (mc - wlead + gstride - 1) / gstride : 0;
+                    const int nst = (njw + R - 1) / R;
+                    auto issue = [&](int t) {
+                        float4 *buf = ring + (t & 1) * (R * 32);
 #pragma unroll
-                    for (int z = 0; z < R; z++) {
-                        const int p = gidx + gstride * (t * R + z);
-                        if (p < mc && col < nv)
-                            cp_async16(buf + z * 32 + lane, Xv + (int64_t)s_mem[p] * ldv + col);
-                    }
-                    cp_async_commit();
-                };
-                if (nst > 0)
-                    issue(0);
-                for (int t = 0; t < nst; t++) {
-                    if (t + 1 < nst)
-                        issue(t + 1);
-                    else
-                        cp_async_commit();  // empty group: the wait below always leaves one
-                    cp_async_wait<1>();
-                    __syncwarp();
-                    const float4 *buf = ring + (t & 1) * (R * 32);
-#pragma unroll
-                    for (int z = 0; z < R; z++) {
-                        if (gidx + gstride * (t * R + z) < mc) {
-                            const V vz[1] = {buf[z * 32 + lane]};
-                            accumulate<VEC, 1, std::is_same_v<XT, __nv_bfloat16>>(vz, s, c, qs, qc, cb, sub, L, nv);
+                        for (int z = 0; z < R; z++) {
+                            const int p = gidx + gstride * (t * R + z);
+                            if (p < mc && col < nv)
+                                cp_async16(buf + z * 32 + lane, Xv + (int64_t)s_mem[p] * ldv + col);
                         }
-                    }
-                    __syncwarp();  // stage t & 1 is refilled by issue(t + 2)
-                }
-            } else {
-                for (int p0 = gidx; p0 < mc; p0 += UNR * gstride) {
-                    V v[UNR][1];
+                        cp_async_commit();
+                    };
+                    if (nst > 0)
+                        issue(0);
+                    for (int t = 0; t < nst; t++) {
+                        if (t + 1 < nst)
+                            issue(t + 1);
+                        else
+                            cp_async_commit();  // empty group: the wait below always leaves one
+                        cp_async_wait<1>();
+                        __syncwarp();
+                        const float4 *buf = ring + (t & 1) * (R * 32);
 #pragma unroll
-                    for (int z = 0; z < UNR; z++) {
-                        const int p = p0 + z * gstride;
-                        if (p < mc && col < nv)
-                            v[z][0] = load_vec<VEC>(X + (int64_t)s_mem[p] * ld + (int64_t)col * VEC);
+                        for (int z = 0; z < R; z++) {
+                            if (gidx + gstride * (t * R + z) < mc) {
+                                const V vz[1] = {buf[z * 32 + lane]};
+                                accumulate<VEC, 1, std::is_same_v<XT, __nv_bfloat16>>(vz, s, c, qs, qc, cb, sub, L, nv);
+                            }
+                        }
+                        __syncwarp();  // stage t & 1 is refilled by issue(t + 2)
                     }
+                } else {
+                    for (int p0 = gidx; p0 < mc; p0 += UNR * gstride) {
+                        V v[UNR][1];
 #pragma unroll
-                    for (int z = 0; z < UNR; z++)
-                        if (p0 + z * gstride < mc)
-                            accumulate<VEC, 1, std::is_same_v<XT, __nv_bfloat16>>(v[z], s, c, qs, qc, cb, sub, L, nv);
+                        for (int z = 0; z < UNR; z++) {
+                            const int p = p0 + z * gstride;
+                            if (p < mc && col < nv)
+                                v[z][0] = load_vec<VEC>(X + (int64_t)s_mem[p] * ld + (int64_t)col * VEC);
+                        }
+#pragma unroll
+                        for (int z = 0; z < UNR; z++)
+                            if (p0 + z * gstride < mc)
+                                accumulate<VEC, 1, std::is_same_v<XT, __nv_bfloat16>>(v[z], s, c, qs, qc, cb, sub, L, nv);
+                    }
                 }
             }
-        }
-        if constexpr (PIPE)
-            __syncthreads();  // every warp is done with the ring before the partial sums overwrite it
-        sq_lane = df_add(sq_lane, chains_sum(qs, qc));
-        // combine the G groups of the warp, then the warps of the block, in a fixed order
+            if constexpr (PIPE)
+                __syncthreads();  // every warp is done with the ring before the partial sums overwrite it
+            sq_lane = df_add(sq_lane, chains_sum(qs, qc));
+            // combine the G groups of the warp, then the warps of the block, in a fixed order
 #pragma unroll
-        for (int q = 0; q < VEC; q++) {
-            DF S = fast_two_sum(s[0][q], -c[0][q]);  // the Kahan sum s - c, exactly
-            for (int o = L; o < 32; o <<= 1)
-                S = df_add(S, df_shfl_xor(S, o));
-            if (g == 0)
-                s_part[w][sub * VEC + q] = make_float2(S.hi, S.lo);
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < L * VEC; e += UP_WARPS * 32) {
-            const int colv = cb + e / VEC;  // entry e: component e % VEC of column vector colv
-            if (colv < nv) {
-                DF S = {s_part[0][e].x, s_part[0][e].y};
-                for (int ww = 1; ww < UP_WARPS; ww++)
-                    S = df_add(S, DF{s_part[ww][e].x, s_part[ww][e].y});
-                C[(int64_t)r * d + (int64_t)colv * VEC + (e % VEC)] = df_div(S, mf, inv_m);
-                dd_lane = df_add(dd_lane, df_sqr(S));
+            for (int q = 0; q < VEC; q++) {
+                DF S = fast_two_sum(s[0][q], -c[0][q]);  // the Kahan sum s - c, exactly
+                for (int o = L; o < 32; o <<= 1)
+                    S = df_add(S, df_shfl_xor(S, o));
+                if (g == 0)
+                    s_part[w][sub * VEC + q] = make_float2(S.hi, S.lo);
             }
+            __syncthreads();
+            for (int e = threadIdx.x; e < L * VEC; e += UP_WARPS * 32) {
+                const int colv = cb + e / VEC;  // entry e: component e % VEC of column vector colv
+                if (colv < nv) {
+                    DF S = {s_part[0][e].x, s_part[0][e].y};
+                    for (int ww = 1; ww < UP_WARPS; ww++)
+                        S = df_add(S, DF{s_part[ww][e].x, s_part[ww][e].y});
+                    C[(int64_t)r * d + (int64_t)colv * VEC + (e % VEC)] = df_div(S, mf, inv_m);
+                    dd_lane = df_add(dd_lane, df_sqr(S));
+                }
+            }
+            __syncthreads();
+        }
+        // sum of ||x||^2 over all lanes, sum of D_t^2 over the threads that wrote means
+        for (int o = 1; o < 32; o <<= 1) {
+            sq_lane = df_add(sq_lane, df_shfl_xor(sq_lane, o));
+            dd_lane = df_add(dd_lane, df_shfl_xor(dd_lane, o));
+        }
+        if (lane == 0) {
+            s_sq[w] = make_float2(sq_lane.hi, sq_lane.lo);
+            s_dd[w] = make_float2(dd_lane.hi, dd_lane.lo);
         }
         __syncthreads();
-    }
-    // sum of ||x||^2 over all lanes, sum of D_t^2 over the threads that wrote means
-    for (int o = 1; o < 32; o <<= 1) {
-        sq_lane = df_add(sq_lane, df_shfl_xor(sq_lane, o));
-        dd_lane = df_add(dd_lane, df_shfl_xor(dd_lane, o));
-    }
-    if (lane == 0) {
-        s_sq[w] = make_float2(sq_lane.hi, sq_lane.lo);
-        s_dd[w] = make_float2(dd_lane.hi, dd_lane.lo);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        DF sq = {s_sq[0].x, s_sq[0].y}, dd = {s_dd[0].x, s_dd[0].y};
-        for (int ww = 1; ww < UP_WARPS; ww++) {
-            sq = df_add(sq, DF{s_sq[ww].x, s_sq[ww].y});
-            dd = df_add(dd, DF{s_dd[ww].x, s_dd[ww].y});
+        if (threadIdx.x == 0) {
+            DF sq = {s_sq[0].x, s_sq[0].y}, dd = {s_dd[0].x, s_dd[0].y};
+            for (int ww = 1; ww < UP_WARPS; ww++) {
+                sq = df_add(sq, DF{s_sq[ww].x, s_sq[ww].y});
+                dd = df_add(dd, DF{s_dd[ww].x, s_dd[ww].y});
+            }
+            if (nb > 1)
+                st_rank(&s_terms[turn][rank], 0, make_float4(sq.hi, sq.lo, dd.hi, dd.lo));
+            else
+                s_terms[0][0] = make_float4(sq.hi, sq.lo, dd.hi, dd.lo);
         }
         if (nb > 1)
-            st_rank(&s_terms[turn][rank], 0, make_float4(sq.hi, sq.lo, dd.hi, dd.lo));
-        else
-            s_terms[0][0] = make_float4(sq.hi, sq.lo, dd.hi, dd.lo);
-    }
-    if (nb > 1)
-        cluster_barrier();  // the next cluster's terms go to the other slots, the one after that waits for its barrier
-    if (threadIdx.x == 0 && rank == 0) {
-        const float4 *terms = s_terms[nb > 1 ? turn : 0];
-        DF sq = {terms[0].x, terms[0].y}, dd = {terms[0].z, terms[0].w};
-        for (int b = 1; b < nb; b++) {
-            sq = df_add(sq, DF{terms[b].x, terms[b].y});
-            dd = df_add(dd, DF{terms[b].z, terms[b].w});
+            cluster_barrier();  // the next cluster's terms go to the other slots, the one after that waits for its barrier
+        if (threadIdx.x == 0 && rank == 0) {
+            const float4 *terms = s_terms[nb > 1 ? turn : 0];
+            DF sq = {terms[0].x, terms[0].y}, dd = {terms[0].z, terms[0].w};
+            for (int b = 1; b < nb; b++) {
+                sq = df_add(sq, DF{terms[b].x, terms[b].y});
+                dd = df_add(dd, DF{terms[b].z, terms[b].w});
+            }
+            const double cr = df_to_double(sq) - df_to_double(dd) / (double)m;
+            contrib[r] = cr;
+            if (!isfinite(cr))  // a non-finite sample in the cluster (Inf or NaN spreads into its sums)
+                flag_error(st, GK_ERR_NUMERIC, (unsigned)r);
         }
-        const double cr = df_to_double(sq) - df_to_double(dd) / (double)m;
-        contrib[r] = cr;
-        if (!isfinite(cr))  // a non-finite sample in the cluster (Inf or NaN spreads into its sums)
-            flag_error(st, GK_ERR_NUMERIC, (unsigned)r);
-    }
-    turn ^= 1;
-    __syncthreads();  // s_sq / s_dd are read above before the next cluster writes them
+        turn ^= 1;
+        __syncthreads();  // s_sq / s_dd are read above before the next cluster writes them
     };
     // a thread per cluster finds the large ones, `chunk` of this block's clusters c, c + stride, ... at a time (large ones
     // often follow one another: 300k x 200 took 195 us with neighbouring clusters on one block)
@@ -779,13 +780,12 @@ static cudaError_t update_t(const XT *X, int64_t n, int64_t d, int64_t ld, const
     }
     // the block kernel walks the clusters grid-stride on a one-wave grid (at most k blocks)
     int bg = 0;
-    if ((e = resident_grid(reinterpret_cast<const void *>(vec4 ? (need <= 1 ? (const void *)k_update<4, 1, PIPE, XT>
-                                                                                         : (const void *)k_update<4, 8, PIPE, XT>)
-                                                                 : (need <= 1 ? (const void *)k_update<1, 1, false, XT>
-                                                                             : need <= 2 ? (const void *)k_update<1, 2, false, XT>
-                                                                             : need <= 4 ? (const void *)k_update<1, 4, false, XT>
-                                                                                         : (const void *)k_update<1, 8, false, XT>)),
-                           UP_WARPS * 32, 0, &bg)) != cudaSuccess)
+    const void *block = vec4 ? (need <= 1 ? (const void *)k_update<4, 1, PIPE, XT> : (const void *)k_update<4, 8, PIPE, XT>)
+                             : (need <= 1   ? (const void *)k_update<1, 1, false, XT>
+                                : need <= 2 ? (const void *)k_update<1, 2, false, XT>
+                                : need <= 4 ? (const void *)k_update<1, 4, false, XT>
+                                            : (const void *)k_update<1, 8, false, XT>);
+    if ((e = resident_grid(block, UP_WARPS * 32, 0, &bg)) != cudaSuccess)
         return e;
     // one block per cluster while the clusters are mostly the block kernel's (the hardware then hands clusters
     // of uneven sizes to SMs as blocks finish); where most clusters are small, a one-wave grid walks the few
