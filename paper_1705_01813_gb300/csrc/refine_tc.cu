@@ -29,7 +29,10 @@
 // with u = 2^-8, a term that vanishes when every staged coordinate is a BF16
 // value already, as for BF16 samples; plus FP32 accumulation and combination),
 // marked (recorded by its column in the run instead of its id), and the run is
-// flagged.
+// flagged.  A distance that is no number (a sample with NaN or infinity in the
+// run; in FP32 the run's first member, the centre, spoils all of it) passes, as
+// every distance does in a row whose kappa-th one is none: the recompute and
+// the merge decide, and the graph is that of the FP32 path.
 //
 // k_refine_exact, over the listed inexact runs: the run's FP32 rows are staged in
 // shared memory once and every marked pair is recomputed exactly in the order
@@ -210,7 +213,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
     const int my_prev = prev && gi_row >= 0 ? prev[gi_row] : -1;
     rpr[tid] = my_prev;
     srt[tid] = tid < sz ? sqrtf(pnrm[p0 + tid]) : 0.f;
-    nrm[tid] = tid < sz ? pnrm[p0 + tid] : __int_as_float(0x7f800000);  // no distance to a column past the run passes
+    nrm[tid] = tid < sz ? pnrm[p0 + tid] : 1e37f;  // a column past the run (rid -1) seldom passes
     float thd = 0.f;
     int thi = 0;
     if (gi_row >= 0) {
@@ -296,7 +299,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
                     const int jid = rid[j];
                     // exact: the whole key decides; a marked pair records the run column of j (k_refine_exact
                     // writes the id back)
-                    if (j != row && jid >= 0 && (tag || key_less(d2, jid, thd, thi))) {
+                    if (j != row && jid >= 0 && (tag || !key_less(thd, thi, d2, jid))) {
                         bid[buf_slot(row, m)] = tag ? (int)(TC_RERANK | (unsigned)j) : jid;
                         bdv[buf_slot(row, m)] = d2;
                         m++;
@@ -312,7 +315,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
 #pragma unroll
                         for (int e = 0; e < 4; e++) {
                             const float d2 = (n_i + nn[e]) - 2.f * g[q4 + e];
-                            if (d2 <= thd && pp[e] != skip)
+                            if (!(d2 > thd) && pp[e] != skip)
                                 keep(c0 + q4 + e, d2, 0u);
                         }
                     }
@@ -328,7 +331,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
                         for (int e = 0; e < 4; e++) {
                             const float d2 = (n_i + nn[e]) - 2.f * g[q4 + e];
                             const float err = c1 * ss[e] + c2 * (n_i + nn[e]);
-                            if (d2 - err <= thd && pp[e] != skip)
+                            if (!(d2 - err > thd) && pp[e] != skip)
                                 keep(c0 + q4 + e, d2, TC_RERANK);
                         }
                     }
