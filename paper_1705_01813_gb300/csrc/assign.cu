@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV == 1 ? AS_ROWS_PER_SM : NV =
 // winner alone), with the lane partials and summation tree of k_assign_rows,
 // so the winner and its distance are that kernel's bit for bit.  The samples
 // (FP32 or BF16, widened exactly) enter both passes unrounded: the bound covers
-// the centroids' rounding alone.
+// the centroids' rounding alone.  A bound that is no number keeps its candidate.
 template <int NV, typename XT, int GS, bool LISTS>
 __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV == 4 ? 4 : 3)) k_assign_rows_scr(
     const XT *__restrict__ X, int64_t n, int d, int64_t ld, const int32_t *__restrict__ G, int kappa,
@@ -578,7 +578,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV 
         // pass 2: exact FP32 distances of the candidates that may be the minimum
         for (int g0 = 0; g0 < u; g0 += 32) {
             const int cnt = min(32, u - g0);
-            unsigned sel = __ballot_sync(FULL_MASK, lane < cnt && lov[g0 + lane] <= best_up);
+            unsigned sel = __ballot_sync(FULL_MASK, lane < cnt && !(lov[g0 + lane] > best_up));
             while (sel) {
                 const int c = __ffs(sel) - 1;
                 sel &= sel - 1;
@@ -1013,7 +1013,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign_rows_bf(const float *_
     #pragma unroll 1
             for (int g0 = 0; g0 < u; g0 += 32) {
                 const int cnt = min(32, u - g0);
-                unsigned sel = __ballot_sync(FULL_MASK, lane < cnt && lov[g0 + lane] <= best_up);
+                unsigned sel = __ballot_sync(FULL_MASK, lane < cnt && !(lov[g0 + lane] > best_up));
                 while (sel) {
                     const int c = __ffs(sel) - 1;
                     sel &= sel - 1;

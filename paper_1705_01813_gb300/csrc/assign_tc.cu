@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_assign_tc(const float *__restric
                         const float e = c1 * xc + c2 * (x2 + c2n) + gp * fabsf(approx) + 1e-30f;
                         const float lo_v = approx - e, up_v = approx + e;
                         best_up = fminf(best_up, up_v);
-                        if (lo_v <= best_up) {
+                        if (!(lo_v > best_up)) {  // a bound that is no number keeps its candidate
                             if (nsel < AT_SEL) {
                                 sel_col[nsel] = c0 + s0 + q;
                                 sel_lo[nsel] = lo_v;
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_assign_tc(const float *__restric
                                 int kept = 0;
 #pragma unroll
                                 for (int z = 0; z < AT_SEL; z++)
-                                    if (sel_lo[z] <= best_up) {
+                                    if (!(sel_lo[z] > best_up)) {
                                         sel_col[kept] = sel_col[z];
                                         sel_lo[kept] = sel_lo[z];
                                         kept++;
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_assign_tc(const float *__restric
             if (!sel_over) {
 #pragma unroll
                 for (int z = 0; z < AT_SEL; z++)
-                    if (z < nsel && sel_lo[z] <= best_up)
+                    if (z < nsel && !(sel_lo[z] > best_up))
                         out[cnt++] = ulab[sel_col[z]];
             }
             sel_n[i] = sel_over ? -1 : cnt;
