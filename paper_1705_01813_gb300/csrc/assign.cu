@@ -501,7 +501,11 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV == 1 ? AS_ROWS_PER_SM : NV =
 // winner alone), with the lane partials and summation tree of k_assign_rows,
 // so the winner and its distance are that kernel's bit for bit.  The samples
 // (FP32 or BF16, widened exactly) enter both passes unrounded: the bound covers
-// the centroids' rounding alone.  A bound that is no number keeps its candidate.
+// the centroids' rounding alone.  SCR_TINY covers what the sums lose below
+// FP32's normal range (at most 2^-150 a term); a bound that is no number keeps
+// its candidate.
+constexpr float SCR_TINY = 1e-41f;
+
 template <int NV, typename XT, int GS, bool LISTS>
 __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV == 4 ? 4 : 3)) k_assign_rows_scr(
     const XT *__restrict__ X, int64_t n, int d, int64_t ld, const int32_t *__restrict__ G, int kappa,
@@ -566,7 +570,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV 
             const int cl = lane / (32 / GS);
             const float dl = __ldg(delta + qlist[g0 + cl]);
             const float sq = sqrtf(fmaxf(dt, 0.f));
-            const float e = 1.01f * (dl * (2.f * sq + dl) + gam * (2.f * dt + dl * (2.f * sq + dl)));
+            const float e = fmaf(1.01f, dl * (2.f * sq + dl) + gam * (2.f * dt + dl * (2.f * sq + dl)), SCR_TINY);
             if (lane % (32 / GS) == 0)
                 lov[g0 + cl] = dt - e;
             best_up = fminf(best_up, dt + e);
@@ -998,7 +1002,8 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign_rows_bf(const float *_
                 if (lane < cnt) {
                     const float dl = delta[qlist[g0 + lane]];
                     const float sq = sqrtf(fmaxf(dt, 0.f));
-                    const float e = 1.01f * (dl * (2.f * sq + dl) + gam * (2.f * dt + dl * (2.f * sq + dl)));
+                    const float e =
+                        fmaf(1.01f, dl * (2.f * sq + dl) + gam * (2.f * dt + dl * (2.f * sq + dl)), SCR_TINY);
                     lov[g0 + lane] = dt - e;
                     best_up = fminf(best_up, dt + e);
                 }

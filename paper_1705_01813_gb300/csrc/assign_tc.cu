@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_assign_tc(const float *__restric
                 xn[row] = part;
         }
         __syncthreads();
-        const float x2 = xn[tid];
+        const float x2 = xn[tid], sx = sqrtf(x2);
         const float u = 1.0f / 256.0f;
         const float c1 = 1.05f * (4.f * u + 2.f * u * u + 4.f * (d + 2) * 1.1920929e-7f);
         const float c2 = 1.05f * 4.f * (d + 2) * 1.1920929e-7f;
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_assign_tc(const float *__restric
                         m &= m - 1;
                         const float c2n = cn[s0 + q];
                         const float approx = (x2 + c2n) - 2.f * vrow[q];
-                        const float xc = sqrtf(x2 * c2n);
+                        const float xc = sx * sqrtf(c2n);  // |x|^2 |C|^2 might leave FP32's range
                         const float e = c1 * xc + c2 * (x2 + c2n) + gp * fabsf(approx) + 1e-30f;
                         const float lo_v = approx - e, up_v = approx + e;
                         best_up = fminf(best_up, up_v);

@@ -283,7 +283,8 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
     const float rnd = (rf & 2) != 0 ? 4.f * u + 2.f * u * u : 0.f;  // BF16 rounding of the operands
     // accumulation of G: exact products, each 16-deep step aligned to its largest term and truncated (an
     // error below 16 units of 2^-23 of the step's terms), over d / 16 steps, doubled by the factor 2 of
-    // 2 G and once more as a margin.  The factor 1.02 covers the rounding of the bound's own terms (|x_t| |x_j| is
+    // 2 G and once more as a margin; 6e-36 for what products and sums lose below FP32's normal range (at most 2^-126
+    // a term).  The factor 1.02 covers the rounding of the bound's own terms (|x_t| |x_j| is
     // a product of two rounded square roots).
     const float c1 = 1.02f * (rnd + 8.f * (d + 2) * 5.9604645e-8f) * s_i;
     const float c2 = 1.02f * (d + 8) * 1.1920929e-7f;
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_refine_gram(const __grid_constan
 #pragma unroll
                         for (int e = 0; e < 4; e++) {
                             const float d2 = (n_i + nn[e]) - 2.f * g[q4 + e];
-                            const float err = c1 * ss[e] + c2 * (n_i + nn[e]);
+                            const float err = fmaf(c1, ss[e], fmaf(c2, n_i + nn[e], 6e-36f));
                             if (!(d2 - err > thd) && pp[e] != skip)
                                 keep(c0 + q4 + e, d2, TC_RERANK);
                         }
