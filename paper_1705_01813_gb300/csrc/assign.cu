@@ -510,7 +510,8 @@ template <int NV, typename XT, int GS, bool LISTS>
 __global__ void __launch_bounds__(AS_WARPS * 32, NV <= 2 ? AS_ROWS_PER_SM : (NV == 4 ? 4 : 3)) k_assign_rows_scr(
     const XT *__restrict__ X, int64_t n, int d, int64_t ld, const int32_t *__restrict__ G, int kappa,
     const float *__restrict__ C, const void *__restrict__ Cs, const float *__restrict__ delta, int k,
-    const int32_t *__restrict__ Lin, int32_t *__restrict__ Lout, float *__restrict__ best_out, DevStatus *st, const Track trk, const int32_t *__restrict__ todo)
+    const int32_t *__restrict__ Lin, int32_t *__restrict__ Lout, float *__restrict__ best_out, DevStatus *st,
+    const Track trk, const int32_t *__restrict__ todo)
 {
     __shared__ __align__(16) int s_q[AS_WARPS][AS_QROW];
     __shared__ __align__(16) int s_h[AS_WARPS][AS_HASH];
@@ -985,11 +986,11 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign_rows_bf(const float *_
             // pass 1: BF16 distances of every candidate (lane l holds candidate g0 + l of each group)
             float *lov = s_lo[w];
             float best_up = __int_as_float(0x7f800000);
-    #pragma unroll 1
+#pragma unroll 1
             for (int g0 = 0; g0 < u; g0 += 32) {
                 const int cnt = min(32, u - g0);
                 float part[32];
-    #pragma unroll
+#pragma unroll
                 for (int c = 0; c < 32; c++) {
                     float acc = 0.f;
                     if (c < cnt) {
@@ -1008,14 +1009,14 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign_rows_bf(const float *_
                     best_up = fminf(best_up, dt + e);
                 }
             }
-    #pragma unroll
+#pragma unroll
             for (int o = 16; o > 0; o >>= 1)
                 best_up = fminf(best_up, __shfl_xor_sync(FULL_MASK, best_up, o));
             __syncwarp();
             // pass 2: FP32 distances of the candidates that may be the minimum, one at a
             // time; the xor butterfly groups the lane partials as transpose_reduce32 does,
             // so each total has the bits of the FP32 kernel
-    #pragma unroll 1
+#pragma unroll 1
             for (int g0 = 0; g0 < u; g0 += 32) {
                 const int cnt = min(32, u - g0);
                 unsigned sel = __ballot_sync(FULL_MASK, lane < cnt && !(lov[g0 + lane] > best_up));
@@ -1025,7 +1026,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_assign_rows_bf(const float *_
                     const int r = qlist[g0 + c];
                     const float4 *row = C4 + (int64_t)r * d4;
                     float tot = lane_partial<NV>(xv, d4, [&](int col) { return __ldg(row + col); });
-    #pragma unroll
+#pragma unroll
                     for (int o = 16; o > 0; o >>= 1)
                         tot += __shfl_xor_sync(FULL_MASK, tot, o);
                     if (key_less(tot, r, bd, br)) {

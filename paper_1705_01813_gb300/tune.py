@@ -100,7 +100,7 @@ def tune_precision(X: torch.Tensor, g_idx: torch.Tensor, g_dist: torch.Tensor, l
              for p in levels}
     best = min(levels, key=lambda p: (score[p], p))
     res = {"precision": best | (group_width[best] << 8), "level": best, "group_width": group_width[best],
-           "assign_ms": assign_ms, "fit_ms": fit_ms, "group_width_by_level": group_width, "refine_ms": refine_ms, "score_ms": score,
-           "key": list(key)}
+           "assign_ms": assign_ms, "fit_ms": fit_ms, "group_width_by_level": group_width, "refine_ms": refine_ms,
+           "score_ms": score, "key": list(key)}
     _CACHE[key] = res
     return res
