@@ -344,7 +344,7 @@ GK_API int gk_update_step_noalloc(const float *X, int64_t n, int64_t d, int64_t 
  * Sec. 5, take 10 GB this way.)  At precision 2 the assignment screens its
  * candidates against BF16 centroids with the samples unrounded, as for FP32
  * samples.  The tensor-core screening (precision 3) reads FP32 samples only:
- * with BF16 samples the assignment takes precision 0, 1 or 2
+ * with BF16 samples the assignment takes precision 0, 1, 2 or 4
  * (gk_assign_step_bf16, gk_kmeans_fit_bf16, and p->precision of
  * gk_build_knn_graph_bf16), else GK_ERR_INVALID.
  */

@@ -73,7 +73,7 @@ int check_precision(int32_t precision, bool bf16)
                     "4: int8 screening, each + exact recompute; bits 8-15: 0, 4 or 8 candidates per group)",
                     precision);
     if (bf16 && level == 3)
-        return fail(GK_ERR_INVALID, "BF16 samples: precision must be 0, 1 or 2 (3 screens on FP32 samples)");
+        return fail(GK_ERR_INVALID, "BF16 samples: precision must be 0, 1, 2 or 4 (3 screens on FP32 samples)");
     return GK_OK;
 }
 
