@@ -633,7 +633,8 @@ def run_gpu(args):
                    "parallelism": f"replicas x{world}"},
         "fit_s": step_s,
         "precision": {0: "fp32 throughout",
-                      1: "bf16 tcgen05 gram in the refinement with exact fp32 recompute inside its error bound",
+                      1: "bf16 tcgen05 gram in the refinement with exact fp32 recompute inside its error bound"
+                         if 64 <= w.d <= 128 else "fp32 tiles in the refinement (its tensor-core path: 64 <= d <= 128)",
                       2: "1 plus bf16 screening of assignment candidates (simt) with exact fp32 recompute",
                       3: "1 plus bf16 tcgen05 screening of assignment candidates with exact fp32 recompute",
                       4: "1 plus int8 (per-row scale) screening of assignment candidates (simt) with exact fp32 "
@@ -901,7 +902,7 @@ def time_tree(gkm, torch, X, w, iters=2, reps=3):
     return {"ms": round(ms, 3), "k": w.k, "iters": iters, "complete_depths": depths,
             "x_read_GB": round(x_bytes / 1e9, 3), "x_read_GBs": round(x_bytes / ms / 1e6, 1),
             "device_status": status,
-            "note": "Alg. 1 initial partition (equal halves, Lloyd 2-means per bisection, FP64 sums); "
+            "note": "Alg. 1 initial partition (equal halves, Lloyd 2-means per bisection, FP64 means); "
                     "not part of the timed step"}
 
 
